@@ -172,12 +172,18 @@ r3_status_t score_simt(r3_gp* gp, const float* Xcand, long long m, float* mu, fl
 struct GuardBuffers {
     float* err_mu;      // [batch][m]
     float* err_q;       // [batch][m]
-    int* count;         // [batch]
+    int* list;          // [batch][m] candidates to recompute
+    int* count;         // [batch] entries of the list
+    int* total;         // [batch] candidates flagged
     unsigned* maxbits;  // [batch] bit pattern of the largest EI
+    unsigned* done;     // [batch] slices selected
+    unsigned* barrier;  // grid barrier of the guard kernel
+    double *ks, *qpart, *mupart;   // the rescue's slab
 };
 size_t guard_workspace_bytes(const r3_gp* gp, long long m);
-// Zeroes the pool's maximum EI and the rescue counters; the engines call it before their first scoring kernel.
-r3_status_t guard_begin(r3_gp* gp, const GuardBuffers& b, cudaStream_t stream);
+// The pool's maximum EI and the guard kernel's counters start at zero: the engines' first kernel of a pool clears this
+// many ints from GuardBuffers::count on.
+int guard_zero_ints(const r3_gp* gp);
 // Key storage the guard kernel needs to leave the first level of a top-k of k (see TopkRequest).
 size_t guard_topk_workspace_bytes(int batch, long long m, int k);
 GuardBuffers guard_carve(const r3_gp* gp, long long m, void* ws);

@@ -1,20 +1,37 @@
-// Accuracy guard, FP64 rescue pass and the first level of the pool's top-k, in one kernel.
+// What follows a pool's scoring, in one cooperatively launched kernel: the pool's largest EI, the accuracy guard,
+// the FP64 rescue pass and the selection.
 //
 // The scoring engines work at FP32 level.  That is enough for almost every candidate of a
 // well-conditioned GP, but not where the posterior variance sf2 - |W k*|^2 is a small difference of
 // two numbers close to sf2 (a candidate on top of an observation), nor where mu = k*.alpha cancels
 // heavily (an ill-conditioned history with large weights).  Each engine therefore writes, next to
-// its results, an estimate of its own rounding error in mu and in q, and raises the pool's largest EI
-// (the EI tolerance is relative to it) with one atomic maximum per warp.  Once the whole pool is scored,
-// guard_kernel gives every block a slice of candidates, and the block
-//   flags    the candidates of its slice whose estimated error exceeds half of the accuracy contract
-//            (1e-4 relative on mu and sigma with absolute floors, 1e-5 max(EI) on EI),
+// its results, an estimate of its own rounding error in mu and in q.  Once the whole pool is scored, guard_kernel
+//   finds    the pool's largest EI (the EI tolerance is relative to it), unless the engine already has,
+//   flags    the candidates whose estimated error exceeds half of the accuracy contract
+//            (1e-4 relative on mu and sigma with absolute floors, 1e-5 max(EI) on EI) in a list per GP,
 //   rescues  them: recomputes them from the raw inputs entirely in FP64 -- direct-difference distances with
 //            FP64 reciprocal lengthscales, FP64 weights and the FP64 inverse factor -- and overwrites
 //            their mu, sigma and EI,
-//   selects  (when the call asked for a top-k) the k largest final EI of its slice as 64-bit keys: the first
-//            level of the selection, taken while the slice's values are at hand; r3_topk.cu finishes it.
+//   selects  (when the call asked for a top-k) the k largest final EI of every slice of the pool as 64-bit keys; when
+//            a GP's slices leave at most 4096 keys the block that finishes its last slice writes the answer,
+//            otherwise r3_topk.cu goes on from the keys.
+//
+// The rescue is a matrix product, V = W Ks with Ks the FP64 cross-covariance of all listed candidates, of which only
+// the column sums of squares are kept.  Blocks compute Ks into a slab of the workspace, meet at a grid barrier, and
+// share out (64 rows of W) x (64 candidates) tiles that run on the FP64 tensor path.  Few listed candidates (less
+// than two tiles per block) get 16 x 16 tiles instead, whose reductions the block's eight warps split, so that W is
+// read once by the whole GPU.  With at most 128 observations a block recomputes the first 16 it flags in a slice by
+// itself, which saves a small call the barriers (64 observations, 4096 candidates: 27.7 us to 19.8 us; with 256 the rows
+// of W cost one block more than the barriers: 45.8 us against 32.9 us).
+// Bound: the FP64 rate for long lists, one read of W otherwise.  Measured, before (the block that met a flagged candidate
+// recomputed it alone, four at a time) and now: 65,536 candidates at n = 4096, most of them listed, 300-600 ms and
+// 36 ms (31 TFLOP/s of FP64); 2222 candidates at n = 701 1.50 ms and 0.14 ms; one pool of 262,144 with four listed
+// (n = 256) 54 us and 33 us; 64 pools of 65,536 with three listed (n = 512) 318 us (with the kernel that found the
+// largest EI) and 201 us.
+#include <algorithm>
+
 #include "r3_epilogue.cuh"
+#include "r3_f64.cuh"
 #include "r3_internal.cuh"
 #include "r3_topk.cuh"
 
@@ -22,280 +39,626 @@ namespace r3 {
 
 namespace {
 
-constexpr int RESCUE_GROUP = 4;   // candidates recomputed together (they share every read of W)
+constexpr int kThreads = 256;
+constexpr int kTile = 64;        // rows of W and candidates of a tile of the long-list form
+constexpr int kSmallTile = 16;   // of the short-list form
+constexpr int kStages = 3;       // 16-deep operand stages in flight
+constexpr size_t kSlabBytes = 64ull << 20;   // FP64 cross-covariances in flight: they stay in L2 beside W
+constexpr int kOwnMaxN = 128;                // histories whose flagged candidates the flagging block recomputes itself
+constexpr size_t kOwnKs = 12 * 1024;         // byte offset of its k* behind the staged coordinates (10.9 KB)
+constexpr size_t kMaxSmem = 80 * 1024;       // operand stages (60 KB) and the tile prefix of 4096 GPs
+constexpr int kFinishKeys = 4096;            // a GP whose slices leave at most this many keys is finished in the kernel
 
 struct GuardArgs {
     const float *X, *ell, *sf2v, *bestv, *yabsv, *Xcand;
     const double *alpha64, *W64;
-    int n, d, npad;
+    int batch, n, d, npad;
     long long m;
-    int slice;                    // candidates per block, a power of two in [32, 4096]
+    int slice;                    // candidates per slice, a power of two in [32, 4096]
+    int slices_per_gp;
     float *mu, *sigma, *ei;
     const float *err_mu, *err_q;
-    const unsigned* maxbits;      // [batch] bit pattern of the pool's largest EI
-    int* count;                   // [batch] candidates recomputed (diagnostics)
-    int* status;                  // the handle's status words (index checks of the bounds-checking build)
-    int k, K2;                    // top-k request (k = 0: none); K2 = min(k, slice): keys a block selects
+    int* list;                    // [batch][m] flagged candidates of each GP
+    unsigned* maxbits;            // [batch] bit pattern of the pool's largest EI
+    int* count;                   // [batch] candidates in the list
+    int* total;                   // [batch] candidates flagged (and recomputed)
+    int* rescued_h;               // pinned host [64]: the same for the caller
+    unsigned* done;               // [batch] slices selected so far
+    unsigned* barrier;            // grid barrier
+    int* status;                  // the handle's status words
+    bool have_max;
+    double *ks, *qpart, *mupart;  // slab: [slab][npad], [slab][npad / 16], [slab][ceil(npad / 64)]
+    int slab;                     // candidates per slab, a multiple of 64
+    int k, K2;                    // top-k request (k = 0: none); K2 = min(k, slice): keys a slice yields
     unsigned select_offset;       // byte offset of the selection's scratch in the dynamic shared memory
-    unsigned long long* keys;     // [batch][blocks][k]
+    unsigned pref_offset;         // byte offset of the tile prefix
+    unsigned long long* keys;     // [batch][slices_per_gp][k]
+    bool finish;                  // the last slice of a GP writes the answer
+    int* idx;
+    float* val;
 };
 
-// The pool's largest EI for an engine whose scoring kernel does not raise it itself (the tensor-core kernel's
-// registers are spoken for).
-__global__ void max_ei_kernel(const float* __restrict__ ei, long long m, unsigned* __restrict__ maxbits)
+// k* and the partial means of (CT candidates) x (64 observations): 256 threads, CT / 16 candidates x 4 observations
+// each.  store(c, k, k*) for every candidate c of the tile and every k < npad of the block (zero beyond n and beyond the
+// listed candidates), mean(c, sum) once per candidate.
+template <int CT, class List, class Store, class Mean>
+__device__ __forceinline__ void kstar_tile(const GuardArgs& a, int g, List list, int in_tile, int kb, unsigned char* smem,
+                                           Store store, Mean mean)
 {
-    const int g = blockIdx.y;
-    const float* e = ei + (size_t)g * m;
-    float v = 0.f;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < m; i += (long long)gridDim.x * blockDim.x)
-        v = fmaxf(v, e[i]);  // EI >= 0; NaN is ignored by fmaxf
-    for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
-    if ((threadIdx.x & 31) == 0) atomicMax(&maxbits[g], __float_as_uint(v));  // order-preserving for v >= 0
-}
-
-template <int R>
-__global__ void __launch_bounds__(256) guard_kernel(const GuardArgs a)
-{
-    extern __shared__ double smem[];
-    // rescue: ks [R][npad], zs [R][d], ls [d]; afterwards the same bytes hold the slice's keys
-    double* ks = smem;
-    double* zs = smem + (size_t)R * a.npad;
-    double* ls = zs + (size_t)R * a.d;   // [d] reciprocal lengthscales
-    __shared__ double red[2][R][8];
-    __shared__ int nflag_s;
-    const int g = blockIdx.y;
-    const int t = threadIdx.x, lane = t % 32, warp = t / 32;
-    const long long m = a.m;
-    const long long c_begin = (long long)blockIdx.x * a.slice;
-    const long long c_end = c_begin + a.slice < m ? c_begin + a.slice : m;
-    // the list of flagged candidates sits after the larger of the two uses of the dynamic region
-    size_t region = sizeof(double) * ((size_t)R * a.npad + (size_t)R * a.d + a.d);
-    if (region < sizeof(unsigned long long) * (size_t)a.slice) region = sizeof(unsigned long long) * (size_t)a.slice;
-    int* list = reinterpret_cast<int*>(reinterpret_cast<char*>(smem) + region);
-    if (t == 0) nflag_s = 0;
-    __syncthreads();
-
-    // ---- flag
-    {
-        const float sf2 = a.sf2v[g], best = a.bestv[g];
-        const float tol_ei = 1e-5f * __uint_as_float(a.maxbits[g]);
-        const float mu_floor = 1e-6f * a.yabsv[g], sd_floor = 1e-6f * sqrtf(sf2);
-        for (long long i = c_begin + t; i < c_end; i += 256) {
-            const size_t f = (size_t)g * m + i;
-            const float mu_i = a.mu[f], sd = a.sigma[f], dmu = a.err_mu[f], dq = a.err_q[f];
-            // d sigma = dq / (2 sigma); with sigma -> 0 every rounding error in q matters
-            const float dsd = (sd > 0.f) ? dq / (2.f * sd) : ((dq > 0.f) ? INFINITY : 0.f);
-            const float tol_mu = 1e-4f * fabsf(mu_i) + mu_floor;
-            const float tol_sd = 1e-4f * sd + sd_floor;
-            bool flag = !(dmu <= 0.5f * tol_mu) || !(dsd <= 0.5f * tol_sd);
-            // EI: dEI = Phi(z) dmu + phi(z) dsigma against 1e-5 of the pool's largest EI
-            const float z = (sd > 0.f) ? (best - mu_i) / sd : 0.f;
-            const float Phi = 0.5f * erfcf(-z * 0.70710678f);
-            const float phi = expf(-0.5f * z * z) * 0.39894228f;
-            if (isfinite(dsd)) flag |= !(Phi * dmu + phi * dsd <= 0.5f * tol_ei);
-            flag |= !(sd * sd >= 1e-3f * sf2);   // deep cancellation: do not trust the estimates either
-            if (flag) list[R3_IDX(atomicAdd(&nflag_s, 1), a.slice, a.status)] = (int)i;
+    constexpr int U = CT / 16;
+    float* zs = reinterpret_cast<float*>(smem);   // [CT][33]
+    float* xs = zs + CT * 33;                     // [64][33]
+    double* il = reinterpret_cast<double*>(xs + 64 * 33 + (CT * 33) % 2);   // [32] reciprocal lengthscales
+    const int t = threadIdx.x, tx = t % 16, ty = t / 16;
+    const int n = a.n, d = a.d, k0 = kb * 64;
+    double r2[U][4] = {};
+    for (int c0 = 0; c0 < d; c0 += 32) {
+        __syncthreads();
+        for (int e = t; e < CT * 32; e += kThreads) {
+            const int r = e / 32, c = e % 32;
+            float z = 0.f;
+            if (r < in_tile && c0 + c < d) {
+                const int cand = list(r);
+                z = a.Xcand[(size_t)R3_IDX((long long)g * a.m + cand, (long long)a.batch * a.m, a.status) * d + c0 + c];
+            }
+            zs[r * 33 + c] = z;
+        }
+        for (int e = t; e < 64 * 32; e += kThreads) {
+            const int r = e / 32, c = e % 32;
+            xs[r * 33 + c] = (k0 + r < n && c0 + c < d) ? a.X[((size_t)g * n + k0 + r) * d + c0 + c] : 0.f;
+        }
+        if (t < 32) il[t] = (c0 + t < d) ? 1.0 / (double)a.ell[(size_t)g * d + c0 + t] : 0.0;
+        __syncthreads();
+        const int cmax = min(32, d - c0);
+        for (int c = 0; c < cmax; ++c) {
+            double z[U], x[4];
+#pragma unroll
+            for (int u = 0; u < U; ++u) z[u] = (double)zs[(ty + 16 * u) * 33 + c];
+#pragma unroll
+            for (int v = 0; v < 4; ++v) x[v] = (double)xs[(tx + 16 * v) * 33 + c];
+            const double w = il[c];
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+#pragma unroll
+                for (int v = 0; v < 4; ++v) {
+                    const double df = (x[v] - z[u]) * w;
+                    r2[u][v] = fma(df, df, r2[u][v]);
+                }
         }
     }
-    __syncthreads();
-    const int total = nflag_s;
-    if (t == 0 && total > 0) atomicAdd(&a.count[g], total);
-
-    // ---- rescue
-    if (total > 0) {
-        const float* Xg = a.X + (size_t)g * a.n * a.d;
-        const double* Wg = a.W64 + (size_t)g * a.npad * a.npad;
-        const double* ag = a.alpha64 + (size_t)g * a.npad;
-        const double sf2 = (double)a.sf2v[g];
-        const int n = a.n, d = a.d, npad = a.npad;
-        // reciprocal lengthscales in FP64: one rounding of 2^-53 per difference against an FP64 division per
-        // difference (the divisions were most of a rescue's time at d = 128)
-        for (int j = t; j < d; j += 256) ls[j] = 1.0 / (double)a.ell[(size_t)g * d + j];
-        for (int e0 = 0; e0 < total; e0 += R) {
-            const int nr = min(R, total - e0);
-            __syncthreads();
-            for (int e = t; e < R * d; e += 256) {
-                const int r = e / d, j = e % d;
-                const int c = list[R3_IDX(e0 + min(r, nr - 1), a.slice, a.status)];
-                zs[e] = (double)a.Xcand[(size_t)R3_IDX((long long)g * m + c, (long long)gridDim.y * m, a.status) * d + j];
+    const double sf2 = (double)a.sf2v[g];
+    const double* alpha = a.alpha64 + (size_t)g * a.npad;
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+        double part = 0.0;
+#pragma unroll
+        for (int v = 0; v < 4; ++v) {
+            const int k = k0 + tx + 16 * v;
+            if (k >= a.npad) continue;
+            double kv = 0.0;
+            if (k < n) {
+                const double sq = sqrt(5.0) * sqrt(r2[u][v]);
+                kv = sf2 * (1.0 + sq + sq * sq / 3.0) * exp(-sq);
+                part = fma(kv, alpha[k], part);
             }
+            store(ty + 16 * u, k, kv);
+        }
+        for (int o = 8; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
+        if (tx == 0) mean(ty + 16 * u, part);
+    }
+}
+
+__device__ __forceinline__ void write_result(const GuardArgs& a, int g, int cand, double mu, double q)
+{
+    const size_t f = (size_t)R3_IDX((long long)g * a.m + cand, (long long)a.batch * a.m, a.status);
+    const CandidateResult res = finalize_candidate(mu, q, (double)a.sf2v[g], (double)a.bestv[g]);
+    a.mu[f] = res.mu;
+    a.sigma[f] = res.sigma;
+    a.ei[f] = res.ei;
+}
+
+// 64 rows of W times 64 candidates: column sums of squares to qpart[slot][rt].
+__device__ __forceinline__ void rescue_tile(const GuardArgs& a, const double* __restrict__ Wg, size_t slot0, int rt,
+                                            unsigned char* smem)
+{
+    double* sA = reinterpret_cast<double*>(smem);         // [stages][64][20]
+    double* sB = sA + kStages * kTile * kStageLd;
+    const int t = threadIdx.x, w = t / 32, l = t % 32;
+    const int wm = (w % 4) * 16, wn = (w / 4) * 32;       // 16 x 32 per warp
+    const int npad = a.npad, i0 = rt * kTile;
+    const int kend = min(npad, i0 + kTile);               // W is lower triangular
+    const int steps = kend / 16;
+    auto load = [&](int s, int k0) {
+#pragma unroll
+        for (int it = 0; it < 2; ++it) {
+            const int e = t + kThreads * it, r = e / 8, q = e % 8;
+            const bool ok = i0 + r < npad;
+            cp_async16(sA + (s * kTile + r) * kStageLd + 2 * q, Wg + (size_t)(ok ? i0 + r : 0) * npad + k0 + 2 * q, ok);
+            cp_async16(sB + (s * kTile + r) * kStageLd + 2 * q,
+                       a.ks + (size_t)R3_IDX(slot0 + r, a.slab, a.status) * npad + k0 + 2 * q);
+        }
+    };
+    double c[2][4][2] = {};
+    __syncthreads();   // the previous item's reads of the stages are done
+#pragma unroll
+    for (int s = 0; s < kStages - 1; ++s) {
+        if (s < steps) load(s, s * 16);
+        cp_async_commit();
+    }
+    for (int kb = 0; kb < steps; ++kb) {
+        cp_async_wait<kStages - 2>();
+        __syncthreads();
+        if (kb + kStages - 1 < steps) load((kb + kStages - 1) % kStages, (kb + kStages - 1) * 16);
+        cp_async_commit();
+        const double* pa = sA + ((kb % kStages) * kTile + wm + l / 4) * kStageLd + l % 4;
+        const double* pb = sB + ((kb % kStages) * kTile + wn + l / 4) * kStageLd + l % 4;
+#pragma unroll
+        for (int kk = 0; kk < 16; kk += 4) {
+            double fa[2], fb[4];
+#pragma unroll
+            for (int i = 0; i < 2; ++i) fa[i] = pa[i * 8 * kStageLd + kk];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) fb[j] = pb[j * 8 * kStageLd + kk];
+#pragma unroll
+            for (int i = 0; i < 2; ++i)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) dmma(c[i][j], fa[i], fb[j]);
+        }
+    }
+    cp_async_wait<0>();
+    __syncthreads();
+    double* red = reinterpret_cast<double*>(smem);        // [4 row warps][64 candidates]
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            double s = fma(c[0][j][h], c[0][j][h], c[1][j][h] * c[1][j][h]);
+            for (int o = 4; o < 32; o <<= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+            if (l < 4) red[(w % 4) * kTile + wn + j * 8 + 2 * l + h] = s;
+        }
+    __syncthreads();
+    if (t < kTile)
+        a.qpart[(slot0 + t) * (npad / 16) + rt] = (red[t] + red[kTile + t]) + (red[2 * kTile + t] + red[3 * kTile + t]);
+}
+
+// 16 rows of W times 16 candidates, the reduction split over the block's eight warps; operands straight from L2.
+// Within a group of eight k the lanes hold pairs (2 l, 2 l + 1): the two products of a pair take the even and the odd
+// k, for both operands alike.
+__device__ __forceinline__ void rescue_small_tile(const GuardArgs& a, const double* __restrict__ Wg, size_t slot0, int rt,
+                                                  unsigned char* smem)
+{
+    double* red = reinterpret_cast<double*>(smem);        // [8 warps][16][17], then [16][17]
+    const int t = threadIdx.x, w = t / 32, l = t % 32;
+    const int npad = a.npad, i0 = rt * kSmallTile;
+    const int groups = min(npad, (i0 + kSmallTile + 7) / 8 * 8) / 8;
+    const double* wa = Wg + (size_t)(i0 + l / 4) * npad + 2 * (l % 4);
+    const double* kb = a.ks + ((size_t)R3_IDX(slot0, a.slab - (kSmallTile - 1), a.status) + l / 4) * npad + 2 * (l % 4);
+    double c[2][2][2] = {};
+#pragma unroll 4
+    for (int gk = w; gk < groups; gk += 8) {
+        double2 fa[2], fb[2];
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            fa[i] = __ldcg(reinterpret_cast<const double2*>(wa + (size_t)i * 8 * npad + gk * 8));
+            fb[i] = __ldcg(reinterpret_cast<const double2*>(kb + (size_t)i * 8 * npad + gk * 8));
+        }
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+                dmma(c[i][j], fa[i].x, fb[j].x);
+                dmma(c[i][j], fa[i].y, fb[j].y);
+            }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+        for (int j = 0; j < 2; ++j)
+#pragma unroll
+            for (int h = 0; h < 2; ++h) red[(w * 16 + i * 8 + l / 4) * 17 + j * 8 + 2 * (l % 4) + h] = c[i][j][h];
+    __syncthreads();
+    const int row = t / 16, col = t % 16;
+    double v = 0.0;
+#pragma unroll
+    for (int ww = 0; ww < 8; ++ww) v += red[(ww * 16 + row) * 17 + col];
+    __syncthreads();
+    red[row * 17 + col] = v * v;
+    __syncthreads();
+    if (t < kSmallTile) {
+        double s = 0.0;
+#pragma unroll
+        for (int r = 0; r < 16; ++r) s += red[r * 17 + t];
+        a.qpart[(slot0 + t) * (npad / 16) + rt] = s;
+    }
+}
+
+// Every listed candidate recomputed in FP64, tiles of CT candidates, a slab of tiles at a time.  Returns false when a
+// grid barrier ran out.
+template <int CT>
+__device__ __forceinline__ bool rescue(const GuardArgs& a, const int* pref, int tiles, unsigned& target, unsigned char* smem)
+{
+    const int nb = (a.npad + 63) / 64, row_tiles = (a.npad + CT - 1) / CT;
+    const int slab_tiles = a.slab / CT;
+    auto gp_of = [&](int tile) {   // last g with pref[g] <= tile
+        int lo = 0, hi = a.batch - 1;
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) / 2;
+            if (pref[mid] <= tile) lo = mid;
+            else hi = mid - 1;
+        }
+        return lo;
+    };
+    for (int t0 = 0; t0 < tiles; t0 += slab_tiles) {
+        const int nt = min(slab_tiles, tiles - t0);
+        for (int item = blockIdx.x; item < nt * nb; item += gridDim.x) {
+            const int tile = item % nt, g = gp_of(t0 + tile), first = (t0 + tile - pref[g]) * CT;
+            const int* list_g = a.list + (size_t)g * a.m + first;
+            const int kb = item / nt;
+            const size_t slot0 = R3_IDX((size_t)tile * CT, a.slab - (CT - 1), a.status);
+            kstar_tile<CT>(
+                a, g, [&](int r) { return __ldcg(list_g + r); }, min(CT, __ldcg(a.count + g) - first), kb, smem,
+                [&](int c, int k, double kv) { a.ks[(slot0 + c) * a.npad + k] = kv; },
+                [&](int c, double part) { a.mupart[(slot0 + c) * nb + kb] = part; });
+        }
+        if (!grid_barrier(a.barrier, target, a.status)) return false;
+        for (int item = blockIdx.x; item < nt * row_tiles; item += gridDim.x) {   // the longest rows first
+            const int tile = item % nt, rt = row_tiles - 1 - item / nt;
+            const double* Wg = a.W64 + (size_t)gp_of(t0 + tile) * a.npad * a.npad;
+            if (CT == kTile) rescue_tile(a, Wg, (size_t)tile * CT, rt, smem);
+            else rescue_small_tile(a, Wg, (size_t)tile * CT, rt, smem);
+        }
+        if (!grid_barrier(a.barrier, target, a.status)) return false;
+        for (int s = blockIdx.x * kThreads + threadIdx.x; s < nt * CT; s += gridDim.x * kThreads) {
+            const int tile = s / CT, g = gp_of(t0 + tile), pos = (t0 + tile - pref[g]) * CT + s % CT;
+            if (pos >= __ldcg(a.count + g)) continue;
+            double mu = 0.0, q = 0.0;
+            for (int b = 0; b < nb; ++b) mu += __ldcg(a.mupart + (size_t)s * nb + b);
+            for (int r = 0; r < row_tiles; ++r) q += __ldcg(a.qpart + (size_t)s * (a.npad / 16) + r);
+            write_result(a, g, __ldcg(a.list + (size_t)g * a.m + pos), mu, q);
+        }
+        // the next slab overwrites the partial sums that other blocks may still be adding up
+        if (t0 + slab_tiles < tiles && !grid_barrier(a.barrier, target, a.status)) return false;
+    }
+    return true;
+}
+
+// Short histories: the block that flags a candidate recomputes it at once, up to 16 per slice, without meeting the other
+// blocks: k* of the tile in shared memory, every warp 8 rows of W times the 16 candidates at a time.
+__device__ __forceinline__ void rescue_own(const GuardArgs& a, int g, const int* own, int count, unsigned char* smem)
+{
+    double* ks = reinterpret_cast<double*>(smem + kOwnKs);   // [16][npad + 8]: fragment reads on different banks
+    const int ld = a.npad + 8;
+    double* mu_s = ks + kSmallTile * ld;                      // [16]
+    double* q_s = mu_s + kSmallTile;                          // [8][16]
+    const int t = threadIdx.x, w = t / 32, l = t % 32;
+    if (t < kSmallTile) mu_s[t] = 0.0;
+    for (int kb = 0; kb < (a.npad + 63) / 64; ++kb)
+        kstar_tile<kSmallTile>(
+            a, g, [&](int r) { return own[r]; }, count, kb, smem, [&](int c, int k, double kv) { ks[c * ld + k] = kv; },
+            [&](int c, double part) { mu_s[c] += part; });
+    __syncthreads();
+    const double* Wg = a.W64 + (size_t)g * a.npad * a.npad;
+    double q[2][2] = {};
+    for (int i0 = w * 8; i0 < a.npad; i0 += 64) {
+        const double* wa = Wg + (size_t)(i0 + l / 4) * a.npad + 2 * (l % 4);
+        const double* kb = ks + (l / 4) * ld + 2 * (l % 4);
+        double c[2][2][2] = {};   // [even and odd k][candidates]
+#pragma unroll 4
+        for (int k = 0; k < i0 + 8; k += 8) {
+            const double2 fa = *reinterpret_cast<const double2*>(wa + k);
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+                const double2 fb = *reinterpret_cast<const double2*>(kb + j * 8 * ld + k);
+                dmma(c[0][j], fa.x, fb.x);
+                dmma(c[1][j], fa.y, fb.y);
+            }
+        }
+#pragma unroll
+        for (int j = 0; j < 2; ++j)
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const double v = c[0][j][h] + c[1][j][h];
+                q[j][h] = fma(v, v, q[j][h]);
+            }
+    }
+#pragma unroll
+    for (int j = 0; j < 2; ++j)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            double s = q[j][h];
+            for (int o = 4; o < 32; o <<= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+            if (l < 4) q_s[w * kSmallTile + j * 8 + 2 * l + h] = s;
+        }
+    __syncthreads();
+    if (t < count) {
+        double s = 0.0;
+        for (int ww = 0; ww < 8; ++ww) s += q_s[ww * kSmallTile + t];
+        write_result(a, g, own[t], mu_s[t], s);
+    }
+}
+
+__global__ void __launch_bounds__(kThreads, 2) guard_kernel(const GuardArgs a)
+{
+    extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ int own[kSmallTile], own_count;
+    __shared__ int warp_sum[8];
+    __shared__ bool last_slice;
+    const int t = threadIdx.x, lane = t % 32, warp = t / 32;
+    const long long m = a.m;
+    const int slices = a.slices_per_gp * a.batch;
+    const bool own_rescue = a.npad <= kOwnMaxN;
+    unsigned target = 0;
+
+    // ---- the pool's largest EI
+    if (!a.have_max) {
+        for (int s = blockIdx.x; s < slices; s += gridDim.x) {
+            const int g = s / a.slices_per_gp;
+            const long long c0 = (long long)(s % a.slices_per_gp) * a.slice, c1 = min(m, c0 + a.slice);
+            float v = 0.f;
+            for (long long i = c0 + t; i < c1; i += kThreads) v = fmaxf(v, __ldcg(a.ei + (size_t)g * m + i));  // EI >= 0; fmaxf ignores NaN
+            const unsigned top = __reduce_max_sync(0xffffffffu, __float_as_uint(v));   // order-preserving for v >= 0
+            if (lane == 0 && top) atomicMax(&a.maxbits[g], top);
+        }
+        if (!grid_barrier(a.barrier, target, a.status)) return;
+    }
+
+    // ---- flag
+    for (int s = blockIdx.x; s < slices; s += gridDim.x) {
+        const int g = s / a.slices_per_gp;
+        const long long c0 = (long long)(s % a.slices_per_gp) * a.slice, c1 = min(m, c0 + a.slice);
+        const float sf2 = a.sf2v[g], best = a.bestv[g];
+        const float tol_ei = 1e-5f * __uint_as_float(__ldcg(a.maxbits + g));
+        const float mu_floor = 1e-6f * a.yabsv[g], sd_floor = 1e-6f * sqrtf(sf2);
+        if (own_rescue) {
             __syncthreads();
-            double mu_part[R];
-#pragma unroll
-            for (int r = 0; r < R; ++r) mu_part[r] = 0.0;
-            for (int i = t; i < n; i += 256) {
-                double r2[R];
-#pragma unroll
-                for (int r = 0; r < R; ++r) r2[r] = 0.0;
-                for (int j = 0; j < d; ++j) {
-                    const double x = (double)Xg[(size_t)i * d + j], il = ls[j];
-#pragma unroll
-                    for (int r = 0; r < R; ++r) {
-                        const double df = (x - zs[r * d + j]) * il;
-                        r2[r] += df * df;
+            if (t == 0) own_count = 0;
+            __syncthreads();
+        }
+        for (long long i0 = c0; i0 < c1; i0 += kThreads) {
+            const long long i = i0 + t;
+            bool flag = false;
+            if (i < c1) {
+                const size_t f = (size_t)g * m + i;
+                const float mu_i = __ldcs(a.mu + f), sd = __ldcs(a.sigma + f), dmu = __ldcs(a.err_mu + f), dq = __ldcs(a.err_q + f);
+                // d sigma = dq / (2 sigma); with sigma -> 0 every rounding error in q matters
+                const float dsd = (sd > 0.f) ? dq / (2.f * sd) : ((dq > 0.f) ? INFINITY : 0.f);
+                const float tol_mu = 1e-4f * fabsf(mu_i) + mu_floor;
+                const float tol_sd = 1e-4f * sd + sd_floor;
+                flag = !(dmu <= 0.5f * tol_mu) || !(dsd <= 0.5f * tol_sd);
+                // EI: dEI = Phi(z) dmu + phi(z) dsigma against 1e-5 of the pool's largest EI
+                const float z = (sd > 0.f) ? (best - mu_i) / sd : 0.f;
+                const float Phi = 0.5f * erfcf(-z * 0.70710678f);
+                const float phi = expf(-0.5f * z * z) * 0.39894228f;
+                if (isfinite(dsd)) flag |= !(Phi * dmu + phi * dsd <= 0.5f * tol_ei);
+                flag |= !(sd * sd >= 1e-3f * sf2);   // deep cancellation: do not trust the estimates either
+            }
+            const unsigned votes = __ballot_sync(0xffffffffu, flag);   // one counter update per warp
+            if (votes) {
+                const int rank = __popc(votes & ((1u << lane) - 1u)), all = __popc(votes);
+                int mine = 0, base = 0;   // the first `mine` of the warp's go to the block's own list
+                if (lane == 0) {
+                    atomicAdd(&a.total[g], all);
+                    if (own_rescue) {
+                        base = atomicAdd(&own_count, all);
+                        mine = max(0, min(all, kSmallTile - base));
                     }
                 }
-                const double al = ag[i];
-#pragma unroll
-                for (int r = 0; r < R; ++r) {
-                    const double sq = sqrt(5.0) * sqrt(r2[r]);
-                    const double kv = sf2 * (1.0 + sq + sq * sq / 3.0) * exp(-sq);
-                    ks[(size_t)R3_IDX((long long)r * npad + i, (long long)R * npad, a.status)] = kv;
-                    mu_part[r] += kv * al;
+                if (own_rescue) {
+                    base = __shfl_sync(0xffffffffu, base, 0);
+                    mine = __shfl_sync(0xffffffffu, mine, 0);
+                    if (flag && rank < mine) own[base + rank] = (int)i;
                 }
+                if (mine < all) {
+                    if (lane == 0) base = atomicAdd(&a.count[g], all - mine);
+                    base = __shfl_sync(0xffffffffu, base, 0);
+                    if (flag && rank >= mine) a.list[(size_t)g * m + R3_IDX(base + rank - mine, m, a.status)] = (int)i;
+                }
+            }
+        }
+        if (own_rescue) {
+            __syncthreads();
+            if (own_count > 0) rescue_own(a, g, own, min(own_count, kSmallTile), smem);
+        }
+    }
+    if (!grid_barrier(a.barrier, target, a.status)) return;
+    if (blockIdx.x == 0 && t < min(a.batch, 64)) a.rescued_h[t] = __ldcg(a.total + t);   // pinned host memory
+
+    // ---- rescue
+    {
+        int* pref = reinterpret_cast<int*>(smem + a.pref_offset);   // [batch + 1] tiles before each GP
+        auto prefix = [&](int ct) {
+            const int per = (a.batch + kThreads - 1) / kThreads, g0 = t * per, g1 = min(a.batch, g0 + per);
+            int mine = 0;
+            for (int g = g0; g < g1; ++g) mine += (__ldcg(a.count + g) + ct - 1) / ct;
+            int incl = mine;
+            for (int o = 1; o < 32; o <<= 1) {
+                const int v = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += v;
             }
             __syncthreads();
-            double q_part[R];
-#pragma unroll
-            for (int r = 0; r < R; ++r) q_part[r] = 0.0;
-            for (int i = warp; i < n; i += 8) {
-                const double* Wr = Wg + (size_t)i * npad;
-                double v[R];
-#pragma unroll
-                for (int r = 0; r < R; ++r) v[r] = 0.0;
-                for (int kk = lane; kk <= i; kk += 32) {
-                    const double w = Wr[kk];
-#pragma unroll
-                    for (int r = 0; r < R; ++r) v[r] += w * ks[(size_t)r * npad + kk];
-                }
-#pragma unroll
-                for (int r = 0; r < R; ++r) {
-                    for (int o = 16; o > 0; o >>= 1) v[r] += __shfl_xor_sync(0xffffffffu, v[r], o);
-                    q_part[r] += v[r] * v[r];  // identical in every lane; lane 0's copy is used
-                }
-            }
-#pragma unroll
-            for (int r = 0; r < R; ++r) {
-                for (int o = 16; o > 0; o >>= 1) mu_part[r] += __shfl_xor_sync(0xffffffffu, mu_part[r], o);
-                if (lane == 0) {
-                    red[0][r][warp] = mu_part[r];
-                    red[1][r][warp] = q_part[r];
-                }
-            }
+            if (lane == 31) warp_sum[warp] = incl;
             __syncthreads();
-            if (t < nr) {
-                double mu_s = 0.0, q = 0.0;
-                for (int w = 0; w < 8; ++w) {
-                    mu_s += red[0][t][w];
-                    q += red[1][t][w];
-                }
-                const size_t f = (size_t)R3_IDX((long long)g * m + list[e0 + t], (long long)gridDim.y * m, a.status);
-                const CandidateResult res = finalize_candidate(mu_s, q, sf2, (double)a.bestv[g]);
-                a.mu[f] = res.mu;
-                a.sigma[f] = res.sigma;
-                a.ei[f] = res.ei;
+            int before = incl - mine;
+            for (int w = 0; w < warp; ++w) before += warp_sum[w];
+            for (int g = g0; g < g1; ++g) {
+                pref[g] = before;
+                before += (__ldcg(a.count + g) + ct - 1) / ct;
             }
+            if (g1 == a.batch && g0 < g1) pref[a.batch] = before;
+            __syncthreads();
+            return pref[a.batch];
+        };
+        const int big = prefix(kTile);
+        if (big > 0) {
+            // 64 x 64 tiles once they give every block two; below that 16 x 16 tiles spread the work
+            const long long items = (long long)big * ((a.npad + kTile - 1) / kTile);
+            if (items >= 2ll * gridDim.x) {
+                if (!rescue<kTile>(a, pref, big, target, smem)) return;
+            } else {
+                const int small = prefix(kSmallTile);
+                if (!rescue<kSmallTile>(a, pref, small, target, smem)) return;
+            }
+            if (a.k > 0 && !grid_barrier(a.barrier, target, a.status)) return;
         }
     }
     if (a.k == 0) return;
 
-    // ---- the k largest final EI of the slice (the rescued values were written by this block)
-    __syncthreads();
+    // ---- the k largest final EI of every slice
     unsigned long long* keys_s = reinterpret_cast<unsigned long long*>(smem);
-    const float* e = a.ei + (size_t)g * m;
-    for (int i = t; i < a.slice; i += 256) {
-        const long long c = c_begin + i;
-        keys_s[i] = (c < m) ? topk_make_key(e[c], (unsigned)c) : 0ull;
+    for (int s = blockIdx.x; s < slices; s += gridDim.x) {
+        const int g = s / a.slices_per_gp;
+        const long long c0 = (long long)(s % a.slices_per_gp) * a.slice;
+        const float* e = a.ei + (size_t)g * m;
+        __syncthreads();
+        for (int i = t; i < a.slice; i += kThreads) {
+            const long long c = c0 + i;
+            keys_s[i] = (c < m) ? topk_make_key(__ldcg(e + c), (unsigned)c) : 0ull;
+        }
+        __syncthreads();
+        block_select_desc(keys_s, a.slice, a.K2, smem + a.select_offset);
+        unsigned long long* out = a.keys + (size_t)s * a.k;
+        for (int i = t; i < a.k; i += kThreads) out[i] = i < a.slice ? keys_s[R3_IDX(i, a.slice, a.status)] : 0ull;
+        if (a.finish) {
+            __threadfence();
+            __syncthreads();
+            if (t == 0) last_slice = atomicAdd(&a.done[g], 1u) == (unsigned)a.slices_per_gp - 1u;
+            __syncthreads();
+            if (last_slice) {   // this block saw the GP's last slice: its keys are all there
+                __threadfence();
+                const int nk = a.slices_per_gp * a.k;
+                const unsigned long long* in = a.keys + (size_t)g * nk;
+                for (int i = t; i < nk; i += kThreads) keys_s[i] = __ldcg(in + i);
+                __syncthreads();
+                block_select_desc(keys_s, nk, a.k, smem + a.select_offset);
+                for (int i = t; i < a.k; i += kThreads) {
+                    const unsigned c = topk_key_index(keys_s[i]);
+                    a.idx[(size_t)g * a.k + i] = (int)c;
+                    if (a.val) a.val[(size_t)g * a.k + i] = ((long long)c < m) ? __ldcg(e + c) : __int_as_float(0x7fc00000);
+                }
+            }
+        }
     }
-    block_select_desc(keys_s, a.slice, a.K2, reinterpret_cast<char*>(smem) + a.select_offset);
-    unsigned long long* out = a.keys + ((size_t)g * gridDim.x + blockIdx.x) * a.k;
-    for (int i = t; i < a.k; i += 256) out[i] = i < a.slice ? keys_s[R3_IDX(i, a.slice, a.status)] : 0ull;
 }
+
+// candidates whose FP64 cross-covariances are in the workspace at a time
+int slab_candidates(const r3_gp* gp, long long m)
+{
+    const size_t fit = kSlabBytes / (sizeof(double) * (size_t)gp->npad) / kTile * kTile;
+    const size_t all = ((size_t)m + kTile - 1) / kTile * kTile * gp->batch;
+    return (int)std::max<size_t>(kTile, std::min(fit, all));
+}
+
+size_t up16(size_t b) { return (b + 15) & ~(size_t)15; }
 
 }  // namespace
 
 size_t guard_workspace_bytes(const r3_gp* gp, long long m)
 {
-    const size_t bm = (size_t)gp->batch * m;
-    return 2 * bm * sizeof(float) + 2 * (size_t)gp->batch * sizeof(int) + 256;
+    const size_t bm = (size_t)gp->batch * m, slab = slab_candidates(gp, m), npad = gp->npad;
+    return 3 * up16(bm * sizeof(float)) + up16((4 * (size_t)gp->batch + 1) * sizeof(int)) +
+           sizeof(double) * slab * (npad + npad / 16 + (npad + 63) / 64) + 256;
 }
 
 GuardBuffers guard_carve(const r3_gp* gp, long long m, void* ws)
 {
     GuardBuffers b;
-    const size_t bm = (size_t)gp->batch * m;
-    char* p = (char*)ws;
+    const size_t bm = up16((size_t)gp->batch * m * sizeof(float));
+    char* p = (char*)(((uintptr_t)ws + 15) & ~(uintptr_t)15);
     b.err_mu = (float*)p;
-    p += bm * sizeof(float);
+    p += bm;
     b.err_q = (float*)p;
-    p += bm * sizeof(float);
+    p += bm;
+    b.list = (int*)p;
+    p += bm;
     b.count = (int*)p;
-    p += (size_t)gp->batch * sizeof(int);
-    b.maxbits = (unsigned*)p;
+    b.total = b.count + gp->batch;
+    b.maxbits = (unsigned*)b.total + gp->batch;
+    b.done = b.maxbits + gp->batch;
+    b.barrier = b.done + gp->batch;
+    p += up16((4 * (size_t)gp->batch + 1) * sizeof(int));
+    const size_t slab = slab_candidates(gp, m), npad = gp->npad;
+    b.ks = (double*)p;
+    b.qpart = b.ks + slab * npad;
+    b.mupart = b.qpart + slab * (npad / 16);
     return b;
 }
 
-// Candidates per block of the guard kernel: enough blocks to fill the GPU on a large pool, small slices on a
-// small one (a power of two: the slice is also the chunk of the first top-k level).
-int guard_slice(long long m, int k)
+// Candidates per slice: enough slices to fill the GPU on a large pool, small ones on a small pool.
+static int guard_slice(int batch, long long m, int k)
 {
-    long long s = k > 32 ? 128 : 32;   // small pools: many blocks (the rescues of a block run one after another)
-    while (s < 4096 && s * 148 < m) s <<= 1;
+    long long s = 128;
+    while (s < 4096 && s < m && s * 296 < (long long)batch * m) s <<= 1;
     return (int)s;
 }
 
 size_t guard_topk_workspace_bytes(int batch, long long m, int k)
 {
-    const long long blocks = (m + guard_slice(m, k) - 1) / guard_slice(m, k);
-    return 2 * (size_t)batch * blocks * k * sizeof(unsigned long long) + 64;
+    const int slice = guard_slice(batch, m, k);
+    const long long slices = (m + slice - 1) / slice;
+    return 2 * (size_t)batch * slices * k * sizeof(unsigned long long) + 64;
 }
 
-r3_status_t guard_begin(r3_gp* gp, const GuardBuffers& b, cudaStream_t stream)
-{
-    R3_CUDA_TRY(cudaMemsetAsync(b.count, 0, 2 * (size_t)gp->batch * sizeof(int), stream));  // count and maxbits
-    return R3_OK;
-}
+// counts, maxima, finished slices and the grid barrier
+int guard_zero_ints(const r3_gp* gp) { return 4 * gp->batch + 1; }
 
 r3_status_t guard_and_rescue(r3_gp* gp, const float* Xcand, long long m, const GuardBuffers& b, float* mu,
                              float* sigma, float* ei, bool have_max, cudaStream_t stream)
 {
     const int B = gp->batch;
-    if (!have_max) {
-        const unsigned gx = (unsigned)((m + 1023) / 1024);
-        R3_LAUNCH(max_ei_kernel, dim3(gx < 592u ? gx : 592u, B), 256, 0, stream, ei, m, b.maxbits);
-    }
     const TopkRequest req = gp->topk_req;
     gp->topk_req = TopkRequest();
     GuardArgs a;
     a.X = gp->X; a.ell = gp->ell_d; a.sf2v = gp->sf2_d; a.bestv = gp->best_d; a.yabsv = gp->yabs_d; a.Xcand = Xcand;
     a.alpha64 = gp->alpha64; a.W64 = gp->W64;
-    a.n = gp->n; a.d = gp->d; a.npad = gp->npad;
+    a.batch = B; a.n = gp->n; a.d = gp->d; a.npad = gp->npad;
     a.m = m;
-    a.slice = guard_slice(m, req.k);
+    a.slice = guard_slice(B, m, req.k);
+    a.slices_per_gp = (int)((m + a.slice - 1) / a.slice);
     a.mu = mu; a.sigma = sigma; a.ei = ei;
     a.err_mu = b.err_mu; a.err_q = b.err_q;
+    a.list = b.list;
     a.maxbits = b.maxbits;
     a.count = b.count;
+    a.total = b.total;
+    a.rescued_h = gp->rescued_h;
+    a.done = b.done;
+    a.barrier = b.barrier;
     a.status = gp->status_d;
+    a.have_max = have_max;
+    a.ks = b.ks; a.qpart = b.qpart; a.mupart = b.mupart;
+    a.slab = slab_candidates(gp, m);
     a.k = req.k;
-    a.K2 = req.k > 0 ? std::min(req.k, a.slice) : 1;   // keys a block selects
+    a.K2 = req.k > 0 ? std::min(req.k, a.slice) : 1;
     a.keys = (unsigned long long*)req.ws;
-    const long long blocks = (m + a.slice - 1) / a.slice;
+    a.idx = req.idx;
+    a.val = req.val;
+    const long long keys_per_gp = (long long)a.slices_per_gp * req.k;
+    a.finish = req.k > 0 && keys_per_gp <= kFinishKeys;
     if (req.k > 0 && req.ws_bytes < guard_topk_workspace_bytes(B, m, req.k)) {
         set_error("internal: top-k workspace of the guard too small");
         return R3_ERR_INVALID_ARG;
     }
-    const int R = gp->npad <= 4096 ? RESCUE_GROUP : 1;
-    size_t region = sizeof(double) * ((size_t)R * gp->npad + (size_t)R * gp->d + gp->d);
-    region = std::max(region, sizeof(unsigned long long) * (size_t)a.slice);
-    // after the flag list (unused by then, but kept apart): the scratch of the slice's top-k selection
-    a.select_offset = (unsigned)((region + sizeof(int) * (size_t)a.slice + 7) & ~(size_t)7);
-    const size_t smem = a.select_offset + (req.k > 0 ? topk_select_scratch_bytes(a.K2) : 0);
-    if (R == RESCUE_GROUP) {
-        if (smem + 1024 > 48 * 1024)   // the kernel's static shared memory counts against the same limit
-            R3_CUDA_TRY(cudaFuncSetAttribute(guard_kernel<RESCUE_GROUP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        R3_LAUNCH(guard_kernel<RESCUE_GROUP>, dim3((unsigned)blocks, B), 256, smem, stream, a);
-    } else {
-        if (smem + 1024 > 48 * 1024)   // the kernel's static shared memory counts against the same limit
-            R3_CUDA_TRY(cudaFuncSetAttribute(guard_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        R3_LAUNCH(guard_kernel<1>, dim3((unsigned)blocks, B), 256, smem, stream, a);
-    }
-    R3_CUDA_TRY(cudaMemcpyAsync(gp->rescued_h, b.count, sizeof(int) * (B < 64 ? B : 64), cudaMemcpyDeviceToHost,
-                                stream));
-    if (req.k == 0) return R3_OK;
+    // dynamic shared memory: operand stages / slice keys, then the selection's scratch, then the tile prefix
+    size_t region = sizeof(double) * kStages * 2 * kTile * kStageLd;
+    a.select_offset = (unsigned)(sizeof(unsigned long long) * (a.finish ? (size_t)kFinishKeys : (size_t)a.slice));
+    if (req.k > 0) region = std::max(region, a.select_offset + topk_select_scratch_bytes(a.finish ? req.k : a.K2));
+    a.pref_offset = (unsigned)up16(region);
+    const size_t smem = a.pref_offset + sizeof(int) * ((size_t)B + 1);
+    int sms = 148;
+    R3_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, gp->device));
+    // the cap belongs to the kernel, not to the call: always the most that any call asks for
+    R3_CUDA_TRY(cudaFuncSetAttribute(guard_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem));
+    // two blocks per SM (launch bounds and 112 KB of shared memory allow it); a small pool is served by half of them,
+    // because the barriers then cost more than the work between them
+    const long long slices = (long long)a.slices_per_gp * B;
+    const unsigned grid = (unsigned)(slices <= sms ? sms : 2 * sms);
+    void* params[] = {&a};
+    R3_CUDA_TRY(cudaLaunchCooperativeKernel((const void*)guard_kernel, dim3(grid), dim3(kThreads), params, smem, stream));
+    ++g_launches;
+    if (req.k == 0 || a.finish) return R3_OK;
     unsigned long long* keys = (unsigned long long*)req.ws;
-    return topk_finish_from_keys(keys, keys + (size_t)B * blocks * req.k, B, blocks * req.k, req.k, ei, m, req.idx,
-                                 req.val, stream);
+    return topk_finish_from_keys(keys, keys + (size_t)B * keys_per_gp, B, keys_per_gp, req.k, ei, m, req.idx, req.val, stream);
 }
 
 }  // namespace r3

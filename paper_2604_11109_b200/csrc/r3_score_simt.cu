@@ -56,8 +56,12 @@ __global__ void __launch_bounds__(256) kstar_kernel(const float* __restrict__ X,
                                                     float sf2, int n, int d, int npad,
                                                     const float* __restrict__ Z,       // [mc][d] this slab
                                                     long long mc, float* __restrict__ ks,
-                                                    double* __restrict__ mu64, int* status)
+                                                    double* __restrict__ mu64, int* __restrict__ zero, int zero_ints,
+                                                    int* status)
 {
+    // the call's first launch clears the guard's counters
+    if (blockIdx.x == 0)
+        for (int i = threadIdx.x; i < zero_ints; i += blockDim.x) zero[i] = 0;
     __shared__ float sz[64][33], sx[64][33], sl[32];
     const int t = threadIdx.x, ty = t / 16, tx = t % 16;
     const long long c0 = (long long)blockIdx.x * 64;
@@ -236,10 +240,6 @@ r3_status_t score_simt(r3_gp* gp, const float* Xcand, long long m, float* mu, fl
     }
     SimtWorkspace w = carve(gp, m, ws);
     const int n = gp->n, d = gp->d, npad = gp->npad;
-    {
-        const r3_status_t st0 = guard_begin(gp, w.guard, stream);
-        if (st0 != R3_OK) return st0;
-    }
     for (int g = 0; g < gp->batch; ++g) {
         for (long long s0 = 0; s0 < m; s0 += w.slab) {
             const long long mc = (m - s0) < w.slab ? (m - s0) : w.slab;
@@ -248,7 +248,7 @@ r3_status_t score_simt(r3_gp* gp, const float* Xcand, long long m, float* mu, fl
             R3_LAUNCH(kstar_kernel, (unsigned)((mc + 63) / 64), 256, 0, stream,
                       gp->X + (size_t)g * n * d, gp->inv_ell + (size_t)g * d,
                       gp->alpha32 + (size_t)g * npad, gp->sf2[g], n, d, npad, Z, mc, w.ks, w.mu64,
-                      gp->status_d);
+                      w.guard.count, g == 0 && s0 == 0 ? guard_zero_ints(gp) : 0, gp->status_d);
             prof_begin(gp, stream);
             R3_LAUNCH(trigemm_sq_kernel, (unsigned)((mc + 127) / 128), 256, 0, stream,
                       gp->W32 + (size_t)g * npad * npad, w.ks, w.mu64, npad, mc, (double)gp->sf2[g],

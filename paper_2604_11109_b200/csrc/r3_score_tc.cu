@@ -170,6 +170,8 @@ __global__ void __launch_bounds__(128 + 128 * G, 1) score_tc_kernel(const TcPara
     if (threadIdx.x == 0) {
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
+    if (blockIdx.x == 0)
+        for (int i = threadIdx.x; i < prm.zero_ints; i += blockDim.x) prm.zero[i] = 0;
     if (warp == 2) {
         __syncwarp();
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
@@ -1343,10 +1345,8 @@ r3_status_t score_tc_part(r3_gp* gp, const float* Xcand, long long m, float* mu,
     }
     const long long launch_tiles = prm.total_tiles - prm.tile_begin;
     if (launch_tiles <= 0) return R3_OK;
-    if (prm.tile_begin == 0) {   // the pool's first (or only) piece: the rescue counters start at zero
-        const r3_status_t st0 = guard_begin(gp, gb, stream);
-        if (st0 != R3_OK) return st0;
-    }
+    prm.zero = gb.count;
+    prm.zero_ints = guard_zero_ints(gp);
     int sms = 148;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, gp->device);
     const unsigned grid = (unsigned)(launch_tiles < sms ? launch_tiles : sms);

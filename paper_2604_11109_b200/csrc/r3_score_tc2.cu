@@ -198,6 +198,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(128 + 128 * G2, 1) s
         abort_flag[1] = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
+    if (blockIdx.x == 0)
+        for (int i = threadIdx.x; i < prm.zero_ints; i += blockDim.x) prm.zero[i] = 0;
     if (warp == 2) {
         __syncwarp();
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(

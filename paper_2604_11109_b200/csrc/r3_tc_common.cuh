@@ -45,6 +45,8 @@ struct TcParams {
     const double* wnorm;
     int DP, NP, P, ws;
     int* status;
+    int* zero;          // the guard's counters, cleared by the first block (nothing reads them before the guard's kernel)
+    int zero_ints;
     long long tiles_per_gp, total_tiles;   // total_tiles: one past the last tile of this launch
     long long tile_begin;                  // first tile of this launch (the single-CTA kernel; 0 for a whole pool)
     long long* trace;   // optional [grid][4 roles][8] cycle counters (diagnostics)
