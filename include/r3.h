@@ -76,7 +76,8 @@ typedef enum {
  *
  * Synchronises `cuda_stream` before returning, so that R3_ERR_NOT_PD and
  * R3_ERR_NONFINITE are reported by this call.  No jitter is added: a
- * non-positive-definite K is an error, never silently repaired.
+ * non-positive-definite K is an error, never silently repaired (a pivot below
+ * four roundings of sf2 + noise, such as a duplicated row without noise leaves, counts as non-positive).
  */
 r3_status_t r3_gp_fit(const float* X, const float* y, const float* lengthscales,
                       const float* signal_var, const float* noise_var, int batch, int n, int d,
@@ -312,10 +313,9 @@ r3_status_t r3_gp_propose(r3_gp_t* gp, const float* Xcand, long long m, int q, i
  * With K' = [[K, B], [B^T, C]]:  L21 = (L^-1 B)^T,  L22 L22^T = C - L21 L21^T,  W' = L'^-1 by blocks,
  * alpha' = K'^-1 y'.  The handle afterwards equals, up to FP64 rounding, the one r3_gp_fit returns for
  * the concatenated history with the same hyper-parameters; best becomes min(y') (an incumbent set
- * with r3_gp_set_best is replaced) and the scoring engine is chosen again for the new size.  L21 is
- * formed with the stored inverse factor; when K is ill-conditioned (|L^-1|_2^2 (signal_var + noise_var)
- * above 1e8) one step of iterative refinement with L itself follows, so that the extension stays as
- * accurate as a fit there.
+ * with r3_gp_set_best is replaced) and the scoring engine is chosen again for the new size.  The new rows
+ * are computed as a fit computes them (substitution with the stored L), so the extension is as accurate as
+ * a fit for ill-conditioned histories too.
  *
  *   Xnew  device [batch][k][d]     ynew  device [batch][k]      1 <= k <= 128,  n + k <= 8192
  *

@@ -255,6 +255,10 @@ r3_status_t r3_gp_fit(const float* X, const float* y, const float* lengthscales,
 
     r3_status_t st = fit_device(gp, y, stream);  // synchronises, fills status_h
     if (st != R3_OK) return bail(st);
+    if (gp->status_h[0] & DEV_TIMEOUT) {
+        set_error("r3_gp_fit: a bounded device-side wait ran out");
+        return bail(R3_ERR_DEVICE_TIMEOUT);
+    }
     if (gp->status_h[0] & DEV_NONFINITE) {
         set_error("r3_gp_fit: X or y contains a non-finite value");
         return bail(R3_ERR_NONFINITE);
@@ -417,12 +421,16 @@ r3_status_t r3_gp_append(r3_gp_t* gp, const float* Xnew, const float* ynew, int 
             return R3_ERR_CUDA;
         }
     }
-    if (st == R3_OK && (bits & (DEV_NONFINITE | DEV_NOT_PD))) {
+    if (st == R3_OK && (bits & (DEV_NONFINITE | DEV_NOT_PD | DEV_TIMEOUT))) {
         // the handle was not touched; clear this call's bits so that it stays usable
         gp->status_h[0] = latched;
         gp->status_h[1] = INT_MAX;
         R3_CUDA_TRY(cudaMemcpyAsync(gp->status_d, gp->status_h, 2 * sizeof(int), cudaMemcpyHostToDevice, stream));
         R3_CUDA_TRY(cudaStreamSynchronize(stream));
+        if (bits & DEV_TIMEOUT) {
+            set_error("r3_gp_append: a bounded device-side wait ran out");
+            return R3_ERR_DEVICE_TIMEOUT;
+        }
         if (bits & DEV_NONFINITE) {
             set_error("r3_gp_append: Xnew or ynew contains a non-finite value");
             return R3_ERR_NONFINITE;

@@ -155,6 +155,19 @@ struct r3_gp {
 
 namespace r3 {
 
+// factor and inverse factor (r3_factor.cu)
+constexpr int kFactorTile = 64;
+struct FactorProblem {
+    const float *X, *y, *ell, *sf2, *sn2;   // [batch][n][d], [batch][n], [batch][d], [batch], [batch]
+    int batch, n, d, npad;
+    int rows_done;          // rows of L and W that are there already: a multiple of kFactorTile
+    double *L, *W;          // [batch][npad][npad]
+    float *best, *yabs;     // [batch] min y, max |y|
+};
+size_t factor_scratch_bytes(int batch, int npad);
+// Asynchronous; non-finite inputs and non-positive pivots are latched in `status`.
+r3_status_t factor_device(const FactorProblem& p, void* scratch, int* status, int device, cudaStream_t stream);
+
 // fit (r3_fit.cu)
 r3_status_t fit_device(r3_gp* gp, const float* y, cudaStream_t stream);
 // Appends k observations per GP (r3_gp_append): extends L, W, alpha, X, y in O(k n^2); synchronises.  On

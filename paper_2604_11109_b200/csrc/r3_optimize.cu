@@ -32,6 +32,10 @@ r3_status_t refit_device(r3_gp* gp, cudaStream_t stream, int* bits, int* pivot =
     R3_CUDA_TRY(cudaStreamSynchronize(stream));   // `inv` is a pageable temporary
     const r3_status_t st = fit_device(gp, gp->y, stream);   // synchronises, fills status_h
     if (st != R3_OK) return st;
+    if (gp->status_h[0] & DEV_TIMEOUT) {
+        set_error("a bounded device-side wait ran out");
+        return R3_ERR_DEVICE_TIMEOUT;
+    }
     *bits = gp->status_h[0];
     if (pivot) *pivot = gp->status_h[1];
     if (*bits & (DEV_NOT_PD | DEV_NONFINITE)) {

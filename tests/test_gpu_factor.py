@@ -1,0 +1,41 @@
+"""Factor and inverse factor at the edges of their 64-row tiles: the whole computation (fit) and its tail (append), for one
+GP and for several, against the oracle's factor; the inverse is checked through the scores, which contract with it."""
+import numpy as np
+import pytest
+
+from paper_2604_11109_b200 import binding as b
+from tests.test_gpu_append import check_handle, check_scoring, dev, problem
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("batch,n", [(1, 1), (1, 32), (3, 63), (1, 64), (2, 65), (1, 96), (1, 128), (5, 129), (1, 320), (1, 833)])
+def test_fit_at_tile_edges(batch, n):
+    g = problem(1300 + n, batch, n, 7, 150)
+    gp = b.r3_gp_fit(dev(g["X"]), dev(g["y"]), g["ell"], g["sf2"], g["sn2"])
+    check_scoring(gp, g, check_handle(gp, g, n))
+    gp.close()
+
+
+@pytest.mark.parametrize("batch,n0,k", [(1, 63, 1), (2, 64, 1), (1, 64, 64), (1, 120, 128), (3, 191, 2), (1, 640, 3)])
+def test_append_at_tile_edges(batch, n0, k):
+    g = problem(1700 + n0, batch, n0 + k, 7, 150)
+    gp = b.r3_gp_fit(dev(g["X"][:, :n0]), dev(g["y"][:, :n0]), g["ell"], g["sf2"], g["sn2"])
+    b.r3_gp_append(gp, dev(g["X"][:, n0:]), dev(g["y"][:, n0:]))
+    check_scoring(gp, g, check_handle(gp, g, n0 + k))
+    # the tail of the computation gives the bits of the whole
+    whole = b.r3_gp_fit(dev(g["X"]), dev(g["y"]), g["ell"], g["sf2"], g["sn2"])
+    for x, y in zip(b.r3_gp_get_factor(gp), b.r3_gp_get_factor(whole)):
+        assert np.array_equal(x, y)
+    gp.close()
+    whole.close()
+
+
+@pytest.mark.parametrize("n,twin", [(40, 3), (100, 70), (200, 10)])
+def test_duplicated_row_without_noise_is_not_positive_definite(n, twin):
+    g = problem(2100 + n, 1, n, 5, 4)
+    g["X"][0, -1] = g["X"][0, twin]
+    with pytest.raises(b.R3Error) as e:
+        b.r3_gp_fit(dev(g["X"]), dev(g["y"]), g["ell"], g["sf2"], np.zeros(1, np.float32))
+    assert e.value.status == 3 and f"pivot {n - 1} " in str(e.value)
