@@ -50,6 +50,10 @@ size_t bin_of(size_t bytes)
 
 }  // namespace
 
+static thread_local int t_no_wait = 0;
+FreeScope::FreeScope() { ++t_no_wait; }
+FreeScope::~FreeScope() { --t_no_wait; }
+
 cudaError_t dev_malloc_bytes(void** p, size_t bytes)
 {
     *p = nullptr;
@@ -109,7 +113,7 @@ void dev_free(void* p)
         cudaFree(p);
         return;
     }
-    cudaDeviceSynchronize();   // as cudaFree would: nothing in flight may still use the block
+    if (t_no_wait == 0) cudaDeviceSynchronize();   // as cudaFree would: nothing in flight may still use the block
     std::lock_guard<std::mutex> lock(g_mutex);
     DeviceCache& c = g_cache[dev];
     if (c.cached_bytes + bin > kCacheLimit || c.free_blocks.size() >= kCacheBlocks) {

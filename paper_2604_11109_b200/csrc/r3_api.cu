@@ -136,23 +136,11 @@ void r3_launch_count_reset(void) { g_launches = 0; }
 void r3_gp_free(r3_gp_t* gp)
 {
     if (!gp) return;
-    tc_release(gp);
-    dev_free(gp->X);
-    dev_free(gp->y);
-    dev_free(gp->ell_d);
-    dev_free(gp->inv_ell);
-    dev_free(gp->sn2_d);
-    dev_free(gp->sf2_d);
-    dev_free(gp->best_d);
-    dev_free(gp->yabs_d);
-    dev_free(gp->wnorm_d);
-    dev_free(gp->L64);
-    dev_free(gp->W64);
-    dev_free(gp->W32);
-    dev_free(gp->alpha64);
-    dev_free(gp->alpha32);
+    cudaDeviceSynchronize();   // nothing in flight uses the handle any more
+    FreeScope no_wait;
+    state_free(*gp);
     dev_free(gp->status_d);
-    pinned_word_release(gp->status_h);   // rescued_h lives in the same block
+    pinned_word_release(gp->status_h);   // rescued_h and stage_h live in the same block
     for (cudaEvent_t e : gp->events) cudaEventDestroy(e);
     for (cudaEvent_t e : gp->copy_events) cudaEventDestroy(e);
     if (gp->copy_stream) cudaStreamDestroy(gp->copy_stream);
@@ -209,76 +197,35 @@ r3_status_t r3_gp_fit(const float* X, const float* y, const float* lengthscales,
     gp->batch = batch;
     gp->n = n;
     gp->d = d;
-    gp->npad = round_up(n, kFitBlock);
     gp->ell.assign(lengthscales, lengthscales + (size_t)batch * d);
     gp->sf2.assign(signal_var, signal_var + batch);
     gp->sn2.assign(noise_var, noise_var + batch);
-    gp->best.assign(batch, 0.f);
-    std::vector<float> inv((size_t)batch * d);
-    for (size_t i = 0; i < inv.size(); ++i) inv[i] = (float)(1.0 / (double)gp->ell[i]);
-
-    const size_t mat = (size_t)gp->npad * gp->npad;
-    TRY_BAIL(dev_malloc(&gp->X, sizeof(float) * batch * (size_t)n * d));
-    TRY_BAIL(dev_malloc(&gp->y, sizeof(float) * batch * (size_t)n));
-    TRY_BAIL(dev_malloc(&gp->ell_d, sizeof(float) * batch * d));
-    TRY_BAIL(dev_malloc(&gp->inv_ell, sizeof(float) * batch * d));
-    TRY_BAIL(dev_malloc(&gp->sn2_d, sizeof(float) * batch));
-    TRY_BAIL(dev_malloc(&gp->sf2_d, sizeof(float) * batch));
-    TRY_BAIL(dev_malloc(&gp->best_d, sizeof(float) * batch));
-    TRY_BAIL(dev_malloc(&gp->yabs_d, sizeof(float) * batch));
-    TRY_BAIL(dev_malloc(&gp->wnorm_d, sizeof(double) * batch));
-    TRY_BAIL(dev_malloc(&gp->L64, sizeof(double) * batch * mat));
-    TRY_BAIL(dev_malloc(&gp->W64, sizeof(double) * batch * mat));
-    TRY_BAIL(dev_malloc(&gp->W32, sizeof(float) * batch * mat));
-    TRY_BAIL(dev_malloc(&gp->alpha64, sizeof(double) * batch * gp->npad));
-    TRY_BAIL(dev_malloc(&gp->alpha32, sizeof(float) * batch * gp->npad));
+    r3_status_t st = state_alloc(*gp);
+    if (st != R3_OK) return bail(st);
     TRY_BAIL(dev_malloc(&gp->status_d, 4 * sizeof(int)));
     TRY_BAIL(cudaMemsetAsync(gp->status_d, 0, 4 * sizeof(int), stream));
-    gp->status_h = pinned_word_acquire();   // [4] status words, then [64] rescue counters
+    gp->status_h = pinned_word_acquire();   // [4] status words, [64] rescue counters, then the staging area
     if (!gp->status_h) {
         set_error("r3_gp_fit: no pinned host memory");
         return bail(R3_ERR_ALLOC);
     }
     gp->rescued_h = gp->status_h + 4;
+    gp->stage_h = reinterpret_cast<char*>(gp->status_h + kStageInt);
     for (int i = 0; i < 64; ++i) gp->rescued_h[i] = 0;
-    gp->status_h[0] = 0;
-    gp->status_h[1] = INT_MAX;
-    TRY_BAIL(cudaMemcpyAsync(gp->status_d, gp->status_h, 2 * sizeof(int), cudaMemcpyHostToDevice, stream));
     TRY_BAIL(cudaMemcpyAsync(gp->X, X, sizeof(float) * batch * (size_t)n * d, cudaMemcpyDeviceToDevice, stream));
     TRY_BAIL(cudaMemcpyAsync(gp->y, y, sizeof(float) * batch * (size_t)n, cudaMemcpyDeviceToDevice, stream));
-    TRY_BAIL(cudaMemcpyAsync(gp->ell_d, gp->ell.data(), sizeof(float) * batch * d, cudaMemcpyHostToDevice, stream));
-    TRY_BAIL(cudaMemcpyAsync(gp->inv_ell, inv.data(), sizeof(float) * batch * d, cudaMemcpyHostToDevice, stream));
-    TRY_BAIL(cudaMemcpyAsync(gp->sn2_d, gp->sn2.data(), sizeof(float) * batch, cudaMemcpyHostToDevice, stream));
-    TRY_BAIL(cudaMemcpyAsync(gp->sf2_d, gp->sf2.data(), sizeof(float) * batch, cudaMemcpyHostToDevice, stream));
-    TRY_BAIL(cudaStreamSynchronize(stream));  // `inv` is a pageable temporary
 #undef TRY_BAIL
 
-    r3_status_t st = fit_device(gp, y, stream);  // synchronises, fills status_h
+    int bits = 0, pivot = 0;
+    st = state_fit(gp, *gp, 0, true, true, stream, &bits, &pivot);
     if (st != R3_OK) return bail(st);
-    if (gp->status_h[0] & DEV_TIMEOUT) {
-        set_error("r3_gp_fit: a bounded device-side wait ran out");
-        return bail(R3_ERR_DEVICE_TIMEOUT);
-    }
-    if (gp->status_h[0] & DEV_NONFINITE) {
+    if (bits & DEV_NONFINITE) {
         set_error("r3_gp_fit: X or y contains a non-finite value");
         return bail(R3_ERR_NONFINITE);
     }
-    if (gp->status_h[0] & DEV_NOT_PD) {
-        set_error("r3_gp_fit: pivot %d of K + noise*I is not positive (duplicate rows with zero noise?)",
-                  gp->status_h[1]);
+    if (bits & DEV_NOT_PD) {
+        set_error("r3_gp_fit: pivot %d of K + noise*I is not positive (duplicate rows with zero noise?)", pivot);
         return bail(R3_ERR_NOT_PD);
-    }
-    gp->y_absmax.assign(batch, 0.f);
-    gp->wnorm.assign(batch, 0.0);
-    if (cudaMemcpy(gp->best.data(), gp->best_d, sizeof(float) * batch, cudaMemcpyDeviceToHost) != cudaSuccess ||
-        cudaMemcpy(gp->y_absmax.data(), gp->yabs_d, sizeof(float) * batch, cudaMemcpyDeviceToHost) != cudaSuccess ||
-        cudaMemcpy(gp->wnorm.data(), gp->wnorm_d, sizeof(double) * batch, cudaMemcpyDeviceToHost) != cudaSuccess) {
-        set_error("r3_gp_fit: reading back the incumbent failed");
-        return bail(R3_ERR_CUDA);
-    }
-    if (tc_supported(n, d)) {
-        st = tc_prepare(gp, stream);
-        if (st != R3_OK) return bail(st);
     }
     *out = gp;
     return R3_OK;
@@ -335,6 +282,7 @@ r3_status_t r3_gp_propose(r3_gp_t* gp, const float* Xcand, long long m, int q, i
     const size_t bm = (size_t)B * m, tbytes = topk_workspace_bytes(B, m, Rk);
     auto done = [&](r3_status_t s) {
         cudaStreamSynchronize(stream);
+        FreeScope no_wait;
         dev_free(scores); dev_free(sval); dev_free(sidx); dev_free(tws); dev_free(pws);
         return s;
     };
@@ -404,51 +352,17 @@ r3_status_t r3_gp_append(r3_gp_t* gp, const float* Xnew, const float* ynew, int 
         return R3_ERR_INVALID_ARG;
     }
     cudaStream_t stream = (cudaStream_t)cuda_stream;
-    // Bits that an earlier scoring call latched (a non-finite candidate, a wait that ran out) are not this
-    // call's: they are taken out of the status word while the append's own checks use it, and put back after.
-    R3_CUDA_TRY(cudaMemcpyAsync(gp->status_h, gp->status_d, 2 * sizeof(int), cudaMemcpyDeviceToHost, stream));
-    R3_CUDA_TRY(cudaStreamSynchronize(stream));
-    const int latched = gp->status_h[0] & (DEV_NONFINITE | DEV_TIMEOUT);
-    if (latched) R3_CUDA_TRY(cudaMemsetAsync(gp->status_d, 0, sizeof(int), stream));
-    r3_status_t st = append_device(gp, Xnew, ynew, k, stream);
-    const int bits = gp->status_h ? gp->status_h[0] : 0;
-    const int pivot = gp->status_h ? gp->status_h[1] : 0;
-    if (latched) {
-        gp->status_h[0] = latched;
-        if (cudaMemcpyAsync(gp->status_d, gp->status_h, sizeof(int), cudaMemcpyHostToDevice, stream) != cudaSuccess ||
-            cudaStreamSynchronize(stream) != cudaSuccess) {
-            set_error("r3_gp_append: restoring the latched status failed");
-            return R3_ERR_CUDA;
-        }
+    int bits = 0, pivot = 0;   // the append's own status words: what scoring calls have latched stays where it is
+    const r3_status_t st = append_device(gp, Xnew, ynew, k, stream, &bits, &pivot);
+    if (st != R3_OK) return st;
+    if (bits & DEV_NONFINITE) {
+        set_error("r3_gp_append: Xnew or ynew contains a non-finite value");
+        return R3_ERR_NONFINITE;
     }
-    if (st == R3_OK && (bits & (DEV_NONFINITE | DEV_NOT_PD | DEV_TIMEOUT))) {
-        // the handle was not touched; clear this call's bits so that it stays usable
-        gp->status_h[0] = latched;
-        gp->status_h[1] = INT_MAX;
-        R3_CUDA_TRY(cudaMemcpyAsync(gp->status_d, gp->status_h, 2 * sizeof(int), cudaMemcpyHostToDevice, stream));
-        R3_CUDA_TRY(cudaStreamSynchronize(stream));
-        if (bits & DEV_TIMEOUT) {
-            set_error("r3_gp_append: a bounded device-side wait ran out");
-            return R3_ERR_DEVICE_TIMEOUT;
-        }
-        if (bits & DEV_NONFINITE) {
-            set_error("r3_gp_append: Xnew or ynew contains a non-finite value");
-            return R3_ERR_NONFINITE;
-        }
+    if (bits & DEV_NOT_PD) {
         set_error("r3_gp_append: pivot %d of the extended K + noise*I is not positive (duplicate rows with zero noise?)",
                   pivot);
         return R3_ERR_NOT_PD;
-    }
-    if (st != R3_OK) return st;
-    R3_CUDA_TRY(cudaMemcpy(gp->best.data(), gp->best_d, sizeof(float) * gp->batch, cudaMemcpyDeviceToHost));
-    R3_CUDA_TRY(cudaMemcpy(gp->y_absmax.data(), gp->yabs_d, sizeof(float) * gp->batch, cudaMemcpyDeviceToHost));
-    R3_CUDA_TRY(cudaMemcpy(gp->wnorm.data(), gp->wnorm_d, sizeof(double) * gp->batch, cudaMemcpyDeviceToHost));
-    tc_release(gp);
-    if (tc_supported(gp->n, gp->d)) {
-        st = tc_prepare(gp, stream);
-        // The history is extended at this point.  If only the tensor engine's operands could not be allocated,
-        // the append stands and the CUDA-core engine serves the handle (r3_gp_engine tells).
-        if (st != R3_OK && st != R3_ERR_ALLOC) return st;
     }
     return R3_OK;
 }
@@ -497,6 +411,7 @@ r3_status_t r3_topk(const float* ei, int batch, long long m, int k, int* idx, fl
     R3_CUDA_TRY(dev_malloc(&ws, bytes));
     st = topk_device(ei, batch, m, k, idx, val, ws, bytes, stream);
     cudaError_t e = cudaStreamSynchronize(stream);
+    FreeScope no_wait;
     dev_free(ws);
     if (st == R3_OK && e != cudaSuccess) {
         set_error("r3_topk: %s", cudaGetErrorString(e));

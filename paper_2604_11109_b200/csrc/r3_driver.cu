@@ -91,6 +91,7 @@ r3_status_t r3_bo_run(const float* X0, const float* y0, int n0, int d, const flo
     void* topk_ws = nullptr;
     auto done = [&](r3_status_t s) {
         cudaStreamSynchronize(stream);
+        FreeScope no_wait;
         dev_free(work);
         dev_free(rows_d);
         dev_free(y_d);

@@ -46,15 +46,15 @@ __device__ __forceinline__ unsigned load_acquire(const unsigned* p)
     return v;
 }
 
-// Barrier over all blocks of a cooperatively launched grid.  `counter` starts at zero and only grows; `target` is the
+// Barrier over `blocks` blocks (grid_barrier: all) of a cooperatively launched grid.  `counter` starts at zero and only grows; `target` is the
 // caller's running count.  Bounded like every device-side wait: after about two seconds the status word gets
 // DEV_TIMEOUT and false is returned, on which the block leaves the kernel.
 constexpr long long kGridWaitCycles = 4000000000ll;
-__device__ __forceinline__ bool grid_barrier(unsigned* counter, unsigned& target, int* status)
+__device__ __forceinline__ bool team_barrier(unsigned* counter, unsigned& target, unsigned blocks, int* status)
 {
     bool ok = true;
     __syncthreads();
-    target += gridDim.x;
+    target += blocks;
     if (threadIdx.x == 0) {
         __threadfence();
         atomicAdd(counter, 1u);
@@ -70,6 +70,10 @@ __device__ __forceinline__ bool grid_barrier(unsigned* counter, unsigned& target
         }
     }
     return __syncthreads_and(ok);
+}
+__device__ __forceinline__ bool grid_barrier(unsigned* counter, unsigned& target, int* status)
+{
+    return team_barrier(counter, target, gridDim.x, status);
 }
 
 }  // namespace r3

@@ -582,7 +582,7 @@ size_t factor_scratch_bytes(int batch, int npad)
     return sizeof(int) * (2 * (size_t)batch * T + 1);
 }
 
-r3_status_t factor_device(const FactorProblem& p, void* scratch, int* status, int device, cudaStream_t stream)
+r3_status_t factor_device(const FactorProblem& p, void* scratch, int extra_ints, int* status, int device, cudaStream_t stream)
 {
     FactorArgs a;
     a.X = p.X; a.ell = p.ell; a.sf2 = p.sf2; a.sn2 = p.sn2;
@@ -598,7 +598,7 @@ r3_status_t factor_device(const FactorProblem& p, void* scratch, int* status, in
     for (int j = 0; j < a.T; ++j)   // column j of L below the finished rows, then row j of W
         a.first[j + 1] = a.first[j] + (a.T - std::max(j, a.i0)) + (j >= a.i0 ? j : 0);
     const size_t xcount = (size_t)p.batch * p.n * p.d;
-    const int zeros = (int)(factor_scratch_bytes(p.batch, p.npad) / sizeof(int));
+    const int zeros = (int)(factor_scratch_bytes(p.batch, p.npad) / sizeof(int)) + extra_ints;
     const unsigned gx = (unsigned)std::max<size_t>(1, std::min<size_t>(148, (xcount + 2047) / 2048) / p.batch);
     R3_LAUNCH(fit_begin_kernel, dim3(gx, p.batch), 256, 0, stream, p.X, xcount, p.y, p.n, p.best, p.yabs,
               reinterpret_cast<int*>(scratch), zeros, status);

@@ -1,145 +1,105 @@
-// r3_gp_fit and r3_gp_append on the device: factor and inverse factor (r3_factor.cu), weights, norm estimate.
+// r3_gp_fit and r3_gp_append on the device: one upload, the factorisation (r3_factor.cu), the weights (r3_weights.cu), the
+// tensor operands (r3_score_tc.cu), one read-back.
 //
-// Everything here runs once per BO round, in FP64, and is rounded to FP32 once at the end:
-//   K = L L^T, W = L^-1          factor_device
-//   alpha = W^T (W y)            two triangular matrix-vector products
-//   |W|_2                        power iteration, for the scoring engines' error estimates
-// `batch` GPs go together.  n is padded to a multiple of 32 with an identity block, which leaves L, W and alpha unchanged.
+// Everything here runs once per BO round, in FP64, and is rounded to FP32 once at the end.  n is padded to a multiple of
+// 32 with an identity block, which leaves L, W and alpha unchanged.
+#include <limits.h>
+#include <string.h>
+
+#include <algorithm>
+
 #include "r3_internal.cuh"
 
 namespace r3 {
 
 namespace {
 
-// ------------------------------------------------------------------------------------ weights
-// u = W y (lower-triangular W, one warp per row); rows >= n give 0.
+// The block of small arrays: what the device reports first, then what it is told.
+size_t carve_block(r3_fit_state& s, char* base, size_t* results)
+{
+    char* p = base;
+    const size_t B = s.batch;
+    auto take = [&](size_t bytes) {
+        char* r = p;
+        p += (bytes + 15) & ~(size_t)15;
+        return r;
+    };
+    s.block = base;
+    s.fit_status = (int*)take(4 * sizeof(int));
+    s.best_d = (float*)take(sizeof(float) * B);
+    s.yabs_d = (float*)take(sizeof(float) * B);
+    s.wmax_d = (unsigned*)take(sizeof(unsigned) * B);
+    s.xamax_d = (unsigned*)take(sizeof(unsigned));
+    s.xnmax_d = (unsigned*)take(sizeof(unsigned) * B);
+    s.wnorm_d = (double*)take(sizeof(double) * B);
+    if (results) *results = (size_t)(p - base);
+    s.ell_d = (float*)take(sizeof(float) * B * s.d);
+    s.inv_ell = (float*)take(sizeof(float) * B * s.d);
+    s.sf2_d = (float*)take(sizeof(float) * B);
+    s.sn2_d = (float*)take(sizeof(float) * B);
+    return (size_t)(p - base);
+}
+
+// Where an array of the device block lies in its host image
 template <typename T>
-__global__ void w_times_y_kernel(const double* __restrict__ W, const T* __restrict__ y, int ystride, int n,
-                                 int npad, double* __restrict__ u)
-{
-    const int g = blockIdx.y;
-    const int row = blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
-    const int lane = threadIdx.x % 32;
-    if (row >= npad) return;
-    const double* Wr = W + (size_t)g * npad * npad + (size_t)row * npad;
-    double s = 0.0;
-    if (row < n)
-        for (int k = lane; k <= row; k += 32) s += Wr[k] * (double)y[(size_t)g * ystride + k];
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (lane == 0) u[(size_t)g * npad + row] = s;
-}
+T* mirror(const r3_fit_state& s, T* device, char* image) { return (T*)(image + ((char*)device - s.block)); }
 
-// alpha = W^T u in two steps so that n = 4096 still fills the GPU: the rows are cut into kRowSlabs
-// slabs, each block sums one slab for 128 columns (coalesced across columns), then the slabs are added
-// in a fixed order (deterministic).
-constexpr int kRowSlabs = 32;
-__global__ void wt_times_u_partial_kernel(const double* __restrict__ W, const double* __restrict__ u, int n,
-                                          int npad, double* __restrict__ partial)
-{
-    const int g = blockIdx.z, slab = blockIdx.y;
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= npad) return;
-    const int rows = (npad + kRowSlabs - 1) / kRowSlabs;
-    const int i0 = max(slab * rows, j), i1 = min(min((slab + 1) * rows, npad), n);
-    const double* Wg = W + (size_t)g * npad * npad;
-    double s = 0.0;
-    if (j < n)
-        for (int i = i0; i < i1; ++i) s += Wg[(size_t)i * npad + j] * u[(size_t)g * npad + i];
-    partial[((size_t)g * kRowSlabs + slab) * npad + j] = s;
-}
-
-__global__ void wt_times_u_reduce_kernel(const double* __restrict__ partial, int npad,
-                                         double* __restrict__ alpha64, float* __restrict__ alpha32)
-{
-    const int g = blockIdx.y;
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= npad) return;
-    double s = 0.0;
-    for (int r = 0; r < kRowSlabs; ++r) s += partial[((size_t)g * kRowSlabs + r) * npad + j];
-    alpha64[(size_t)g * npad + j] = s;
-    alpha32[(size_t)g * npad + j] = (float)s;
-}
-
-// Power iteration on W^T W: v holds the current vector (unit norm after the call), lam its norm
-// before normalisation, i.e. the current estimate of |W|_2^2.
-__global__ void power_init_kernel(double* __restrict__ v, int n, int npad)
-{
-    const int g = blockIdx.x;
-    for (int i = threadIdx.x; i < npad; i += blockDim.x)
-        v[(size_t)g * npad + i] = (i < n) ? (1.0 + 0.37 * ((i * 2654435761u >> 16) & 0xff) / 255.0) : 0.0;
-}
-
-__global__ void power_normalize_kernel(double* __restrict__ v, int npad, double* __restrict__ lam)
-{
-    __shared__ double s[256];
-    const int g = blockIdx.x;
-    double* vg = v + (size_t)g * npad;
-    double acc = 0.0;
-    for (int i = threadIdx.x; i < npad; i += 256) acc += vg[i] * vg[i];
-    s[threadIdx.x] = acc;
-    __syncthreads();
-    for (int o = 128; o > 0; o >>= 1) {
-        if (threadIdx.x < o) s[threadIdx.x] += s[threadIdx.x + o];
-        __syncthreads();
-    }
-    const double nrm = sqrt(s[0]);
-    if (threadIdx.x == 0) lam[g] = nrm;
-    const double inv = nrm > 0.0 ? 1.0 / nrm : 0.0;
-    for (int i = threadIdx.x; i < npad; i += 256) vg[i] *= inv;
-}
-
-__global__ void power_finish_kernel(const double* __restrict__ lam, double* __restrict__ wnorm, int batch)
-{
-    // lam ~ |W|_2^2 from below; 1.5 covers slow convergence
-    const int g = blockIdx.x * blockDim.x + threadIdx.x;
-    if (g < batch) wnorm[g] = 1.5 * sqrt(lam[g]);
-}
-
-__global__ void to_float_kernel(const double* __restrict__ a, float* __restrict__ b, size_t count)
-{
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < count;
-         i += (size_t)gridDim.x * blockDim.x)
-        b[i] = (float)a[i];
-}
-
-// From W and y: the estimate of |W|_2 (power iteration on W^T W; alpha64/alpha32 serve as scratch first),
-// alpha = W^T (W y) in FP64 and FP32, and W rounded to FP32.  u: [B][npad] scratch; slabs: [B + B*kRowSlabs*npad].
-r3_status_t finish_weights(int B, int n, int npad, const double* W64, const float* y, double* alpha64, float* alpha32,
-                           float* W32, double* wnorm_d, double* u, double* slabs, cudaStream_t stream)
-{
-    double* pv = alpha64;
-    double* lam = slabs;  // [B], followed by the row-slab partial sums
-    double* part = slabs + B;
-    R3_LAUNCH(power_init_kernel, B, 256, 0, stream, pv, n, npad);
-    R3_LAUNCH(power_normalize_kernel, B, 256, 0, stream, pv, npad, lam);
-    for (int it = 0; it < 12; ++it) {
-        R3_LAUNCH(w_times_y_kernel<double>, dim3((npad + 7) / 8, B), 256, 0, stream, W64, pv, npad, n, npad, u);
-        R3_LAUNCH(wt_times_u_partial_kernel, dim3((npad + 127) / 128, kRowSlabs, B), 128, 0, stream, W64, u, n, npad,
-                  part);
-        R3_LAUNCH(wt_times_u_reduce_kernel, dim3((npad + 127) / 128, B), 128, 0, stream, part, npad, pv, alpha32);
-        R3_LAUNCH(power_normalize_kernel, B, 256, 0, stream, pv, npad, lam);
-    }
-    R3_LAUNCH(power_finish_kernel, (B + 255) / 256, 256, 0, stream, lam, wnorm_d, B);
-    R3_LAUNCH(w_times_y_kernel<float>, dim3((npad + 7) / 8, B), 256, 0, stream, W64, y, n, n, npad, u);
-    R3_LAUNCH(wt_times_u_partial_kernel, dim3((npad + 127) / 128, kRowSlabs, B), 128, 0, stream, W64, u, n, npad, part);
-    R3_LAUNCH(wt_times_u_reduce_kernel, dim3((npad + 127) / 128, B), 128, 0, stream, part, npad, alpha64, alpha32);
-    R3_LAUNCH(to_float_kernel, 1184, 256, 0, stream, W64, W32, (size_t)B * npad * npad);
-    return R3_OK;
-}
+#define TRY_ST(expr)                                                                               \
+    do {                                                                                           \
+        cudaError_t e__ = (expr);                                                                  \
+        if (e__ != cudaSuccess) {                                                                  \
+            set_error("%s failed: %s", #expr, cudaGetErrorString(e__));                            \
+            return e__ == cudaErrorMemoryAllocation ? R3_ERR_ALLOC : R3_ERR_CUDA;                  \
+        }                                                                                          \
+    } while (0)
 
 }  // namespace
 
-// Runs the whole fit on `stream`.  gp->X, ell (device copies) and the scalar arrays are already in
-// place; L64, W64, W32, alpha*, best_d are filled.  The caller synchronises and reads status_d.
-r3_status_t fit_device(r3_gp* gp, const float* y, cudaStream_t stream)
+r3_status_t state_alloc(r3_fit_state& s)
 {
-    const int B = gp->batch, npad = gp->npad;
-    double *u = nullptr, *slabs = nullptr;
-    void* scratch = nullptr;
+    s.npad = round_up(s.n, kFitBlock);
+    const size_t B = s.batch, mat = (size_t)s.npad * s.npad;
+    r3_fit_state layout = s;
+    const size_t bytes = carve_block(layout, nullptr, nullptr);
+    char* block = nullptr;
+    TRY_ST(dev_malloc(&s.X, sizeof(float) * B * (size_t)s.n * s.d));
+    TRY_ST(dev_malloc(&s.y, sizeof(float) * B * (size_t)s.n));
+    TRY_ST(dev_malloc(&block, bytes));
+    carve_block(s, block, nullptr);
+    TRY_ST(dev_malloc(&s.L64, sizeof(double) * B * mat));
+    TRY_ST(dev_malloc(&s.W64, sizeof(double) * B * mat));
+    TRY_ST(dev_malloc(&s.W32, sizeof(float) * B * mat));
+    TRY_ST(dev_malloc(&s.alpha64, sizeof(double) * B * s.npad));
+    TRY_ST(dev_malloc(&s.alpha32, sizeof(float) * B * s.npad));
+    return R3_OK;
+}
+
+void state_free(r3_fit_state& s)
+{
+    tc_release(s);
+    dev_free(s.X);
+    dev_free(s.y);
+    dev_free(s.block);
+    dev_free(s.L64);
+    dev_free(s.W64);
+    dev_free(s.W32);
+    dev_free(s.alpha64);
+    dev_free(s.alpha32);
+    s = r3_fit_state();
+}
+
+r3_status_t state_fit(r3_gp* gp, r3_fit_state& s, int rows_done, bool full, bool need_tc, cudaStream_t stream, int* bits,
+                      int* pivot)
+{
+    const int B = s.batch, npad = s.npad;
+    void* ints = nullptr;
+    double* doubles = nullptr;
     auto done = [&](r3_status_t st) {
-        dev_free(u);
-        dev_free(slabs);
-        dev_free(scratch);
+        // on an error something may still be in flight on the stream
+        if (st != R3_OK) cudaStreamSynchronize(stream);
+        FreeScope no_wait;
+        dev_free(ints);
+        dev_free(doubles);
         return st;
     };
 #define TRY_DONE(expr)                                                                             \
@@ -150,22 +110,74 @@ r3_status_t fit_device(r3_gp* gp, const float* y, cudaStream_t stream)
             return done(e__ == cudaErrorMemoryAllocation ? R3_ERR_ALLOC : R3_ERR_CUDA);            \
         }                                                                                          \
     } while (0)
-    TRY_DONE(dev_malloc(&u, sizeof(double) * B * npad));
-    TRY_DONE(dev_malloc(&slabs, sizeof(double) * ((size_t)B + (size_t)B * kRowSlabs * npad)));
-    TRY_DONE(dev_malloc(&scratch, factor_scratch_bytes(B, npad)));
+    const size_t fbytes = factor_scratch_bytes(B, npad);
+    TRY_DONE(dev_malloc(&ints, fbytes + sizeof(unsigned) * B));
+    TRY_DONE(dev_malloc(&doubles, sizeof(double) * weights_scratch_doubles(B, npad)));
+
+    // the block: results cleared, hyper-parameters filled in
+    size_t results = 0;
+    const size_t bytes = carve_block(s, s.block, &results);
+    char* image = gp->stage_h;
+    if (bytes > kStageBytes) {
+        gp->image.resize(bytes);
+        image = gp->image.data();
+    }
+    memset(image, 0, results);
+    mirror(s, s.fit_status, image)[1] = INT_MAX;
+    memcpy(mirror(s, s.ell_d, image), gp->ell.data(), sizeof(float) * gp->ell.size());
+    float* inv = mirror(s, s.inv_ell, image);
+    for (size_t i = 0; i < gp->ell.size(); ++i) inv[i] = (float)(1.0 / (double)gp->ell[i]);
+    memcpy(mirror(s, s.sf2_d, image), gp->sf2.data(), sizeof(float) * B);
+    memcpy(mirror(s, s.sn2_d, image), gp->sn2.data(), sizeof(float) * B);
+    TRY_DONE(cudaMemcpyAsync(s.block, image, bytes, cudaMemcpyHostToDevice, stream));
+
     FactorProblem f;
-    f.X = gp->X; f.y = y; f.ell = gp->ell_d; f.sf2 = gp->sf2_d; f.sn2 = gp->sn2_d;
-    f.batch = B; f.n = gp->n; f.d = gp->d; f.npad = npad; f.rows_done = 0;
-    f.L = gp->L64; f.W = gp->W64;
-    f.best = gp->best_d; f.yabs = gp->yabs_d;
-    r3_status_t st = factor_device(f, scratch, gp->status_d, gp->device, stream);
+    f.X = s.X; f.y = s.y; f.ell = s.ell_d; f.sf2 = s.sf2_d; f.sn2 = s.sn2_d;
+    f.batch = B; f.n = s.n; f.d = s.d; f.npad = npad; f.rows_done = rows_done;
+    f.L = s.L64; f.W = s.W64;
+    f.best = s.best_d; f.yabs = s.yabs_d;
+    r3_status_t st = factor_device(f, ints, B, s.fit_status, gp->device, stream);
     if (st != R3_OK) return done(st);
-    st = finish_weights(B, gp->n, npad, gp->W64, y, gp->alpha64, gp->alpha32, gp->W32, gp->wnorm_d, u, slabs, stream);
+    WeightProblem w;
+    w.W = s.W64; w.y = s.y;
+    w.batch = B; w.n = s.n; w.npad = npad;
+    w.alpha64 = s.alpha64; w.alpha32 = s.alpha32;
+    w.W32 = full ? s.W32 : nullptr;
+    w.wnorm = full ? s.wnorm_d : nullptr;
+    w.wmax = full ? s.wmax_d : nullptr;
+    st = weights_device(w, doubles, (unsigned*)((char*)ints + fbytes), s.fit_status, gp->device, stream);
     if (st != R3_OK) return done(st);
-    TRY_DONE(cudaMemcpyAsync(gp->status_h, gp->status_d, 2 * sizeof(int), cudaMemcpyDeviceToHost, stream));
+    if (full) {
+        if (s.tc) {   // a refit: calls that still use the old operands end first
+            cudaDeviceSynchronize();
+            FreeScope no_wait;
+            tc_release(s);
+        }
+        if (tc_supported(s.n, s.d)) {
+            st = tc_prepare(s, gp->device, stream);
+            if (st != R3_OK && (need_tc || st != R3_ERR_ALLOC)) return done(st);
+        }
+    }
+    TRY_DONE(cudaMemcpyAsync(image, s.block, results, cudaMemcpyDeviceToHost, stream));
     TRY_DONE(cudaStreamSynchronize(stream));
 #undef TRY_DONE
-    return done(R3_OK);  // frees the temporaries
+    const int* fs = mirror(s, s.fit_status, image);
+    *bits = fs[0];
+    if (pivot) *pivot = fs[1];
+    if (fs[0] & DEV_TIMEOUT) {
+        set_error("a bounded device-side wait of the fit ran out");
+        return done(R3_ERR_DEVICE_TIMEOUT);
+    }
+    if (full) {
+        s.best.assign(mirror(s, s.best_d, image), mirror(s, s.best_d, image) + B);
+        s.y_absmax.assign(mirror(s, s.yabs_d, image), mirror(s, s.yabs_d, image) + B);
+        s.wnorm.assign(mirror(s, s.wnorm_d, image), mirror(s, s.wnorm_d, image) + B);
+        if (s.tc && !tc_accept(s, gp->sf2.data(), mirror(s, s.wmax_d, image), *mirror(s, s.xamax_d, image))) {
+            FreeScope no_wait;   // nothing has used them yet
+            tc_release(s);
+        }
+    }
+    return done(R3_OK);
 }
 
 // =====================================================================================================
@@ -174,108 +186,62 @@ r3_status_t fit_device(r3_gp* gp, const float* y, cudaStream_t stream)
 // against the fit's O(n^3 / 3), and the result is the one a fit of the concatenated history gives.
 namespace {
 
-// Rows [0, rows) of L and W of every GP into matrices with another leading dimension (the columns right of the copied
-// triangle are zeroed by the factorisation, or lie within the copied width and are zero there).
+// The old state's part of the new one, per GP: rows [0, rows) of L and W into matrices with another leading dimension
+// (blockIdx.z = 0, 1; the columns right of the copied triangle are zeroed by the factorisation, or lie within the copied
+// width and are zero there), old and new rows of X and y (blockIdx.z = 2).
 __global__ void embed_kernel(const double* __restrict__ L0, const double* __restrict__ W0, int np0, double* __restrict__ L1,
-                             double* __restrict__ W1, int np1, int rows)
+                             double* __restrict__ W1, int np1, int rows, const float* __restrict__ X0,
+                             const float* __restrict__ Xnew, const float* __restrict__ y0, const float* __restrict__ ynew,
+                             int n0, int k, int d, float* __restrict__ X1, float* __restrict__ y1)
 {
-    const int g = blockIdx.y, i = blockIdx.x;
+    const int g = blockIdx.y;
+    if (blockIdx.z == 2) {
+        const size_t n1 = n0 + k, old = (size_t)n0 * d, all = n1 * d, step = (size_t)gridDim.x * blockDim.x;
+        const size_t at = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
+        for (size_t e = at; e < all; e += step)
+            X1[g * all + e] = e < old ? X0[g * old + e] : Xnew[(size_t)g * k * d + (e - old)];
+        for (size_t e = at; e < n1; e += step) y1[g * n1 + e] = e < (size_t)n0 ? y0[(size_t)g * n0 + e] : ynew[(size_t)g * k + (e - n0)];
+        return;
+    }
+    const int i = blockIdx.x;
+    if (i >= rows) return;
     const double* src = (blockIdx.z ? W0 : L0) + (size_t)g * np0 * np0 + (size_t)i * np0;
     double* dst = (blockIdx.z ? W1 : L1) + (size_t)g * np1 * np1 + (size_t)i * np1;
     for (int c = 2 * threadIdx.x; c < rows; c += 2 * blockDim.x)
         *reinterpret_cast<double2*>(dst + c) = *reinterpret_cast<const double2*>(src + c);
 }
 
-struct AppendBuffers {
-    float *X = nullptr, *y = nullptr, *W32 = nullptr, *alpha32 = nullptr, *best = nullptr;   // best: [2][B]
-    double *L64 = nullptr, *W64 = nullptr, *alpha64 = nullptr, *u = nullptr, *slabs = nullptr, *wnorm = nullptr;
-    void* scratch = nullptr;
-    void release()
-    {
-        dev_free(X); dev_free(y); dev_free(W32); dev_free(alpha32); dev_free(L64); dev_free(W64); dev_free(alpha64);
-        dev_free(u); dev_free(slabs); dev_free(best); dev_free(wnorm); dev_free(scratch);
-        *this = AppendBuffers();
-    }
-};
-
 }  // namespace
 
-r3_status_t append_device(r3_gp* gp, const float* Xnew, const float* ynew, int k, cudaStream_t stream)
+r3_status_t append_device(r3_gp* gp, const float* Xnew, const float* ynew, int k, cudaStream_t stream, int* bits, int* pivot)
 {
-    const size_t xnew_gp_stride = (size_t)k * gp->d, ynew_gp_stride = (size_t)k;
-    const int B = gp->batch, d = gp->d, n0 = gp->n, n1 = n0 + k, np0 = gp->npad, np1 = round_up(n1, kFitBlock);
-    const size_t mat1 = (size_t)np1 * np1;
-    AppendBuffers nb;
-    auto fail = [&](r3_status_t st) {
-        nb.release();
+    r3_fit_state s;
+    s.batch = gp->batch;
+    s.d = gp->d;
+    s.n = gp->n + k;
+    auto drop = [&](r3_status_t st) {
+        cudaStreamSynchronize(stream);
+        FreeScope no_wait;
+        state_free(s);
         return st;
     };
-#define TRY_OR_FAIL(expr)                                                                          \
-    do {                                                                                           \
-        cudaError_t e__ = (expr);                                                                  \
-        if (e__ != cudaSuccess) {                                                                  \
-            set_error("%s failed: %s", #expr, cudaGetErrorString(e__));                            \
-            return fail(e__ == cudaErrorMemoryAllocation ? R3_ERR_ALLOC : R3_ERR_CUDA);            \
-        }                                                                                          \
-    } while (0)
-    TRY_OR_FAIL(dev_malloc(&nb.X, sizeof(float) * B * (size_t)n1 * d));
-    TRY_OR_FAIL(dev_malloc(&nb.y, sizeof(float) * B * (size_t)n1));
-    TRY_OR_FAIL(dev_malloc(&nb.L64, sizeof(double) * B * mat1));
-    TRY_OR_FAIL(dev_malloc(&nb.W64, sizeof(double) * B * mat1));
-    TRY_OR_FAIL(dev_malloc(&nb.W32, sizeof(float) * B * mat1));
-    TRY_OR_FAIL(dev_malloc(&nb.alpha64, sizeof(double) * B * np1));
-    TRY_OR_FAIL(dev_malloc(&nb.alpha32, sizeof(float) * B * np1));
-    TRY_OR_FAIL(dev_malloc(&nb.u, sizeof(double) * B * np1));
-    TRY_OR_FAIL(dev_malloc(&nb.slabs, sizeof(double) * ((size_t)B + (size_t)B * kRowSlabs * np1)));
-    TRY_OR_FAIL(dev_malloc(&nb.best, sizeof(float) * 2 * B));
-    TRY_OR_FAIL(dev_malloc(&nb.wnorm, sizeof(double) * B));
-    TRY_OR_FAIL(dev_malloc(&nb.scratch, factor_scratch_bytes(B, np1)));
-
-    // histories: old rows then new rows, per GP
-    TRY_OR_FAIL(cudaMemcpy2DAsync(nb.X, sizeof(float) * (size_t)n1 * d, gp->X, sizeof(float) * (size_t)n0 * d,
-                                  sizeof(float) * (size_t)n0 * d, B, cudaMemcpyDeviceToDevice, stream));
-    TRY_OR_FAIL(cudaMemcpy2DAsync(nb.X + (size_t)n0 * d, sizeof(float) * (size_t)n1 * d, Xnew,
-                                  sizeof(float) * xnew_gp_stride, sizeof(float) * (size_t)k * d, B,
-                                  cudaMemcpyDeviceToDevice, stream));
-    TRY_OR_FAIL(cudaMemcpy2DAsync(nb.y, sizeof(float) * n1, gp->y, sizeof(float) * n0, sizeof(float) * n0, B,
-                                  cudaMemcpyDeviceToDevice, stream));
-    TRY_OR_FAIL(cudaMemcpy2DAsync(nb.y + n0, sizeof(float) * n1, ynew, sizeof(float) * ynew_gp_stride, sizeof(float) * k,
-                                  B, cudaMemcpyDeviceToDevice, stream));
-    const int kept = n0 / kFactorTile * kFactorTile;   // rows of whole tiles of old observations
-    if (kept > 0) {
-        embed_kernel<<<dim3(kept, B, 2), 128, 0, stream>>>(gp->L64, gp->W64, np0, nb.L64, nb.W64, np1, kept);
-        ++g_launches;
-        TRY_OR_FAIL(cudaGetLastError());
+    r3_status_t st = state_alloc(s);
+    if (st != R3_OK) return drop(st);
+    const int kept = gp->n / kFactorTile * kFactorTile;   // rows of whole tiles of old observations
+    embed_kernel<<<dim3(std::max(kept, 64), s.batch, 3), 128, 0, stream>>>(gp->L64, gp->W64, gp->npad, s.L64, s.W64, s.npad,
+                                                                           kept, gp->X, Xnew, gp->y, ynew, gp->n, k, s.d, s.X, s.y);
+    ++g_launches;
+    if (cudaError_t e = cudaGetLastError(); e != cudaSuccess) {
+        set_error("launch of embed_kernel failed: %s", cudaGetErrorString(e));
+        return drop(R3_ERR_CUDA);
     }
-    FactorProblem f;
-    f.X = nb.X; f.y = nb.y; f.ell = gp->ell_d; f.sf2 = gp->sf2_d; f.sn2 = gp->sn2_d;
-    f.batch = B; f.n = n1; f.d = d; f.npad = np1; f.rows_done = kept;
-    f.L = nb.L64; f.W = nb.W64;
-    f.best = nb.best; f.yabs = nb.best + B;
-    r3_status_t st = factor_device(f, nb.scratch, gp->status_d, gp->device, stream);
-    if (st != R3_OK) return fail(st);
-    st = finish_weights(B, n1, np1, nb.W64, nb.y, nb.alpha64, nb.alpha32, nb.W32, nb.wnorm, nb.u, nb.slabs, stream);
-    if (st != R3_OK) return fail(st);
-    TRY_OR_FAIL(cudaMemcpyAsync(gp->status_h, gp->status_d, 2 * sizeof(int), cudaMemcpyDeviceToHost, stream));
-    TRY_OR_FAIL(cudaStreamSynchronize(stream));
-#undef TRY_OR_FAIL
-    if (gp->status_h[0] & (DEV_NOT_PD | DEV_NONFINITE | DEV_TIMEOUT)) return fail(R3_OK);   // the caller reports; nothing swapped
-    // success: the new arrays replace the old ones
-    if (cudaMemcpy(gp->best_d, nb.best, sizeof(float) * B, cudaMemcpyDeviceToDevice) != cudaSuccess ||
-        cudaMemcpy(gp->yabs_d, nb.best + B, sizeof(float) * B, cudaMemcpyDeviceToDevice) != cudaSuccess ||
-        cudaMemcpy(gp->wnorm_d, nb.wnorm, sizeof(double) * B, cudaMemcpyDeviceToDevice) != cudaSuccess) {
-        set_error("r3_gp_append: copying the incumbent failed");
-        return fail(R3_ERR_CUDA);
-    }
-    dev_free(gp->X); dev_free(gp->y); dev_free(gp->L64); dev_free(gp->W64); dev_free(gp->W32);
-    dev_free(gp->alpha64); dev_free(gp->alpha32);
-    gp->X = nb.X; gp->y = nb.y; gp->L64 = nb.L64; gp->W64 = nb.W64; gp->W32 = nb.W32;
-    gp->alpha64 = nb.alpha64; gp->alpha32 = nb.alpha32;
-    nb.X = nullptr; nb.y = nullptr; nb.L64 = nullptr; nb.W64 = nullptr; nb.W32 = nullptr;
-    nb.alpha64 = nullptr; nb.alpha32 = nullptr;
-    nb.release();
-    gp->n = n1;
-    gp->npad = np1;
+    st = state_fit(gp, s, kept, true, false, stream, bits, pivot);
+    if (st != R3_OK || (*bits & (DEV_NOT_PD | DEV_NONFINITE))) return drop(st);   // the caller reports; nothing swapped
+    // success: the new state takes the old one's place (calls that still use the old one end first)
+    cudaDeviceSynchronize();
+    FreeScope no_wait;
+    std::swap(static_cast<r3_fit_state&>(*gp), s);
+    state_free(s);
     return R3_OK;
 }
 

@@ -81,8 +81,18 @@ inline cudaError_t dev_malloc(T** p, size_t bytes)
     return dev_malloc_bytes(reinterpret_cast<void**>(p), bytes);
 }
 void dev_free(void* p);
+// While one lives, dev_free on this thread does not wait for the device: whoever opens it knows that nothing in flight
+// still uses what is freed (temporaries after their stream has been synchronised).
+struct FreeScope {
+    FreeScope();
+    ~FreeScope();
+    FreeScope(const FreeScope&) = delete;
+    FreeScope& operator=(const FreeScope&) = delete;
+};
 void trim_cache();
-constexpr int kPinnedInts = 128;
+constexpr int kPinnedInts = 1024;
+constexpr int kStageInt = 128;       // where a handle's staging area begins in its pinned block
+constexpr size_t kStageBytes = sizeof(int) * (kPinnedInts - kStageInt);
 int* pinned_word_acquire();          // kPinnedInts pinned host ints from a process-wide pool (nullptr on failure)
 void pinned_word_release(int* w);
 size_t cached_bytes();
@@ -102,35 +112,49 @@ struct TopkRequest {
     size_t ws_bytes = 0;
 };
 
-// The handle.  Device arrays are allocated at fit time and freed by r3_gp_free.
-struct r3_gp {
+// Everything a fit produces.  A handle is one of these and what goes with it; r3_gp_append builds the next one beside
+// the handle's and puts it in its place.
+struct r3_fit_state {
     int batch = 0, n = 0, d = 0;
     int npad = 0;              // n rounded up to kFitBlock; padded rows/cols are identity / zero
-    int device = 0;
-    std::vector<float> ell, sf2, sn2, best;   // host copies [batch][d], [batch], [batch], [batch]
-    std::vector<float> y_absmax;              // [batch] max |y|
+    std::vector<float> best, y_absmax;        // host copies [batch]: incumbent, max |y|
     std::vector<double> wnorm;                // [batch] estimate of |L^-1|_2 (power iteration x 1.5)
 
     float* X = nullptr;        // [batch][n][d]   raw observations (FP32 as given)
     float* y = nullptr;        // [batch][n]      observed values as given (kept for r3_gp_append)
-    float* ell_d = nullptr;    // [batch][d]      lengthscales as given
-    float* inv_ell = nullptr;  // [batch][d]      1/lengthscale
-    float* sn2_d = nullptr;    // [batch]
-    float* sf2_d = nullptr;    // [batch]
-    float* best_d = nullptr;   // [batch]
-    float* yabs_d = nullptr;   // [batch] max |y|
-    double* wnorm_d = nullptr; // [batch]
     double* L64 = nullptr;     // [batch][npad][npad] lower Cholesky factor (upper part zero)
     double* W64 = nullptr;     // [batch][npad][npad] W = L^-1, lower
     float* W32 = nullptr;      // [batch][npad][npad] W rounded to FP32
     double* alpha64 = nullptr; // [batch][npad]  (zero in the padding)
     float* alpha32 = nullptr;  // [batch][npad]
-    int* status_d = nullptr;   // [4]: status bits, first bad pivot index, line of a failed index check, unused
+
+    // the small arrays, in one block that a fit uploads and whose first part it reads back
+    char* block = nullptr;
+    int* fit_status = nullptr; // [4] status bits, first bad pivot index
+    float* best_d = nullptr;   // [batch]
+    float* yabs_d = nullptr;   // [batch] max |y|
+    unsigned* wmax_d = nullptr;   // [batch] bits of max |W|
+    unsigned* xamax_d = nullptr;  // bits of the largest scaled coordinate
+    unsigned* xnmax_d = nullptr;  // [batch] bits of max |x~|^2
+    double* wnorm_d = nullptr; // [batch]
+    float* ell_d = nullptr;    // [batch][d]      lengthscales as given
+    float* inv_ell = nullptr;  // [batch][d]      1/lengthscale
+    float* sf2_d = nullptr;    // [batch]
+    float* sn2_d = nullptr;    // [batch]
+
+    // tensor-core operands (built by the fit when the tensor engine can serve (n, d))
+    void* tc = nullptr;        // r3::TensorOperands*, see r3_score_tc.cu
+};
+
+// The handle.  Device arrays are allocated at fit time and freed by r3_gp_free.
+struct r3_gp : r3_fit_state {
+    int device = 0;
+    std::vector<float> ell, sf2, sn2;         // host copies [batch][d], [batch], [batch]
+    int* status_d = nullptr;   // [4]: status bits of the scoring calls, pivot, line of a failed index check, unused
     int* status_h = nullptr;   // pinned mirror of status_d
     int* rescued_h = nullptr;  // pinned [64]: candidates recomputed in FP64 by the last scoring call, per GP
-
-    // tensor-core operands (built by fit when the tensor engine can serve (n, d))
-    void* tc = nullptr;        // r3::TensorOperands*, see r3_score_tc.cu
+    char* stage_h = nullptr;   // pinned [kStageBytes]: uploads and read-backs of a fit's block
+    std::vector<char> image;   // the same for blocks that do not fit there
 
     // grow-only private workspace used by scoring and top-k
     void* ws = nullptr;
@@ -166,13 +190,37 @@ struct FactorProblem {
 };
 size_t factor_scratch_bytes(int batch, int npad);
 // Asynchronous; non-finite inputs and non-positive pivots are latched in `status`.
-r3_status_t factor_device(const FactorProblem& p, void* scratch, int* status, int device, cudaStream_t stream);
+// `scratch`: factor_scratch_bytes, followed by extra_ints more ints that are cleared with it.
+r3_status_t factor_device(const FactorProblem& p, void* scratch, int extra_ints, int* status, int device, cudaStream_t stream);
+
+// weights, norm estimate and FP32 copy of the inverse factor (r3_weights.cu)
+struct WeightProblem {
+    const double* W;        // [batch][npad][npad]
+    const float* y;         // [batch][n]
+    int batch, n, npad;
+    double* alpha64;        // [batch][npad]
+    float* alpha32;         // [batch][npad]
+    float* W32;             // [batch][npad][npad], or nullptr
+    double* wnorm;          // [batch], or nullptr: weights only
+    unsigned* wmax;         // [batch] bits of max |W|, zero on entry, or nullptr
+};
+size_t weights_scratch_doubles(int batch, int npad);
+// barrier: [batch] words, zero on entry.  Asynchronous.
+r3_status_t weights_device(const WeightProblem& p, double* scratch, unsigned* barrier, int* status, int device,
+                           cudaStream_t stream);
 
 // fit (r3_fit.cu)
-r3_status_t fit_device(r3_gp* gp, const float* y, cudaStream_t stream);
+r3_status_t state_alloc(r3_fit_state& s);    // arrays for s.batch, s.n, s.d
+void state_free(r3_fit_state& s);
+// The fit of s (histories in place, hyper-parameters from gp's host copies), rows below rows_done of L and W given.
+// full: everything a handle needs, tensor operands included; otherwise L, W, alpha and the status only (an evaluation of
+// the evidence).  Synchronises; *bits and *pivot are what the device found.  need_tc: a failed allocation of the tensor
+// operands is an error (otherwise the CUDA-core engine serves the state).
+r3_status_t state_fit(r3_gp* gp, r3_fit_state& s, int rows_done, bool full, bool need_tc, cudaStream_t stream, int* bits,
+                      int* pivot);
 // Appends k observations per GP (r3_gp_append): extends L, W, alpha, X, y in O(k n^2); synchronises.  On
-// any error the handle is left as it was.
-r3_status_t append_device(r3_gp* gp, const float* Xnew, const float* ynew, int k, cudaStream_t stream);
+// any error (and when *bits says so) the handle is left as it was.
+r3_status_t append_device(r3_gp* gp, const float* Xnew, const float* ynew, int k, cudaStream_t stream, int* bits, int* pivot);
 
 // SIMT scoring (r3_score_simt.cu)
 size_t score_simt_workspace_bytes(const r3_gp* gp, long long m);
@@ -206,8 +254,12 @@ r3_status_t guard_and_rescue(r3_gp* gp, const float* Xcand, long long m, const G
 
 // tensor-core scoring (r3_score_tc.cu)
 bool tc_supported(int n, int d);
-r3_status_t tc_prepare(r3_gp* gp, cudaStream_t stream);
-void tc_release(r3_gp* gp);
+// Allocates the tensor operands of a state whose weights are under way on `stream` and launches their preparation;
+// s.tc stays nullptr when no shape fits.  tc_accept, after the stream has been synchronised and the block read back:
+// false when the values do not suit the FP16 planes (the caller releases the operands and the CUDA-core engine serves).
+r3_status_t tc_prepare(r3_fit_state& s, int device, cudaStream_t stream);
+bool tc_accept(const r3_fit_state& s, const float* sf2, const unsigned* wmax, unsigned xamax);
+void tc_release(r3_fit_state& s);
 void tc_info(const r3_gp* gp, int* info);   // r3_gp_tensor_info
 size_t score_tc_workspace_bytes(const r3_gp* gp, long long m);
 r3_status_t score_tc(r3_gp* gp, const float* Xcand, long long m, float* mu, float* sigma, float* ei,

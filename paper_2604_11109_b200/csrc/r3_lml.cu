@@ -225,6 +225,8 @@ r3_status_t lml_device(r3_gp* gp, double* out_h, cudaStream_t stream)
     const int t32 = (n + 31) / 32, tiles = t32 * (t32 + 1) / 2;
     double *M = nullptr, *partial = nullptr, *out = nullptr;
     auto done = [&](r3_status_t st) {
+        if (st != R3_OK) cudaStreamSynchronize(stream);   // otherwise it has been
+        FreeScope no_wait;
         dev_free(M);
         dev_free(partial);
         dev_free(out);

@@ -16,47 +16,6 @@ namespace r3 {
 
 namespace {
 
-// Uploads the handle's host hyper-parameters, refits, returns the latched status bits in *bits.
-r3_status_t refit_device(r3_gp* gp, cudaStream_t stream, int* bits, int* pivot = nullptr)
-{
-    const int B = gp->batch, d = gp->d;
-    std::vector<float> inv((size_t)B * d);
-    for (size_t i = 0; i < inv.size(); ++i) inv[i] = (float)(1.0 / (double)gp->ell[i]);
-    gp->status_h[0] = 0;
-    gp->status_h[1] = INT_MAX;
-    R3_CUDA_TRY(cudaMemcpyAsync(gp->status_d, gp->status_h, 2 * sizeof(int), cudaMemcpyHostToDevice, stream));
-    R3_CUDA_TRY(cudaMemcpyAsync(gp->ell_d, gp->ell.data(), sizeof(float) * B * d, cudaMemcpyHostToDevice, stream));
-    R3_CUDA_TRY(cudaMemcpyAsync(gp->inv_ell, inv.data(), sizeof(float) * B * d, cudaMemcpyHostToDevice, stream));
-    R3_CUDA_TRY(cudaMemcpyAsync(gp->sf2_d, gp->sf2.data(), sizeof(float) * B, cudaMemcpyHostToDevice, stream));
-    R3_CUDA_TRY(cudaMemcpyAsync(gp->sn2_d, gp->sn2.data(), sizeof(float) * B, cudaMemcpyHostToDevice, stream));
-    R3_CUDA_TRY(cudaStreamSynchronize(stream));   // `inv` is a pageable temporary
-    const r3_status_t st = fit_device(gp, gp->y, stream);   // synchronises, fills status_h
-    if (st != R3_OK) return st;
-    if (gp->status_h[0] & DEV_TIMEOUT) {
-        set_error("a bounded device-side wait ran out");
-        return R3_ERR_DEVICE_TIMEOUT;
-    }
-    *bits = gp->status_h[0];
-    if (pivot) *pivot = gp->status_h[1];
-    if (*bits & (DEV_NOT_PD | DEV_NONFINITE)) {
-        gp->status_h[0] = 0;
-        gp->status_h[1] = INT_MAX;
-        R3_CUDA_TRY(cudaMemcpy(gp->status_d, gp->status_h, 2 * sizeof(int), cudaMemcpyHostToDevice));
-    }
-    return R3_OK;
-}
-
-// After the last refit: host copies of the incumbent and the norm estimate, tensor-engine operands.
-r3_status_t refresh_after_fit(r3_gp* gp, cudaStream_t stream)
-{
-    R3_CUDA_TRY(cudaMemcpy(gp->best.data(), gp->best_d, sizeof(float) * gp->batch, cudaMemcpyDeviceToHost));
-    R3_CUDA_TRY(cudaMemcpy(gp->y_absmax.data(), gp->yabs_d, sizeof(float) * gp->batch, cudaMemcpyDeviceToHost));
-    R3_CUDA_TRY(cudaMemcpy(gp->wnorm.data(), gp->wnorm_d, sizeof(double) * gp->batch, cudaMemcpyDeviceToHost));
-    tc_release(gp);
-    if (tc_supported(gp->n, gp->d)) return tc_prepare(gp, stream);
-    return R3_OK;
-}
-
 // Minimises F = -lml over a box by L-BFGS with backtracking; the caller evaluates the points it asks for.
 class Lbfgs {
 public:
@@ -251,20 +210,20 @@ r3_status_t r3_gp_refit(r3_gp_t* gp, const float* lengthscales, const float* sig
     gp->sf2.assign(signal_var, signal_var + B);
     gp->sn2.assign(noise_var, noise_var + B);
     int bits = 0, pivot = 0;
-    r3_status_t st = refit_device(gp, stream, &bits, &pivot);
+    r3_status_t st = state_fit(gp, *gp, 0, true, true, stream, &bits, &pivot);
     if (st != R3_OK) return st;
     if (bits & DEV_NOT_PD) {
         gp->ell = ell0;
         gp->sf2 = sf0;
         gp->sn2 = sn0;
-        st = refit_device(gp, stream, &bits);
-        if (st == R3_OK) st = refresh_after_fit(gp, stream);
+        int bits0 = 0;
+        st = state_fit(gp, *gp, 0, true, true, stream, &bits0, nullptr);
         if (st != R3_OK) return st;
         set_error("r3_gp_refit: K + noise*I is not positive definite with these hyper-parameters (pivot %d); the "
                   "previous ones were kept", pivot);
         return R3_ERR_NOT_PD;
     }
-    return refresh_after_fit(gp, stream);
+    return R3_OK;
 }
 
 r3_status_t r3_gp_optimize(r3_gp_t* gp, int max_evals, double gtol, float* lengthscales, float* signal_var,
@@ -315,7 +274,7 @@ r3_status_t r3_gp_optimize(r3_gp_t* gp, int max_evals, double gtol, float* lengt
         if (!any) break;
         load(false);
         int bits = 0;
-        st = refit_device(gp, stream, &bits);
+        st = state_fit(gp, *gp, 0, false, false, stream, &bits, nullptr);
         if (st != R3_OK) return st;
         ++used;
         const bool ok = !(bits & (DEV_NOT_PD | DEV_NONFINITE));
@@ -332,14 +291,12 @@ r3_status_t r3_gp_optimize(r3_gp_t* gp, int max_evals, double gtol, float* lengt
     // leave the handle at the best point of every GP
     load(true);
     int bits = 0;
-    st = refit_device(gp, stream, &bits);
+    st = state_fit(gp, *gp, 0, true, true, stream, &bits, nullptr);
     if (st != R3_OK) return st;
     if (bits & (DEV_NOT_PD | DEV_NONFINITE)) {
         set_error("r3_gp_optimize: the starting hyper-parameters do not give a positive definite covariance matrix");
         return R3_ERR_NOT_PD;
     }
-    st = refresh_after_fit(gp, stream);
-    if (st != R3_OK) return st;
     for (int g = 0; g < B; ++g) {
         if (lengthscales)
             for (int j = 0; j < d; ++j) lengthscales[(size_t)g * d + j] = gp->ell[(size_t)g * d + j];

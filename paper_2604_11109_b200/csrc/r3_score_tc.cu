@@ -41,6 +41,7 @@
 #include <math.h>
 #include <stdio.h>
 #include <stdlib.h>
+#include <string.h>
 
 #include "r3_epilogue.cuh"
 #include "r3_internal.cuh"
@@ -967,9 +968,11 @@ __global__ void centre_kernel(const float* __restrict__ X, const float* __restri
 __global__ void xt_build_kernel(const float* __restrict__ X, const float* __restrict__ centre,
                                 const float* __restrict__ scale, const float* __restrict__ alpha32, int n, int d,
                                 int npad_fit, int DP, int NP, int KD, __half* __restrict__ xt,
-                                float* __restrict__ xs32, float* __restrict__ xnorm, float* __restrict__ alpha, unsigned* __restrict__ xamax_bits)
+                                float* __restrict__ xs32, float* __restrict__ xnorm, float* __restrict__ alpha, unsigned* __restrict__ xamax_bits,
+                                unsigned* __restrict__ xnmax_bits)
 {
     const int g = blockIdx.y, c = blockIdx.x;
+    float nmax = 0.f;
     __half* blob = xt + ((size_t)g * (NP / KD) + c) * (2 * DP * KD);
     const float* cen = centre + (size_t)g * DP;
     const float* scl = scale + (size_t)g * DP;
@@ -997,36 +1000,21 @@ __global__ void xt_build_kernel(const float* __restrict__ X, const float* __rest
                 nrm += (double)xv * (double)xv;
             }
         xnorm[(size_t)g * NP + k] = (float)nrm;
+        nmax = fmaxf(nmax, (float)nrm);
         alpha[(size_t)g * NP + k] = (k < n) ? alpha32[(size_t)g * npad_fit + k] : 0.f;
     }
+    const unsigned top = __reduce_max_sync(0xffffffffu, __float_as_uint(nmax));   // order-preserving for nmax >= 0
+    if ((threadIdx.x & 31) == 0) atomicMax(xnmax_bits + g, top);
 }
 
-__global__ void xnmax_kernel(const float* __restrict__ xnorm, int NP, float* __restrict__ xnmax)
+// Powers of two that the operands of the variance product are multiplied by: 2^sw W and 2^sk k*.
+__host__ __device__ inline void operand_scales(float wmax, float sf2, bool f8, int& sw, int& sk)
 {
-    __shared__ float s[256];
-    float v = 0.f;
-    for (int i = threadIdx.x; i < NP; i += 256) v = fmaxf(v, xnorm[(size_t)blockIdx.x * NP + i]);
-    s[threadIdx.x] = v;
-    __syncthreads();
-    for (int o = 128; o > 0; o >>= 1) {
-        if (threadIdx.x < o) s[threadIdx.x] = fmaxf(s[threadIdx.x], s[threadIdx.x + o]);
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) xnmax[blockIdx.x] = s[0];
-}
-
-// Largest |W| entry of each GP (bit pattern of a non-negative float, so atomicMax orders it).
-__global__ void wmax_kernel(const double* __restrict__ W64, int n, int npad_fit, unsigned* __restrict__ wmax_bits)
-{
-    const int g = blockIdx.y;
-    const double* Wg = W64 + (size_t)g * npad_fit * npad_fit;
-    float v = 0.f;
-    for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < (size_t)n * n; e += (size_t)gridDim.x * blockDim.x) {
-        const int i = (int)(e / n), k = (int)(e % n);
-        if (k <= i) v = fmaxf(v, fabsf((float)Wg[(size_t)i * npad_fit + k]));
-    }
-    for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
-    if ((threadIdx.x & 31) == 0) atomicMax(&wmax_bits[g], __float_as_uint(v));
+    int ew = 0, ek = 0;
+    frexp((double)wmax, &ew);   // wmax < 2^ew
+    frexp((double)sf2, &ek);    // sf2  < 2^ek  (k* <= sf2)
+    sw = (f8 ? kScaleExpF8 : kScaleExp) - ew;
+    sk = kScaleExp - ek;
 }
 
 // One block per (chunk c, pass p, GP): the KC x NV block of 2^eW W (rows p NV.., columns c KC..) as
@@ -1035,7 +1023,8 @@ __global__ void wmax_kernel(const double* __restrict__ W64, int n, int npad_fit,
 // layout (16 k-elements per 16-byte slice): the hi parts as E4M3 (|2^eW W| < 2^8 for these histories), then the
 // lo parts as E5M2.
 __global__ void wt_build_kernel(const double* __restrict__ W64, int n, int npad_fit, int NV, size_t gp_stride,
-                                const float* __restrict__ wscale, __half* __restrict__ wt, bool f8)
+                                const unsigned* __restrict__ wmax, const float* __restrict__ sf2, float* __restrict__ kscale,
+                                double* __restrict__ vinv2, __half* __restrict__ wt, bool f8)
 {
     const int c = blockIdx.x, p = blockIdx.y, g = blockIdx.z;
     const int CPP = NV / KC;
@@ -1043,7 +1032,13 @@ __global__ void wt_build_kernel(const double* __restrict__ W64, int n, int npad_
     const size_t tile = (size_t)CPP * p * (p + 1) / 2 + c;
     __half* dst = wt + (size_t)g * gp_stride + tile * (2 * KC * NV);
     const double* Wg = W64 + (size_t)g * npad_fit * npad_fit;
-    const double sc = (double)wscale[g];
+    int sw, sk;
+    operand_scales(__uint_as_float(wmax[g]), sf2[g], f8, sw, sk);
+    const double sc = ldexp(1.0, sw);
+    if (c == 0 && p == 0 && threadIdx.x == 0) {
+        kscale[g] = (float)ldexp(1.0, sk);
+        vinv2[g] = ldexp(1.0, -2 * (sw + sk));
+    }
     for (int e = threadIdx.x; e < KC * NV; e += blockDim.x) {
         const int kk = e % KC, r = e / KC;   // consecutive threads walk k: coalesced reads of a W row
         const int i = p * NV + r, k = c * KC + kk;
@@ -1064,7 +1059,7 @@ __global__ void wt_build_kernel(const double* __restrict__ W64, int n, int npad_
     }
 }
 
-TensorOperands* ops_of(const r3_gp* gp) { return static_cast<TensorOperands*>(gp->tc); }
+TensorOperands* ops_of(const r3_fit_state* gp) { return static_cast<TensorOperands*>(gp->tc); }
 
 void (*kernel_for(int NV, int G, bool kt, int nbk, bool f8, bool putoff, bool zs))(const TcParams)
 {
@@ -1103,33 +1098,32 @@ int env_int(const char* name, int fallback)
 
 bool tc_supported(int n, int d) { return n >= 1 && n <= kMaxN && d >= 1 && d <= 128; }
 
-void tc_release(r3_gp* gp)
+void tc_release(r3_fit_state& st)
 {
-    TensorOperands* t = ops_of(gp);
+    TensorOperands* t = ops_of(&st);
     if (!t) return;
     dev_free(t->centre);
     dev_free(t->scale);
     dev_free(t->xt);
     dev_free(t->xs32);
     dev_free(t->xnorm);
-    dev_free(t->xnmax);
     dev_free(t->alpha);
     dev_free(t->wt);
     dev_free(t->kscale);
     dev_free(t->vinv2);
     delete t;
-    gp->tc = nullptr;
+    st.tc = nullptr;
 }
 
-r3_status_t tc_prepare(r3_gp* gp, cudaStream_t stream)
+r3_status_t tc_prepare(r3_fit_state& st, int device, cudaStream_t stream)
 {
-    const int B = gp->batch, n = gp->n, d = gp->d;
+    const int B = st.batch, n = st.n, d = st.d;
     TensorOperands* t = new (std::nothrow) TensorOperands;
     if (!t) {
         set_error("out of host memory");
         return R3_ERR_ALLOC;
     }
-    gp->tc = t;
+    st.tc = t;
     t->DP = round_up(d, 16);
     t->NV = n > 128 ? 256 : 128;
     t->NP = round_up(n, t->NV);
@@ -1165,7 +1159,7 @@ r3_status_t tc_prepare(r3_gp* gp, cudaStream_t stream)
         found = t->ws >= pr.min_ws;
     }
     if (!found) {
-        tc_release(gp);   // does not fit: the SIMT engine serves this shape
+        tc_release(st);   // does not fit: the SIMT engine serves this shape
         return R3_OK;
     }
     t->smem_bytes = smem_map(t->DP, t->NV, t->G, t->KD, t->ws, t->kt).bar + kBarBytes + 1024;
@@ -1175,20 +1169,12 @@ r3_status_t tc_prepare(r3_gp* gp, cudaStream_t stream)
     const int CPP = t->NV / KC;
     const size_t tiles = (size_t)CPP * t->P * (t->P + 1) / 2;
     t->wt_gp_stride = tiles * (2 * (size_t)KC * t->NV);
-    unsigned* wmax_bits = nullptr;
-    float* wscale_d = nullptr;
     auto fail = [&](const char* what, cudaError_t e) {
         set_error("%s failed: %s", what, cudaGetErrorString(e));
-        dev_free(wmax_bits);
-        dev_free(wscale_d);
-        tc_release(gp);
+        cudaStreamSynchronize(stream);
+        FreeScope no_wait;
+        tc_release(st);
         return e == cudaErrorMemoryAllocation ? R3_ERR_ALLOC : R3_ERR_CUDA;
-    };
-    auto decline = [&]() {   // the SIMT engine serves this history
-        dev_free(wmax_bits);
-        dev_free(wscale_d);
-        tc_release(gp);
-        return R3_OK;
     };
     cudaError_t e;
     if ((e = dev_malloc(&t->centre, sizeof(float) * B * t->DP)) != cudaSuccess) return fail("cudaMalloc", e);
@@ -1197,71 +1183,54 @@ r3_status_t tc_prepare(r3_gp* gp, cudaStream_t stream)
         return fail("cudaMalloc", e);
     if ((e = dev_malloc(&t->xs32, sizeof(float) * B * (size_t)t->NP * t->DP)) != cudaSuccess) return fail("cudaMalloc", e);
     if ((e = dev_malloc(&t->xnorm, sizeof(float) * B * t->NP)) != cudaSuccess) return fail("cudaMalloc", e);
-    if ((e = dev_malloc(&t->xnmax, sizeof(float) * (B > 2 ? B : 2))) != cudaSuccess) return fail("cudaMalloc", e);
     if ((e = dev_malloc(&t->alpha, sizeof(float) * B * t->NP)) != cudaSuccess) return fail("cudaMalloc", e);
     if ((e = dev_malloc(&t->wt, sizeof(__half) * B * t->wt_gp_stride)) != cudaSuccess) return fail("cudaMalloc", e);
     if ((e = dev_malloc(&t->kscale, sizeof(float) * B)) != cudaSuccess) return fail("cudaMalloc", e);
     if ((e = dev_malloc(&t->vinv2, sizeof(double) * B)) != cudaSuccess) return fail("cudaMalloc", e);
-    if ((e = dev_malloc(&wmax_bits, sizeof(unsigned) * B)) != cudaSuccess) return fail("cudaMalloc", e);
-    if ((e = dev_malloc(&wscale_d, sizeof(float) * B)) != cudaSuccess) return fail("cudaMalloc", e);
+    t->xnmax = reinterpret_cast<float*>(st.xnmax_d);   // lives in the state's block
 
-    // scaled observations (their largest coordinate decides whether the FP16 planes can hold them) and
-    // the largest |W| of each GP (it decides the power-of-two scale of its W planes)
-    unsigned* xamax_bits = reinterpret_cast<unsigned*>(t->xnmax);   // borrowed until xnmax_kernel overwrites it
-    if ((e = cudaMemsetAsync(xamax_bits, 0, sizeof(unsigned), stream)) != cudaSuccess) return fail("cudaMemsetAsync", e);
-    if ((e = cudaMemsetAsync(wmax_bits, 0, sizeof(unsigned) * B, stream)) != cudaSuccess) return fail("cudaMemsetAsync", e);
-    centre_kernel<<<dim3(t->DP, B), 256, 0, stream>>>(gp->X, gp->inv_ell, n, d, t->DP, t->centre, t->scale);
-    xt_build_kernel<<<dim3(t->NP / t->KD, B), 256, 0, stream>>>(gp->X, t->centre, t->scale, gp->alpha32, n, d, gp->npad,
-                                                                t->DP, t->NP, t->KD, t->xt, t->xs32, t->xnorm, t->alpha, xamax_bits);
-    wmax_kernel<<<dim3(296, B), 256, 0, stream>>>(gp->W64, n, gp->npad, wmax_bits);
+    // scaled observations (their largest coordinate decides whether the FP16 planes can hold them), then the planes of W,
+    // scaled by a power of two that the largest |W| decides
+    centre_kernel<<<dim3(t->DP, B), 256, 0, stream>>>(st.X, st.inv_ell, n, d, t->DP, t->centre, t->scale);
+    xt_build_kernel<<<dim3(t->NP / t->KD, B), 256, 0, stream>>>(st.X, t->centre, t->scale, st.alpha32, n, d, st.npad, t->DP,
+                                                                t->NP, t->KD, t->xt, t->xs32, t->xnorm, t->alpha, st.xamax_d,
+                                                                st.xnmax_d);
+    wt_build_kernel<<<dim3(t->P * CPP, t->P, B), 256, 0, stream>>>(st.W64, n, st.npad, t->NV, t->wt_gp_stride, st.wmax_d,
+                                                                   st.sf2_d, t->kscale, t->vinv2, t->wt, t->f8);
     g_launches += 3;
-    float xamax = 0.f;
-    std::vector<float> wmax(B);
-    if ((e = cudaMemcpyAsync(&xamax, xamax_bits, sizeof(float), cudaMemcpyDeviceToHost, stream)) != cudaSuccess)
-        return fail("cudaMemcpyAsync", e);
-    if ((e = cudaMemcpyAsync(wmax.data(), wmax_bits, sizeof(float) * B, cudaMemcpyDeviceToHost, stream)) != cudaSuccess)
-        return fail("cudaMemcpyAsync", e);
-    if ((e = cudaStreamSynchronize(stream)) != cudaSuccess) return fail("operand preparation", e);
-    if (!(xamax <= kMaxScaled)) return decline();   // scaled coordinates beyond the FP16 planes
-    std::vector<float> wscale(B), kscale(B);
-    std::vector<double> vinv2(B);
-    for (int g = 0; g < B; ++g) {
-        int ew = 0, ek = 0;
-        frexp((double)wmax[g], &ew);               // wmax < 2^ew
-        frexp((double)gp->sf2[g], &ek);            // sf2  < 2^ek  (k* <= sf2)
-        const int sw = (t->f8 ? kScaleExpF8 : kScaleExp) - ew, sk = kScaleExp - ek;
-        if (!(wmax[g] > 0.f) || sw < -60 || sw > 60 || sk < -60 || sk > 60) return decline();   // degenerate scales
-        wscale[g] = (float)ldexp(1.0, sw);
-        kscale[g] = (float)ldexp(1.0, sk);
-        vinv2[g] = ldexp(1.0, -2 * (sw + sk));
-    }
-    if ((e = cudaMemcpyAsync(wscale_d, wscale.data(), sizeof(float) * B, cudaMemcpyHostToDevice, stream)) != cudaSuccess)
-        return fail("cudaMemcpyAsync", e);
-    if ((e = cudaMemcpyAsync(t->kscale, kscale.data(), sizeof(float) * B, cudaMemcpyHostToDevice, stream)) != cudaSuccess)
-        return fail("cudaMemcpyAsync", e);
-    if ((e = cudaMemcpyAsync(t->vinv2, vinv2.data(), sizeof(double) * B, cudaMemcpyHostToDevice, stream)) != cudaSuccess)
-        return fail("cudaMemcpyAsync", e);
-    xnmax_kernel<<<B, 256, 0, stream>>>(t->xnorm, t->NP, t->xnmax);
-    wt_build_kernel<<<dim3(t->P * CPP, t->P, B), 256, 0, stream>>>(gp->W64, n, gp->npad, t->NV, t->wt_gp_stride,
-                                                                   wscale_d, t->wt, t->f8);
-    g_launches += 2;
     if ((e = cudaGetLastError()) != cudaSuccess) return fail("operand preparation launch", e);
-    if ((e = cudaStreamSynchronize(stream)) != cudaSuccess) return fail("operand preparation", e);
-    dev_free(wmax_bits);
-    dev_free(wscale_d);
-    wmax_bits = nullptr;
-    wscale_d = nullptr;
     // The cap on dynamic shared memory belongs to the kernel, not to the handle, and handles with different
     // feature counts share an instantiation with different sizes: raise it to the device's limit (the kernel
     // has no static shared memory), so that no handle's preparation lowers it for another.
     int smem_optin = 0;
-    if ((e = cudaDeviceGetAttribute(&smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, gp->device)) != cudaSuccess)
+    if ((e = cudaDeviceGetAttribute(&smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, device)) != cudaSuccess)
         return fail("cudaDeviceGetAttribute", e);
-    if ((size_t)smem_optin < t->smem_bytes) return decline();
+    if ((size_t)smem_optin < t->smem_bytes) {
+        cudaStreamSynchronize(stream);
+        FreeScope no_wait;
+        tc_release(st);   // the SIMT engine serves this history
+        return R3_OK;
+    }
     e = cudaFuncSetAttribute(kernel_for(t->NV, t->G, t->kt, t->nbk, t->f8, t->P >= 2 && t->P < kF8MinPasses, t->DP <= kZsMaxDP), cudaFuncAttributeMaxDynamicSharedMemorySize,
                              smem_optin);
     if (e != cudaSuccess) return fail("cudaFuncSetAttribute", e);
     return R3_OK;
+}
+
+bool tc_accept(const r3_fit_state& st, const float* sf2, const unsigned* wmax, unsigned xamax)
+{
+    auto value = [](unsigned bits) {
+        float v;
+        memcpy(&v, &bits, sizeof(v));
+        return v;
+    };
+    if (!(value(xamax) <= kMaxScaled)) return false;   // scaled coordinates beyond the FP16 planes
+    for (int g = 0; g < st.batch; ++g) {
+        int sw, sk;
+        operand_scales(value(wmax[g]), sf2[g], ops_of(&st)->f8, sw, sk);
+        if (!(value(wmax[g]) > 0.f) || sw < -60 || sw > 60 || sk < -60 || sk > 60) return false;   // degenerate scales
+    }
+    return true;
 }
 
 void tc_info(const r3_gp* gp, int* info)
