@@ -239,6 +239,7 @@ struct GuardBuffers {
     unsigned* maxbits;  // [batch] bit pattern of the largest EI
     unsigned* done;     // [batch] slices selected
     unsigned* barrier;  // grid barrier of the guard kernel
+    int* mode;          // what guard_pilot decided
     double *ks, *qpart, *mupart;   // the rescue's slab
 };
 size_t guard_workspace_bytes(const r3_gp* gp, long long m);
@@ -247,6 +248,10 @@ size_t guard_workspace_bytes(const r3_gp* gp, long long m);
 int guard_zero_ints(const r3_gp* gp);
 // Key storage the guard kernel needs to leave the first level of a top-k of k (see TopkRequest).
 size_t guard_topk_workspace_bytes(int batch, long long m, int k);
+// Looks at the first `rows` scored candidates and decides (b.mode, on the device) whether so many of them miss the accuracy
+// contract that the engine should score the pool in its more accurate form.
+r3_status_t guard_pilot(r3_gp* gp, long long m, long long rows, const GuardBuffers& b, const float* mu, const float* sigma,
+                        const float* ei, cudaStream_t stream);
 GuardBuffers guard_carve(const r3_gp* gp, long long m, void* ws);
 // have_max: the engine's kernels have already raised maxbits to the pool's largest EI
 r3_status_t guard_and_rescue(r3_gp* gp, const float* Xcand, long long m, const GuardBuffers& b, float* mu,

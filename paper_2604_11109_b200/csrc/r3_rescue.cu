@@ -78,6 +78,57 @@ struct GuardArgs {
     float* val;
 };
 
+// Whether a candidate's estimated errors may exceed half of the accuracy contract.
+__device__ __forceinline__ bool misses_contract(float mu, float sd, float dmu, float dq, float tol_ei, float mu_floor,
+                                                float sd_floor, float best, float sf2)
+{
+    // d sigma = dq / (2 sigma); with sigma -> 0 every rounding error in q matters
+    const float dsd = (sd > 0.f) ? dq / (2.f * sd) : ((dq > 0.f) ? INFINITY : 0.f);
+    const float tol_mu = 1e-4f * fabsf(mu) + mu_floor;
+    const float tol_sd = 1e-4f * sd + sd_floor;
+    bool flag = !(dmu <= 0.5f * tol_mu) || !(dsd <= 0.5f * tol_sd);
+    // EI: dEI = Phi(z) dmu + phi(z) dsigma against 1e-5 of the pool's largest EI
+    const float z = (sd > 0.f) ? (best - mu) / sd : 0.f;
+    const float Phi = 0.5f * erfcf(-z * 0.70710678f);
+    const float phi = expf(-0.5f * z * z) * 0.39894228f;
+    if (isfinite(dsd)) flag |= !(Phi * dmu + phi * dsd <= 0.5f * tol_ei);
+    flag |= !(sd * sd >= 1e-3f * sf2);   // deep cancellation: do not trust the estimates either
+    return flag;
+}
+
+// One block looks at the first `rows` candidates (GP after GP) of a pool that the engine has scored in its cheaper form:
+// mode <- 1 when more than one in 32 of them would have to be recomputed, 0 otherwise.
+__global__ void __launch_bounds__(1024) pilot_kernel(const GuardArgs a, long long rows, int* __restrict__ mode)
+{
+    __shared__ unsigned top_s;
+    __shared__ int count_s;
+    const int t = threadIdx.x;
+    if (t == 0) {
+        top_s = 0u;
+        count_s = 0;
+    }
+    __syncthreads();
+    float v = 0.f;
+#pragma unroll 8
+    for (long long f = t; f < rows; f += 1024) v = fmaxf(v, a.ei[f]);
+    const unsigned top = __reduce_max_sync(0xffffffffu, __float_as_uint(v));
+    if (t % 32 == 0) atomicMax(&top_s, top);
+    __syncthreads();
+    const float tol_ei = 1e-5f * __uint_as_float(top_s);
+    int mine = 0;
+#pragma unroll 4
+    for (long long f = t; f < rows; f += 1024) {
+        const int g = (int)(f / a.m);
+        const float sf2 = a.sf2v[g];
+        mine += misses_contract(a.mu[f], a.sigma[f], a.err_mu[f], a.err_q[f], tol_ei, 1e-6f * a.yabsv[g], 1e-6f * sqrtf(sf2),
+                                a.bestv[g], sf2) ? 1 : 0;
+    }
+    mine = __reduce_add_sync(0xffffffffu, mine);
+    if (t % 32 == 0 && mine) atomicAdd(&count_s, mine);
+    __syncthreads();
+    if (t == 0) *mode = (long long)count_s * 32 > rows ? 1 : 0;
+}
+
 // k* and the partial means of (CT candidates) x (64 observations): 256 threads, CT / 16 candidates x 4 observations
 // each.  store(c, k, k*) for every candidate c of the tile and every k < npad of the block (zero beyond n and beyond the
 // listed candidates), mean(c, sum) once per candidate.
@@ -421,17 +472,7 @@ __global__ void __launch_bounds__(kThreads, 2) guard_kernel(const GuardArgs a)
             if (i < c1) {
                 const size_t f = (size_t)g * m + i;
                 const float mu_i = __ldcs(a.mu + f), sd = __ldcs(a.sigma + f), dmu = __ldcs(a.err_mu + f), dq = __ldcs(a.err_q + f);
-                // d sigma = dq / (2 sigma); with sigma -> 0 every rounding error in q matters
-                const float dsd = (sd > 0.f) ? dq / (2.f * sd) : ((dq > 0.f) ? INFINITY : 0.f);
-                const float tol_mu = 1e-4f * fabsf(mu_i) + mu_floor;
-                const float tol_sd = 1e-4f * sd + sd_floor;
-                flag = !(dmu <= 0.5f * tol_mu) || !(dsd <= 0.5f * tol_sd);
-                // EI: dEI = Phi(z) dmu + phi(z) dsigma against 1e-5 of the pool's largest EI
-                const float z = (sd > 0.f) ? (best - mu_i) / sd : 0.f;
-                const float Phi = 0.5f * erfcf(-z * 0.70710678f);
-                const float phi = expf(-0.5f * z * z) * 0.39894228f;
-                if (isfinite(dsd)) flag |= !(Phi * dmu + phi * dsd <= 0.5f * tol_ei);
-                flag |= !(sd * sd >= 1e-3f * sf2);   // deep cancellation: do not trust the estimates either
+                flag = misses_contract(mu_i, sd, dmu, dq, tol_ei, mu_floor, sd_floor, best, sf2);
             }
             const unsigned votes = __ballot_sync(0xffffffffu, flag);   // one counter update per warp
             if (votes) {
@@ -556,7 +597,7 @@ size_t up16(size_t b) { return (b + 15) & ~(size_t)15; }
 size_t guard_workspace_bytes(const r3_gp* gp, long long m)
 {
     const size_t bm = (size_t)gp->batch * m, slab = slab_candidates(gp, m), npad = gp->npad;
-    return 3 * up16(bm * sizeof(float)) + up16((4 * (size_t)gp->batch + 1) * sizeof(int)) +
+    return 3 * up16(bm * sizeof(float)) + up16((4 * (size_t)gp->batch + 2) * sizeof(int)) +
            sizeof(double) * slab * (npad + npad / 16 + (npad + 63) / 64) + 256;
 }
 
@@ -576,7 +617,8 @@ GuardBuffers guard_carve(const r3_gp* gp, long long m, void* ws)
     b.maxbits = (unsigned*)b.total + gp->batch;
     b.done = b.maxbits + gp->batch;
     b.barrier = b.done + gp->batch;
-    p += up16((4 * (size_t)gp->batch + 1) * sizeof(int));
+    b.mode = (int*)b.barrier + 1;
+    p += up16((4 * (size_t)gp->batch + 2) * sizeof(int));
     const size_t slab = slab_candidates(gp, m), npad = gp->npad;
     b.ks = (double*)p;
     b.qpart = b.ks + slab * npad;
@@ -601,6 +643,18 @@ size_t guard_topk_workspace_bytes(int batch, long long m, int k)
 
 // counts, maxima, finished slices and the grid barrier
 int guard_zero_ints(const r3_gp* gp) { return 4 * gp->batch + 1; }
+
+r3_status_t guard_pilot(r3_gp* gp, long long m, long long rows, const GuardBuffers& b, const float* mu, const float* sigma,
+                        const float* ei, cudaStream_t stream)
+{
+    GuardArgs a = {};
+    a.sf2v = gp->sf2_d; a.bestv = gp->best_d; a.yabsv = gp->yabs_d;
+    a.m = m;
+    a.mu = const_cast<float*>(mu); a.sigma = const_cast<float*>(sigma); a.ei = const_cast<float*>(ei);   // only read
+    a.err_mu = b.err_mu; a.err_q = b.err_q;
+    R3_LAUNCH(pilot_kernel, 1, 1024, 0, stream, a, rows, b.mode);
+    return R3_OK;
+}
 
 r3_status_t guard_and_rescue(r3_gp* gp, const float* Xcand, long long m, const GuardBuffers& b, float* mu,
                              float* sigma, float* ei, bool have_max, cudaStream_t stream)

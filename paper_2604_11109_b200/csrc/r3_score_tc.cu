@@ -116,6 +116,7 @@ template <int NV, int G, int KD, bool KT, int NBK = G, bool F8 = false, bool PUT
 __global__ void __launch_bounds__(128 + 128 * G, 1) score_tc_kernel(const TcParams prm)
 {
     static_assert(NBK == G || (KT && NBK >= 2 && NBK < G), "ring of k* buffers: TMEM only");
+    if (prm.mode && *prm.mode != prm.want_mode) return;   // the other form of the kernel serves this pool
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw = smem_u32(smem_raw);
     const uint32_t base = (raw + 1023u) & ~1023u;
@@ -1088,6 +1089,12 @@ void (*kernel_for(int NV, int G, bool kt, int nbk, bool f8, bool putoff, bool zs
 
 constexpr int kF8MinPasses = 8;   // n > 1792: below that the guard hands more candidates to the FP64 pass than the cheaper MMAs save
 
+// The kernel a set of operands runs on, with or without FP8 cross terms
+void (*kernel_of(const TensorOperands* t, bool f8))(const TcParams)
+{
+    return kernel_for(t->NV, t->G, t->kt, t->nbk, f8, t->P >= 2 && t->P < kF8MinPasses, t->DP <= kZsMaxDP);
+}
+
 int env_int(const char* name, int fallback)
 {
     const char* v = getenv(name);
@@ -1111,6 +1118,8 @@ void tc_release(r3_fit_state& st)
     dev_free(t->wt);
     dev_free(t->kscale);
     dev_free(t->vinv2);
+    dev_free(t->wt16);
+    dev_free(t->vinv2_16);
     delete t;
     st.tc = nullptr;
 }
@@ -1187,6 +1196,10 @@ r3_status_t tc_prepare(r3_fit_state& st, int device, cudaStream_t stream)
     if ((e = dev_malloc(&t->wt, sizeof(__half) * B * t->wt_gp_stride)) != cudaSuccess) return fail("cudaMalloc", e);
     if ((e = dev_malloc(&t->kscale, sizeof(float) * B)) != cudaSuccess) return fail("cudaMalloc", e);
     if ((e = dev_malloc(&t->vinv2, sizeof(double) * B)) != cudaSuccess) return fail("cudaMalloc", e);
+    if (t->f8) {
+        if ((e = dev_malloc(&t->wt16, sizeof(__half) * B * t->wt_gp_stride)) != cudaSuccess) return fail("cudaMalloc", e);
+        if ((e = dev_malloc(&t->vinv2_16, sizeof(double) * B)) != cudaSuccess) return fail("cudaMalloc", e);
+    }
     t->xnmax = reinterpret_cast<float*>(st.xnmax_d);   // lives in the state's block
 
     // scaled observations (their largest coordinate decides whether the FP16 planes can hold them), then the planes of W,
@@ -1198,6 +1211,11 @@ r3_status_t tc_prepare(r3_fit_state& st, int device, cudaStream_t stream)
     wt_build_kernel<<<dim3(t->P * CPP, t->P, B), 256, 0, stream>>>(st.W64, n, st.npad, t->NV, t->wt_gp_stride, st.wmax_d,
                                                                    st.sf2_d, t->kscale, t->vinv2, t->wt, t->f8);
     g_launches += 3;
+    if (t->f8) {
+        wt_build_kernel<<<dim3(t->P * CPP, t->P, B), 256, 0, stream>>>(st.W64, n, st.npad, t->NV, t->wt_gp_stride, st.wmax_d,
+                                                                       st.sf2_d, t->kscale, t->vinv2_16, t->wt16, false);
+        ++g_launches;
+    }
     if ((e = cudaGetLastError()) != cudaSuccess) return fail("operand preparation launch", e);
     // The cap on dynamic shared memory belongs to the kernel, not to the handle, and handles with different
     // feature counts share an instantiation with different sizes: raise it to the device's limit (the kernel
@@ -1211,9 +1229,10 @@ r3_status_t tc_prepare(r3_fit_state& st, int device, cudaStream_t stream)
         tc_release(st);   // the SIMT engine serves this history
         return R3_OK;
     }
-    e = cudaFuncSetAttribute(kernel_for(t->NV, t->G, t->kt, t->nbk, t->f8, t->P >= 2 && t->P < kF8MinPasses, t->DP <= kZsMaxDP), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             smem_optin);
-    if (e != cudaSuccess) return fail("cudaFuncSetAttribute", e);
+    for (int form = 0; form < (t->f8 ? 2 : 1); ++form) {
+        e = cudaFuncSetAttribute(kernel_of(t, t->f8 && form == 0), cudaFuncAttributeMaxDynamicSharedMemorySize, smem_optin);
+        if (e != cudaSuccess) return fail("cudaFuncSetAttribute", e);
+    }
     return R3_OK;
 }
 
@@ -1316,6 +1335,8 @@ r3_status_t score_tc_part(r3_gp* gp, const float* Xcand, long long m, float* mu,
     if (launch_tiles <= 0) return R3_OK;
     prm.zero = gb.count;
     prm.zero_ints = guard_zero_ints(gp);
+    prm.mode = nullptr;
+    prm.want_mode = 0;
     int sms = 148;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, gp->device);
     const unsigned grid = (unsigned)(launch_tiles < sms ? launch_tiles : sms);
@@ -1334,8 +1355,42 @@ r3_status_t score_tc_part(r3_gp* gp, const float* Xcand, long long m, float* mu,
         const r3_status_t st = launch_tc_pair(t, prm, sms, stream);
         if (st != R3_OK) return st;
     } else {
-        void (*kernel)(const TcParams) = kernel_for(t->NV, t->G, t->kt, t->nbk, t->f8, t->P >= 2 && t->P < kF8MinPasses, t->DP <= kZsMaxDP);
-        R3_LAUNCH(kernel, grid, 128 + 128 * t->G, t->smem_bytes, stream, prm);
+        auto launch = [&](bool f8, long long begin, long long end, int want_mode) -> r3_status_t {
+            TcParams q = prm;
+            q.tile_begin = begin;
+            q.total_tiles = end;
+            q.mode = want_mode < 0 ? nullptr : gb.mode;
+            q.want_mode = want_mode;
+            if (t->f8 && !f8) {
+                q.wt = t->wt16;
+                q.vinv2 = t->vinv2_16;
+            }
+            void (*kernel)(const TcParams) = kernel_of(t, f8);
+            R3_LAUNCH(kernel, (unsigned)std::min<long long>(end - begin, sms), 128 + 128 * t->G, t->smem_bytes, stream, q);
+            return R3_OK;
+        };
+        const long long begin = prm.tile_begin, end = prm.total_tiles;
+        r3_status_t st = R3_OK;
+        if (!t->f8) {
+            st = launch(false, begin, end, -1);
+        } else {
+            // The FP8 cross terms save a fifth of the time where the posterior is tame and send most of a pool to the FP64
+            // pass where it is not (few features, long lengthscales): 65,536 candidates at n = 4096 with 41,604 recomputed
+            // 41.6 ms, with FP16 cross terms and none recomputed 4.1 ms.  So the pool's first wave of tiles is scored with
+            // them, the guard's own test decides on the device, and of the two launches for the rest (for all of it, in the
+            // FP16 form) one returns at once.  A first wave costs no more alone than as part of the whole.
+            long long rest = begin;
+            if (begin == 0) {
+                rest = std::min<long long>(end, sms);
+                st = launch(true, 0, rest, -1);
+                // candidates of the first `rest` tiles that lie together in memory: whole GPs and a part of the next
+                const long long whole = rest / prm.tiles_per_gp, part = std::min(m, rest % prm.tiles_per_gp * TILE_M);
+                if (st == R3_OK) st = guard_pilot(gp, m, whole * m + part, gb, mu, sigma, ei, stream);
+            }
+            if (st == R3_OK && rest < end) st = launch(true, rest, end, 0);
+            if (st == R3_OK) st = launch(false, begin, end, 1);
+        }
+        if (st != R3_OK) return st;
     }
     prof_end(gp, stream);
     if (prm.trace) {

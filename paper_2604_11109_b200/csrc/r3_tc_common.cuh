@@ -30,6 +30,8 @@ struct TensorOperands {
                                // second plane is two 8-bit planes [2][KC/16][NV][16]: hi parts (E4M3), then lo parts (E5M2)
     float* kscale = nullptr;   // [B]  2^eK, applied to k* before its split
     double* vinv2 = nullptr;   // [B]  2^(-2 (eK + eW)): scales sum V^2 back
+    __half* wt16 = nullptr;    // with f8: the chunks as FP16 hi/lo planes too, for pools that need them
+    double* vinv2_16 = nullptr;
 };
 
 struct TcParams {
@@ -47,6 +49,8 @@ struct TcParams {
     int* status;
     int* zero;          // the guard's counters, cleared by the first block (nothing reads them before the guard's kernel)
     int zero_ints;
+    const int* mode;    // nullptr, or: the launch does nothing unless *mode == want_mode
+    int want_mode;
     long long tiles_per_gp, total_tiles;   // total_tiles: one past the last tile of this launch
     long long tile_begin;                  // first tile of this launch (the single-CTA kernel; 0 for a whole pool)
     long long* trace;   // optional [grid][4 roles][8] cycle counters (diagnostics)

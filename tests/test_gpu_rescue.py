@@ -6,7 +6,9 @@ import numpy as np
 import pytest
 
 from paper_2604_11109_b200 import binding as b
-from tests.test_gpu_parity import compare_everything, fit_gpu, rand_problem
+from oracle import gp_oracle as o
+from tests.parity import check_scores
+from tests.test_gpu_parity import compare_everything, dev, fit_gpu, rand_problem
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
@@ -30,4 +32,26 @@ def test_flagged_candidates_are_recomputed(engine, batch, n, m, near):
     gp = fit_gpu(g, engine)
     compare_everything(g, gp, min(m, 40), f"rescue n{n} m{m}")
     assert b.r3_gp_last_rescued(gp) >= 0.9 * near * batch
+    gp.close()
+
+
+@pytest.mark.parametrize("batch,n,d,m,sn2", [
+    (1, 1900, 4, 700, 1e-2),      # a single wave of tiles: scored again with FP16 cross terms
+    (1, 2048, 4, 20000, 1e-2),    # more than one wave: the pilot decides
+    (2, 1800, 5, 15000, 1e-2),    # the first wave spans both GPs
+    (1, 1900, 40, 21000, 1e-3),   # a tame pool: the FP8 form serves it
+])
+def test_long_histories_on_pools_that_need_fp16_cross_terms(batch, n, d, m, sn2):
+    g = rand_problem(77 + n, batch, n, d, m, sn2=sn2, spread=2.0 if d < 10 else 0.4)
+    gp = fit_gpu(g, b.ENGINE_TENSOR)
+    assert b.r3_gp_tensor_info(gp)["f8_cross_terms"] == 1
+    rows = np.sort(np.random.default_rng(3).choice(m, size=min(m, 1500), replace=False))
+    mu, sd, ei, idx, val = (t.cpu().numpy() for t in b.r3_gp_score_topk(gp, dev(g["Xcand"]), 20))
+    b.r3_gp_check(gp)
+    for q, f in enumerate(o.fit_batch(g["X"], g["y"], g["ell"], g["sf2"], g["sn2"])):
+        mu_r, sd_r, ei_r = o.score(f, g["Xcand"][q][rows])
+        check_scores(mu[q][rows], sd[q][rows], ei[q][rows], mu_r, sd_r, ei_r, float(np.abs(g["y"][q]).max()),
+                     float(g["sf2"][q]), ei_max=float(ei[q].max()), what=f"n{n} m{m}")
+        assert np.array_equal(val[q], ei[q][idx[q]])
+        assert np.array_equal(idx[q], o.topk(ei[q], 20)[0])
     gp.close()
