@@ -274,16 +274,18 @@ r3_status_t r3_gp_propose(r3_gp_t* gp, const float* Xcand, long long m, int q, i
     const int B = gp->batch;
     const int Rk = (long long)R < m ? R + 1 : R;   // one more than the shortlist: the certificate's bound
     cudaStream_t stream = (cudaStream_t)cuda_stream;
-    r3_status_t st = ensure_workspace(gp, score_workspace_bytes(gp, m));
+    const size_t sb = align256(score_workspace_bytes(gp, m));
+    const size_t tb = guard_topk_workspace_bytes(B, m, Rk);
+    r3_status_t st = ensure_workspace(gp, sb + tb);
     if (st != R3_OK) return st;
+    const size_t bm = (size_t)B * m;
     float *scores = nullptr, *sval = nullptr;
     int* sidx = nullptr;
-    void *tws = nullptr, *pws = nullptr;
-    const size_t bm = (size_t)B * m, tbytes = topk_workspace_bytes(B, m, Rk);
+    void* pws = nullptr;
     auto done = [&](r3_status_t s) {
         cudaStreamSynchronize(stream);
         FreeScope no_wait;
-        dev_free(scores); dev_free(sval); dev_free(sidx); dev_free(tws); dev_free(pws);
+        dev_free(scores); dev_free(sval); dev_free(sidx); dev_free(pws);
         return s;
     };
 #define TRY_DONE(expr)                                                                             \
@@ -297,23 +299,27 @@ r3_status_t r3_gp_propose(r3_gp_t* gp, const float* Xcand, long long m, int q, i
     TRY_DONE(dev_malloc(&scores, sizeof(float) * 3 * bm));
     TRY_DONE(dev_malloc(&sval, sizeof(float) * (size_t)B * Rk));
     TRY_DONE(dev_malloc(&sidx, sizeof(int) * (size_t)B * Rk));
-    TRY_DONE(dev_malloc(&tws, tbytes));
     TRY_DONE(dev_malloc(&pws, propose_workspace_bytes(B, gp->npad, R, q)));
     float *mu = scores, *sigma = scores + bm, *ei = scores + 2 * bm;
-    st = run_score(gp, Xcand, m, mu, sigma, ei, gp->ws, gp->ws_bytes, stream);
+    gp->topk_req.k = Rk;   // the shortlist rides on the scoring call
+    gp->topk_req.idx = sidx;
+    gp->topk_req.val = sval;
+    gp->topk_req.ws = (char*)gp->ws + sb;
+    gp->topk_req.ws_bytes = tb;
+    st = run_score(gp, Xcand, m, mu, sigma, ei, gp->ws, sb, stream);
+    gp->topk_req = TopkRequest();
     if (st != R3_OK) return done(st);
-    st = topk_device(ei, B, m, Rk, sidx, sval, tws, tbytes, stream);
-    if (st != R3_OK) return done(st);
-    st = propose_shortlist(gp, Xcand, m, sidx, Rk, R, q, lie, idx, ei_pick, pws, stream);
+    int* cert_d = nullptr;
+    st = propose_shortlist(gp, Xcand, m, sidx, sval, Rk, R, q, lie, idx, ei_pick, &cert_d, pws, stream);
     if (st != R3_OK) return done(st);
     // certificate and latched device status
-    std::vector<float> hval((size_t)B * Rk), hpick;
-    TRY_DONE(cudaMemcpyAsync(hval.data(), sval, sizeof(float) * hval.size(), cudaMemcpyDeviceToHost, stream));
-    TRY_DONE(cudaMemcpyAsync(gp->status_h, gp->status_d, 2 * sizeof(int), cudaMemcpyDeviceToHost, stream));
-    if (ei_pick) {
-        hpick.resize((size_t)B * q);
-        TRY_DONE(cudaMemcpyAsync(hpick.data(), ei_pick, sizeof(float) * hpick.size(), cudaMemcpyDeviceToHost, stream));
+    int* cert = reinterpret_cast<int*>(gp->stage_h);
+    if (sizeof(int) * B > kStageBytes) {
+        gp->image.resize(sizeof(int) * B);
+        cert = reinterpret_cast<int*>(gp->image.data());
     }
+    TRY_DONE(cudaMemcpyAsync(cert, cert_d, sizeof(int) * B, cudaMemcpyDeviceToHost, stream));
+    TRY_DONE(cudaMemcpyAsync(gp->status_h, gp->status_d, 2 * sizeof(int), cudaMemcpyDeviceToHost, stream));
     TRY_DONE(cudaStreamSynchronize(stream));
 #undef TRY_DONE
     if (gp->status_h[0] & DEV_NOT_PD) {
@@ -323,21 +329,8 @@ r3_status_t r3_gp_propose(r3_gp_t* gp, const float* Xcand, long long m, int q, i
                   "observation); nothing to condition on");
         return done(R3_ERR_NOT_PD);
     }
-    if (certified) {
-        for (int g = 0; g < B; ++g) {
-            if (Rk == R) {
-                certified[g] = 1;   // the shortlist is the whole pool
-            } else if (lie != 0 || !ei_pick) {
-                certified[g] = 0;
-            } else {
-                // the first excluded candidate's initial EI (FP32, within the scoring tolerance of 1e-5 max EI)
-                const double bound = hval[(size_t)g * Rk + R], top = hval[(size_t)g * Rk];
-                double lowest = hpick[(size_t)g * q];
-                for (int t = 1; t < q; ++t) lowest = hpick[(size_t)g * q + t] < lowest ? hpick[(size_t)g * q + t] : lowest;
-                certified[g] = lowest >= bound + 4e-5 * top ? 1 : 0;
-            }
-        }
-    }
+    if (certified)
+        for (int g = 0; g < B; ++g) certified[g] = Rk == R || ei_pick ? cert[g] : 0;
     return done(R3_OK);
 }
 

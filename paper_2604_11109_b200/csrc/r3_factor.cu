@@ -92,10 +92,19 @@ __device__ __forceinline__ void gram_tile(const FactorArgs& a, int g, int ti, in
     double r2[2][4][2] = {};
     for (int c0 = 0; c0 < d; c0 += 32) {
         __syncthreads();
-        for (int e = t; e < TB * 32; e += kThreads) {
-            const int r = e / 32, f = e % 32, gi = ti * TB + r, gj = tj * TB + r;
-            xi[r * 33 + f] = (gi < n && c0 + f < d) ? (double)Xg[(size_t)gi * d + c0 + f] : 0.0;
-            xj[r * 33 + f] = (gj < n && c0 + f < d) ? (double)Xg[(size_t)gj * d + c0 + f] : 0.0;
+        // all of a thread's loads are under way before the first is stored
+        const int f0 = t % 32, q0 = t / 32;
+        float vi[8], vj[8];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+            const int gi = ti * TB + q0 + 8 * e, gj = tj * TB + q0 + 8 * e;
+            vi[e] = (gi < n && c0 + f0 < d) ? __ldg(Xg + (size_t)gi * d + c0 + f0) : 0.f;
+            vj[e] = (gj < n && c0 + f0 < d) ? __ldg(Xg + (size_t)gj * d + c0 + f0) : 0.f;
+        }
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+            xi[(q0 + 8 * e) * 33 + f0] = (double)vi[e];
+            xj[(q0 + 8 * e) * 33 + f0] = (double)vj[e];
         }
         // FP64 reciprocal of the lengthscale: one rounding more than a division per difference, a third of its time
         if (t < 32) il[t] = (c0 + t < d) ? 1.0 / (double)a.ell[(size_t)g * d + c0 + t] : 0.0;

@@ -7,22 +7,33 @@
 // is a rank-one change of the posterior:
 //     c(x) = cov(x, x_t),  s = var(x_t) + noise,
 //     mu(x) += c(x) (value - mu(x_t)) / s,     var(x) -= c(x)^2 / s,
-//     cov(x, x_t) = k(x, x_t) - v(x).v(x_t) - sum_{earlier picks u} c_u(x) c_u(x_t) / s_u,   v(x) = W k*(x),
+//     cov(x, x_t) = C0(x, x_t) - sum_{earlier picks u} c_u(x) c_u(x_t) / s_u,   C0(x, z) = k(x, z) - v(x).v(z),  v = W k*
 // and with the believer's value the means never move while the variances only shrink, so EI (fixed
 // incumbent) only drops: a candidate outside the R best of the first scoring can be picked only if some
-// pick's EI falls below the (R+1)-th initial EI.  So: one full scoring, top-(R+1), then the q picks on the
-// shortlist alone, in FP64 (k*, v = W k* by one triangular product, the moments recomputed), two small
-// launches per pick.  The (R+1)-th initial EI is returned as the certificate's bound.
+// pick's EI falls below the (R+1)-th initial EI.  So: one full scoring with its top-(R+1), then the q picks on the
+// shortlist alone, in FP64, in two kernels:
+//   build_kernel  (cooperative) k* of the shortlist, V = W k*, C0 for all its pairs, as tiles on the FP64 tensor path;
+//   pick_kernel   (one cluster per GP) the q picks: a candidate per thread and part, the columns c_u in shared memory, one
+//                 cluster barrier per pick.
+// Bound: R n^2 / 2 + R^2 n / 2 FP64 multiply-adds, then the latency of a pick.  One GP of 4096 observations, 1023
+// shortlisted, 128 picks: 6.1 ms as 259 launches (R n multiply-adds per pick), 1.8 ms now; 72 observations, 256
+// shortlisted, 8 picks: 100 us in 19 launches and 62 us.
+#include <cooperative_groups.h>
+
+#include <algorithm>
+
+#include "r3_cross.cuh"
 #include "r3_epilogue.cuh"
-#include "r3_gemm64.cuh"
 #include "r3_internal.cuh"
 
 namespace r3 {
 
 namespace {
 
-// All GPs of the handle are processed together: blockIdx.z (or .y) is the GP.  Per-GP scalars come from
-// device arrays; the shortlist state of GP g starts at g times the per-GP stride of each array.
+namespace cg = cooperative_groups;
+
+// All GPs of the handle are processed together; the shortlist state of GP g starts at g times the per-GP stride of each
+// array.
 struct ProposeArrays {
     const float* X;        // [B][n][d]
     const float* ell;      // [B][d]
@@ -30,237 +41,331 @@ struct ProposeArrays {
     const float* sn2;      // [B]
     const float* best;     // [B]
     const double* alpha;   // [B][npad]
+    const double* W;       // [B][npad][npad]
     const float* Xcand;    // [B][m][d]
     const int* sidx;       // [B][Rk] shortlist (pool indices), Rk >= R
+    const float* sval;     // [B][Rk] their EI in the scoring of the pool
     long long m;
-    int n, d, npad, R, Rk, q;
+    int B, n, d, npad, R, Rk, q;
     double *Ks, *V;        // [B][R][npad]
-    double *C;             // [B][q][R]
-    double *mu, *var;      // [B][R]
-    double *S, *delta;     // [B][q]
-    int *picked, *sel;     // [B][R], [B][q]
+    double *C0;            // [B][R][R] posterior covariances
+    double *mupart;        // [B][R][ceil(npad / 64)]
+    double *qpart;         // [B][R][ceil(npad / 64)]
+    double *C;             // [B][q][R] columns of picks that do not fit shared memory
+    int *cert;             // [B] the shortlist is certified to lose nothing
+    unsigned* barrier;     // grid barrier, zero on entry
+    int* status;
 };
 
-// Ks[r][i] = k(x_i, candidate sidx[r]) in FP64 by direct differences; zero in the padding columns.
-__global__ void shortlist_kstar_kernel(const ProposeArrays a)
+__device__ __forceinline__ const float* short_row(const ProposeArrays& a, int g, int r)
 {
-    const int g = blockIdx.z, r = blockIdx.y;
-    const int n = a.n, d = a.d, npad = a.npad;
-    const float* X = a.X + (size_t)g * n * d;
-    const float* ell = a.ell + (size_t)g * d;
-    const float* Xcand = a.Xcand + (size_t)g * a.m * d;
-    const int* sidx = a.sidx + (size_t)g * a.Rk;
-    double* Ks = a.Ks + (size_t)g * a.R * npad;
-    const double sf2 = (double)a.sf2[g];
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    __shared__ double inv[kMaxD];   // FP64 reciprocals of the lengthscales, as the fit's Gram kernel uses them
-    for (int j = threadIdx.x; j < d; j += blockDim.x) inv[j] = 1.0 / (double)ell[j];
-    __syncthreads();
-    if (i >= npad) return;
-    double v = 0.0;
-    if (i < n) {
-        const float* z = Xcand + (size_t)sidx[r] * d;
-        const float* x = X + (size_t)i * d;
-        double r2 = 0.0;
-        for (int j = 0; j < d; ++j) {
-            const double diff = ((double)x[j] - (double)z[j]) * inv[j];
-            r2 += diff * diff;
-        }
-        const double s = sqrt(5.0) * sqrt(r2);
-        v = sf2 * (1.0 + s + s * s / 3.0) * exp(-s);
-    }
-    Ks[(size_t)r * npad + i] = v;
+    return r < a.R ? a.Xcand + ((size_t)g * a.m + a.sidx[(size_t)g * a.Rk + r]) * a.d : nullptr;
 }
 
-// mu[r] = Ks[r].alpha, var[r] = sf2 - |V[r]|^2 (one warp per shortlisted candidate).
-__global__ void shortlist_moments_kernel(const ProposeArrays a)
+__global__ void __launch_bounds__(kCrossThreads, 2) build_kernel(const ProposeArrays a)
 {
-    const int g = blockIdx.y;
-    const int n = a.n, npad = a.npad, R = a.R;
-    const double* Ks = a.Ks + (size_t)g * R * npad;
-    const double* V = a.V + (size_t)g * R * npad;
-    const double* alpha = a.alpha + (size_t)g * npad;
-    double* mu = a.mu + (size_t)g * R;
-    double* var = a.var + (size_t)g * R;
-    int* picked = a.picked + (size_t)g * R;
-    const double sf2 = (double)a.sf2[g];
-    const int r = blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
-    const int lane = threadIdx.x % 32;
-    if (r >= R) return;
-    double m = 0.0, q = 0.0;
-    for (int i = lane; i < n; i += 32) {
-        m = fma(Ks[(size_t)r * npad + i], alpha[i], m);
-        const double v = V[(size_t)r * npad + i];
-        q = fma(v, v, q);
+    extern __shared__ __align__(16) unsigned char smem[];
+    const int t = threadIdx.x, w = t / 32, l = t % 32, wm = (w % 4) * 16, wn = (w / 4) * 32;
+    const int npad = a.npad, R = a.R, RT = (R + 63) / 64, NT = (npad + 63) / 64;
+    unsigned target = 0;
+    // ---- k* and the partial means
+    for (int item = blockIdx.x; item < a.B * RT * NT; item += gridDim.x) {
+        const int g = item / (RT * NT), rt = item % (RT * NT) / NT, kb = item % NT;
+        double* Ks = a.Ks + ((size_t)g * R + rt * 64) * npad;
+        cross_tile<64>(
+            a.n, a.d, npad, a.ell + (size_t)g * a.d, (double)a.sf2[g], a.alpha + (size_t)g * npad,
+            [&](int r) { return short_row(a, g, rt * 64 + r); }, [&](int k) { return a.X + ((size_t)g * a.n + k) * a.d; }, kb,
+            smem, [&](int c, int k, double v) { if (rt * 64 + c < R) Ks[(size_t)c * npad + k] = v; },
+            [&](int c, double s) { if (rt * 64 + c < R) a.mupart[((size_t)g * R + rt * 64 + c) * NT + kb] = s; });
     }
-    for (int o = 16; o > 0; o >>= 1) {
-        m += __shfl_xor_sync(0xffffffffu, m, o);
-        q += __shfl_xor_sync(0xffffffffu, q, o);
-    }
-    if (lane == 0) {
-        mu[r] = m;
-        var[r] = sf2 - q;
-        picked[r] = 0;
-    }
-}
-
-// One block: EI of every unpicked shortlisted candidate, the largest (ties: lower pool index) is pick t.
-__global__ void __launch_bounds__(1024) pick_kernel(const ProposeArrays a, int liar, int t, int* __restrict__ idx_all,
-                                                    float* __restrict__ ei_all, int* __restrict__ status)
-{
-    __shared__ double se[1024];
-    __shared__ int sr[1024];
-    const int g = blockIdx.x;
-    const int R = a.R;
-    const double* mu = a.mu + (size_t)g * R;
-    const double* var = a.var + (size_t)g * R;
-    int* picked = a.picked + (size_t)g * R;
-    const int* sidx = a.sidx + (size_t)g * a.Rk;
-    int* sel = a.sel + (size_t)g * a.q;
-    double* S = a.S + (size_t)g * a.q;
-    double* delta = a.delta + (size_t)g * a.q;
-    int* idx_out = idx_all + (size_t)g * a.q;
-    float* ei_out = ei_all ? ei_all + (size_t)g * a.q : nullptr;
-    const double best = (double)a.best[g], sn2 = (double)a.sn2[g];
-    const int r = threadIdx.x;
-    double e = -1.0;
-    if (r < R && !picked[r]) e = ei_closed_form(mu[r], sqrt(fmax(var[r], 0.0)), best);
-    se[r] = e;
-    sr[r] = r;
-    __syncthreads();
-    for (int o = 512; o > 0; o >>= 1) {
-        if (r < o) {
-            const double ea = se[r], eb = se[r + o];
-            const int ra = sr[r], rb = sr[r + o];
-            // an entry that is not a candidate (e < 0) always loses; equal EI: the lower pool index wins
-            const bool take_b = (eb > ea) || (eb == ea && eb >= 0.0 && sidx[rb] < sidx[ra]);
-            if (take_b) {
-                se[r] = eb;
-                sr[r] = rb;
+    if (!grid_barrier(a.barrier, target, a.status)) return;
+    // ---- V[r][i] = sum_k Ks[r][k] W[i][k], the longest rows of W first, and the partial sums of squares
+    for (int item = blockIdx.x; item < a.B * RT * NT; item += gridDim.x) {
+        const int it = NT - 1 - item / (a.B * RT), g = item % (a.B * RT) / RT, rt = item % RT;
+        double c[2][4][2] = {};
+        nt_tile(a.Ks + ((size_t)g * R + rt * 64) * npad, R - rt * 64, a.W + ((size_t)g * npad + it * 64) * npad, npad - it * 64,
+                npad, min(npad, it * 64 + 64), smem, c);
+        double* red = reinterpret_cast<double*>(smem);   // [2 column warps][64 rows]
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            const int r = rt * 64 + wm + 8 * i + l / 4;
+            double s = 0.0;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const int col = it * 64 + wn + 8 * j + 2 * (l % 4);
+                s = fma(c[i][j][0], c[i][j][0], fma(c[i][j][1], c[i][j][1], s));
+                if (r < R && col < npad)
+                    *reinterpret_cast<double2*>(a.V + ((size_t)g * R + r) * npad + col) = make_double2(c[i][j][0], c[i][j][1]);
             }
+            s += __shfl_xor_sync(0xffffffffu, s, 1);
+            s += __shfl_xor_sync(0xffffffffu, s, 2);
+            if (l % 4 == 0) red[(w / 4) * 64 + wm + 8 * i + l / 4] = s;
         }
         __syncthreads();
+        if (t < 64 && rt * 64 + t < R) a.qpart[((size_t)g * R + rt * 64 + t) * NT + it] = red[t] + red[64 + t];
+        __syncthreads();
     }
-    if (r == 0) {
-        const int j = sr[0];
-        sel[t] = j;
-        picked[j] = 1;
-        idx_out[t] = sidx[j];
-        if (ei_out) ei_out[t] = (float)se[0];
-        const double s = fmax(var[j], 0.0) + sn2;
-        if (!(s > 0.0)) {   // a candidate on top of an observation with zero noise: nothing to condition on
-            atomicOr(status, DEV_NOT_PD);
-            S[t] = INFINITY;
-            delta[t] = 0.0;
-        } else {
-            S[t] = s;
-            // the fantasised value enters the history as an observation, i.e. rounded to FP32
-            const double value = liar ? best : (double)(float)mu[j];
-            delta[t] = (value - mu[j]) / s;
-        }
+    if (a.q < 2) return;
+    if (!grid_barrier(a.barrier, target, a.status)) return;
+    // ---- C0 = k(z, z') - V V^T, tiles of the lower triangle, written on both sides
+    const int pairs = RT * (RT + 1) / 2;
+    for (int item = blockIdx.x; item < a.B * pairs; item += gridDim.x) {
+        const int g = item / pairs, p = item % pairs;
+        int ta = 0;
+        while ((ta + 1) * (ta + 2) / 2 <= p) ++ta;
+        const int tb = p - ta * (ta + 1) / 2;
+        double c[2][4][2] = {};
+        const double* Vg = a.V + (size_t)g * R * npad;
+        nt_tile(Vg + (size_t)ta * 64 * npad, R - ta * 64, Vg + (size_t)tb * 64 * npad, R - tb * 64, npad, npad, smem, c);
+        double* tile = reinterpret_cast<double*>(smem + 20 * 1024);   // [64][65], behind the staged coordinates (17 KB)
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+#pragma unroll
+                for (int h = 0; h < 2; ++h) tile[(wm + 8 * i + l / 4) * 65 + wn + 8 * j + 2 * (l % 4) + h] = c[i][j][h];
+        double* C0 = a.C0 + (size_t)g * R * R;
+        cross_tile<64>(
+            R, a.d, R, a.ell + (size_t)g * a.d, (double)a.sf2[g], nullptr, [&](int r) { return short_row(a, g, ta * 64 + r); },
+            [&](int k) { return short_row(a, g, k); }, tb, smem,
+            [&](int r, int k, double v) {
+                const int row = ta * 64 + r;
+                if (row >= R) return;
+                v -= tile[r * 65 + k - tb * 64];
+                C0[(size_t)row * R + k] = v;
+                if (ta != tb) C0[(size_t)k * R + row] = v;
+            },
+            [](int, double) {});
+        __syncthreads();
     }
 }
 
-// One warp per shortlisted candidate r: c = cov(x_r, x_pick) under the posterior before pick t, then the
-// rank-one update of its mean and variance.  C[t][r] keeps c for the later picks.
-__global__ void condition_kernel(const ProposeArrays a, int t)
+constexpr int kPickThreads = 1024;
+constexpr int kMaxCluster = 8;
+constexpr int kMaxPicks = 256;
+struct Best {
+    unsigned long long key;   // bits of the EI plus one, 0: no candidate
+    int idx, r;               // pool index, place in the shortlist
+    double mu, var;
+};
+struct PickShared {
+    Best slot[2][kMaxCluster];
+    Best warp_best[kPickThreads / 32];
+    double w[kMaxPicks], inv_s[kMaxPicks], part[kPickThreads];
+};
+constexpr size_t kPickSmem = 224 * 1024;
+
+__device__ __forceinline__ bool better(unsigned long long ka, int ia, unsigned long long kb, int ib)
 {
-    const int g = blockIdx.y;
-    const int n = a.n, d = a.d, npad = a.npad, R = a.R;
-    const float* Xcand = a.Xcand + (size_t)g * a.m * d;
-    const int* sidx = a.sidx + (size_t)g * a.Rk;
-    const float* ell = a.ell + (size_t)g * d;
-    const double sf2 = (double)a.sf2[g];
-    const double* V = a.V + (size_t)g * R * npad;
-    double* C = a.C + (size_t)g * a.q * R;
-    const double* S = a.S + (size_t)g * a.q;
-    const double* delta = a.delta + (size_t)g * a.q;
-    const int* sel = a.sel + (size_t)g * a.q;
-    double* mu = a.mu + (size_t)g * R;
-    double* var = a.var + (size_t)g * R;
-    const int r = blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
-    const int lane = threadIdx.x % 32;
-    if (r >= R) return;
-    const int j = sel[t];
-    const float* xr = Xcand + (size_t)sidx[r] * d;
-    const float* xj = Xcand + (size_t)sidx[j] * d;
-    double r2 = 0.0, dot = 0.0, prev = 0.0;
-    for (int f = lane; f < d; f += 32) {
-        const double diff = ((double)xr[f] - (double)xj[f]) / (double)ell[f];
-        r2 = fma(diff, diff, r2);
-    }
-    for (int i = lane; i < n; i += 32) dot = fma(V[(size_t)r * npad + i], V[(size_t)j * npad + i], dot);
-    for (int u = lane; u < t; u += 32) prev += C[(size_t)u * R + r] * C[(size_t)u * R + j] / S[u];
-    for (int o = 16; o > 0; o >>= 1) {
-        r2 += __shfl_xor_sync(0xffffffffu, r2, o);
-        dot += __shfl_xor_sync(0xffffffffu, dot, o);
-        prev += __shfl_xor_sync(0xffffffffu, prev, o);
-    }
-    if (lane == 0) {
-        const double s = sqrt(5.0) * sqrt(r2);
-        const double c = sf2 * (1.0 + s + s * s / 3.0) * exp(-s) - dot - prev;
-        C[(size_t)t * R + r] = c;
-        mu[r] += c * delta[t];
-        var[r] -= c * c / S[t];
-    }
+    return ka > kb || (ka == kb && ia < ib);   // equal EI: the lower pool index
 }
+
+// One cluster per GP, the shortlist cut into one piece of Rl candidates per block; `held` columns c_u in shared memory.
+__global__ void __launch_bounds__(kPickThreads, 1) pick_kernel(const ProposeArrays a, int liar, int Rl, int held,
+                                                               int* __restrict__ idx_all, float* __restrict__ ei_all)
+{
+    extern __shared__ __align__(16) unsigned char smem[];
+    PickShared& sh = *reinterpret_cast<PickShared*>(smem);
+    double* cols = reinterpret_cast<double*>(smem + sizeof(PickShared));   // [held][Rl]
+    cg::cluster_group cluster = cg::this_cluster();
+    const int CS = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
+    const int g = blockIdx.x / CS, t = threadIdx.x, lane = t % 32, warp = t / 32;
+    const int R = a.R, NT = (a.npad + 63) / 64;
+    const int parts = kPickThreads / Rl, part = t / Rl, mine = t % Rl;   // Rl is a multiple of 32
+    const int r = rank * Rl + mine;
+    const bool active = part < parts && r < R, owner = active && part == 0;
+    const double best = (double)a.best[g], sn2 = (double)a.sn2[g];
+    const double* C0 = a.C0 + (size_t)g * R * R;
+    double* Cg = a.C + (size_t)g * a.q * R;
+    double mu = 0.0, var = 0.0;
+    int idx = 0;
+    bool picked = true;
+    if (owner) {
+        double s = 0.0;
+        for (int b = 0; b < NT; ++b) {
+            mu += a.mupart[((size_t)g * R + r) * NT + b];
+            s += a.qpart[((size_t)g * R + r) * NT + b];
+        }
+        var = (double)a.sf2[g] - s;
+        idx = a.sidx[(size_t)g * a.Rk + r];
+        picked = false;
+    }
+    double lowest = INFINITY;
+    for (int step = 0; step < a.q; ++step) {
+        // ---- the largest EI of the block, then of the cluster
+        Best m = {0ull, 0x7fffffff, 0, 0.0, 0.0};
+        if (owner && !picked) {
+            const double ei = ei_closed_form(mu, sqrt(fmax(var, 0.0)), best), e = ei >= 0.0 ? ei : 0.0;   // NaN counts as 0
+            m = {(unsigned long long)__double_as_longlong(e) + 1ull, idx, r, mu, var};   // e >= 0
+        }
+        unsigned long long key = m.key;
+        int who = m.idx, from = lane;
+        if (warp * 32 < Rl) {
+            for (int o = 16; o > 0; o >>= 1) {
+                const unsigned long long k2 = __shfl_xor_sync(0xffffffffu, key, o);
+                const int i2 = __shfl_xor_sync(0xffffffffu, who, o), f2 = __shfl_xor_sync(0xffffffffu, from, o);
+                if (better(k2, i2, key, who)) {
+                    key = k2;
+                    who = i2;
+                    from = f2;
+                }
+            }
+            if (lane == from) sh.warp_best[warp] = m;
+        }
+        __syncthreads();
+        if (warp == 0) {
+            m = lane < Rl / 32 ? sh.warp_best[lane] : Best{0ull, 0x7fffffff, 0, 0.0, 0.0};
+            key = m.key;
+            who = m.idx;
+            from = lane;
+            for (int o = 16; o > 0; o >>= 1) {
+                const unsigned long long k2 = __shfl_xor_sync(0xffffffffu, key, o);
+                const int i2 = __shfl_xor_sync(0xffffffffu, who, o), f2 = __shfl_xor_sync(0xffffffffu, from, o);
+                if (better(k2, i2, key, who)) {
+                    key = k2;
+                    who = i2;
+                    from = f2;
+                }
+            }
+            if (lane == from)
+                for (int b = 0; b < CS; ++b) *cluster.map_shared_rank(&sh.slot[step & 1][rank], b) = m;
+        }
+        cluster.sync();
+        Best win = sh.slot[step & 1][0];
+        for (int b = 1; b < CS; ++b)
+            if (better(sh.slot[step & 1][b].key, sh.slot[step & 1][b].idx, win.key, win.idx)) win = sh.slot[step & 1][b];
+        const int j = win.r;
+        const double e = __longlong_as_double((long long)(win.key - 1ull));
+        double s = fmax(win.var, 0.0) + sn2, delta = 0.0;
+        if (!(s > 0.0)) {   // a candidate on top of an observation with zero noise: nothing to condition on
+            if (rank == 0 && t == 0) atomicOr(a.status, DEV_NOT_PD);
+            s = INFINITY;
+        } else {
+            // the fantasised value enters the history as an observation, i.e. rounded to FP32
+            const double value = liar ? best : (double)(float)win.mu;
+            delta = (value - win.mu) / s;
+        }
+        lowest = fmin(lowest, (double)(float)e);
+        if (rank == 0 && t == 0) {
+            idx_all[(size_t)g * a.q + step] = win.idx;
+            if (ei_all) ei_all[(size_t)g * a.q + step] = (float)e;
+        }
+        if (owner && r == j) picked = true;
+        if (step + 1 == a.q) break;
+        // ---- c(x) = C0(x, x_j) - sum_u c_u(x) c_u(x_j) / s_u
+        double c = owner ? C0[(size_t)j * R + r] : 0.0;
+        const int jr = j / Rl, jl = j % Rl;
+        const double* theirs = cluster.map_shared_rank(cols, jr);
+        for (int u = t; u < step; u += kPickThreads)
+            sh.w[u] = (u < held ? theirs[(size_t)u * Rl + jl] : __ldcg(Cg + (size_t)u * R + j)) * sh.inv_s[u];
+        if (t == 0) sh.inv_s[step] = 1.0 / s;
+        __syncthreads();
+        double s0 = 0.0, s1 = 0.0;
+        if (active) {
+            int u = part;
+            for (; u + parts < step; u += 2 * parts) {
+                const double x = u < held ? cols[(size_t)u * Rl + mine] : Cg[(size_t)u * R + r];
+                const double y = u + parts < held ? cols[(size_t)(u + parts) * Rl + mine] : Cg[(size_t)(u + parts) * R + r];
+                s0 = fma(x, sh.w[u], s0);
+                s1 = fma(y, sh.w[u + parts], s1);
+            }
+            if (u < step) s0 = fma(u < held ? cols[(size_t)u * Rl + mine] : Cg[(size_t)u * R + r], sh.w[u], s0);
+        }
+        sh.part[t] = s0 + s1;
+        __syncthreads();
+        if (owner) {
+            for (int p = 0; p < parts; ++p) c -= sh.part[p * Rl + mine];
+            if (step < held) cols[(size_t)step * Rl + mine] = c;
+            else Cg[(size_t)step * R + r] = c;
+            mu = fma(c, delta, mu);
+            var -= c * c / s;
+        }
+    }
+    if (rank == 0 && t == 0) {
+        // The believer's EI only drops: nothing outside the shortlist could have been picked while the picks stayed above
+        // the best EI left out (FP32, within the scoring tolerance of 1e-5 max EI).
+        int cert = 1;
+        if (a.Rk > R) {
+            const double bound = a.sval[(size_t)g * a.Rk + R], top = a.sval[(size_t)g * a.Rk];
+            cert = !liar && lowest >= bound + 4e-5 * top ? 1 : 0;
+        }
+        a.cert[g] = cert;
+    }
+    cluster.sync();   // no block leaves while another may read its shared memory
+}
+
+size_t up16(size_t b) { return (b + 15) & ~(size_t)15; }
 
 }  // namespace
 
 size_t propose_workspace_bytes(int batch, int npad, int R, int q)
 {
-    return (size_t)batch * (sizeof(double) * (2 * (size_t)R * npad + (size_t)q * R + 2 * (size_t)R + 2 * (size_t)q) +
-                            sizeof(int) * ((size_t)R + q)) + 1024;
+    const size_t B = batch, NT = (npad + 63) / 64;
+    return up16(sizeof(double) * B * R * (2 * (size_t)npad + R + 2 * NT)) + up16(sizeof(double) * B * q * R) +
+           up16(sizeof(int) * B) + 256;
 }
 
-// The q picks of every GP of the handle.  sidx: device [batch][Rk] pool indices of the shortlists (by initial
-// EI, descending; the first R of each row are used); idx_out / ei_out: device [batch][q].
+// The q picks of every GP of the handle.  sidx, sval: device [batch][Rk] pool indices and EI of the shortlists (by initial
+// EI, descending; the first R of each row are used); idx_out / ei_out: device [batch][q]; *cert: device [batch].
 // ws: propose_workspace_bytes(batch, npad, R, q) bytes.
-r3_status_t propose_shortlist(r3_gp* gp, const float* Xcand, long long m, const int* sidx, int Rk, int R, int q, int liar,
-                              int* idx_out, float* ei_out, void* ws, cudaStream_t stream)
+r3_status_t propose_shortlist(r3_gp* gp, const float* Xcand, long long m, const int* sidx, const float* sval, int Rk, int R,
+                              int q, int liar, int* idx_out, float* ei_out, int** cert, void* ws, cudaStream_t stream)
 {
-    const int B = gp->batch, n = gp->n, d = gp->d, npad = gp->npad;
-    char* p = (char*)ws;
-    auto carve = [&](size_t bytes) {
-        char* r = p;
-        p += (bytes + 15) / 16 * 16;
-        return r;
-    };
     ProposeArrays a;
-    a.X = gp->X;
-    a.ell = gp->ell_d;
-    a.sf2 = gp->sf2_d;
-    a.sn2 = gp->sn2_d;
-    a.best = gp->best_d;
-    a.alpha = gp->alpha64;
-    a.Xcand = Xcand;
-    a.sidx = sidx;
+    a.X = gp->X; a.ell = gp->ell_d; a.sf2 = gp->sf2_d; a.sn2 = gp->sn2_d; a.best = gp->best_d; a.alpha = gp->alpha64;
+    a.W = gp->W64; a.Xcand = Xcand; a.sidx = sidx; a.sval = sval;
     a.m = m;
-    a.n = n;
-    a.d = d;
-    a.npad = npad;
-    a.R = R;
-    a.Rk = Rk;
-    a.q = q;
-    a.Ks = (double*)carve(sizeof(double) * (size_t)B * R * npad);
-    a.V = (double*)carve(sizeof(double) * (size_t)B * R * npad);
-    a.C = (double*)carve(sizeof(double) * (size_t)B * q * R);
-    a.mu = (double*)carve(sizeof(double) * (size_t)B * R);
-    a.var = (double*)carve(sizeof(double) * (size_t)B * R);
-    a.S = (double*)carve(sizeof(double) * (size_t)B * q);
-    a.delta = (double*)carve(sizeof(double) * (size_t)B * q);
-    a.picked = (int*)carve(sizeof(int) * (size_t)B * R);
-    a.sel = (int*)carve(sizeof(int) * (size_t)B * q);
+    a.B = gp->batch; a.n = gp->n; a.d = gp->d; a.npad = gp->npad; a.R = R; a.Rk = Rk; a.q = q;
+    const size_t B = a.B, npad = a.npad, NT = (npad + 63) / 64;
+    a.Ks = (double*)ws;
+    a.V = a.Ks + B * R * npad;
+    a.C0 = a.V + B * R * npad;
+    a.mupart = a.C0 + B * R * R;
+    a.qpart = a.mupart + B * R * NT;
+    char* p = (char*)ws + up16(sizeof(double) * B * R * (2 * npad + R + 2 * NT));
+    a.C = (double*)p;
+    p += up16(sizeof(double) * B * q * R);
+    a.cert = (int*)p;
+    p += up16(sizeof(int) * B);
+    a.barrier = (unsigned*)p;
+    a.status = gp->status_d;
+    *cert = a.cert;
+    R3_CUDA_TRY(cudaMemsetAsync(a.barrier, 0, sizeof(unsigned), stream));
 
-    R3_LAUNCH(shortlist_kstar_kernel, dim3((npad + 127) / 128, R, B), 128, 0, stream, a);
-    // V = Ks W^T (v_r = W k*_r): the same triangular product as the append step of the fit
-    R3_LAUNCH((tri_gemm_kernel<true, 64>), dim3((n + 63) / 64, (R + 63) / 64, B), 256, 0, stream, a.Ks, npad,
-              (size_t)R * npad, gp->W64, npad, (size_t)npad * npad, a.V, npad, (size_t)R * npad, R, n);
-    R3_LAUNCH(shortlist_moments_kernel, dim3((R + 7) / 8, B), 256, 0, stream, a);
-    for (int t = 0; t < q; ++t) {
-        R3_LAUNCH(pick_kernel, B, 1024, 0, stream, a, liar, t, idx_out, ei_out, gp->status_d);
-        if (t + 1 < q) R3_LAUNCH(condition_kernel, dim3((R + 7) / 8, B), 256, 0, stream, a, t);
+    int sms = 148;
+    R3_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, gp->device));
+    R3_CUDA_TRY(cudaFuncSetAttribute(build_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCrossStageBytes));
+    const long long items = (long long)B * ((R + 63) / 64) * NT;
+    const unsigned grid = (unsigned)std::min<long long>(2ll * sms, std::max<long long>(items, (long long)B * 4));
+    void* params[] = {&a};
+    R3_CUDA_TRY(cudaLaunchCooperativeKernel((const void*)build_kernel, dim3(grid), dim3(kCrossThreads), params, kCrossStageBytes,
+                                            stream));
+    ++g_launches;
+
+    // One block as long as its shared memory holds the columns of all picks (or nearly nothing would be gained by more),
+    // else a cluster of eight.
+    const size_t room = (kPickSmem - sizeof(PickShared)) / sizeof(double);
+    int CS = 1, Rl = round_up(R, 32);
+    if ((size_t)Rl * (q - 1) > room) {
+        CS = kMaxCluster;
+        Rl = round_up((R + CS - 1) / CS, 32);
     }
+    const int held = (int)std::min<size_t>(q, room / Rl);
+    R3_CUDA_TRY(cudaFuncSetAttribute(pick_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPickSmem));
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(B * CS));
+    cfg.blockDim = dim3(kPickThreads);
+    cfg.dynamicSmemBytes = sizeof(PickShared) + sizeof(double) * (size_t)held * Rl;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = CS;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    R3_CUDA_TRY(cudaLaunchKernelEx(&cfg, pick_kernel, a, liar, Rl, held, idx_out, ei_out));
+    ++g_launches;
     return R3_OK;
 }
 

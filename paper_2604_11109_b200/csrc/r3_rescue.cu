@@ -30,8 +30,8 @@
 // largest EI) and 201 us.
 #include <algorithm>
 
+#include "r3_cross.cuh"
 #include "r3_epilogue.cuh"
-#include "r3_f64.cuh"
 #include "r3_internal.cuh"
 #include "r3_topk.cuh"
 
@@ -39,13 +39,12 @@ namespace r3 {
 
 namespace {
 
-constexpr int kThreads = 256;
-constexpr int kTile = 64;        // rows of W and candidates of a tile of the long-list form
+constexpr int kThreads = kCrossThreads;
+constexpr int kTile = kCrossTile;   // rows of W and candidates of a tile of the long-list form
 constexpr int kSmallTile = 16;   // of the short-list form
-constexpr int kStages = 3;       // 16-deep operand stages in flight
 constexpr size_t kSlabBytes = 64ull << 20;   // FP64 cross-covariances in flight: they stay in L2 beside W
 constexpr int kOwnMaxN = 128;                // histories whose flagged candidates the flagging block recomputes itself
-constexpr size_t kOwnKs = 12 * 1024;         // byte offset of its k* behind the staged coordinates (10.9 KB)
+constexpr size_t kOwnKs = 12 * 1024;         // byte offset of its k* behind the staged coordinates (11.5 KB)
 constexpr size_t kMaxSmem = 80 * 1024;       // operand stages (60 KB) and the tile prefix of 4096 GPs
 constexpr int kFinishKeys = 4096;            // a GP whose slices leave at most this many keys is finished in the kernel
 
@@ -54,8 +53,8 @@ struct GuardArgs {
     const double *alpha64, *W64;
     int batch, n, d, npad;
     long long m;
-    int slice;                    // candidates per slice, a power of two in [32, 4096]
-    int slices_per_gp;
+    int chunk, chunks_per_gp;     // candidates a block looks over at a time (largest EI, flags)
+    int slice, slices_per_gp;     // candidates of which a block selects the k largest, a multiple of a chunk; at most 4096
     float *mu, *sigma, *ei;
     const float *err_mu, *err_q;
     int* list;                    // [batch][m] flagged candidates of each GP
@@ -72,7 +71,7 @@ struct GuardArgs {
     int k, K2;                    // top-k request (k = 0: none); K2 = min(k, slice): keys a slice yields
     unsigned select_offset;       // byte offset of the selection's scratch in the dynamic shared memory
     unsigned pref_offset;         // byte offset of the tile prefix
-    unsigned long long* keys;     // [batch][slices_per_gp][k]
+    unsigned long long* keys;     // [batch][slices_per_gp][K2]
     bool finish;                  // the last slice of a GP writes the answer
     int* idx;
     float* val;
@@ -129,74 +128,9 @@ __global__ void __launch_bounds__(1024) pilot_kernel(const GuardArgs a, long lon
     if (t == 0) *mode = (long long)count_s * 32 > rows ? 1 : 0;
 }
 
-// k* and the partial means of (CT candidates) x (64 observations): 256 threads, CT / 16 candidates x 4 observations
-// each.  store(c, k, k*) for every candidate c of the tile and every k < npad of the block (zero beyond n and beyond the
-// listed candidates), mean(c, sum) once per candidate.
-template <int CT, class List, class Store, class Mean>
-__device__ __forceinline__ void kstar_tile(const GuardArgs& a, int g, List list, int in_tile, int kb, unsigned char* smem,
-                                           Store store, Mean mean)
+__device__ __forceinline__ const float* cand_row(const GuardArgs& a, int g, int cand)
 {
-    constexpr int U = CT / 16;
-    float* zs = reinterpret_cast<float*>(smem);   // [CT][33]
-    float* xs = zs + CT * 33;                     // [64][33]
-    double* il = reinterpret_cast<double*>(xs + 64 * 33 + (CT * 33) % 2);   // [32] reciprocal lengthscales
-    const int t = threadIdx.x, tx = t % 16, ty = t / 16;
-    const int n = a.n, d = a.d, k0 = kb * 64;
-    double r2[U][4] = {};
-    for (int c0 = 0; c0 < d; c0 += 32) {
-        __syncthreads();
-        for (int e = t; e < CT * 32; e += kThreads) {
-            const int r = e / 32, c = e % 32;
-            float z = 0.f;
-            if (r < in_tile && c0 + c < d) {
-                const int cand = list(r);
-                z = a.Xcand[(size_t)R3_IDX((long long)g * a.m + cand, (long long)a.batch * a.m, a.status) * d + c0 + c];
-            }
-            zs[r * 33 + c] = z;
-        }
-        for (int e = t; e < 64 * 32; e += kThreads) {
-            const int r = e / 32, c = e % 32;
-            xs[r * 33 + c] = (k0 + r < n && c0 + c < d) ? a.X[((size_t)g * n + k0 + r) * d + c0 + c] : 0.f;
-        }
-        if (t < 32) il[t] = (c0 + t < d) ? 1.0 / (double)a.ell[(size_t)g * d + c0 + t] : 0.0;
-        __syncthreads();
-        const int cmax = min(32, d - c0);
-        for (int c = 0; c < cmax; ++c) {
-            double z[U], x[4];
-#pragma unroll
-            for (int u = 0; u < U; ++u) z[u] = (double)zs[(ty + 16 * u) * 33 + c];
-#pragma unroll
-            for (int v = 0; v < 4; ++v) x[v] = (double)xs[(tx + 16 * v) * 33 + c];
-            const double w = il[c];
-#pragma unroll
-            for (int u = 0; u < U; ++u)
-#pragma unroll
-                for (int v = 0; v < 4; ++v) {
-                    const double df = (x[v] - z[u]) * w;
-                    r2[u][v] = fma(df, df, r2[u][v]);
-                }
-        }
-    }
-    const double sf2 = (double)a.sf2v[g];
-    const double* alpha = a.alpha64 + (size_t)g * a.npad;
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-        double part = 0.0;
-#pragma unroll
-        for (int v = 0; v < 4; ++v) {
-            const int k = k0 + tx + 16 * v;
-            if (k >= a.npad) continue;
-            double kv = 0.0;
-            if (k < n) {
-                const double sq = sqrt(5.0) * sqrt(r2[u][v]);
-                kv = sf2 * (1.0 + sq + sq * sq / 3.0) * exp(-sq);
-                part = fma(kv, alpha[k], part);
-            }
-            store(ty + 16 * u, k, kv);
-        }
-        for (int o = 8; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
-        if (tx == 0) mean(ty + 16 * u, part);
-    }
+    return a.Xcand + (size_t)R3_IDX((long long)g * a.m + cand, (long long)a.batch * a.m, a.status) * a.d;
 }
 
 __device__ __forceinline__ void write_result(const GuardArgs& a, int g, int cand, double mu, double q)
@@ -212,52 +146,12 @@ __device__ __forceinline__ void write_result(const GuardArgs& a, int g, int cand
 __device__ __forceinline__ void rescue_tile(const GuardArgs& a, const double* __restrict__ Wg, size_t slot0, int rt,
                                             unsigned char* smem)
 {
-    double* sA = reinterpret_cast<double*>(smem);         // [stages][64][20]
-    double* sB = sA + kStages * kTile * kStageLd;
-    const int t = threadIdx.x, w = t / 32, l = t % 32;
-    const int wm = (w % 4) * 16, wn = (w / 4) * 32;       // 16 x 32 per warp
+    const int t = threadIdx.x, w = t / 32, l = t % 32, wn = (w / 4) * 32;
     const int npad = a.npad, i0 = rt * kTile;
-    const int kend = min(npad, i0 + kTile);               // W is lower triangular
-    const int steps = kend / 16;
-    auto load = [&](int s, int k0) {
-#pragma unroll
-        for (int it = 0; it < 2; ++it) {
-            const int e = t + kThreads * it, r = e / 8, q = e % 8;
-            const bool ok = i0 + r < npad;
-            cp_async16(sA + (s * kTile + r) * kStageLd + 2 * q, Wg + (size_t)(ok ? i0 + r : 0) * npad + k0 + 2 * q, ok);
-            cp_async16(sB + (s * kTile + r) * kStageLd + 2 * q,
-                       a.ks + (size_t)R3_IDX(slot0 + r, a.slab, a.status) * npad + k0 + 2 * q);
-        }
-    };
     double c[2][4][2] = {};
-    __syncthreads();   // the previous item's reads of the stages are done
-#pragma unroll
-    for (int s = 0; s < kStages - 1; ++s) {
-        if (s < steps) load(s, s * 16);
-        cp_async_commit();
-    }
-    for (int kb = 0; kb < steps; ++kb) {
-        cp_async_wait<kStages - 2>();
-        __syncthreads();
-        if (kb + kStages - 1 < steps) load((kb + kStages - 1) % kStages, (kb + kStages - 1) * 16);
-        cp_async_commit();
-        const double* pa = sA + ((kb % kStages) * kTile + wm + l / 4) * kStageLd + l % 4;
-        const double* pb = sB + ((kb % kStages) * kTile + wn + l / 4) * kStageLd + l % 4;
-#pragma unroll
-        for (int kk = 0; kk < 16; kk += 4) {
-            double fa[2], fb[4];
-#pragma unroll
-            for (int i = 0; i < 2; ++i) fa[i] = pa[i * 8 * kStageLd + kk];
-#pragma unroll
-            for (int j = 0; j < 4; ++j) fb[j] = pb[j * 8 * kStageLd + kk];
-#pragma unroll
-            for (int i = 0; i < 2; ++i)
-#pragma unroll
-                for (int j = 0; j < 4; ++j) dmma(c[i][j], fa[i], fb[j]);
-        }
-    }
-    cp_async_wait<0>();
-    __syncthreads();
+    // W is lower triangular: columns up to the tile's last row
+    nt_tile(Wg + (size_t)i0 * npad, npad - i0, a.ks + (size_t)R3_IDX(slot0, a.slab - (kTile - 1), a.status) * npad, kTile, npad,
+            min(npad, i0 + kTile), smem, c);
     double* red = reinterpret_cast<double*>(smem);        // [4 row warps][64 candidates]
 #pragma unroll
     for (int j = 0; j < 4; ++j)
@@ -347,8 +241,11 @@ __device__ __forceinline__ bool rescue(const GuardArgs& a, const int* pref, int 
             const int* list_g = a.list + (size_t)g * a.m + first;
             const int kb = item / nt;
             const size_t slot0 = R3_IDX((size_t)tile * CT, a.slab - (CT - 1), a.status);
-            kstar_tile<CT>(
-                a, g, [&](int r) { return __ldcg(list_g + r); }, min(CT, __ldcg(a.count + g) - first), kb, smem,
+            const int in_tile = min(CT, __ldcg(a.count + g) - first);
+            cross_tile<CT>(
+                a.n, a.d, a.npad, a.ell + (size_t)g * a.d, (double)a.sf2v[g], a.alpha64 + (size_t)g * a.npad,
+                [&](int r) { return r < in_tile ? cand_row(a, g, __ldcg(list_g + r)) : nullptr; },
+                [&](int k) { return a.X + ((size_t)g * a.n + k) * a.d; }, kb, smem,
                 [&](int c, int k, double kv) { a.ks[(slot0 + c) * a.npad + k] = kv; },
                 [&](int c, double part) { a.mupart[(slot0 + c) * nb + kb] = part; });
         }
@@ -364,7 +261,9 @@ __device__ __forceinline__ bool rescue(const GuardArgs& a, const int* pref, int 
             const int tile = s / CT, g = gp_of(t0 + tile), pos = (t0 + tile - pref[g]) * CT + s % CT;
             if (pos >= __ldcg(a.count + g)) continue;
             double mu = 0.0, q = 0.0;
+#pragma unroll 4
             for (int b = 0; b < nb; ++b) mu += __ldcg(a.mupart + (size_t)s * nb + b);
+#pragma unroll 4
             for (int r = 0; r < row_tiles; ++r) q += __ldcg(a.qpart + (size_t)s * (a.npad / 16) + r);
             write_result(a, g, __ldcg(a.list + (size_t)g * a.m + pos), mu, q);
         }
@@ -385,8 +284,10 @@ __device__ __forceinline__ void rescue_own(const GuardArgs& a, int g, const int*
     const int t = threadIdx.x, w = t / 32, l = t % 32;
     if (t < kSmallTile) mu_s[t] = 0.0;
     for (int kb = 0; kb < (a.npad + 63) / 64; ++kb)
-        kstar_tile<kSmallTile>(
-            a, g, [&](int r) { return own[r]; }, count, kb, smem, [&](int c, int k, double kv) { ks[c * ld + k] = kv; },
+        cross_tile<kSmallTile>(
+            a.n, a.d, a.npad, a.ell + (size_t)g * a.d, (double)a.sf2v[g], a.alpha64 + (size_t)g * a.npad,
+            [&](int r) { return r < count ? cand_row(a, g, own[r]) : nullptr; },
+            [&](int k) { return a.X + ((size_t)g * a.n + k) * a.d; }, kb, smem, [&](int c, int k, double kv) { ks[c * ld + k] = kv; },
             [&](int c, double part) { mu_s[c] += part; });
     __syncthreads();
     const double* Wg = a.W64 + (size_t)g * a.npad * a.npad;
@@ -437,16 +338,17 @@ __global__ void __launch_bounds__(kThreads, 2) guard_kernel(const GuardArgs a)
     __shared__ bool last_slice;
     const int t = threadIdx.x, lane = t % 32, warp = t / 32;
     const long long m = a.m;
-    const int slices = a.slices_per_gp * a.batch;
+    const int slices = a.slices_per_gp * a.batch, chunks = a.chunks_per_gp * a.batch;
     const bool own_rescue = a.npad <= kOwnMaxN;
     unsigned target = 0;
 
     // ---- the pool's largest EI
     if (!a.have_max) {
-        for (int s = blockIdx.x; s < slices; s += gridDim.x) {
-            const int g = s / a.slices_per_gp;
-            const long long c0 = (long long)(s % a.slices_per_gp) * a.slice, c1 = min(m, c0 + a.slice);
+        for (int s = blockIdx.x; s < chunks; s += gridDim.x) {
+            const int g = s / a.chunks_per_gp;
+            const long long c0 = (long long)(s % a.chunks_per_gp) * a.chunk, c1 = min(m, c0 + a.chunk);
             float v = 0.f;
+#pragma unroll 8
             for (long long i = c0 + t; i < c1; i += kThreads) v = fmaxf(v, __ldcg(a.ei + (size_t)g * m + i));  // EI >= 0; fmaxf ignores NaN
             const unsigned top = __reduce_max_sync(0xffffffffu, __float_as_uint(v));   // order-preserving for v >= 0
             if (lane == 0 && top) atomicMax(&a.maxbits[g], top);
@@ -455,9 +357,9 @@ __global__ void __launch_bounds__(kThreads, 2) guard_kernel(const GuardArgs a)
     }
 
     // ---- flag
-    for (int s = blockIdx.x; s < slices; s += gridDim.x) {
-        const int g = s / a.slices_per_gp;
-        const long long c0 = (long long)(s % a.slices_per_gp) * a.slice, c1 = min(m, c0 + a.slice);
+    for (int s = blockIdx.x; s < chunks; s += gridDim.x) {
+        const int g = s / a.chunks_per_gp;
+        const long long c0 = (long long)(s % a.chunks_per_gp) * a.chunk, c1 = min(m, c0 + a.chunk);
         const float sf2 = a.sf2v[g], best = a.bestv[g];
         const float tol_ei = 1e-5f * __uint_as_float(__ldcg(a.maxbits + g));
         const float mu_floor = 1e-6f * a.yabsv[g], sd_floor = 1e-6f * sqrtf(sf2);
@@ -466,6 +368,7 @@ __global__ void __launch_bounds__(kThreads, 2) guard_kernel(const GuardArgs a)
             if (t == 0) own_count = 0;
             __syncthreads();
         }
+#pragma unroll 2
         for (long long i0 = c0; i0 < c1; i0 += kThreads) {
             const long long i = i0 + t;
             bool flag = false;
@@ -552,14 +455,15 @@ __global__ void __launch_bounds__(kThreads, 2) guard_kernel(const GuardArgs a)
         const long long c0 = (long long)(s % a.slices_per_gp) * a.slice;
         const float* e = a.ei + (size_t)g * m;
         __syncthreads();
+#pragma unroll 8
         for (int i = t; i < a.slice; i += kThreads) {
             const long long c = c0 + i;
             keys_s[i] = (c < m) ? topk_make_key(__ldcg(e + c), (unsigned)c) : 0ull;
         }
         __syncthreads();
         block_select_desc(keys_s, a.slice, a.K2, smem + a.select_offset);
-        unsigned long long* out = a.keys + (size_t)s * a.k;
-        for (int i = t; i < a.k; i += kThreads) out[i] = i < a.slice ? keys_s[R3_IDX(i, a.slice, a.status)] : 0ull;
+        unsigned long long* out = a.keys + (size_t)s * a.K2;
+        for (int i = t; i < a.K2; i += kThreads) out[i] = keys_s[R3_IDX(i, a.slice, a.status)];
         if (a.finish) {
             __threadfence();
             __syncthreads();
@@ -567,8 +471,9 @@ __global__ void __launch_bounds__(kThreads, 2) guard_kernel(const GuardArgs a)
             __syncthreads();
             if (last_slice) {   // this block saw the GP's last slice: its keys are all there
                 __threadfence();
-                const int nk = a.slices_per_gp * a.k;
+                const int nk = a.slices_per_gp * a.K2;
                 const unsigned long long* in = a.keys + (size_t)g * nk;
+#pragma unroll 8
                 for (int i = t; i < nk; i += kThreads) keys_s[i] = __ldcg(in + i);
                 __syncthreads();
                 block_select_desc(keys_s, nk, a.k, smem + a.select_offset);
@@ -626,19 +531,30 @@ GuardBuffers guard_carve(const r3_gp* gp, long long m, void* ws)
     return b;
 }
 
-// Candidates per slice: enough slices to fill the GPU on a large pool, small ones on a small pool.
-static int guard_slice(int batch, long long m, int k)
+// Candidates per chunk: enough chunks to fill the GPU on a large pool, small ones on a small pool.
+static int guard_chunk(int batch, long long m)
 {
     long long s = 128;
     while (s < 4096 && s < m && s * 296 < (long long)batch * m) s <<= 1;
     return (int)s;
 }
 
+// Candidates per slice of the selection: a chunk, or more when that brings the slices' keys down to what the kernel
+// finishes by itself (262,144 candidates, k = 32: two more launches and 8192 keys 15 us, one block over 8192 keys 25 us).
+static int guard_slice(int batch, long long m, int k)
+{
+    const long long s = guard_chunk(batch, m);
+    auto keys = [&](long long v) { return (m + v - 1) / v * std::min<long long>(k, v); };
+    long long v = s;
+    while (v < 4096 && v < m && keys(v) > kFinishKeys) v <<= 1;
+    return (int)(keys(v) <= kFinishKeys ? v : s);
+}
+
 size_t guard_topk_workspace_bytes(int batch, long long m, int k)
 {
     const int slice = guard_slice(batch, m, k);
     const long long slices = (m + slice - 1) / slice;
-    return 2 * (size_t)batch * slices * k * sizeof(unsigned long long) + 64;
+    return 2 * (size_t)batch * slices * std::min(k, slice) * sizeof(unsigned long long) + 64;
 }
 
 // counts, maxima, finished slices and the grid barrier
@@ -667,6 +583,8 @@ r3_status_t guard_and_rescue(r3_gp* gp, const float* Xcand, long long m, const G
     a.alpha64 = gp->alpha64; a.W64 = gp->W64;
     a.batch = B; a.n = gp->n; a.d = gp->d; a.npad = gp->npad;
     a.m = m;
+    a.chunk = guard_chunk(B, m);
+    a.chunks_per_gp = (int)((m + a.chunk - 1) / a.chunk);
     a.slice = guard_slice(B, m, req.k);
     a.slices_per_gp = (int)((m + a.slice - 1) / a.slice);
     a.mu = mu; a.sigma = sigma; a.ei = ei;
@@ -687,14 +605,14 @@ r3_status_t guard_and_rescue(r3_gp* gp, const float* Xcand, long long m, const G
     a.keys = (unsigned long long*)req.ws;
     a.idx = req.idx;
     a.val = req.val;
-    const long long keys_per_gp = (long long)a.slices_per_gp * req.k;
+    const long long keys_per_gp = (long long)a.slices_per_gp * a.K2;
     a.finish = req.k > 0 && keys_per_gp <= kFinishKeys;
     if (req.k > 0 && req.ws_bytes < guard_topk_workspace_bytes(B, m, req.k)) {
         set_error("internal: top-k workspace of the guard too small");
         return R3_ERR_INVALID_ARG;
     }
     // dynamic shared memory: operand stages / slice keys, then the selection's scratch, then the tile prefix
-    size_t region = sizeof(double) * kStages * 2 * kTile * kStageLd;
+    size_t region = kCrossStageBytes;
     a.select_offset = (unsigned)(sizeof(unsigned long long) * (a.finish ? (size_t)kFinishKeys : (size_t)a.slice));
     if (req.k > 0) region = std::max(region, a.select_offset + topk_select_scratch_bytes(a.finish ? req.k : a.K2));
     a.pref_offset = (unsigned)up16(region);
@@ -705,8 +623,8 @@ r3_status_t guard_and_rescue(r3_gp* gp, const float* Xcand, long long m, const G
     R3_CUDA_TRY(cudaFuncSetAttribute(guard_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem));
     // two blocks per SM (launch bounds and 112 KB of shared memory allow it); a small pool is served by half of them,
     // because the barriers then cost more than the work between them
-    const long long slices = (long long)a.slices_per_gp * B;
-    const unsigned grid = (unsigned)(slices <= sms ? sms : 2 * sms);
+    const long long chunks = (long long)a.chunks_per_gp * B;
+    const unsigned grid = (unsigned)(chunks <= sms ? sms : 2 * sms);
     void* params[] = {&a};
     R3_CUDA_TRY(cudaLaunchCooperativeKernel((const void*)guard_kernel, dim3(grid), dim3(kThreads), params, smem, stream));
     ++g_launches;

@@ -135,3 +135,31 @@ def test_errors():
         assert e.value.status == 3
         b.r3_gp_check(gp)        # the handle stays usable
     gp.close()
+
+
+@pytest.mark.parametrize("batch,n,m,q,shortlist", [
+    (1, 40, 1500, 1, 0),          # a single pick: no conditioning
+    (3, 70, 900, 20, 0),          # one block per GP
+    (1, 90, 3000, 60, 600),       # a cluster of eight
+    (2, 64, 1200, 256, 1023),     # more picks than fit shared memory
+    (1, 200, 33, 33, 33),         # every candidate is picked
+])
+def test_picks_follow_the_definition_at_every_split(batch, n, m, q, shortlist):
+    """Each pick must be the best (to the contract) of the posterior conditioned on the picks before it: the oracle
+    conditions on the library's own picks, at a few places of the sequence."""
+    g = problem(4000 + n, batch, n, 4, m, sn2=1e-2)
+    gp = b.r3_gp_fit(dev(g["X"]), dev(g["y"]), g["ell"], g["sf2"], g["sn2"])
+    idx, val, cert = b.r3_gp_propose(gp, dev(g["Xcand"]), q, shortlist=shortlist)
+    b.r3_gp_check(gp)
+    idx, val = idx.cpu().numpy(), val.cpu().numpy()
+    for q_ in range(batch):
+        assert len(set(idx[q_].tolist())) == q
+        first = oracle_ei_at_step(g, q_, [], "believer")
+        tol = max(1e-5 * first.max(), EI_ABS_FLOOR)
+        for t in sorted({0, 1, q // 2, q - 1} & set(range(q))):
+            e = oracle_ei_at_step(g, q_, idx[q_][:t].tolist(), "believer")
+            left = np.setdiff1d(np.arange(m), idx[q_][:t])
+            assert abs(val[q_][t] - e[idx[q_][t]]) <= tol
+            if cert[q_]:
+                assert e[idx[q_][t]] >= e[left].max() - tol
+    gp.close()
