@@ -6,8 +6,10 @@
 // rounded up to five significant bits so that neighbouring sizes (a history that grew by a few
 // rows) share a bin; blocks below 1 MiB -- a small history's fit is two dozen of them, and their cudaMalloc and
 // cudaFree calls were most of its time -- are rounded up to a multiple of 512 bytes and kept as well.  dev_free waits for the device like cudaFree does, which makes the block safe to
-// reuse at once.  The cache holds at most kCacheLimit bytes per device; r3_trim_cache() returns
-// everything to the driver.
+// reuse at once.  The cache holds at most kCacheLimit bytes per device: a block that would go over the limit pushes out
+// the ones that have lain there longest (a program whose sizes change would otherwise fill the cache with sizes it no
+// longer asks for, and pay the driver for every block from then on).  r3_trim_cache() returns everything to the driver.
+#include <list>
 #include <map>
 #include <mutex>
 #include <vector>
@@ -22,8 +24,14 @@ constexpr size_t kCacheLimit = 2ull << 30;
 constexpr size_t kSmall = 1 << 20;   // below 1 MiB: bins of 512 bytes
 constexpr size_t kCacheBlocks = 4096;   // at most this many kept blocks per device
 
+struct FreeBlock {
+    size_t bin;
+    void* p;
+};
+
 struct DeviceCache {
-    std::multimap<size_t, void*> free_blocks;   // bin size -> block
+    std::list<FreeBlock> by_age;                                         // oldest first
+    std::multimap<size_t, std::list<FreeBlock>::iterator> free_blocks;   // bin size -> block
     std::map<void*, size_t> live;               // block -> bin size (only blocks handed out by dev_malloc)
     size_t cached_bytes = 0;
 };
@@ -71,7 +79,8 @@ cudaError_t dev_malloc_bytes(void** p, size_t bytes)
         DeviceCache& c = g_cache[dev];
         auto it = c.free_blocks.find(bin);
         if (it != c.free_blocks.end()) {
-            *p = it->second;
+            *p = it->second->p;
+            c.by_age.erase(it->second);
             c.free_blocks.erase(it);
             c.cached_bytes -= bin;
             c.live[*p] = bin;
@@ -116,11 +125,20 @@ void dev_free(void* p)
     if (t_no_wait == 0) cudaDeviceSynchronize();   // as cudaFree would: nothing in flight may still use the block
     std::lock_guard<std::mutex> lock(g_mutex);
     DeviceCache& c = g_cache[dev];
-    if (c.cached_bytes + bin > kCacheLimit || c.free_blocks.size() >= kCacheBlocks) {
+    if (bin > kCacheLimit) {
         cudaFree(p);
         return;
     }
-    c.free_blocks.emplace(bin, p);
+    while (c.cached_bytes + bin > kCacheLimit || c.free_blocks.size() >= kCacheBlocks) {
+        const auto oldest = c.by_age.begin();
+        auto it = c.free_blocks.lower_bound(oldest->bin);
+        while (it->second != oldest) ++it;
+        c.free_blocks.erase(it);
+        c.cached_bytes -= oldest->bin;
+        cudaFree(oldest->p);
+        c.by_age.erase(oldest);
+    }
+    c.free_blocks.emplace(bin, c.by_age.insert(c.by_age.end(), FreeBlock{bin, p}));
     c.cached_bytes += bin;
 }
 
@@ -132,8 +150,9 @@ void trim_cache()
     {
         std::lock_guard<std::mutex> lock(g_mutex);
         DeviceCache& c = g_cache[dev];
-        for (auto& kv : c.free_blocks) blocks.push_back(kv.second);
+        for (const FreeBlock& b : c.by_age) blocks.push_back(b.p);
         c.free_blocks.clear();
+        c.by_age.clear();
         c.cached_bytes = 0;
     }
     for (void* b : blocks) cudaFree(b);

@@ -168,3 +168,19 @@ def test_two_live_handles_that_share_a_kernel_instantiation():
     _scores_match(gb, bb, "B after C")
     for h in (a, bb, c):
         h.close()
+
+
+def test_the_cache_makes_room_for_sizes_that_are_still_in_use():
+    """A program that changes its sizes must not fill the cache with blocks of sizes it has left: beyond the limit the
+    block that has lain there longest goes, and the newest is kept."""
+    b.r3_trim_cache()
+    for n in (2048, 2304, 2560, 2816, 3072, 3328, 3584, 3840):   # fits of 120 to 420 MB, over 2 GiB together
+        g = rand_problem(30, 1, n, 3, 8)
+        fit_gpu(g).close()
+    full = b.r3_cached_bytes()
+    assert (1 << 30) < full <= (2 << 30)
+    gp = fit_gpu(g)                       # the last size is served from the cache
+    assert b.r3_cached_bytes() < full - (200 << 20)
+    gp.close()
+    b.r3_trim_cache()
+    assert b.r3_cached_bytes() == 0
