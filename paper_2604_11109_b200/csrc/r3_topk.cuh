@@ -49,7 +49,7 @@ __host__ __device__ inline size_t topk_select_scratch_bytes(int K)
 // 1 <= K <= n; blockDim.x is a multiple of 32; all threads of the block call it.
 //
 // Radix selection, then a rank sort of the K survivors -- no sorting network over the n keys:
-//  1. the K-th largest key is found digit by digit from the top (8 bits per step): a histogram of the digit
+//  1. the K-th largest key is found digit by digit (8 bits per step) from the highest bit in which the keys differ: a histogram of the digit
 //     over the keys that match the digits found so far (lanes that share a digit with the warp's first active lane add once, so a
 //     pool whose values share their exponent does not serialise on one bin), a walk over the 256 bins from the top by one
 //     warp; it stops as soon as the chosen bin holds one key, typically after three or four steps;
@@ -74,17 +74,34 @@ __device__ __forceinline__ void block_select_desc(unsigned long long* s, int n, 
     if (K >= n) {
         for (int i = tid; i < n; i += T) tmp[i] = s[i];
     } else {
-        unsigned long long prefix = 0ull;   // the digits of the K-th largest key found so far, in place
+        const int n_up = (n + 31) & ~31;    // whole warps take part in the votes below
+        // the bits above the highest one in which the keys differ need no step (values of a pool share their exponent)
+        __syncthreads();                    // the caller's keys are in place
+        const unsigned long long first_key = s[0];
+        unsigned long long diff = 0ull;
+#pragma unroll 4
+        for (int i = tid; i < n; i += T) diff |= s[i] ^ first_key;
+        const unsigned dh = __reduce_or_sync(0xffffffffu, (unsigned)(diff >> 32)), dl = __reduce_or_sync(0xffffffffu, (unsigned)diff);
+        if (tid == 0) sel[6] = sel[7] = 0u;
+        __syncthreads();
+        if (lane == 0) {
+            if (dh) atomicOr(&sel[6], dh);
+            if (dl) atomicOr(&sel[7], dl);
+        }
+        __syncthreads();
+        diff = ((unsigned long long)sel[6] << 32) | sel[7];
+        int shift = diff ? max(0, 63 - __clzll((long long)diff) - 7) : 0;
+        // the digits of the K-th largest key found so far, in place
+        unsigned long long decided = shift == 56 ? 0ull : ~0ull << (shift + 8);   // the bits they cover
+        unsigned long long prefix = first_key & decided;
         unsigned want = (unsigned)K;        // its rank among the keys that share them
-        int shift = 56;
-        const int n_up = (n + 31) & ~31;    // whole warps take part in the vote below
-        for (;; shift -= 8) {
+        for (;; shift = max(0, shift - 8)) {
             for (int b = tid; b < 256; b += T) hist[b] = 0u;
             __syncthreads();
-            const unsigned long long himask = shift == 56 ? 0ull : (~0ull << (shift + 8));
+#pragma unroll 4
             for (int i = tid; i < n_up; i += T) {
                 const unsigned long long key = i < n ? s[i] : 0ull;
-                const bool act = i < n && (key & himask) == prefix;
+                const bool act = i < n && (key & decided) == prefix;
                 const unsigned dgt = (unsigned)(key >> shift) & 255u;
                 // the lanes that share the first active lane's digit add once (pools whose values share their
                 // exponent would otherwise serialise on one bin); the others add for themselves
@@ -124,12 +141,14 @@ __device__ __forceinline__ void block_select_desc(unsigned long long* s, int n, 
                 }
             }
             __syncthreads();
-            prefix |= (unsigned long long)sel[0] << shift;
+            prefix |= (unsigned long long)sel[0] << shift;   // the last step's window may overlap the one before
+            decided = ~0ull << shift;
             want = sel[1];
             if (sel[2] == 1u || shift == 0) break;
         }
         // gather: the keys above the chosen bin (K - want of them), then `want` keys of the bin
         const unsigned long long ph = prefix >> shift;
+#pragma unroll 4
         for (int i = tid; i < n_up; i += T) {
             const unsigned long long key = i < n ? s[i] : 0ull, hi = key >> shift;
             const bool above = i < n && hi > ph;
