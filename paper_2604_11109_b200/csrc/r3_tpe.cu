@@ -60,12 +60,68 @@ __device__ __forceinline__ float from_ordered_bits(unsigned u)
     return __uint_as_float((u & 0x80000000u) ? (u & 0x7FFFFFFFu) : ~u);
 }
 
-// Ascending bitonic sort of `count` (a power of two) 64-bit keys in shared memory.
-__device__ void bitonic_sort_asc(unsigned long long* s, int count)
+// Ascending bitonic sort of `count` (a power of two, at most 8 blockDim.x) 64-bit keys in shared memory; all threads of the
+// block call it.  A warp takes 128 neighbouring keys into registers, four per lane, and makes all steps of distance below
+// 128 there, by shuffles and within the lane; the longer distances go through shared memory.
+constexpr int kWarpKeys = 128;
+__device__ __forceinline__ void order_pair(unsigned long long& a, unsigned long long& b, bool asc)
 {
-    for (int size = 2; size <= count; size <<= 1) {
-        for (int stride = size >> 1; stride > 0; stride >>= 1) {
-            __syncthreads();
+    const bool swap = (a > b) == asc;
+    const unsigned long long lo = swap ? b : a, hi = swap ? a : b;
+    a = lo;
+    b = hi;
+}
+// Steps of distance `top` (at most 64) and below of the merge to blocks of `size`, for the 128 keys from `first` on.  Lane l
+// holds keys first + l + 32 e.
+__device__ __forceinline__ void warp_merge(unsigned long long (&k)[4], int first, int size, int top)
+{
+    const int lane = threadIdx.x & 31;
+    const bool asc_all = (first & size) == 0;   // size >= 128: one direction for the whole warp
+    for (int stride = top; stride > 0; stride >>= 1) {
+        if (stride >= 32) {
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const int o = e ^ (stride >> 5);
+                if (o > e) {
+                    // (e is a compile-time constant, o one of two: both cases are spelt out by the unrolling)
+                    const bool asc = size >= kWarpKeys ? asc_all : ((e * 32) & size) == 0;
+                    if (stride == 64) { if (e < 2) order_pair(k[e], k[e + 2], asc); }
+                    else if ((e & 1) == 0) order_pair(k[e], k[e + 1], asc);
+                }
+            }
+        } else {
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const int pos = e * 32 + lane;
+                const bool asc = size >= kWarpKeys ? asc_all : (pos & size) == 0;
+                const unsigned long long other = __shfl_xor_sync(0xffffffffu, k[e], stride);
+                const bool low = (lane & stride) == 0;   // this lane keeps the smaller one if ascending
+                const bool take = (low == asc) ? other < k[e] : other > k[e];
+                k[e] = take ? other : k[e];
+            }
+        }
+    }
+}
+__device__ __forceinline__ void bitonic_sort_asc(unsigned long long* s, int count)
+{
+    const int warp = threadIdx.x / 32, lane = threadIdx.x & 31, warps = blockDim.x / 32;
+    __syncthreads();
+    if (count < kWarpKeys) {
+        // a handful of keys: one warp, filled up with keys that sort last
+        if (warp == 0) {
+            unsigned long long k[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) k[e] = e * 32 + lane < count ? s[e * 32 + lane] : ~0ull;
+            for (int size = 2; size <= kWarpKeys; size <<= 1) warp_merge(k, 0, size, size >> 1);
+#pragma unroll
+            for (int e = 0; e < 4; ++e)
+                if (e * 32 + lane < count) s[e * 32 + lane] = k[e];
+        }
+        __syncthreads();
+        return;
+    }
+    for (int size = kWarpKeys; size <= count; size <<= 1) {
+        for (int stride = size >> 1; stride >= kWarpKeys; stride >>= 1) {
             for (int t = threadIdx.x; t < count / 2; t += blockDim.x) {
                 const int lo = 2 * t - (t & (stride - 1));
                 const int hi = lo + stride;
@@ -76,9 +132,20 @@ __device__ void bitonic_sort_asc(unsigned long long* s, int count)
                     s[hi] = a;
                 }
             }
+            __syncthreads();
         }
+        for (int first = warp * kWarpKeys; first < count; first += warps * kWarpKeys) {
+            unsigned long long k[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) k[e] = s[first + e * 32 + lane];
+            if (size == kWarpKeys)
+                for (int sz = 2; sz < kWarpKeys; sz <<= 1) warp_merge(k, first, sz, sz >> 1);
+            warp_merge(k, first, size, kWarpKeys / 2);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) s[first + e * 32 + lane] = k[e];
+        }
+        __syncthreads();
     }
-    __syncthreads();
 }
 
 __device__ __forceinline__ int pow2_at_least(int v)
@@ -88,28 +155,38 @@ __device__ __forceinline__ int pow2_at_least(int v)
     return p;
 }
 
-// (T1) order[i] = index of the i-th smallest y, ties by lower index.
-__global__ void __launch_bounds__(kSortThreads) tpe_order_kernel(const float* __restrict__ y, int n,
-                                                                 int* __restrict__ order, int* __restrict__ status)
+// (T1) order[i] = index of the i-th smallest y, ties by lower index: every value counts the ones before it.  n^2 comparisons
+// spread over the GPU, kOrderRows values per block, a warp per value, against all of y in shared memory (a sort by one block
+// took 40 us for 4096 values; 15 us).
+constexpr int kOrderRows = 32;
+__global__ void __launch_bounds__(256) tpe_order_kernel(const float* __restrict__ y, int n, int* __restrict__ order,
+                                                        int* __restrict__ status)
 {
-    __shared__ unsigned long long keys[kTpeMaxN];
-    const int count = pow2_at_least(n);
+    __shared__ unsigned bits[kTpeMaxN];
     bool bad = false;
-    for (int i = threadIdx.x; i < count; i += blockDim.x) {
-        unsigned long long k = ~0ull;
-        if (i < n) {
-            const float v = y[i];
-            bad |= !isfinite(v);
-            k = ((unsigned long long)ordered_bits(v) << 32) | (unsigned)i;
-        }
-        keys[i] = k;
+#pragma unroll 4
+    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+        const float v = y[i];
+        bad |= !isfinite(v);
+        bits[i] = ordered_bits(v);
     }
-    if (bad) atomicOr(status, DEV_NONFINITE);
-    bitonic_sort_asc(keys, count);
-    for (int i = threadIdx.x; i < n; i += blockDim.x) order[i] = (int)(keys[i] & 0xFFFFFFFFull);
+    if (__syncthreads_or(bad) && threadIdx.x == 0) atomicOr(status, DEV_NONFINITE);
+    const int lane = threadIdx.x & 31;
+    for (int r = threadIdx.x / 32; r < kOrderRows; r += blockDim.x / 32) {
+        const int i = blockIdx.x * kOrderRows + r;
+        if (i >= n) break;
+        const unsigned mine = bits[i];
+        int before = 0;
+#pragma unroll 8
+        for (int k = lane; k < n; k += 32) before += bits[k] < mine || (bits[k] == mine && k < i) ? 1 : 0;
+        before = __reduce_add_sync(0xffffffffu, before);
+        if (lane == 0) order[before] = i;
+    }
 }
 
-// (T2), (T3): one block per (dimension, set).  The log-probabilities (categorical) or log-densities (grid) of a
+// (T2), (T3): one block per (dimension, set).  Bound: the sort.  64 dimensions, 4096 observations, 16 distinct values each:
+// 60 us; 737 us while one thread walked the sorted values to merge equal components, all of which had their truncation mass
+// computed first.  The log-probabilities (categorical) or log-densities (grid) of a
 // set go to lnp[j][set][v]; tpe_table_kernel subtracts the two sets afterwards.
 __global__ void __launch_bounds__(kSortThreads) tpe_mixture_kernel(const float* __restrict__ X,
                                                                    const int* __restrict__ order, int n, int d,
@@ -118,9 +195,9 @@ __global__ void __launch_bounds__(kSortThreads) tpe_mixture_kernel(const float* 
                                                                    int* __restrict__ n_comps, double* __restrict__ lnp_out,
                                                                    int* __restrict__ status)
 {
-    extern __shared__ unsigned long long keys[];   // pow2 >= n + 1 keys, then (grid dimensions) 2 (n + 1) doubles
+    extern __shared__ unsigned long long keys[];   // pow2 >= n + 1 keys, then 3 (n + 2) doubles
     __shared__ int counts[kTpeMaxLevels];
-    __shared__ double wsum_s[32];
+    __shared__ int warp_count[32];
     const int j = blockIdx.x >> 1;
     const int code = levels[j];
     const int C = code > 0 ? code : 0;      // categorical levels
@@ -166,87 +243,98 @@ __global__ void __launch_bounds__(kSortThreads) tpe_mixture_kernel(const float* 
         bitonic_sort_asc(keys, count);
         const double sigma_lo = 1.0 / fmin(100.0, (double)s + 1.0);
         const double wsum = (double)s + prior_weight;
-        for (int t = threadIdx.x; t <= s; t += blockDim.x) {
-            const unsigned long long k = keys[t];
-            const bool is_prior = (int)(k & 0xFFFFFFFFull) == s;
-            const double mu = (double)from_ordered_bits((unsigned)(k >> 32));
-            double sigma = 1.0;
-            if (!is_prior) {
-                double gap = -1.0;
-                if (t > 0) gap = fmax(gap, mu - (double)from_ordered_bits((unsigned)(keys[t - 1] >> 32)));
-                if (t < s) gap = fmax(gap, (double)from_ordered_bits((unsigned)(keys[t + 1] >> 32)) - mu);
-                sigma = fmin(fmax(gap, sigma_lo), 1.0);
+        auto mean_bits = [&](int t) { return (unsigned)(keys[t] >> 32); };
+        auto mean_of = [&](int t) { return (double)from_ordered_bits(mean_bits(t)); };
+        auto sigma_of = [&](int t) {
+            if ((int)(keys[t] & 0xFFFFFFFFull) == s) return 1.0;   // the prior
+            const double mu = mean_of(t);
+            double gap = -1.0;
+            if (t > 0) gap = fmax(gap, mu - mean_of(t - 1));
+            if (t < s) gap = fmax(gap, mean_of(t + 1) - mu);
+            return fmin(fmax(gap, sigma_lo), 1.0);
+        };
+        // Components with the same mean and bandwidth (repeated values of a discrete feature) are one component with the
+        // summed coefficient: the density is the same sum, with far fewer terms.  Equal means are neighbours in the sorted
+        // order, and such a run has at most four bandwidths: its first value, the values inside, its last value, the prior.
+        // The first value of a run with its bandwidth stands for all of them; every thread finds that out for its own.
+        double* comp = reinterpret_cast<double*>(keys + count);   // [c][3]: mean, sigma, coefficient
+        int done_before = 0;
+        for (int t0 = 0; t0 <= s; t0 += blockDim.x) {
+            const int t = t0 + threadIdx.x;
+            bool leader = false;
+            double sigma = 0.0, coef = 0.0;
+            if (t <= s) {
+                const unsigned mu_bits = mean_bits(t);
+                sigma = sigma_of(t);
+                leader = true;
+                if (t > 0 && mean_bits(t - 1) == mu_bits) {
+                    int lo = 0, hi = t;   // the run's first position
+                    while (lo < hi) {
+                        const int mid = (lo + hi) / 2;
+                        if (mean_bits(mid) < mu_bits) lo = mid + 1;
+                        else hi = mid;
+                    }
+                    leader = sigma_of(lo) != sigma && (lo + 1 >= t || sigma_of(lo + 1) != sigma) && sigma_of(t - 1) != sigma;
+                }
+                if (leader) {
+                    // how many values of the run share the bandwidth, and whether the prior does
+                    int lo = t, hi = s + 1;   // one past the run
+                    while (lo < hi) {
+                        const int mid = (lo + hi) / 2;
+                        if (mean_bits(mid) <= mu_bits) lo = mid + 1;
+                        else hi = mid;
+                    }
+                    const int last = lo - 1;
+                    const bool with_prior = (int)(keys[last] & 0xFFFFFFFFull) == s;
+                    const int last_value = with_prior ? last - 1 : last;
+                    double weight = with_prior && sigma == 1.0 ? prior_weight : 0.0;
+                    // values t .. last_value: itself, those strictly inside (one bandwidth), the last
+                    if (t <= last_value) {
+                        weight += 1.0;
+                        if (t < last_value) {
+                            const int inside = last_value - t - 1;
+                            if (inside > 0 && sigma_of(t + 1) == sigma) weight += (double)inside;
+                            if (sigma_of(last_value) == sigma) weight += 1.0;
+                        }
+                    }
+                    const double mu = mean_of(t);
+                    const double Z = 0.5 * erfc(-(1.0 - mu) / sigma * 0.70710678118654752440) -
+                                     0.5 * erfc(-(0.0 - mu) / sigma * 0.70710678118654752440);
+                    coef = weight / (wsum * sigma * Z * 2.5066282746310005024);
+                }
             }
-            const double w = is_prior ? prior_weight : 1.0;
-            const double Z = 0.5 * erfc(-(1.0 - mu) / sigma * 0.70710678118654752440) -
-                             0.5 * erfc(-(0.0 - mu) / sigma * 0.70710678118654752440);
-            double* par = reinterpret_cast<double*>(keys + count);
-            par[2 * t] = sigma;
-            par[2 * t + 1] = w / (wsum * sigma * Z * 2.5066282746310005024);
+            // place among the leaders: order of the sorted positions
+            const unsigned votes = __ballot_sync(0xffffffffu, leader);
+            __syncthreads();
+            if ((threadIdx.x & 31) == 0) warp_count[threadIdx.x / 32] = __popc(votes);
+            __syncthreads();
+            int before = done_before, all = 0;
+            for (int w = 0; w < (int)blockDim.x / 32; ++w) {
+                if (w < (int)threadIdx.x / 32) before += warp_count[w];
+                all += warp_count[w];
+            }
+            done_before += all;
+            if (leader) {
+                const int c = before + __popc(votes & ((1u << (threadIdx.x & 31)) - 1u));
+                comp[3 * c] = mean_of(t);
+                comp[3 * c + 1] = sigma;
+                comp[3 * c + 2] = coef;
+                const double a = 1.4426950408889634074 / (2.0 * sigma * sigma);
+                out[c] = make_float4(from_ordered_bits(mean_bits(t)), (float)a, (float)log2(coef), (float)sigma);
+            }
         }
+        if (threadIdx.x == 0) n_comps[2 * j + set] = done_before;
         __syncthreads();
-        if (threadIdx.x == 0) {
-            // Components with the same mean and bandwidth (repeated values of a discrete feature) are one
-            // component with the summed coefficient: the density is the same sum, with far fewer terms.
-            // Equal means are neighbours in the sorted order; among them a run of equal values has one
-            // bandwidth inside and one at each end, so a handful of open slots per mean is enough (a full
-            // set of slots emits its oldest one, which only costs a missed merge).
-            constexpr int kSlots = 4;
-            const double* par = reinterpret_cast<const double*>(keys + count);
-            int c = 0, open = 0;
-            unsigned run_mu = 0;
-            double slot_sigma[kSlots], slot_coef[kSlots];
-            auto emit = [&](int i) {
-                const double a = 1.4426950408889634074 / (2.0 * slot_sigma[i] * slot_sigma[i]);
-                out[c++] = make_float4(from_ordered_bits(run_mu), (float)a, (float)log2(slot_coef[i]), (float)slot_sigma[i]);
-            };
-            for (int t = 0; t <= s; ++t) {
-                const unsigned mu_bits = (unsigned)(keys[t] >> 32);
-                if (mu_bits != run_mu) {
-                    for (int i = 0; i < open; ++i) emit(i);
-                    open = 0;
-                    run_mu = mu_bits;
-                }
-                const double sigma = par[2 * t], coef = par[2 * t + 1];
-                int hit = -1;
-                for (int i = 0; i < open; ++i)
-                    if (slot_sigma[i] == sigma) hit = i;
-                if (hit >= 0) {
-                    slot_coef[hit] += coef;
-                    continue;
-                }
-                if (open == kSlots) {
-                    emit(0);
-                    for (int i = 1; i < kSlots; ++i) slot_sigma[i - 1] = slot_sigma[i], slot_coef[i - 1] = slot_coef[i];
-                    --open;
-                }
-                slot_sigma[open] = sigma;
-                slot_coef[open++] = coef;
+        // (T3g) the mixture at each of the G grid values, in FP64, a warp per value
+        for (int v = threadIdx.x / 32; v < G; v += blockDim.x / 32) {
+            const double xg = (double)(float)((double)v / (double)(G - 1));
+            double acc = 0.0;
+            for (int c = threadIdx.x & 31; c < done_before; c += 32) {
+                const double z = (xg - comp[3 * c]) / comp[3 * c + 1];
+                acc += comp[3 * c + 2] * exp(-0.5 * z * z);
             }
-            for (int i = 0; i < open; ++i) emit(i);
-            n_comps[2 * j + set] = c;
-        }
-        __syncthreads();
-        if (G > 0) {
-            // (T3g) the mixture at each of the G grid values, in FP64; the warps' sums are added in order
-            const double* par = reinterpret_cast<const double*>(keys + count);
-            for (int v = 0; v < G; ++v) {
-                const double xg = (double)(float)((double)v / (double)(G - 1));
-                double acc = 0.0;
-                for (int t = threadIdx.x; t <= s; t += blockDim.x) {
-                    const double z = (xg - (double)from_ordered_bits((unsigned)(keys[t] >> 32))) / par[2 * t];
-                    acc += par[2 * t + 1] * exp(-0.5 * z * z);
-                }
-                for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-                if ((threadIdx.x & 31) == 0) wsum_s[threadIdx.x / 32] = acc;
-                __syncthreads();
-                if (threadIdx.x == 0) {
-                    double tot = 0.0;
-                    for (int w = 0; w < (int)blockDim.x / 32; ++w) tot += wsum_s[w];
-                    lnp_set[v] = log(tot);
-                }
-                __syncthreads();
-            }
+            for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+            if ((threadIdx.x & 31) == 0) lnp_set[v] = log(acc);
         }
     }
     if (bad) atomicOr(status, DEV_NONFINITE);
@@ -378,14 +466,37 @@ __global__ void __launch_bounds__(kScoreThreads) tpe_score_kernel(const float* _
     if (bad) atomicOr(status, DEV_NONFINITE);
 }
 
-// One (dimension, set) per block: copy its kept components to their place in the packed model.
-__global__ void __launch_bounds__(256) tpe_pack_kernel(const float4* __restrict__ comps, int n, int n_good,
-                                                       const int* __restrict__ offs, float4* __restrict__ packed)
+// One (dimension, set) per block: where its kept components begin in the packed model, and, if the whole model fits
+// `limit` components, their copy there.
+__global__ void __launch_bounds__(256) tpe_pack_kernel(const float4* __restrict__ comps, const int* __restrict__ counts, int n,
+                                                       int n_good, int sets, int limit, int* __restrict__ offs,
+                                                       float4* __restrict__ packed)
 {
-    const int j = blockIdx.x >> 1, set = blockIdx.x & 1;
+    __shared__ int sums[2];
+    const int b = blockIdx.x, j = b >> 1, set = b & 1;
+    if (threadIdx.x < 2) sums[threadIdx.x] = 0;
+    __syncthreads();
+    int before = 0, all = 0;
+    for (int i = threadIdx.x; i < sets; i += blockDim.x) {
+        const int c = counts[i];
+        all += c;
+        if (i < b) before += c;
+    }
+    before = __reduce_add_sync(0xffffffffu, before);
+    all = __reduce_add_sync(0xffffffffu, all);
+    if ((threadIdx.x & 31) == 0) {
+        atomicAdd(&sums[0], before);
+        atomicAdd(&sums[1], all);
+    }
+    __syncthreads();
+    const int lo = sums[0], cnt = counts[b];
+    if (threadIdx.x == 0) {
+        offs[b] = lo;
+        if (b == sets - 1) offs[sets] = sums[1];
+    }
+    if (sums[1] > limit) return;
     const float4* src = comps + (size_t)j * (n + 2) + (set ? n_good + 1 : 0);
-    const int lo = offs[blockIdx.x], hi = offs[blockIdx.x + 1];
-    for (int i = lo + threadIdx.x; i < hi; i += blockDim.x) packed[i] = src[i - lo];
+    for (int i = threadIdx.x; i < cnt; i += blockDim.x) packed[lo + i] = src[i];
 }
 
 // sum over components [lo, hi) of a model held in shared memory, for R candidates at once
@@ -605,32 +716,27 @@ r3_status_t tpe_fit_impl(r3_tpe* t, const float* X, const float* y, cudaStream_t
     }
     R3_CUDA_TRY(cudaMemcpyAsync(t->levels_d, t->levels.data(), sizeof(int) * d, cudaMemcpyHostToDevice, stream));
     R3_CUDA_TRY(cudaMemsetAsync(t->status_d, 0, sizeof(int), stream));
-    R3_LAUNCH(tpe_order_kernel, 1, kSortThreads, 0, stream, y, n, t->order_d, t->status_d);
+    R3_LAUNCH(tpe_order_kernel, (n + kOrderRows - 1) / kOrderRows, 256, 0, stream, y, n, t->order_d, t->status_d);
     int count = 1;
     while (count < n + 1) count <<= 1;
-    const size_t smem = sizeof(unsigned long long) * (size_t)count + sizeof(double) * 2 * ((size_t)n + 2);
+    const size_t smem = sizeof(unsigned long long) * (size_t)count + sizeof(double) * 3 * ((size_t)n + 2);
     if (smem > 48 * 1024)
         R3_CUDA_TRY(cudaFuncSetAttribute(tpe_mixture_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     R3_LAUNCH(tpe_mixture_kernel, 2 * d, kSortThreads, smem, stream, X, t->order_d, n, d, t->n_good, t->levels_d,
               (double)t->prior_weight, t->comps_d, t->counts_d, lnp_d, t->status_d);
     R3_LAUNCH(tpe_table_kernel, d, kTpeMaxLevels, 0, stream, t->levels_d, lnp_d, d, t->table_d);
+    // a model that a scoring block can hold in shared memory is packed
+    const int limit = (int)((kResidentBytes - resident_bytes(0, d)) / sizeof(float4));
+    R3_LAUNCH(tpe_pack_kernel, 2 * d, 256, 0, stream, t->comps_d, t->counts_d, n, t->n_good, 2 * d, limit, t->offs_d, t->packed_d);
     R3_CUDA_TRY(cudaMemcpyAsync(t->status_h, t->status_d, sizeof(int), cudaMemcpyDeviceToHost, stream));
+    R3_CUDA_TRY(cudaMemcpyAsync(t->status_h + 1, t->offs_d + 2 * d, sizeof(int), cudaMemcpyDeviceToHost, stream));
     R3_CUDA_TRY(cudaStreamSynchronize(stream));
-    if (*t->status_h & DEV_NONFINITE) {
+    if (t->status_h[0] & DEV_NONFINITE) {
         set_error("r3_tpe_fit: X or y contains NaN or Inf");
         return R3_ERR_NONFINITE;
     }
-    // pack a model that a scoring block can hold in shared memory
-    std::vector<int> counts(2 * (size_t)d), offs(2 * (size_t)d + 1, 0);
-    R3_CUDA_TRY(cudaMemcpy(counts.data(), t->counts_d, sizeof(int) * 2 * (size_t)d, cudaMemcpyDeviceToHost));
-    for (int i = 0; i < 2 * d; ++i) offs[i + 1] = offs[i] + counts[i];
-    t->total = offs[2 * d];
-    t->resident = t->total > 0 && resident_bytes(t->total, d) <= kResidentBytes;
-    if (t->resident) {
-        R3_CUDA_TRY(cudaMemcpyAsync(t->offs_d, offs.data(), sizeof(int) * offs.size(), cudaMemcpyHostToDevice, stream));
-        R3_LAUNCH(tpe_pack_kernel, 2 * d, 256, 0, stream, t->comps_d, n, t->n_good, t->offs_d, t->packed_d);
-        R3_CUDA_TRY(cudaStreamSynchronize(stream));   // `offs` leaves scope
-    }
+    t->total = t->status_h[1];
+    t->resident = t->total > 0 && t->total <= limit;
     return R3_OK;
 }
 

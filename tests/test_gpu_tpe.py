@@ -311,3 +311,40 @@ def test_errors():
     b.r3_tpe_score(tpe, dev(np.nan_to_num(Xc)))
     b.r3_tpe_check(tpe)      # the latch was cleared
     tpe.close()
+
+
+@pytest.mark.parametrize("n", [1, 2, 31, 32, 63, 64, 127, 128, 129, 1000, 2048, 4095, 4096])
+def test_fit_at_the_edges_of_the_sort_and_of_runs(n):
+    """Histories of few distinct values (long runs of equal ones, the prior's mean among them) and of distinct ones, at
+    sizes around the sort's blocks: order, component counts and components against the oracle's mixture, merged."""
+    rng = np.random.default_rng(n)
+    X = np.stack([rng.integers(0, 3, n) / 2.0, rng.integers(0, 16, n) / 15.0, rng.uniform(0, 1, n), np.full(n, 0.5)],
+                 axis=1).astype(np.float32)
+    y = rng.integers(0, max(2, n // 3), n).astype(np.float32)
+    t = b.r3_tpe_fit(dev(X), dev(y), np.zeros(4, np.int32))
+    n_good, order, comps, counts, _ = b.r3_tpe_get_model(t)
+    assert np.array_equal(order, np.lexsort((np.arange(n), y)))
+    for j in range(4):
+        for set_, rows in enumerate((order[:n_good], order[n_good:])):
+            v = np.sort(X[rows, j].astype(np.float64))
+            s = v.size
+            means = np.concatenate([v, [0.5]])
+            prior = np.concatenate([np.zeros(s, bool), [True]])
+            at = np.lexsort((prior, means))
+            means, prior = means[at], prior[at]
+            gap = np.diff(means)
+            left, right = np.concatenate([[-1.0], gap]), np.concatenate([gap, [-1.0]])
+            sigma = np.where(prior, 1.0, np.clip(np.maximum(left, right), 1.0 / min(100.0, s + 1.0), 1.0))
+            distinct = sorted(set(zip(means.tolist(), sigma.tolist())))
+            c0 = 0 if set_ == 0 else n_good + 1
+            got = comps[j, c0:c0 + counts[j, set_]]
+            assert counts[j, set_] == len(distinct)
+            assert sorted(zip(got[:, 0].tolist(), got[:, 3].tolist())) == sorted(
+                (float(np.float32(a)), float(np.float32(q))) for a, q in distinct)
+            # the weights add up to one: sum of exp2(b) sigma Z sqrt(2 pi)
+            sg = got[:, 3].astype(np.float64)
+            from scipy.special import ndtr
+            Z = ndtr((1.0 - got[:, 0]) / sg) - ndtr((0.0 - got[:, 0]) / sg)
+            total = (np.exp2(got[:, 2].astype(np.float64)) * sg * Z * np.sqrt(2 * np.pi)).sum()
+            assert abs(total - 1.0) < 1e-5     # b is FP32: 2^-24 |b| ln 2 per component
+    t.close()
