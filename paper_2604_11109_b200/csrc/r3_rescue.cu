@@ -86,11 +86,14 @@ __device__ __forceinline__ bool misses_contract(float mu, float sd, float dmu, f
     const float tol_mu = 1e-4f * fabsf(mu) + mu_floor;
     const float tol_sd = 1e-4f * sd + sd_floor;
     bool flag = !(dmu <= 0.5f * tol_mu) || !(dsd <= 0.5f * tol_sd);
-    // EI: dEI = Phi(z) dmu + phi(z) dsigma against 1e-5 of the pool's largest EI
+    // EI: dEI = Phi(z) dmu + phi(z) dsigma against 1e-5 of the pool's largest EI.  Phi(z) <= exp(-z^2/2) / 2 for z <= 0 (and
+    // <= 1 above) and phi(z) < 0.4 exp(-z^2/2): most candidates pass by that bound and need no erfc.
     const float z = (sd > 0.f) ? (best - mu) / sd : 0.f;
-    const float Phi = 0.5f * erfcf(-z * 0.70710678f);
-    const float phi = expf(-0.5f * z * z) * 0.39894228f;
-    if (isfinite(dsd)) flag |= !(Phi * dmu + phi * dsd <= 0.5f * tol_ei);
+    const float bell = expf(-0.5f * z * z);
+    if (isfinite(dsd) && !((z > 0.f ? dmu : 0.501f * bell * dmu) + 0.4f * bell * dsd <= 0.5f * tol_ei)) {
+        const float Phi = 0.5f * erfcf(-z * 0.70710678f);
+        flag |= !(Phi * dmu + bell * 0.39894228f * dsd <= 0.5f * tol_ei);
+    }
     flag |= !(sd * sd >= 1e-3f * sf2);   // deep cancellation: do not trust the estimates either
     return flag;
 }
@@ -368,35 +371,45 @@ __global__ void __launch_bounds__(kThreads, 2) guard_kernel(const GuardArgs a)
             if (t == 0) own_count = 0;
             __syncthreads();
         }
-#pragma unroll 2
-        for (long long i0 = c0; i0 < c1; i0 += kThreads) {
-            const long long i = i0 + t;
-            bool flag = false;
-            if (i < c1) {
-                const size_t f = (size_t)g * m + i;
-                const float mu_i = __ldcs(a.mu + f), sd = __ldcs(a.sigma + f), dmu = __ldcs(a.err_mu + f), dq = __ldcs(a.err_q + f);
-                flag = misses_contract(mu_i, sd, dmu, dq, tol_ei, mu_floor, sd_floor, best, sf2);
+        constexpr int kBatch = 4;   // loads of so many candidates per thread are under way at a time
+        for (long long b0 = c0; b0 < c1; b0 += kBatch * kThreads) {
+            float mu4[kBatch], sd4[kBatch], dmu4[kBatch], dq4[kBatch];
+#pragma unroll
+            for (int j = 0; j < kBatch; ++j) {
+                if (b0 + j * kThreads >= c1) continue;   // the same for the whole block
+                const long long i = b0 + j * kThreads + t;
+                const size_t f = (size_t)g * m + (i < c1 ? i : c0);
+                mu4[j] = __ldcs(a.mu + f);
+                sd4[j] = __ldcs(a.sigma + f);
+                dmu4[j] = __ldcs(a.err_mu + f);
+                dq4[j] = __ldcs(a.err_q + f);
             }
-            const unsigned votes = __ballot_sync(0xffffffffu, flag);   // one counter update per warp
-            if (votes) {
-                const int rank = __popc(votes & ((1u << lane) - 1u)), all = __popc(votes);
-                int mine = 0, base = 0;   // the first `mine` of the warp's go to the block's own list
-                if (lane == 0) {
-                    atomicAdd(&a.total[g], all);
-                    if (own_rescue) {
-                        base = atomicAdd(&own_count, all);
-                        mine = max(0, min(all, kSmallTile - base));
+#pragma unroll
+            for (int j = 0; j < kBatch; ++j) {
+                if (b0 + j * kThreads >= c1) continue;
+                const long long i = b0 + j * kThreads + t;
+                const bool flag = i < c1 && misses_contract(mu4[j], sd4[j], dmu4[j], dq4[j], tol_ei, mu_floor, sd_floor, best, sf2);
+                const unsigned votes = __ballot_sync(0xffffffffu, flag);   // one counter update per warp
+                if (votes) {
+                    const int rank = __popc(votes & ((1u << lane) - 1u)), all = __popc(votes);
+                    int mine = 0, base = 0;   // the first `mine` of the warp's go to the block's own list
+                    if (lane == 0) {
+                        atomicAdd(&a.total[g], all);
+                        if (own_rescue) {
+                            base = atomicAdd(&own_count, all);
+                            mine = max(0, min(all, kSmallTile - base));
+                        }
                     }
-                }
-                if (own_rescue) {
-                    base = __shfl_sync(0xffffffffu, base, 0);
-                    mine = __shfl_sync(0xffffffffu, mine, 0);
-                    if (flag && rank < mine) own[base + rank] = (int)i;
-                }
-                if (mine < all) {
-                    if (lane == 0) base = atomicAdd(&a.count[g], all - mine);
-                    base = __shfl_sync(0xffffffffu, base, 0);
-                    if (flag && rank >= mine) a.list[(size_t)g * m + R3_IDX(base + rank - mine, m, a.status)] = (int)i;
+                    if (own_rescue) {
+                        base = __shfl_sync(0xffffffffu, base, 0);
+                        mine = __shfl_sync(0xffffffffu, mine, 0);
+                        if (flag && rank < mine) own[base + rank] = (int)i;
+                    }
+                    if (mine < all) {
+                        if (lane == 0) base = atomicAdd(&a.count[g], all - mine);
+                        base = __shfl_sync(0xffffffffu, base, 0);
+                        if (flag && rank >= mine) a.list[(size_t)g * m + R3_IDX(base + rank - mine, m, a.status)] = (int)i;
+                    }
                 }
             }
         }
@@ -455,15 +468,23 @@ __global__ void __launch_bounds__(kThreads, 2) guard_kernel(const GuardArgs a)
         const long long c0 = (long long)(s % a.slices_per_gp) * a.slice;
         const float* e = a.ei + (size_t)g * m;
         __syncthreads();
-#pragma unroll 8
-        for (int i = t; i < a.slice; i += kThreads) {
-            const long long c = c0 + i;
-            keys_s[i] = (c < m) ? topk_make_key(__ldcg(e + c), (unsigned)c) : 0ull;
+#pragma unroll 1
+        for (int i0 = t; i0 < a.slice; i0 += 8 * kThreads) {   // eight loads under way at a time
+            float v[8];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                const int i = i0 + j * kThreads;
+                v[j] = i < a.slice && c0 + i < m ? __ldcg(e + c0 + i) : 0.f;
+            }
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                const int i = i0 + j * kThreads;
+                if (i < a.slice) keys_s[i] = c0 + i < m ? topk_make_key(v[j], (unsigned)(c0 + i)) : 0ull;
+            }
         }
-        __syncthreads();
         block_select_desc(keys_s, a.slice, a.K2, smem + a.select_offset);
         unsigned long long* out = a.keys + (size_t)s * a.K2;
-        for (int i = t; i < a.K2; i += kThreads) out[i] = keys_s[R3_IDX(i, a.slice, a.status)];
+        for (int i = t; i < a.K2; i += kThreads) out[i] = keys_s[i];
         if (a.finish) {
             __threadfence();
             __syncthreads();
@@ -475,7 +496,6 @@ __global__ void __launch_bounds__(kThreads, 2) guard_kernel(const GuardArgs a)
                 const unsigned long long* in = a.keys + (size_t)g * nk;
 #pragma unroll 8
                 for (int i = t; i < nk; i += kThreads) keys_s[i] = __ldcg(in + i);
-                __syncthreads();
                 block_select_desc(keys_s, nk, a.k, smem + a.select_offset);
                 for (int i = t; i < a.k; i += kThreads) {
                     const unsigned c = topk_key_index(keys_s[i]);

@@ -50,8 +50,8 @@ __host__ __device__ inline size_t topk_select_scratch_bytes(int K)
 //
 // Radix selection, then a rank sort of the K survivors -- no sorting network over the n keys:
 //  1. the K-th largest key is found digit by digit (8 bits per step) from the highest bit in which the keys differ: a histogram of the digit
-//     over the keys that match the digits found so far (lanes that share a digit with the warp's first active lane add once, so a
-//     pool whose values share their exponent does not serialise on one bin), a walk over the 256 bins from the top by one
+//     over the keys that match the digits found so far (lanes that share a digit add once, so a pool whose values crowd into a
+//     few bins does not serialise on them), a walk over the 256 bins from the top by one
 //     warp; it stops as soon as the chosen bin holds one key, typically after three or four steps;
 //  2. the keys above that bin, and as many of the bin's as are still wanted (more than one only for the
 //     duplicated padding key 0), are gathered: exactly K;
@@ -98,20 +98,15 @@ __device__ __forceinline__ void block_select_desc(unsigned long long* s, int n, 
         for (;; shift = max(0, shift - 8)) {
             for (int b = tid; b < 256; b += T) hist[b] = 0u;
             __syncthreads();
-#pragma unroll 4
+#pragma unroll 2
             for (int i = tid; i < n_up; i += T) {
                 const unsigned long long key = i < n ? s[i] : 0ull;
                 const bool act = i < n && (key & decided) == prefix;
-                const unsigned dgt = (unsigned)(key >> shift) & 255u;
-                // the lanes that share the first active lane's digit add once (pools whose values share their
-                // exponent would otherwise serialise on one bin); the others add for themselves
-                const unsigned active = __ballot_sync(0xffffffffu, act);
-                if (active) {
-                    const int first = __ffs(active) - 1;
-                    const unsigned d0 = __shfl_sync(0xffffffffu, dgt, first);
-                    const unsigned same = __ballot_sync(0xffffffffu, act && dgt == d0);
-                    if (lane == first) atomicAdd(&hist[d0], (unsigned)__popc(same));
-                    else if (act && dgt != d0) atomicAdd(&hist[dgt], 1u);
+                if (__any_sync(0xffffffffu, act)) {   // few warps find a match after the first step
+                    const unsigned dgt = (unsigned)(key >> shift) & 255u;
+                    // lanes that share a digit add once: a few bins may take most of the keys
+                    const unsigned same = __match_any_sync(0xffffffffu, act ? dgt : 256u);
+                    if (act && lane == __ffs(same) - 1) atomicAdd(&hist[dgt], (unsigned)__popc(same));
                 }
             }
             __syncthreads();
@@ -148,7 +143,7 @@ __device__ __forceinline__ void block_select_desc(unsigned long long* s, int n, 
         }
         // gather: the keys above the chosen bin (K - want of them), then `want` keys of the bin
         const unsigned long long ph = prefix >> shift;
-#pragma unroll 4
+#pragma unroll 2
         for (int i = tid; i < n_up; i += T) {
             const unsigned long long key = i < n ? s[i] : 0ull, hi = key >> shift;
             const bool above = i < n && hi > ph;
@@ -198,6 +193,7 @@ __device__ __forceinline__ void block_select_desc(unsigned long long* s, int n, 
             const unsigned long long key = tmp[i];
             const int j0 = (int)((long long)part * k_cap / parts), j1 = (int)((long long)(part + 1) * k_cap / parts);
             unsigned before = 0u;
+#pragma unroll 4
             for (int j = j0; j < j1; ++j) {
                 const unsigned long long o = tmp[j];
                 before += (o > key || (o == key && j < i)) ? 1u : 0u;
