@@ -89,7 +89,7 @@ void state_free(r3_fit_state& s)
 }
 
 r3_status_t state_fit(r3_gp* gp, r3_fit_state& s, int rows_done, bool full, bool need_tc, cudaStream_t stream, int* bits,
-                      int* pivot)
+                      int* pivot, double* lml)
 {
     const int B = s.batch, npad = s.npad;
     void* ints = nullptr;
@@ -112,7 +112,8 @@ r3_status_t state_fit(r3_gp* gp, r3_fit_state& s, int rows_done, bool full, bool
     } while (0)
     const size_t fbytes = factor_scratch_bytes(B, npad);
     TRY_DONE(dev_malloc(&ints, fbytes + sizeof(unsigned) * B));
-    TRY_DONE(dev_malloc(&doubles, sizeof(double) * weights_scratch_doubles(B, npad)));
+    const size_t wdoubles = weights_scratch_doubles(B, npad);
+    TRY_DONE(dev_malloc(&doubles, sizeof(double) * (wdoubles + (lml ? lml_scratch_doubles(s) : 0))));
 
     // the block: results cleared, hyper-parameters filled in
     size_t results = 0;
@@ -158,8 +159,18 @@ r3_status_t state_fit(r3_gp* gp, r3_fit_state& s, int rows_done, bool full, bool
             if (st != R3_OK && (need_tc || st != R3_ERR_ALLOC)) return done(st);
         }
     }
+    // the evidence goes behind the block's image if there is room
+    const size_t lml_bytes = sizeof(double) * (size_t)B * (s.d + 3);
+    const bool staged = lml && image == gp->stage_h && bytes + lml_bytes <= kStageBytes;
+    if (lml) {
+        double* out = nullptr;
+        st = lml_enqueue(s, doubles + wdoubles, &out, stream);
+        if (st != R3_OK) return done(st);
+        TRY_DONE(cudaMemcpyAsync(staged ? (void*)(image + bytes) : (void*)lml, out, lml_bytes, cudaMemcpyDeviceToHost, stream));
+    }
     TRY_DONE(cudaMemcpyAsync(image, s.block, results, cudaMemcpyDeviceToHost, stream));
     TRY_DONE(cudaStreamSynchronize(stream));
+    if (staged) memcpy(lml, image + bytes, lml_bytes);
 #undef TRY_DONE
     const int* fs = mirror(s, s.fit_status, image);
     *bits = fs[0];

@@ -216,8 +216,9 @@ void state_free(r3_fit_state& s);
 // full: everything a handle needs, tensor operands included; otherwise L, W, alpha and the status only (an evaluation of
 // the evidence).  Synchronises; *bits and *pivot are what the device found.  need_tc: a failed allocation of the tensor
 // operands is an error (otherwise the CUDA-core engine serves the state).
+// lml: if not nullptr receives the evidence and its gradient, host [batch][d + 3] (meaningless when *bits reports a failure).
 r3_status_t state_fit(r3_gp* gp, r3_fit_state& s, int rows_done, bool full, bool need_tc, cudaStream_t stream, int* bits,
-                      int* pivot);
+                      int* pivot, double* lml = nullptr);
 // Appends k observations per GP (r3_gp_append): extends L, W, alpha, X, y in O(k n^2); synchronises.  On
 // any error (and when *bits says so) the handle is left as it was.
 r3_status_t append_device(r3_gp* gp, const float* Xnew, const float* ynew, int k, cudaStream_t stream, int* bits, int* pivot);
@@ -287,6 +288,8 @@ r3_status_t topk_device(const float* ei, int batch, long long m, int k, int* idx
                         size_t ws_bytes, cudaStream_t stream);
 
 // log marginal likelihood and gradient (r3_lml.cu): out_h host [batch][d + 3]
+size_t lml_scratch_doubles(const r3_fit_state& s);
+r3_status_t lml_enqueue(const r3_fit_state& s, double* scratch, double** out, cudaStream_t stream);
 r3_status_t lml_device(r3_gp* gp, double* out_h, cudaStream_t stream);
 
 // greedy batch proposal on a shortlist (r3_propose.cu)

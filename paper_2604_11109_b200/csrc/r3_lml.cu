@@ -1,261 +1,305 @@
 // Log marginal likelihood of the history and its gradient with respect to the logarithms of the
 // hyper-parameters, from what the fit already holds (L, W = L^-1, alpha, X, y):
 //     lml = -1/2 y.alpha - sum_i log L_ii - n/2 log(2 pi)
-//     M   = alpha alpha^T - K^-1,   K^-1 = W^T W                     (kinv_kernel: n^3/3 FP64 FMAs)
+//     M   = alpha alpha^T - K^-1,   K^-1 = W^T W
 //     d lml / d log ell_j = 1/2 sum_ik M_ik sf2 e^-s (5/3)(1 + s) u_j^2     (u_j = (x_ij - x_kj)/ell_j)
 //     d lml / d log sf2   = 1/2 sum_ik M_ik Kf_ik,    d lml / d log sn2 = 1/2 sn2 trace(M)
-// Everything in FP64; the pair sums use the symmetry of M (lower triangle, off-diagonal pairs twice) and
-// are reduced in a fixed order (per-block partial sums, then one block adds them), so results repeat
-// bit for bit.
+// Everything in FP64.  A block forms a 64 x 64 tile of the lower triangle of K^-1 on the FP64 tensor path and, with the
+// tile still in registers, its share of every pair sum; M is never stored.  The sums are reduced in a fixed order (per-tile
+// partial sums, then one warp per derivative adds them), so results repeat bit for bit.
+// Bound: FP64 rate, n^3/3 multiply-adds for K^-1 and 7 n^2 d / 2 operations for the pairs.  64 GPs of 512 observations, 32
+// features: 0.35 ms; K^-1 by 4x4 register tiles, M written and read back, and a warp sum per feature and pair tile: 0.79 ms.
 #include <math.h>
 
+#include <algorithm>
 #include <vector>
 
+#include "r3_f64.cuh"
 #include "r3_internal.cuh"
 
 namespace r3 {
 
 namespace {
 
-// M[i][j] = alpha_i alpha_j - sum_{r >= i} W[r][i] W[r][j] for j <= i (64 x 64 tile per block, 4 x 4 per thread).
-__global__ void __launch_bounds__(256) kinv_kernel(const double* __restrict__ W, const double* __restrict__ alpha, int n,
-                                                   int npad, double* __restrict__ M)
-{
-    const int g = blockIdx.z;
-    const int ti = blockIdx.y, tj = blockIdx.x;
-    if (tj > ti) return;
-    W += (size_t)g * npad * npad;
-    M += (size_t)g * npad * npad;
-    alpha += (size_t)g * npad;
-    __shared__ double Ai[16][65], Aj[16][65];
-    const int i0 = ti * 64, j0 = tj * 64;
-    const int t = threadIdx.x, ty = t / 16, tx = t % 16;
-    double acc[4][4] = {};
-    for (int r0 = i0 / 16 * 16; r0 < n; r0 += 16) {
-        for (int e = t; e < 16 * 64; e += 256) {
-            const int r = e / 64, c = e % 64;
-            const bool ok = r0 + r < n;
-            Ai[r][c] = (ok && i0 + c < n) ? W[(size_t)(r0 + r) * npad + i0 + c] : 0.0;
-            Aj[r][c] = (ok && j0 + c < n) ? W[(size_t)(r0 + r) * npad + j0 + c] : 0.0;
-        }
-        __syncthreads();
-#pragma unroll
-        for (int r = 0; r < 16; ++r) {
-            double a[4], b[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                a[u] = Ai[r][ty * 4 + u];
-                b[u] = Aj[r][tx * 4 + u];
-            }
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-#pragma unroll
-                for (int v = 0; v < 4; ++v) acc[u][v] = fma(a[u], b[v], acc[u][v]);
-        }
-        __syncthreads();
-    }
-#pragma unroll
-    for (int u = 0; u < 4; ++u)
-#pragma unroll
-        for (int v = 0; v < 4; ++v) {
-            const int i = i0 + ty * 4 + u, j = j0 + tx * 4 + v;
-            if (i < n && j <= i) M[(size_t)i * npad + j] = alpha[i] * alpha[j] - acc[u][v];
-        }
-}
+constexpr int kThreads = 256;
+constexpr int kTile = 64;
+constexpr int kStages = 3;
+constexpr int kLd = 68;   // leading dimension of a [16][64] operand stage: 4 mod 16 keeps the fragment reads on different banks
+constexpr size_t kTileSmem = sizeof(double) * kStages * 2 * 16 * kLd;   // 52 KB; the pair sums need 34 KB of it
 
-// One 32 x 32 tile of pairs (i, k), k-tile <= i-tile, per block of 256 threads (thread: one i, four k).
-// partial[block][0 .. d-1] = sum over the tile of w M_ik G_ik u_j^2, partial[block][d] = sum w M_ik Kf_ik,
-// with w = 1 on the diagonal, 2 below it, 0 above.
-__global__ void __launch_bounds__(256) lml_pairs_kernel(const float* __restrict__ X, const float* __restrict__ ell,
-                                                        const float* __restrict__ sf2v, int n, int d, int npad,
-                                                        const double* __restrict__ M, int tiles,
-                                                        double* __restrict__ partial)
-{
-    // blockIdx.y: the GP
-    const int g = blockIdx.y;
-    X += (size_t)g * n * d;
-    ell += (size_t)g * d;
-    M += (size_t)g * npad * npad;
-    partial += (size_t)g * tiles * (d + 1);
-    const double sf2 = (double)sf2v[g];
-    // tile index -> (ti, tk) of the lower triangle
-    const int b = blockIdx.x;
-    int ti = (int)((sqrt(8.0 * b + 1.0) - 1.0) * 0.5);
-    while ((ti + 1) * (ti + 2) / 2 <= b) ++ti;
-    while (ti * (ti + 1) / 2 > b) --ti;
-    const int tk = b - ti * (ti + 1) / 2;
-    __shared__ float xi[32][33], xk[32][33];
-    __shared__ double sl[32];        // 1 / lengthscale (FP64 reciprocal, as in the fit's Gram kernel)
-    __shared__ double red[8];
-    __shared__ double redc[8][32];   // the warps' sums of 32 features' terms
-    const int t = threadIdx.x, li = t % 32, lk0 = (t / 32) * 4;
-    const int i = ti * 32 + li;
-    double r2[4] = {0, 0, 0, 0};
-    for (int c0 = 0; c0 < d; c0 += 32) {
-        __syncthreads();
-        for (int e = t; e < 32 * 32; e += 256) {
-            const int r = e / 32, c = e % 32;
-            const int gi = ti * 32 + r, gk = tk * 32 + r;
-            xi[r][c] = (gi < n && c0 + c < d) ? X[(size_t)gi * d + c0 + c] : 0.f;
-            xk[r][c] = (gk < n && c0 + c < d) ? X[(size_t)gk * d + c0 + c] : 0.f;
-        }
-        if (t < 32) sl[t] = (c0 + t < d) ? 1.0 / (double)ell[c0 + t] : 1.0;
-        __syncthreads();
-        const int cmax = min(32, d - c0);
-        for (int c = 0; c < cmax; ++c) {
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const double u = ((double)xi[li][c] - (double)xk[lk0 + q][c]) * sl[c];
-                r2[q] = fma(u, u, r2[q]);
-            }
-        }
-    }
-    double gk[4], kf_sum = 0.0;
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        const int k = tk * 32 + lk0 + q;
-        double w = 0.0;
-        if (i < n && k < n && k <= i) w = (k == i) ? 1.0 : 2.0;
-        const double m = w != 0.0 ? M[(size_t)i * npad + k] : 0.0;
-        const double s = sqrt(5.0) * sqrt(r2[q]);
-        const double e = exp(-s);
-        gk[q] = w * m * sf2 * e * (5.0 / 3.0) * (1.0 + s);
-        kf_sum += w * m * sf2 * (1.0 + s + s * s / 3.0) * e;
-    }
-    double* out = partial + (size_t)b * (d + 1);
-    // block sums: warp shuffle, then the eight warps in a fixed order
-    auto block_sum = [&](double v, int slot) {
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        __syncthreads();
-        if ((t & 31) == 0) red[t / 32] = v;
-        __syncthreads();
-        if (t == 0) {
-            double s = 0.0;
-            for (int w = 0; w < 8; ++w) s += red[w];
-            out[slot] = s;
-        }
-    };
-    block_sum(kf_sum, d);
-    for (int c0 = 0; c0 < d; c0 += 32) {
-        __syncthreads();
-        for (int e = t; e < 32 * 32; e += 256) {
-            const int r = e / 32, c = e % 32;
-            const int gi = ti * 32 + r, gk_ = tk * 32 + r;
-            xi[r][c] = (gi < n && c0 + c < d) ? X[(size_t)gi * d + c0 + c] : 0.f;
-            xk[r][c] = (gk_ < n && c0 + c < d) ? X[(size_t)gk_ * d + c0 + c] : 0.f;
-        }
-        if (t < 32) sl[t] = (c0 + t < d) ? 1.0 / (double)ell[c0 + t] : 1.0;
-        __syncthreads();
-        const int cmax = min(32, d - c0);
-        for (int c = 0; c < cmax; ++c) {
-            double v = 0.0;
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const double u = ((double)xi[li][c] - (double)xk[lk0 + q][c]) * sl[c];
-                v = fma(gk[q], u * u, v);
-            }
-            // warp sum now, the eight warps in a fixed order once per 32 features
-            for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-            if ((t & 31) == 0) redc[t / 32][c] = v;
-        }
-        __syncthreads();
-        if (t < cmax) {
-            double s = 0.0;
-            for (int w = 0; w < 8; ++w) s += redc[w][t];
-            out[c0 + t] = s;
-        }
-    }
-}
+struct LmlArgs {
+    const float *X, *ell, *sf2, *sn2, *y;
+    const double *W, *L, *alpha;
+    int n, d, npad, tiles;
+    double* partial;   // [batch][tiles][d + 2]: the features' sums, sum w M Kf, trace
+    double* out;       // [batch][d + 3]
+};
 
-// One block per GP: adds the tiles' partial sums in order, the trace term and the value.
-__global__ void __launch_bounds__(256) lml_finish_kernel(const double* __restrict__ partial, int tiles, int d,
-                                                         const double* __restrict__ M, const double* __restrict__ L,
-                                                         const double* __restrict__ alpha, const float* __restrict__ y,
-                                                         int n, int npad, const float* __restrict__ sn2v,
-                                                         double* __restrict__ out)
+__global__ void __launch_bounds__(kThreads, 2) lml_tile_kernel(const LmlArgs a)
 {
-    __shared__ double red[256];
-    const int g = blockIdx.x;
-    partial += (size_t)g * tiles * (d + 1);
-    M += (size_t)g * npad * npad;
-    L += (size_t)g * npad * npad;
-    alpha += (size_t)g * npad;
-    y += (size_t)g * n;
-    out += (size_t)g * (d + 3);
-    const double sn2 = (double)sn2v[g];
-    const int t = threadIdx.x;
-    auto block_sum = [&](double v) {
-        red[t] = v;
-        __syncthreads();
-        for (int o = 128; o > 0; o >>= 1) {
-            if (t < o) red[t] += red[t + o];
+    extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ double red[8][34];   // the warps' sums of 32 features, of M Kf and of the trace
+    const int g = blockIdx.y, n = a.n, d = a.d, npad = a.npad;
+    const int t = threadIdx.x, w = t / 32, l = t % 32, wm = (w % 4) * 16, wn = (w / 4) * 32;
+    // tile index -> (ti, tj) of the lower triangle; small ti have the longest reductions and come first
+    int ti = (int)((sqrtf(8.f * blockIdx.x + 1.f) - 1.f) * 0.5f);
+    while ((ti + 1) * (ti + 2) / 2 <= (int)blockIdx.x) ++ti;
+    while (ti * (ti + 1) / 2 > (int)blockIdx.x) --ti;
+    const int tj = blockIdx.x - ti * (ti + 1) / 2, i0 = ti * kTile, j0 = tj * kTile;
+    const double* Wg = a.W + (size_t)g * npad * npad;
+    // ---- c = sum_{r >= i0} W[r][i] W[r][j]
+    double c[2][4][2] = {};
+    {
+        double* sA = reinterpret_cast<double*>(smem);   // [stages][16][68]
+        double* sB = sA + kStages * 16 * kLd;
+        const int steps = (npad - i0) / 16;             // npad and i0 are multiples of 32
+        auto load = [&](int s, int r0) {
+#pragma unroll
+            for (int it = 0; it < 2; ++it) {
+                const int e = t + kThreads * it, r = e / 32, q = e % 32;
+                const bool ok = i0 + 2 * q < npad;      // j0 <= i0: its columns exist where these do
+                cp_async16(sA + (s * 16 + r) * kLd + 2 * q, Wg + (size_t)(r0 + r) * npad + (ok ? i0 + 2 * q : 0), ok);
+                cp_async16(sB + (s * 16 + r) * kLd + 2 * q, Wg + (size_t)(r0 + r) * npad + j0 + 2 * q);
+            }
+        };
+#pragma unroll
+        for (int s = 0; s < kStages - 1; ++s) {
+            if (s < steps) load(s, i0 + s * 16);
+            cp_async_commit();
+        }
+        for (int s = 0; s < steps; ++s) {
+            cp_async_wait<kStages - 2>();
             __syncthreads();
+            if (s + kStages - 1 < steps) load((s + kStages - 1) % kStages, i0 + (s + kStages - 1) * 16);
+            cp_async_commit();
+            const double* pa = sA + ((s % kStages) * 16 + l % 4) * kLd + wm + l / 4;
+            const double* pb = sB + ((s % kStages) * 16 + l % 4) * kLd + wn + l / 4;
+#pragma unroll
+            for (int kk = 0; kk < 16; kk += 4) {
+                double fa[2], fb[4];
+#pragma unroll
+                for (int i = 0; i < 2; ++i) fa[i] = pa[kk * kLd + 8 * i];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) fb[j] = pb[kk * kLd + 8 * j];
+#pragma unroll
+                for (int i = 0; i < 2; ++i)
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) dmma(c[i][j], fa[i], fb[j]);
+            }
         }
-        const double s = red[0];
+        cp_async_wait<0>();
+    }
+    // ---- the pairs: rows wm + 8 i + l / 4, columns wn + 8 j + 2 (l % 4) + h of the tile
+    double* xi = reinterpret_cast<double*>(smem);   // [64][33]
+    double* xj = xi + kTile * 33;
+    double* il = xj + kTile * 33;                   // [32] reciprocal lengthscales (FP64, as the fit's)
+    const float* Xg = a.X + (size_t)g * n * d;
+    auto stage = [&](int c0) {
         __syncthreads();
-        return s;
+        const int f = t % 32, q = t / 32;
+        float vi[8], vj[8];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+            const int gi = i0 + q + 8 * e, gj = j0 + q + 8 * e;
+            vi[e] = (gi < n && c0 + f < d) ? __ldg(Xg + (size_t)gi * d + c0 + f) : 0.f;
+            vj[e] = (gj < n && c0 + f < d) ? __ldg(Xg + (size_t)gj * d + c0 + f) : 0.f;
+        }
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+            xi[(q + 8 * e) * 33 + f] = (double)vi[e];
+            xj[(q + 8 * e) * 33 + f] = (double)vj[e];
+        }
+        if (t < 32) il[t] = (c0 + t < d) ? 1.0 / (double)a.ell[(size_t)g * d + c0 + t] : 0.0;
+        __syncthreads();
     };
-    for (int j = 0; j <= d; ++j) {
-        double v = 0.0;
-        for (int b = t; b < tiles; b += 256) v += partial[(size_t)b * (d + 1) + j];
-        const double s = block_sum(v);
-        if (t == 0) out[1 + j] = 0.5 * s;
+    double r2[2][4][2] = {};
+    for (int c0 = 0; c0 < d; c0 += 32) {
+        stage(c0);
+        const int cmax = min(32, d - c0);
+        for (int f = 0; f < cmax; ++f) {
+            const double s = il[f];
+            double p[2], q[4][2];
+#pragma unroll
+            for (int i = 0; i < 2; ++i) p[i] = xi[(wm + 8 * i + l / 4) * 33 + f];
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+#pragma unroll
+                for (int h = 0; h < 2; ++h) q[j][h] = xj[(wn + 8 * j + 2 * (l % 4) + h) * 33 + f];
+#pragma unroll
+            for (int i = 0; i < 2; ++i)
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        const double df = (p[i] - q[j][h]) * s;
+                        r2[i][j][h] = fma(df, df, r2[i][j][h]);
+                    }
+        }
     }
-    double tr = 0.0, quad = 0.0, logdet = 0.0;
-    for (int i = t; i < n; i += 256) {
-        tr += M[(size_t)i * npad + i];
-        quad += (double)y[i] * alpha[i];
-        logdet += log(L[(size_t)i * npad + i]);
+    // c becomes the weight of u^2 in the lengthscales' derivatives: w M sf2 e^-s (5/3)(1 + s)
+    const double sf2 = (double)a.sf2[g];
+    const double* alpha = a.alpha + (size_t)g * npad;
+    double kf = 0.0, trace = 0.0;
+#pragma unroll 1
+    for (int j = 0; j < 4; ++j)
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int row = i0 + wm + 8 * i + l / 4, col = j0 + wn + 8 * j + 2 * (l % 4) + h;
+                double r = 0.0, k = 0.0;   // j is not unrolled (code size): pick its entries
+#pragma unroll
+                for (int jj = 0; jj < 4; ++jj) {
+                    r = jj == j ? r2[i][jj][h] : r;
+                    k = jj == j ? c[i][jj][h] : k;
+                }
+                double gk = 0.0;
+                if (row < n && col <= row) {
+                    const double m = fma(alpha[row], alpha[col], -k), wm2 = row == col ? m : 2.0 * m;
+                    const double s = sqrt(5.0) * sqrt(r), e = wm2 * sf2 * exp(-s);
+                    gk = e * (5.0 / 3.0) * (1.0 + s);
+                    kf = fma(e, fma(s, fma(s, 1.0 / 3.0, 1.0), 1.0), kf);
+                    if (row == col) trace += m;
+                }
+#pragma unroll
+                for (int jj = 0; jj < 4; ++jj) c[i][jj][h] = jj == j ? gk : c[i][jj][h];
+            }
+    double* out = a.partial + ((size_t)g * a.tiles + blockIdx.x) * (d + 2);
+    auto warp_sum = [](double v) {
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        return v;
+    };
+    kf = warp_sum(kf);
+    trace = warp_sum(trace);
+    if (l == 0) {
+        red[w][32] = kf;
+        red[w][33] = trace;
     }
-    tr = block_sum(tr);
-    quad = block_sum(quad);
-    logdet = block_sum(logdet);
-    if (t == 0) {
-        out[d + 2] = 0.5 * sn2 * tr;
-        out[0] = -0.5 * quad - logdet - 0.5 * n * 1.8378770664093454836;   // log(2 pi)
+    for (int c0 = 0; c0 < d; c0 += 32) {
+        if (d > 32) stage(c0);   // with one chunk the coordinates are still there
+        const int cmax = min(32, d - c0);
+        // Eight features at a time: every lane has eight sums, and a butterfly that halves their number with the number of
+        // lanes that hold them needs 9 exchanges instead of 40.
+#pragma unroll 1
+        for (int f0 = 0; f0 < cmax; f0 += 8) {
+            double v[8];
+#pragma unroll
+            for (int b = 0; b < 8; ++b) {
+                const int f = f0 + b;   // beyond cmax: coordinates and scale are zeros
+                const double s = il[f];
+                double acc = 0.0, q[4][2];
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) q[j][h] = xj[(wn + 8 * j + 2 * (l % 4) + h) * 33 + f];
+#pragma unroll
+                for (int i = 0; i < 2; ++i) {
+                    const double p = xi[(wm + 8 * i + l / 4) * 33 + f];
+#pragma unroll
+                    for (int j = 0; j < 4; ++j)
+#pragma unroll
+                        for (int h = 0; h < 2; ++h) {
+                            const double u = (p - q[j][h]) * s;
+                            acc = fma(c[i][j][h], u * u, acc);
+                        }
+                }
+                v[b] = acc;
+            }
+#pragma unroll
+            for (int o = 4; o > 0; o >>= 1) {
+                const bool up = (l & o) != 0;
+#pragma unroll
+                for (int b = 0; b < 4; ++b)
+                    if (b < o) {
+                        const double give = up ? v[b] : v[b + o], keep = up ? v[b + o] : v[b];
+                        v[b] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+                    }
+            }
+            double s = v[0];   // of feature f0 + l % 8
+            s += __shfl_xor_sync(0xffffffffu, s, 8);
+            s += __shfl_xor_sync(0xffffffffu, s, 16);
+            if (l < 8) red[w][f0 + l] = s;
+        }
+        __syncthreads();
+        if (t < cmax || (c0 == 0 && t >= 32 && t < 34)) {
+            double s = 0.0;
+            for (int ww = 0; ww < 8; ++ww) s += red[ww][t];
+            out[t < 32 ? c0 + t : d + t - 32] = s;
+        }
+        __syncthreads();
     }
 }
+
+// A warp per derivative (and one each for the trace and the value), the tiles' sums added in a fixed order.
+__global__ void __launch_bounds__(kThreads) lml_finish_kernel(const LmlArgs a)
+{
+    const int g = blockIdx.y, lane = threadIdx.x % 32, what = blockIdx.x * (kThreads / 32) + threadIdx.x / 32, d = a.d, n = a.n;
+    if (what > d + 2) return;
+    double* out = a.out + (size_t)g * (d + 3);
+    double s = 0.0;
+    if (what <= d + 1) {
+        const double* p = a.partial + (size_t)g * a.tiles * (d + 2) + what;
+#pragma unroll 4
+        for (int b = lane; b < a.tiles; b += 32) s += p[(size_t)b * (d + 2)];
+    } else {
+        const double* L = a.L + (size_t)g * a.npad * a.npad;
+#pragma unroll 4
+        for (int i = lane; i < n; i += 32) {
+            s = fma(-0.5 * (double)a.y[(size_t)g * n + i], a.alpha[(size_t)g * a.npad + i], s);
+            s -= log(L[(size_t)i * a.npad + i]);
+        }
+    }
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane == 0) {
+        if (what <= d) out[1 + what] = 0.5 * s;
+        else if (what == d + 1) out[d + 2] = 0.5 * (double)a.sn2[g] * s;
+        else out[0] = s - 0.5 * n * 1.8378770664093454836;   // log(2 pi)
+    }
+}
+
+int lml_tiles(int n) { return ((n + kTile - 1) / kTile) * ((n + kTile - 1) / kTile + 1) / 2; }
 
 }  // namespace
 
-// out_h: host [batch][d + 3] = {lml, d/dlog ell_1..d, d/dlog sf2, d/dlog sn2}.  Synchronises.
+size_t lml_scratch_doubles(const r3_fit_state& s) { return (size_t)s.batch * ((size_t)lml_tiles(s.n) * (s.d + 2) + s.d + 3); }
+
+// Asynchronous: *out (device, inside scratch) becomes [batch][d + 3] = {lml, d/dlog ell_1..d, d/dlog sf2, d/dlog sn2}.
+r3_status_t lml_enqueue(const r3_fit_state& s, double* scratch, double** out, cudaStream_t stream)
+{
+    LmlArgs a;
+    a.X = s.X; a.ell = s.ell_d; a.sf2 = s.sf2_d; a.sn2 = s.sn2_d; a.y = s.y;
+    a.W = s.W64; a.L = s.L64; a.alpha = s.alpha64;
+    a.n = s.n; a.d = s.d; a.npad = s.npad;
+    a.tiles = lml_tiles(s.n);
+    a.out = scratch;
+    a.partial = scratch + (size_t)s.batch * (s.d + 3);
+    *out = a.out;
+    R3_CUDA_TRY(cudaFuncSetAttribute(lml_tile_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTileSmem));
+    R3_LAUNCH(lml_tile_kernel, dim3(a.tiles, s.batch), kThreads, kTileSmem, stream, a);
+    R3_LAUNCH(lml_finish_kernel, dim3((s.d + 3 + kThreads / 32 - 1) / (kThreads / 32), s.batch), kThreads, 0, stream, a);
+    return R3_OK;
+}
+
+// out_h: host [batch][d + 3].  Synchronises.
 r3_status_t lml_device(r3_gp* gp, double* out_h, cudaStream_t stream)
 {
-    const int B = gp->batch, n = gp->n, d = gp->d, npad = gp->npad;
-    const int t32 = (n + 31) / 32, tiles = t32 * (t32 + 1) / 2;
-    double *M = nullptr, *partial = nullptr, *out = nullptr;
+    double* scratch = nullptr;
     auto done = [&](r3_status_t st) {
         if (st != R3_OK) cudaStreamSynchronize(stream);   // otherwise it has been
         FreeScope no_wait;
-        dev_free(M);
-        dev_free(partial);
-        dev_free(out);
+        dev_free(scratch);
         return st;
     };
-#define TRY_DONE(expr)                                                                             \
-    do {                                                                                           \
-        cudaError_t e__ = (expr);                                                                  \
-        if (e__ != cudaSuccess) {                                                                  \
-            set_error("%s failed: %s", #expr, cudaGetErrorString(e__));                            \
-            return done(e__ == cudaErrorMemoryAllocation ? R3_ERR_ALLOC : R3_ERR_CUDA);            \
-        }                                                                                          \
-    } while (0)
-    TRY_DONE(dev_malloc(&M, sizeof(double) * (size_t)B * npad * npad));
-    TRY_DONE(dev_malloc(&partial, sizeof(double) * (size_t)B * tiles * (d + 1)));
-    TRY_DONE(dev_malloc(&out, sizeof(double) * (size_t)B * (d + 3)));
-    const int t64 = (n + 63) / 64;
-    kinv_kernel<<<dim3(t64, t64, B), 256, 0, stream>>>(gp->W64, gp->alpha64, n, npad, M);
-    ++g_launches;
-    TRY_DONE(cudaGetLastError());
-    lml_pairs_kernel<<<dim3(tiles, B), 256, 0, stream>>>(gp->X, gp->ell_d, gp->sf2_d, n, d, npad, M, tiles, partial);
-    ++g_launches;
-    TRY_DONE(cudaGetLastError());
-    lml_finish_kernel<<<B, 256, 0, stream>>>(partial, tiles, d, M, gp->L64, gp->alpha64, gp->y, n, npad, gp->sn2_d, out);
-    ++g_launches;
-    TRY_DONE(cudaGetLastError());
-    TRY_DONE(cudaMemcpyAsync(out_h, out, sizeof(double) * (size_t)B * (d + 3), cudaMemcpyDeviceToHost, stream));
-    TRY_DONE(cudaStreamSynchronize(stream));
-#undef TRY_DONE
+    R3_CUDA_TRY(dev_malloc(&scratch, sizeof(double) * lml_scratch_doubles(*gp)));
+    double* out = nullptr;
+    const r3_status_t st = lml_enqueue(*gp, scratch, &out, stream);
+    if (st != R3_OK) return done(st);
+    cudaError_t e = cudaMemcpyAsync(out_h, out, sizeof(double) * (size_t)gp->batch * (gp->d + 3), cudaMemcpyDeviceToHost, stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
+    if (e != cudaSuccess) {
+        set_error("r3_gp_lml: %s", cudaGetErrorString(e));
+        return done(R3_ERR_CUDA);
+    }
     return done(R3_OK);
 }
 

@@ -274,14 +274,10 @@ r3_status_t r3_gp_optimize(r3_gp_t* gp, int max_evals, double gtol, float* lengt
         if (!any) break;
         load(false);
         int bits = 0;
-        st = state_fit(gp, *gp, 0, false, false, stream, &bits, nullptr);
+        st = state_fit(gp, *gp, 0, false, false, stream, &bits, nullptr, out.data());
         if (st != R3_OK) return st;
         ++used;
         const bool ok = !(bits & (DEV_NOT_PD | DEV_NONFINITE));
-        if (ok) {
-            st = lml_device(gp, out.data(), stream);
-            if (st != R3_OK) return st;
-        }
         for (int g = 0; g < B; ++g) {
             if (opt[g].done()) continue;
             for (int j = 0; j < P; ++j) grad[j] = ok ? -out[(size_t)g * (d + 3) + 1 + j] : 0.0;
