@@ -20,8 +20,8 @@
 // ill-conditioned factor, and the log-determinant of noise-free smooth data came out wrong in the third digit.)
 //
 // Bound: FP64 rate for long histories, the chain of diagonal blocks for short ones.  One GP of 4096 observations (64
-// features): 3.4 ms, 27 TFLOP/s of FP64 without the exponentials (a sequence of 290 launches with 4x4 register tiles and
-// recursive doubling for the inverse: 7.2 ms); 300 observations 0.18 ms (0.41 ms); 64 GPs of 512 0.65 ms (1.26 ms).
+// features): 3.1 ms, 30 TFLOP/s of FP64 without the exponentials (a sequence of 290 launches with 4x4 register tiles and
+// recursive doubling for the inverse: 7.2 ms); 300 observations 0.14 ms (0.41 ms); 64 GPs of 512 0.60 ms (1.26 ms).
 // An append of 128 to 3968 (it was triangular products, a Schur complement and their corrections): 0.6 ms (2.0 ms).
 #include <algorithm>
 
@@ -75,8 +75,7 @@ __device__ __forceinline__ int wait_progress(const int* p, int want, int* status
 
 struct Shared {
     int task, ready, ok;
-    alignas(16) double col[2][32];
-    double rinv[TB];   // the diagonal block's current column; its reciprocal roots
+    double rinv[TB];   // reciprocal roots of the diagonal block's pivots
 };
 
 // This thread's accumulators, -K(i,j): rows wm + 8 a + l / 4, columns wn + 8 b + 2 (l % 4) + h.
@@ -297,12 +296,18 @@ __device__ __forceinline__ double rsqrt_halley(double p)
 }
 
 // Columns b .. b + 31 of the tile, rows b .. 63 (one warp for 32 rows, two for 64): lane = row, the row's 32 entries in
-// registers.  The chain from pivot to pivot is one reciprocal square root, a multiplication, a multiply-add and a
-// shuffle; the rank-one update of a column reads the other rows' entries as broadcasts.
+// registers.  The loop over the columns is not unrolled: the entries move down by one place per step instead, so that the
+// step's column is always the first.  That is twice the multiply-adds (the places beyond the end hold leftovers that nothing
+// uses), but straight code for 32 columns is over 20 KB that a block runs once, and fetching it took longer.
+// The chain from pivot to pivot is a multiplication, a multiply-add and a reciprocal square root: every lane carries the next
+// row's entries on the diagonal and left of it along (fetched by shuffles a step ahead), so that none waits for a broadcast.
+// The two panels of a 64 x 64 block: 17,700 cycles; 22,000 with the shuffle in the chain and unrolled code.  (Letting the
+// second warp follow by a counter instead of the barrier: 24,000, it falls behind.)
 // A pivot of the history must exceed `tiny`, a few roundings of the diagonal entry it was computed from: a duplicated row
-// without noise leaves a pivot of either sign at that level.
-__device__ __forceinline__ void factor_panel(double* tile, int b, int warps, Shared& sh, const FactorArgs& a, int pivot0,
-                                             double tiny)
+// without noise leaves a pivot of either sign at that level.  cols: 32 x 32 doubles of scratch in shared memory; *step: zero
+// on entry, seen by both warps.
+__device__ __forceinline__ void factor_panel(double* tile, int b, int warps, double* cols, double* rinv,
+                                             const FactorArgs& a, int pivot0, double tiny)
 {
     const int w = threadIdx.x / 32, l = threadIdx.x % 32;
     if (w >= warps) return;
@@ -314,43 +319,65 @@ __device__ __forceinline__ void factor_panel(double* tile, int b, int warps, Sha
         x[c] = v.x;
         x[c + 1] = v.y;
     }
-    double p = w == 0 ? __shfl_sync(0xffffffffu, x[0], 0) : 1.0;
-    int failed = 32;   // first column whose pivot was not positive
+    double* out = tile + row * kLd + b;
+    auto update = [&](int k, double x0) {   // the entries move down as they are updated
+        const double* col = cols + 32 * k;
 #pragma unroll
-    for (int k = 0; k < 32; ++k) {
-        if (w == 0) {
-            // the test runs beside the root; a failed pivot becomes 1 (the call reports it)
-            const bool bad = !(p > (pivot0 + b + k < a.n ? tiny : 0.0)) || !isfinite(p);
-            failed = bad ? min(failed, k) : failed;
-            const double r0 = rsqrt_halley(p), r = bad ? 1.0 : r0;
-            p = bad ? 1.0 : p;
-            // sqrt(p) from r with one correction step: s = p r, s += r (p - s^2) / 2
-            const double sq = p * r, root = fma(0.5 * r, fma(-sq, sq, p), sq);
-            x[k] = l == k ? root : x[k] * r;
-            // the next pivot first: its row's own entry is all it needs
-            if (k < 31) p = __shfl_sync(0xffffffffu, fma(-x[k], x[k], x[k + 1]), k + 1);
-            sh.col[k & 1][l] = x[k];
-            if (l == k) sh.rinv[b + k] = r;
+        for (int j = 0; j < 30; j += 2) {
+            const double2 v = *reinterpret_cast<const double2*>(col + j);
+            x[j] = fma(-x0, v.x, x[j + 1]);
+            x[j + 1] = fma(-x0, v.y, x[j + 2]);
         }
+        x[30] = fma(-x0, col[30], x[31]);
+    };
+    auto meet = [&]() {
         if (warps == 2) asm volatile("bar.sync 1, 64;" ::: "memory");
         else __syncwarp();
-        if (w == 1) x[k] *= sh.rinv[b + k];
-        // two entries per read (the column starts on a 16-byte boundary)
-#pragma unroll
-        for (int j = (k + 1) & ~1; j < 32; j += 2) {
-            const double2 v = *reinterpret_cast<const double2*>(&sh.col[k & 1][j]);
-            if (j > k) x[j] = fma(-x[k], v.x, x[j]);
-            x[j + 1] = fma(-x[k], v.y, x[j + 1]);
+    };
+    if (w == 0) {
+        int failed = 32;   // first column whose pivot was not positive
+        // the test of a pivot runs beside its root; a failed one becomes 1 (the call reports it)
+        auto root = [&](int k, double& p) {
+            const bool bad = !(p > (pivot0 + b + k < a.n ? tiny : 0.0)) || !isfinite(p);
+            const double r = rsqrt_halley(p);
+            failed = bad ? min(failed, k) : failed;
+            p = bad ? 1.0 : p;
+            return bad ? 1.0 : r;
+        };
+        double p = __shfl_sync(0xffffffffu, x[0], 0), r = root(0, p);
+        // row k + 1: its entry in column k and on the diagonal, after the updates of the columns before k
+        double left = __shfl_sync(0xffffffffu, x[0], 1), below = __shfl_sync(0xffffffffu, x[1], 1);
+#pragma unroll 1
+        for (int k = 0; k < 32; ++k) {
+            const double lk = left * r;
+            double pn = fma(-lk, lk, below);
+            // sqrt(p) from r with one correction step: s = p r, s += r (p - s^2) / 2
+            const double sq = p * r, diag = fma(0.5 * r, fma(-sq, sq, p), sq);
+            const double x0 = l == k ? diag : x[0] * r;
+            if (l > k) cols[32 * k + l - k - 1] = x0;
+            if (l == k) rinv[b + k] = r;
+            out[k] = l >= k ? x0 : 0.0;
+            meet();
+            const double rn = root(k + 1, pn);   // (beyond the last column: of a leftover, not used)
+            update(k, x0);
+            left = __shfl_sync(0xffffffffu, x[0], (k + 2) & 31);
+            below = __shfl_sync(0xffffffffu, x[1], (k + 2) & 31);
+            p = pn;
+            r = rn;
+        }
+        if (failed < 32 && l == 0) {
+            atomicOr(&a.status[0], DEV_NOT_PD);
+            atomicMin(&a.status[1], pivot0 + b + failed);
+        }
+    } else {
+#pragma unroll 1
+        for (int k = 0; k < 32; ++k) {
+            meet();
+            const double x0 = x[0] * rinv[b + k];
+            out[k] = x0;
+            update(k, x0);
         }
     }
-    if (w == 0 && failed < 32 && l == 0) {
-        atomicOr(&a.status[0], DEV_NOT_PD);
-        atomicMin(&a.status[1], pivot0 + b + failed);
-    }
-#pragma unroll
-    for (int c = 0; c < 32; c += 2)   // zeros above the diagonal
-        *reinterpret_cast<double2*>(tile + row * kLd + b + c) =
-            make_double2(b + c <= row ? x[c] : 0.0, b + c + 1 <= row ? x[c + 1] : 0.0);
 }
 
 // x L^T = a for 64 rows against the 32 columns at b, two warps, lane = row
@@ -443,10 +470,7 @@ __global__ void __launch_bounds__(kThreads, 2) factor_kernel(const __grid_consta
     const int total = a.first[T] * a.batch;
     auto publish = [&](int* p, int v) {   // the tile has been stored by all threads
         __syncthreads();
-        if (t == 0) {
-            __threadfence();
-            store_release_int(p, v);
-        }
+        if (t == 0) store_release_int(p, v);   // (a release covers what the barrier has made this thread see)
     };
     auto await = [&](const int* p, int want) {
         if (t == 0) sh.ok = wait_progress(p, want, a.status);
@@ -483,11 +507,11 @@ __global__ void __launch_bounds__(kThreads, 2) factor_kernel(const __grid_consta
             __syncthreads();
             if (i == j) {
                 const double tiny = 4.0 * 2.220446049250313e-16 * ((double)a.sf2[g] + (double)a.sn2[g]);
-                factor_panel(tile0, 0, 2, sh, a, j * TB, tiny);
+                factor_panel(tile0, 0, 2, tile1, sh.rinv, a, j * TB, tiny);
                 __syncthreads();
                 update_right(tile0, tile0, 32);
                 __syncthreads();
-                factor_panel(tile0, 32, 1, sh, a, j * TB, tiny);
+                factor_panel(tile0, 32, 1, tile1, sh.rinv, a, j * TB, tiny);
                 for (int e = t; e < 32 * 32; e += kThreads) tile0[(e / 32) * kLd + 32 + e % 32] = 0.0;
                 __syncthreads();
                 store_tile(Lg, npad, j, j, tile0);
