@@ -55,3 +55,25 @@ def test_long_histories_on_pools_that_need_fp16_cross_terms(batch, n, d, m, sn2)
         assert np.array_equal(val[q], ei[q][idx[q]])
         assert np.array_equal(idx[q], o.topk(ei[q], 20)[0])
     gp.close()
+
+
+@pytest.mark.parametrize("m,k", [(128, 64), (300, 8), (4096, 1), (4096, 128), (4096, 129), (5000, 320), (20000, 321), (70001, 257)])
+@pytest.mark.parametrize("kind", ["uniform", "crowded", "equal", "clustered"])
+def test_selection_behind_the_guard(m, k, kind):
+    """The scoring call's selection must be the oracle's on the EI it returns, on pools whose best values lie spread out,
+    side by side, among many equal ones, or almost all below the rest."""
+    g = rand_problem(60 + k, 1, 24, 3, m, spread=1.0)
+    rng = np.random.default_rng(m + k)
+    if kind == "crowded":        # the best candidates side by side (one thread's share of a slice at stride 256)
+        best = g["Xcand"][0][:1].repeat(m, axis=0)
+        g["Xcand"][0, ::256] = best[::256] + rng.normal(0, 1e-3, (len(best[::256]), 3)).astype(np.float32)
+    elif kind == "equal":
+        g["Xcand"][0] = g["Xcand"][0][rng.integers(0, 5, m)]
+    elif kind == "clustered":
+        g["Xcand"][0, k // 2:] = 40.0   # far away: prior mean and variance, one EI value for most of the pool
+    gp = fit_gpu(g)
+    mu, sd, ei, idx, val = (t.cpu().numpy()[0] for t in b.r3_gp_score_topk(gp, dev(g["Xcand"]), k))
+    b.r3_gp_check(gp)
+    oidx, oval = o.topk(ei, k)
+    assert np.array_equal(idx, oidx) and np.array_equal(val, oval.astype(np.float32))
+    gp.close()
