@@ -296,18 +296,21 @@ __device__ __forceinline__ double rsqrt_halley(double p)
 }
 
 // Columns b .. b + 31 of the tile, rows b .. 63 (one warp for 32 rows, two for 64): lane = row, the row's 32 entries in
-// registers.  The loop over the columns is not unrolled: the entries move down by one place per step instead, so that the
-// step's column is always the first.  That is twice the multiply-adds (the places beyond the end hold leftovers that nothing
-// uses), but straight code for 32 columns is over 20 KB that a block runs once, and fetching it took longer.
-// The chain from pivot to pivot is a multiplication, a multiply-add and a reciprocal square root: every lane carries the next
-// row's entries on the diagonal and left of it along (fetched by shuffles a step ahead), so that none waits for a broadcast.
-// The two panels of a 64 x 64 block: 17,700 cycles; 22,000 with the shuffle in the chain and unrolled code.  (Letting the
-// second warp follow by a counter instead of the barrier: 24,000, it falls behind.)
+// registers.  The loop over the columns is not unrolled: the entries move down as they are updated instead, so that the
+// step's columns are always the first.  That is twice the multiply-adds (the places beyond the end hold leftovers that
+// nothing uses), but straight code for 32 columns is over 20 KB that a block runs once, and fetching it took longer.
+// Two columns per step, because the latency of the chain from pivot to pivot is what a diagonal block costs.  With the 2 x 2
+// block (p1 . ; s p2) ahead, det = p1 p2 - s^2 and the second pivot is det / p1, so that both reciprocal roots
+//     r1 = p1^-1/2,   r2 = (det / p1)^-1/2 = p1 r1 det^-1/2
+// are under way together (det is as accurate as the second pivot of column-by-column elimination: its rounding is that of
+// p2).  Every lane carries the next block and the entries left of it along, fetched by shuffles a step ahead, so that the
+// chain of a step is r2, one column, one update, det and its root, and waits for no broadcast.
+// The two panels of a 64 x 64 block: 15,500 cycles; 17,700 column by column, 22,000 with a shuffle in the chain and unrolled
+// code.  (Letting the second warp follow by a counter instead of the barrier: 24,000, it falls behind.)
 // A pivot of the history must exceed `tiny`, a few roundings of the diagonal entry it was computed from: a duplicated row
-// without noise leaves a pivot of either sign at that level.  cols: 32 x 32 doubles of scratch in shared memory; *step: zero
-// on entry, seen by both warps.
-__device__ __forceinline__ void factor_panel(double* tile, int b, int warps, double* cols, double* rinv,
-                                             const FactorArgs& a, int pivot0, double tiny)
+// without noise leaves a pivot of either sign at that level.  cols: 16 x 64 doubles of scratch in shared memory.
+__device__ __forceinline__ void factor_panel(double* tile, int b, int warps, double* cols, double* rinv, const FactorArgs& a,
+                                             int pivot0, double tiny)
 {
     const int w = threadIdx.x / 32, l = threadIdx.x % 32;
     if (w >= warps) return;
@@ -320,62 +323,78 @@ __device__ __forceinline__ void factor_panel(double* tile, int b, int warps, dou
         x[c + 1] = v.y;
     }
     double* out = tile + row * kLd + b;
-    auto update = [&](int k, double x0) {   // the entries move down as they are updated
-        const double* col = cols + 32 * k;
+    auto update = [&](int k, double x0, double x1) {   // the entries move down as they are updated
+        const double *c0 = cols + 32 * k, *c1 = c0 + 32;
 #pragma unroll
         for (int j = 0; j < 30; j += 2) {
-            const double2 v = *reinterpret_cast<const double2*>(col + j);
-            x[j] = fma(-x0, v.x, x[j + 1]);
-            x[j + 1] = fma(-x0, v.y, x[j + 2]);
+            const double2 u = *reinterpret_cast<const double2*>(c0 + j), v = *reinterpret_cast<const double2*>(c1 + j);
+            x[j] = fma(-x1, v.x, fma(-x0, u.x, x[j + 2]));
+            x[j + 1] = fma(-x1, v.y, fma(-x0, u.y, x[j + 3]));
         }
-        x[30] = fma(-x0, col[30], x[31]);
     };
     auto meet = [&]() {
         if (warps == 2) asm volatile("bar.sync 1, 64;" ::: "memory");
         else __syncwarp();
     };
     if (w == 0) {
-        int failed = 32;   // first column whose pivot was not positive
-        // the test of a pivot runs beside its root; a failed one becomes 1 (the call reports it)
-        auto root = [&](int k, double& p) {
-            const bool bad = !(p > (pivot0 + b + k < a.n ? tiny : 0.0)) || !isfinite(p);
-            const double r = rsqrt_halley(p);
-            failed = bad ? min(failed, k) : failed;
-            p = bad ? 1.0 : p;
-            return bad ? 1.0 : r;
-        };
-        double p = __shfl_sync(0xffffffffu, x[0], 0), r = root(0, p);
-        // row k + 1: its entry in column k and on the diagonal, after the updates of the columns before k
-        double left = __shfl_sync(0xffffffffu, x[0], 1), below = __shfl_sync(0xffffffffu, x[1], 1);
+        auto from = [&](double v, int lane) { return __shfl_sync(0xffffffffu, v, lane & 31); };
+        double p1 = from(x[0], 0), s = from(x[0], 1), p2 = from(x[1], 1), det = fma(p1, p2, -(s * s));
+        double r1 = rsqrt_halley(p1), rd = rsqrt_halley(det);
+        // rows k + 2 and k + 3: entries in columns k and k + 1, and their own block, after the updates before column k
+        double a0 = from(x[0], 2), a1 = from(x[1], 2), d22 = from(x[2], 2);
+        double b0 = from(x[0], 3), b1 = from(x[1], 3), d32 = from(x[2], 3), d33 = from(x[3], 3);
 #pragma unroll 1
-        for (int k = 0; k < 32; ++k) {
-            const double lk = left * r;
-            double pn = fma(-lk, lk, below);
-            // sqrt(p) from r with one correction step: s = p r, s += r (p - s^2) / 2
-            const double sq = p * r, diag = fma(0.5 * r, fma(-sq, sq, p), sq);
-            const double x0 = l == k ? diag : x[0] * r;
-            if (l > k) cols[32 * k + l - k - 1] = x0;
-            if (l == k) rinv[b + k] = r;
-            out[k] = l >= k ? x0 : 0.0;
+        for (int k = 0; k < 32; k += 2) {
+            const double sq1 = p1 * r1, l21 = s * r1, r2 = sq1 * rd;
+            const double la0 = a0 * r1, la1 = fma(-la0, l21, a1) * r2, lb0 = b0 * r1, lb1 = fma(-lb0, l21, b1) * r2;
+            const double p1n = fma(-la1, la1, fma(-la0, la0, d22)), sn = fma(-lb1, la1, fma(-lb0, la0, d32)),
+                         p2n = fma(-lb1, lb1, fma(-lb0, lb0, d33)), detn = fma(p1n, p2n, -(sn * sn));
+            // this lane's entries of the two columns; on the diagonal sqrt(p) from r with one correction step
+            // (s = p r, s += r (p - s^2) / 2)
+            const double q2 = det * (r1 * r1), sq2 = q2 * r2;
+            const double x0 = l == k ? fma(0.5 * r1, fma(-sq1, sq1, p1), sq1) : x[0] * r1;
+            const double x1 = l == k + 1 ? fma(0.5 * r2, fma(-sq2, sq2, q2), sq2) : fma(-x0, l21, x[1]) * r2;
+            double* c0 = cols + 32 * k;
+            if (l > k + 1) {
+                c0[l - k - 2] = x0;
+                c0[32 + l - k - 2] = x1;
+            }
+            if (l == k) {
+                rinv[b + k] = r1;
+                rinv[b + k + 1] = r2;
+                c0[31] = l21;
+            }
+            *reinterpret_cast<double2*>(out + k) = make_double2(l >= k ? x0 : 0.0, l >= k + 1 ? x1 : 0.0);
             meet();
-            const double rn = root(k + 1, pn);   // (beyond the last column: of a leftover, not used)
-            update(k, x0);
-            left = __shfl_sync(0xffffffffu, x[0], (k + 2) & 31);
-            below = __shfl_sync(0xffffffffu, x[1], (k + 2) & 31);
-            p = pn;
-            r = rn;
+            r1 = rsqrt_halley(p1n);
+            rd = rsqrt_halley(detn);
+            update(k, x0, x1);
+            p1 = p1n;
+            s = sn;
+            det = detn;
+            a0 = from(x[0], k + 4);
+            a1 = from(x[1], k + 4);
+            d22 = from(x[2], k + 4);
+            b0 = from(x[0], k + 5);
+            b1 = from(x[1], k + 5);
+            d32 = from(x[2], k + 5);
+            d33 = from(x[3], k + 5);
         }
-        if (failed < 32 && l == 0) {
+        // the pivots' test, once for all: lane = column; beyond the first bad pivot everything is NaN or means nothing
+        const double d = tile[row * kLd + row];
+        const bool bad = !(d * d > (pivot0 + row < a.n ? tiny : 0.0) * (1.0 + 1e-15)) || !isfinite(d);
+        const unsigned which = __ballot_sync(0xffffffffu, bad);
+        if (which && l == 0) {
             atomicOr(&a.status[0], DEV_NOT_PD);
-            atomicMin(&a.status[1], pivot0 + b + failed);
+            atomicMin(&a.status[1], pivot0 + b + __ffs(which) - 1);
         }
     } else {
 #pragma unroll 1
-        for (int k = 0; k < 32; ++k) {
+        for (int k = 0; k < 32; k += 2) {
             meet();
-            const double x0 = x[0] * rinv[b + k];
-            out[k] = x0;
-            update(k, x0);
+            const double x0 = x[0] * rinv[b + k], x1 = fma(-x0, cols[32 * k + 31], x[1]) * rinv[b + k + 1];
+            *reinterpret_cast<double2*>(out + k) = make_double2(x0, x1);
+            update(k, x0, x1);
         }
     }
 }
