@@ -12,6 +12,8 @@
 // task depends only on tasks before it, all blocks are resident, and a block works its tasks off one by one, so some
 // block can always go on.  Progress is one counter per row of L (its tiles finish from left to right) and one per
 // column of W (from top to bottom); a task adds up the products whose operands are there and waits for the next.
+// A tile of L is handed out in halves of 32 columns: the left half of a column's tiles is solved, stored and multiplied
+// while one warp factors the diagonal tile's second panel (300 observations: 118 -> 93 us; 1000: fit 621 -> 552 us).
 // So a tile is written once and read as an operand, nothing is updated in place, and the factor's critical path --
 // 64 columns in shared memory, one substitution, one product -- runs while the other blocks are busy with tiles far
 // from it.  Products run on the FP64 tensor path with three 16-deep operand stages in flight.
@@ -20,8 +22,8 @@
 // ill-conditioned factor, and the log-determinant of noise-free smooth data came out wrong in the third digit.)
 //
 // Bound: FP64 rate for long histories, the chain of diagonal blocks for short ones.  One GP of 4096 observations (64
-// features): 3.1 ms, 30 TFLOP/s of FP64 without the exponentials (a sequence of 290 launches with 4x4 register tiles and
-// recursive doubling for the inverse: 7.2 ms); 300 observations 0.14 ms (0.41 ms); 64 GPs of 512 0.60 ms (1.26 ms).
+// features): 3.0 ms, 31 TFLOP/s of FP64 without the exponentials (a sequence of 290 launches with 4x4 register tiles and
+// recursive doubling for the inverse: 7.2 ms); 300 observations 0.09 ms (0.41 ms); 64 GPs of 512 0.60 ms (1.26 ms).
 // An append of 128 to 3968 (it was triangular products, a Schur complement and their corrections): 0.6 ms (2.0 ms).
 #include <algorithm>
 
@@ -43,8 +45,8 @@ struct FactorArgs {
     const float *X, *ell, *sf2, *sn2;
     int batch, n, d, npad, T, i0;   // T tile rows; those below i0 are finished
     double *L, *W;                  // [batch][npad][npad]
-    int *lprog;                     // [batch][T] finished tiles of each row of L
-    int *wprog;                     // [batch][T] one past the last finished tile of each column of W
+    int *lprog;                     // [batch][T] finished half tiles (32 columns) of each row of L
+    int *wprog;                     // [batch][T] one past the last finished half tile of each column of W
     unsigned* ticket;
     int* status;
     int first[kMaxTiles + 1];       // tasks per GP before step j
@@ -184,13 +186,13 @@ __device__ __forceinline__ bool accumulate(const FactorArgs& a, int g, int i, in
     const int* li = a.lprog + (size_t)g * a.T + i;
     const int* lj = a.lprog + (size_t)g * a.T + j;
     const int* wj = a.wprog + (size_t)g * a.T + j;
-    // thread 0: the number of tile columns whose operands are there (at least `want`), -1 if a wait ran out
+    // thread 0: the number of half tiles whose operands are there (at least `want`), -1 if a wait ran out
     auto poll = [&](int want) {
-        int v = i < a.i0 ? a.T : wait_progress(li, want, a.status);
+        int v = i < a.i0 ? 2 * a.T : wait_progress(li, want, a.status);
         if (v < 0) return -1;
         int u;
-        if (NT) u = j < a.i0 ? a.T : (j == i ? v : wait_progress(lj, want, a.status));
-        else u = want <= a.i0 ? a.i0 : wait_progress(wj, want, a.status);
+        if (NT) u = j < a.i0 ? 2 * a.T : (j == i ? v : wait_progress(lj, want, a.status));
+        else u = want <= 2 * a.i0 ? 2 * a.i0 : wait_progress(wj, want, a.status);
         return u < 0 ? -1 : min(u, v);
     };
     auto load = [&](int s, int k) {   // stage s <- columns k .. k + 15
@@ -210,20 +212,20 @@ __device__ __forceinline__ bool accumulate(const FactorArgs& a, int g, int i, in
     const int s0 = k0 * 4, s1 = k1 * 4;   // 16-deep steps
     if (s0 >= s1) return true;
     __syncthreads();                      // the stages' bytes were last used for something else
-    if (t == 0) sh.ready = poll(k0 + 1);
+    if (t == 0) sh.ready = poll(2 * k0 + 1);
     __syncthreads();
     int ready = sh.ready;
     if (ready < 0) return false;
 #pragma unroll
     for (int s = 0; s < kStages - 1; ++s) {
-        load(s, (s0 + s) * 16);           // a tile has four steps: the first two are within it
+        load(s, (s0 + s) * 16);           // the first half tile has two steps
         cp_async_commit();
     }
     for (int s = s0; s < s1; ++s) {
         const int nx = s + kStages - 1;   // the step to fetch now
         cp_async_wait<kStages - 2>();
-        const bool ask = nx < s1 && nx / 4 >= ready;
-        if (ask && t == 0) sh.ready = poll(nx / 4 + 1);
+        const bool ask = nx < s1 && nx / 2 >= ready;
+        if (ask && t == 0) sh.ready = poll(nx / 2 + 1);
         __syncthreads();
         if (ask) {
             ready = sh.ready;
@@ -261,6 +263,28 @@ __device__ __forceinline__ void store_tile(double* Mg, int npad, int ti, int tj,
         if (ti * TB + r < npad && tj * TB + 2 * q < npad)
             *reinterpret_cast<double2*>(Mg + (size_t)(ti * TB + r) * npad + tj * TB + 2 * q) =
                 *reinterpret_cast<const double2*>(src + r * kLd + 2 * q);
+    }
+}
+
+// Of a diagonal tile: columns h .. h + 31 from row h on, as fetch_tile
+__device__ __forceinline__ void fetch_half(const double* Mg, int npad, int tj, int h, double* dst)
+{
+    for (int e = threadIdx.x; e < (TB - h) * 16; e += kThreads) {
+        const int r = h + e / 16, c = h + 2 * (e % 16);
+        const bool ok = tj * TB + r < npad && tj * TB + c < npad;
+        cp_async16(dst + r * kLd + c, Mg + (ok ? (size_t)(tj * TB + r) * npad + tj * TB + c : 0), ok);
+    }
+    cp_async_commit();
+}
+
+// Columns h .. h + 31 of a tile, by the threads t of `threads`
+__device__ __forceinline__ void store_half(double* Mg, int npad, int ti, int tj, int h, const double* src, int t, int threads)
+{
+    for (int e = t; e < TB * 16; e += threads) {
+        const int r = e / 16, c = h + 2 * (e % 16);
+        if (ti * TB + r < npad && tj * TB + c < npad)
+            *reinterpret_cast<double2*>(Mg + (size_t)(ti * TB + r) * npad + tj * TB + c) =
+                *reinterpret_cast<const double2*>(src + r * kLd + c);
     }
 }
 
@@ -530,32 +554,39 @@ __global__ void __launch_bounds__(kThreads, 2) factor_kernel(const __grid_consta
                 __syncthreads();
                 update_right(tile0, tile0, 32);
                 __syncthreads();
-                factor_panel(tile0, 32, 1, tile1, sh.rinv, a, j * TB, tiny);
-                for (int e = t; e < 32 * 32; e += kThreads) tile0[(e / 32) * kLd + 32 + e % 32] = 0.0;
+                // one warp takes the second panel; the others hand the first one out meanwhile
+                if (w == 0) {
+                    factor_panel(tile0, 32, 1, tile1, sh.rinv, a, j * TB, tiny);
+                } else {
+                    store_half(Lg, npad, j, j, 0, tile0, t - 32, kThreads - 32);
+                    asm volatile("bar.sync 2, 224;" ::: "memory");
+                    if (t == 32) store_release_int(lp + j, 2 * j + 1);
+                    for (int e = t - 32; e < 32 * 32; e += kThreads - 32) tile0[(e / 32) * kLd + 32 + e % 32] = 0.0;
+                }
                 __syncthreads();
-                store_tile(Lg, npad, j, j, tile0);
-                publish(lp + j, j + 1);
+                store_half(Lg, npad, j, j, 32, tile0, t, kThreads);
+                publish(lp + j, 2 * j + 2);
                 for (int e = t; e < 32 * 32; e += kThreads) tile1[(e / 32) * kLd + 32 + e % 32] = 0.0;
                 if (w < 2) invert_block(tile0, sh.rinv, 32 * w, tile1);
                 __syncthreads();
                 invert_corner(tile0, tile1, tile0);   // L11 is not needed any more
                 store_tile(Wg, npad, j, j, tile1);
-                publish(a.wprog + (size_t)g * T + j, j + 1);
+                publish(a.wprog + (size_t)g * T + j, 2 * j + 2);
             } else {
-                if (j >= a.i0 && !await(lp + j, j + 1)) return;
-                fetch_tile(Lg, npad, j, j, tile1);
-                cp_async_wait<0>();
-                __syncthreads();
-                if (t < TB) sh.rinv[t] = 1.0 / tile1[t * kLd + t];
-                __syncthreads();
-                solve_panel(tile0, tile1, sh.rinv, 0);
-                __syncthreads();
-                update_right(tile0, tile1, 0);
-                __syncthreads();
-                solve_panel(tile0, tile1, sh.rinv, 32);
-                __syncthreads();
-                store_tile(Lg, npad, i, j, tile0);
-                publish(lp + i, j + 1);
+                // the left half against the first panel while the second is being made
+                for (int h = 0; h < 64; h += 32) {
+                    if (j >= a.i0 && !await(lp + j, 2 * j + 1 + h / 32)) return;
+                    fetch_half(Lg, npad, j, h, tile1);
+                    cp_async_wait<0>();
+                    __syncthreads();
+                    if (t < 32) sh.rinv[h + t] = 1.0 / tile1[(h + t) * kLd + h + t];
+                    __syncthreads();
+                    solve_panel(tile0, tile1, sh.rinv, h);
+                    __syncthreads();
+                    store_half(Lg, npad, i, j, h, tile0, t, kThreads);
+                    publish(lp + i, 2 * j + 1 + h / 32);
+                    if (h == 0) update_right(tile0, tile1, 0);
+                }
                 zero_tile(Lg, npad, j, i);
                 zero_tile(Wg, npad, j, i);
             }
@@ -565,7 +596,7 @@ __global__ void __launch_bounds__(kThreads, 2) factor_kernel(const __grid_consta
             Wg = a.W + (size_t)g * npad * npad;
             int* wp = a.wprog + (size_t)g * T;
             if (!accumulate<false>(a, g, i, col, col, i, smem, sh, c)) return;
-            if (!await(wp + i, i + 1)) return;
+            if (!await(wp + i, 2 * i + 2)) return;
             fetch_tile(Wg, npad, i, i, tile0);
             park(c, -1.0, tile1);
             cp_async_wait<0>();
@@ -581,7 +612,7 @@ __global__ void __launch_bounds__(kThreads, 2) factor_kernel(const __grid_consta
             park(c, 1.0, tile0);
             __syncthreads();
             store_tile(Wg, npad, i, col, tile0);
-            publish(wp + col, i + 1);
+            publish(wp + col, 2 * i + 2);
         }
     }
 }
