@@ -7,18 +7,23 @@
 // The weights ride on the first pass.  Vectors sit in shared memory; the norm of a new vector divides the next product, so
 // that normalising costs no barrier.
 //
-// Bound: W from L2, 26 times 4 n^2 bytes, and 25 barriers.  Up to 160 observations one block per GP keeps W in shared
-// memory instead and needs no barriers but its own (64 observations: 118 us by teams, 17 us by one block).  Before, 57
-// launches of three kernels per pass: 0.90 ms for one GP of 4096 observations (now 0.31 ms), 0.12 ms and 0.2 ms of launches
-// for one of 64.
+// Bound: W from L2, 26 times 4 n^2 bytes, and 25 barriers.  Up to 544 observations a cluster of blocks per GP keeps W in
+// shared memory instead and exchanges one vector per pass (one GP of 64 observations: 22 us, 29 us by one block; of 100 to
+// 180: 26 us, 53 us by one block; of 300 with the launch: 44 us, 93 us by a team).  Before, 57 launches of three kernels per
+// pass: 0.90 ms for one GP of 4096 observations (now 0.31 ms), 0.12 ms and 0.2 ms of launches for one of 64.
+#include <cooperative_groups.h>
+
 #include <algorithm>
 
 #include "r3_f64.cuh"
 #include "r3_internal.cuh"
+#include "r3_tc_common.cuh"
 
 namespace r3 {
 
 namespace {
+
+namespace cg = cooperative_groups;
 
 constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;
@@ -154,103 +159,221 @@ __device__ __forceinline__ void columns_pass(const WeightArgs& a, int g, int j0,
     }
 }
 
-// One block, W in shared memory: histories of at most kSmallRows observations.  A thread sums one part of one row (then of
-// one column): the lanes of a warp take 32 neighbouring rows and the same entries of the vector, so that the matrix is read
-// without bank conflicts (odd leading dimension) and the vector as broadcasts; the parts meet in shared memory.
-constexpr int kSmallRows = 160;
-constexpr int kSmallThreads = 1024;
-constexpr int kSmallParts = 16;
-__global__ void __launch_bounds__(kSmallThreads, 1) weights_small_kernel(const WeightArgs a)
+// One cluster of R blocks per GP, W in their shared memory: row i in block i mod R, packed to the diagonal.  A block forms
+// its own rows' products u_i = W_i . x and at once their share sum u_i W_i of the new vector.  The shares are written
+// straight into all blocks' shared memory (asynchronous stores that count on the receiver's mbarrier), which is the only
+// exchange of a pass, and every block adds them up in the same order.  Two sets of shares: a block sends the next set only
+// after it has read this one, so whoever sends the one after next has seen that.
+// Eight lanes take a row (128 contiguous bytes), a thread two columns and every P-th of the block's rows.
+// Bound: instructions issued by all warps alike, so a short history gets few warps and everything that depends only on the
+// thread is worked out before the passes.
+constexpr int kClusterThreads = 512;   // at most
+constexpr int kMaxParts = 4;
+__host__ __device__ inline int cluster_threads(int npad) { return npad <= 128 ? 128 : npad <= 256 ? 256 : 512; }
+__host__ __device__ inline int cluster_parts(int npad) { return min(kMaxParts, cluster_threads(npad) / (npad / 2)); }
+__host__ __device__ inline int packed_doubles(int npad, int R) { return npad / 2 * (npad / R + 1); }
+constexpr size_t kClusterSmem = 226 * 1024;   // dynamic; a block's static arrays take a little more
+inline size_t cluster_smem(int npad, int R)   // W, x, the shares, the parts of a share, u
 {
-    extern __shared__ __align__(16) double vec[];   // W [npad][npad + 1], x [npad], sums [parts][npad]
-    __shared__ double part_norm[kSmallThreads / 32];
-    const int t = threadIdx.x, lane = t % 32, warp = t / 32, npad = a.npad, n = a.n, ld = npad + 1;
-    const int P = min(kSmallParts, kSmallThreads / npad), idx = t % npad, part = t / npad, block = idx & ~31;
-    double *Ws = vec, *x = Ws + npad * ld, *sums = x + npad;
-    // x <- sum of the parts times scale (zero beyond the history when asked for)
-    auto gather = [&](double scale, bool zero_beyond) {
-        __syncthreads();
-        if (t < npad) {
-            double s = 0.0;
-            for (int p = 0; p < P; ++p) s += sums[p * npad + t];
-            x[t] = zero_beyond && t >= n ? 0.0 : s * scale;
-        }
-        __syncthreads();
-    };
-    auto rows = [&]() {
-        if (part < P) {
-            double s[4] = {};
-            const double* w = Ws + idx * ld;
-            int k = part;
-            for (; k + 3 * P < block + 32; k += 4 * P)
-#pragma unroll
-                for (int e = 0; e < 4; ++e) s[e] = fma(w[k + e * P], x[k + e * P], s[e]);
-            for (; k < block + 32; k += P) s[0] = fma(w[k], x[k], s[0]);
-            sums[part * npad + idx] = (s[0] + s[1]) + (s[2] + s[3]);
-        }
-    };
-    auto columns = [&]() {
-        if (part < P) {
-            double s[4] = {};
-            const double* w = Ws + idx;
-            int i = block + part;
-            for (; i + 3 * P < npad; i += 4 * P)
-#pragma unroll
-                for (int e = 0; e < 4; ++e) s[e] = fma(w[(i + e * P) * ld], x[i + e * P], s[e]);
-            for (; i < npad; i += P) s[0] = fma(w[i * ld], x[i], s[0]);
-            sums[part * npad + idx] = (s[0] + s[1]) + (s[2] + s[3]);
-        }
-    };
-    auto norm = [&]() {
-        double s = t < npad ? x[t] * x[t] : 0.0;
-        if (warp < npad / 32) {
-            for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-            if (lane == 0) part_norm[warp] = s;
-        }
-        __syncthreads();
-        double all = 0.0;
-        for (int w = 0; w < npad / 32; ++w) all += part_norm[w];
-        return sqrt(all);
-    };
-    for (int g = blockIdx.x; g < a.batch; g += gridDim.x) {
-        const double* Wg = a.W + (size_t)g * npad * npad;
+    return sizeof(double) * ((size_t)packed_doubles(npad, R) + npad + 2 * R * npad + cluster_parts(npad) * npad + npad / R);
+}
+
+__device__ __forceinline__ uint32_t in_block(uint32_t addr, int block)
+{
+    uint32_t r;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(block));
+    return r;
+}
+__device__ __forceinline__ void send(uint32_t dst, uint32_t bar, double2 v)
+{
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.b64 [%0], {%1, %2}, [%3];" ::"r"(dst),
+                 "l"(__double_as_longlong(v.x)), "l"(__double_as_longlong(v.y)), "r"(bar)
+                 : "memory");
+}
+__device__ __forceinline__ bool arrived(uint32_t bar, uint32_t parity)
+{
+    uint32_t ok;
+    asm volatile("{\n\t.reg .pred p;\n\t"
+                 "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+                 "selp.u32 %0, 1, 0, p;\n\t}"
+                 : "=r"(ok)
+                 : "r"(bar), "r"(parity)
+                 : "memory");
+    return ok != 0;
+}
+
+template <int R>
+__global__ void __launch_bounds__(kClusterThreads, 1) weights_cluster_kernel(const WeightArgs a)
+{
+    extern __shared__ __align__(16) double vec[];
+    __shared__ double warp_sums[kClusterThreads / 32];
+    __shared__ int warp_tops[kClusterThreads / 32];
+    __shared__ __align__(8) unsigned long long bars[2];
+    cg::cluster_group cluster = cg::this_cluster();
+    const int r = (int)cluster.block_rank(), g = blockIdx.x / R, threads = blockDim.x, warps = threads / 32;
+    const int t = threadIdx.x, lane = t % 32, warp = t / 32, npad = a.npad, n = a.n, rows = npad / R, half = npad / 2;
+    const int P = cluster_parts(npad), even = (r & ~1) + 2;
+    double *Ws = vec, *x = Ws + packed_doubles(npad, R), *shares = x + npad, *parts = shares + 2 * R * npad, *u = parts + P * npad;
+    auto at = [&](int q) { return R / 2 * q * (q - 1) + q * even; };   // start of row R q + r: its length is even
+    const double* Wg = a.W + (size_t)g * npad * npad;
+    for (int q = warp; q < rows; q += warps)
+        for (int c = lane; c <= (R * q + r) / 2; c += 32)
+            cp_async16(Ws + at(q) + 2 * c, Wg + (size_t)(R * q + r) * npad + 2 * c);
+    cp_async_commit();
+    for (int j = t; j < npad; j += threads) x[j] = j < n ? (double)a.y[(size_t)g * n + j] : 0.0;
+    if (t == 0) {
+        mbar_init(smem_u32(&bars[0]), 1);
+        mbar_init(smem_u32(&bars[1]), 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (t < kClusterThreads / 32) {
+        warp_sums[t] = 0.0;
+        warp_tops[t] = 0;
+    }
+    cp_async_wait<0>();
+    cluster.sync();
+    if (a.W32 || a.wmax) {
         float top = 0.f;
-        __syncthreads();
-#pragma unroll 4
-        for (int i = warp; i < npad; i += kSmallThreads / 32)
-            for (int k = lane; k < npad; k += 32) {
-                const double w = Wg[i * npad + k];
-                Ws[i * ld + k] = w;
-                if (i < n) top = fmaxf(top, fabsf((float)w));
-                if (a.W32) a.W32[((size_t)g * npad + i) * npad + k] = (float)w;
+        for (int q = warp; q < rows; q += warps) {
+            const int i = R * q + r;
+            for (int c = lane; c < half; c += 32) {
+                float2 f = make_float2(0.f, 0.f);
+                if (c <= i / 2) {
+                    const double2 w = *reinterpret_cast<const double2*>(Ws + at(q) + 2 * c);
+                    f = make_float2((float)w.x, (float)w.y);
+                }
+                if (i < n) top = fmaxf(top, fmaxf(fabsf(f.x), fabsf(f.y)));
+                if (a.W32) *reinterpret_cast<float2*>(a.W32 + ((size_t)g * npad + i) * npad + 2 * c) = f;
             }
-        if (t < npad) x[t] = t < n ? (double)a.y[(size_t)g * n + t] : 0.0;
+        }
         if (a.wmax) {
             const unsigned m = __reduce_max_sync(0xffffffffu, __float_as_uint(top));
             if (lane == 0 && m) atomicMax(&a.wmax[g], m);
         }
-        __syncthreads();
-        rows();
-        gather(1.0, true);
-        columns();
-        gather(1.0, false);
-        if (t < npad) {
-            a.alpha64[(size_t)g * npad + t] = x[t];
-            a.alpha32[(size_t)g * npad + t] = (float)x[t];
-        }
-        if (a.iters == 0) continue;
-        __syncthreads();
-        if (t < npad) x[t] = t < n ? 1.0 + 0.37 * ((t * 2654435761u >> 16) & 0xff) / 255.0 : 0.0;
-        double nrm = norm();
-        for (int it = 0; it < a.iters; ++it) {
-            rows();
-            gather(nrm > 0.0 ? 1.0 / nrm : 0.0, true);
-            columns();
-            gather(1.0, false);
-            nrm = norm();
-        }
-        if (t == 0) a.wnorm[g] = 1.5 * sqrt(nrm);
     }
+    // the sum of all threads' values, to every thread
+    auto total = [&](double v) {
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        if (lane == 0) warp_sums[warp] = v;
+        __syncthreads();
+        double all = 0.0;
+        for (int w = 0; w < warps; ++w) all += warp_sums[w];
+        return all;
+    };
+    // this thread's columns 2 c and 2 c + 1, its first row there and the distance to the next ones in W
+    const int c = t % half, p = t / half, lots = threads / half;
+    const int q0 = p < P ? max(0, (2 * c - r + R - 1) / R) + p : rows;
+    const int off0 = at(q0) + 2 * c, step0 = at(q0 + P) - at(q0), grow = R * P * P;
+    const bool second = rows > threads / 8;
+    const uint32_t mine = smem_u32(shares + r * npad + 2 * c);
+    double2 v = make_double2(0.0, 0.0);   // (thread < half) the new vector's columns 2 t and 2 t + 1
+    bool late = false;                    // a bounded wait ran out: the rest goes through without waiting
+    auto pass = [&](double scale, int turn) {   // x, v <- W^T (scale W x)
+        for (int q = t / 8; q < rows; q += threads / 8) {
+            const int i = R * q + r, m = i < n ? i / 2 : -1;
+            const double* w = Ws + at(q);
+            double s0 = 0.0, s1 = 0.0;
+#pragma unroll 4
+            for (int k = t % 8; k <= m; k += 8) {
+                const double2 e = *reinterpret_cast<const double2*>(w + 2 * k), f = *reinterpret_cast<const double2*>(x + 2 * k);
+                s0 = fma(e.x, f.x, s0);
+                s1 = fma(e.y, f.y, s1);
+            }
+            s0 += s1;
+            const unsigned mask = 0xffu << (lane & 24);
+#pragma unroll
+            for (int o = 4; o > 0; o >>= 1) s0 += __shfl_xor_sync(mask, s0, o);
+            if (t % 8 == 0) u[q] = s0 * scale;
+            if (!second) break;
+        }
+        __syncthreads();
+        const int buffer = turn & 1;
+        const uint32_t bar = smem_u32(&bars[buffer]);
+        if (t == 0) mbar_arrive_expect_tx(bar, (uint32_t)(R * npad * sizeof(double)));
+        if (p < P) {
+            double2 s = make_double2(0.0, 0.0);
+            int off = off0, step = step0;
+#pragma unroll 4
+            for (int q = q0; q < rows; q += P) {   // the rows from the diagonal on
+                const double2 e = *reinterpret_cast<const double2*>(Ws + off);
+                const double uq = u[q];
+                s.x = fma(e.x, uq, s.x);
+                s.y = fma(e.y, uq, s.y);
+                off += step;
+                step += grow;
+            }
+            *reinterpret_cast<double2*>(parts + p * npad + 2 * c) = s;
+        }
+        __syncthreads();
+        if (p < min(lots, R)) {   // two columns to every lots-th block
+            double2 s = *reinterpret_cast<const double2*>(parts + 2 * c);
+#pragma unroll
+            for (int k = 1; k < kMaxParts; ++k)
+                if (k < P) {
+                    const double2 e = *reinterpret_cast<const double2*>(parts + k * npad + 2 * c);
+                    s.x += e.x;
+                    s.y += e.y;
+                }
+            const uint32_t dst = mine + buffer * (uint32_t)(R * npad * sizeof(double));
+#pragma unroll 1
+            for (int b = p; b < R; b += lots) send(in_block(dst, b), in_block(bar, b), s);
+        }
+        if (t < half) {
+            const uint32_t parity = (turn >> 1) & 1;
+            if (!late && !arrived(bar, parity)) {
+                const long long t0 = clock64();
+                while (!arrived(bar, parity))
+                    if (clock64() - t0 > kGridWaitCycles) {
+                        late = true;
+                        break;
+                    }
+            }
+            const double* from = shares + buffer * R * npad + 2 * t;
+            v = make_double2(0.0, 0.0);
+#pragma unroll
+            for (int b = 0; b < R; ++b) {
+                const double2 e = *reinterpret_cast<const double2*>(from + b * npad);
+                v.x += e.x;
+                v.y += e.y;
+            }
+            *reinterpret_cast<double2*>(x + 2 * t) = v;
+        }
+    };
+    double sum = 0.0, before = 0.0, scale = 1.0;
+#pragma unroll 1
+    for (int turn = 0; turn <= a.iters; ++turn) {
+        pass(scale, turn);
+        if (turn == 0) {
+            if (t < half) {
+                if (r == 0) {
+                    *reinterpret_cast<double2*>(a.alpha64 + (size_t)g * npad + 2 * t) = v;
+                    *reinterpret_cast<float2*>(a.alpha32 + (size_t)g * npad + 2 * t) = make_float2((float)v.x, (float)v.y);
+                }
+                auto start = [&](int j) { return j < n ? 1.0 + 0.37 * ((j * 2654435761u >> 16) & 0xff) / 255.0 : 0.0; };
+                v = make_double2(start(2 * t), start(2 * t + 1));
+                *reinterpret_cast<double2*>(x + 2 * t) = v;
+            }
+            if (a.iters == 0) break;
+        }
+        // 2^-e for the largest exponent e in x: a factor that keeps the iteration in range, without rounding and in a
+        // fraction of the time of a norm, its root and the division
+        const int top = __reduce_max_sync(0xffffffffu, max(__double2hiint(fabs(v.x)), __double2hiint(fabs(v.y))));
+        if (lane == 0) warp_tops[warp] = top;
+        if (turn + 1 >= a.iters) {
+            before = sum;
+            sum = total(fma(v.x, v.x, v.y * v.y));
+        } else {
+            __syncthreads();
+        }
+        if (turn < a.iters) {
+            const int e = __reduce_max_sync(0xffffffffu, warp_tops[lane % (kClusterThreads / 32)]) >> 20;
+            scale = e == 0 ? 1.0 : __hiloint2double(max(2046 - e, 0) << 20, 0);
+        }
+    }
+    // the growth of the last pass estimates |W|_2^2 from below; 1.5 covers slow convergence
+    if (a.iters > 0 && r == 0 && t == 0) a.wnorm[g] = before > 0.0 ? 1.5 * sqrt(sqrt(sum) / (sqrt(before) * scale)) : 0.0;
+    if (late) atomicOr(a.status, DEV_TIMEOUT);
+    cluster.sync();   // no block leaves while another may still write to it
 }
 
 __global__ void __launch_bounds__(kThreads, 2) weights_kernel(const WeightArgs a)
@@ -347,12 +470,29 @@ r3_status_t weights_device(const WeightProblem& p, double* scratch, unsigned* ba
     a.status = status;
     int sms = 148;
     R3_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device));
-    if (p.npad <= kSmallRows) {
-        const size_t small = sizeof(double) * ((size_t)p.npad * (p.npad + 2) + std::min(kSmallParts * p.npad, kSmallThreads));
-        a.team = 1;
-        R3_CUDA_TRY(cudaFuncSetAttribute(weights_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)(sizeof(double) * (kSmallRows * (kSmallRows + 2) + kSmallThreads))));
-        R3_LAUNCH(weights_small_kernel, std::min(p.batch, sms), kSmallThreads, small, stream, a);
+    // W in shared memory, as far as that goes (R = 2: 320 observations, R = 8: 544).  Eight blocks per GP while that leaves
+    // at most two on a multiprocessor, or where two do not hold W: one GP of 300 44 us (R = 2: 86, teams: 93), 64 of 300
+    // 201 us (R = 2: 88, teams: 238), 64 of 512 348 us (teams: 479).  Weights alone take one pass, for which loading W
+    // pays less: with more than 320 observations the team has them sooner if every GP gets a full one (8 of 512: 15 us, R = 8: 18).
+    const int resident2 = 2 * sms, R = 8 * p.batch <= resident2 || cluster_smem(p.npad, 2) > kClusterSmem ? 8 : 2;
+    const bool full_teams = p.batch * (p.npad / kCols) <= resident2;
+    if (cluster_smem(p.npad, R) <= kClusterSmem && (a.iters > 0 || p.npad <= 320 || !full_teams)) {
+        auto kernel = R == 8 ? weights_cluster_kernel<8> : weights_cluster_kernel<2>;
+        R3_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kClusterSmem));
+        cudaLaunchConfig_t cfg = {};
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = R;
+        attr[0].val.clusterDim.y = 1;
+        attr[0].val.clusterDim.z = 1;
+        cfg.gridDim = dim3(R * p.batch);
+        cfg.blockDim = dim3(cluster_threads(p.npad));
+        cfg.dynamicSmemBytes = cluster_smem(p.npad, R);
+        cfg.stream = stream;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        R3_CUDA_TRY(cudaLaunchKernelEx(&cfg, kernel, a));
+        ++g_launches;
         return R3_OK;
     }
     const size_t smem = sizeof(double) * 2 * p.npad;

@@ -39,3 +39,13 @@ def test_duplicated_row_without_noise_is_not_positive_definite(n, twin):
     with pytest.raises(b.R3Error) as e:
         b.r3_gp_fit(dev(g["X"]), dev(g["y"]), g["ell"], g["sf2"], np.zeros(1, np.float32))
     assert e.value.status == 3 and f"pivot {n - 1} " in str(e.value)
+
+
+@pytest.mark.parametrize("batch,n", [(1, 31), (2, 129), (40, 33), (40, 320), (40, 321), (1, 544), (1, 545)])
+def test_weights_where_their_split_changes(batch, n):
+    """One GP or many, around the history lengths at which W stops fitting the shared memory of two and of eight blocks: the
+    weights (check_handle) and, through the scores, the norm estimate."""
+    g = problem(2500 + n, batch, n, 4, 40)
+    gp = b.r3_gp_fit(dev(g["X"]), dev(g["y"]), g["ell"], g["sf2"], g["sn2"])
+    check_scoring(gp, g, check_handle(gp, g, n))
+    gp.close()
