@@ -99,12 +99,14 @@ __device__ __forceinline__ bool misses_contract(float mu, float sd, float dmu, f
 }
 
 // One block looks at the first `rows` candidates (GP after GP) of a pool that the engine has scored in its cheaper form:
-// mode <- 1 when more than one in 32 of them would have to be recomputed, 0 otherwise.
-__global__ void __launch_bounds__(1024) pilot_kernel(const GuardArgs a, long long rows, int* __restrict__ mode)
+// mode <- 1 when more than one in 32 of them would have to be recomputed, 0 otherwise.  Clears the guard's counters.
+__global__ void __launch_bounds__(1024) pilot_kernel(const GuardArgs a, long long rows, int* __restrict__ mode, int* __restrict__ zero,
+                                                     int zeros)
 {
     __shared__ unsigned top_s;
     __shared__ int count_s;
     const int t = threadIdx.x;
+    for (int i = t; i < zeros; i += 1024) zero[i] = 0;
     if (t == 0) {
         top_s = 0u;
         count_s = 0;
@@ -588,7 +590,7 @@ r3_status_t guard_pilot(r3_gp* gp, long long m, long long rows, const GuardBuffe
     a.m = m;
     a.mu = const_cast<float*>(mu); a.sigma = const_cast<float*>(sigma); a.ei = const_cast<float*>(ei);   // only read
     a.err_mu = b.err_mu; a.err_q = b.err_q;
-    R3_LAUNCH(pilot_kernel, 1, 1024, 0, stream, a, rows, b.mode);
+    R3_LAUNCH(pilot_kernel, 1, 1024, 0, stream, a, rows, b.mode, b.count, guard_zero_ints(gp));
     return R3_OK;
 }
 
