@@ -8,10 +8,13 @@
 //   L(i,j), i > j   A = K(i,j) - sum_{k<j} L(i,k) L(j,k)^T, then A L(j,j)^-T by forward substitution
 //   L(j,j)          the same sum, factored in shared memory; W(j,j) = L(j,j)^-1 follows
 //   W(i,c), i > c   -W(i,i) sum_{c<=k<i} L(i,k) W(k,c)
-// Blocks draw tasks from a ticket counter in the order: column 0 of L, row 0 of W, column 1 of L, row 1 of W, ...  A
-// task depends only on tasks before it, all blocks are resident, and a block works its tasks off one by one, so some
-// block can always go on.  Progress is one counter per row of L (its tiles finish from left to right) and one per
-// column of W (from top to bottom); a task adds up the products whose operands are there and waits for the next.
+// Blocks draw tasks from a ticket counter in the order: for every j the diagonal tile of column j of L, row j - 1 of W,
+// the rest of column j.  A task depends only on tasks before it, all blocks are resident, and a block works its tasks off
+// one by one, so some block can always go on.  The row of W is work for the blocks while the diagonal tile is factored (64
+// GPs of 512: 515 to 473 us, one of 1000 336 to 305 us against row j after column j; with L(j+1,j) and L(j+1,j+1) before
+// the rest of column j 2048 observations gain 9 % and 64 GPs of 512 lose 3 %).  Progress is one counter per row of L (its
+// tiles finish from left to right) and one per column of W (from top to bottom); a task adds up the products whose
+// operands are there and waits for the next.
 // A tile of L is handed out in halves of 32 columns: the left half of a column's tiles is solved, stored and multiplied
 // while one warp factors the diagonal tile's second panel (300 observations: 118 -> 93 us; 1000: fit 621 -> 552 us).
 // So a tile is written once and read as an operand, nothing is updated in place, and the factor's critical path --
@@ -22,8 +25,8 @@
 // ill-conditioned factor, and the log-determinant of noise-free smooth data came out wrong in the third digit.)
 //
 // Bound: FP64 rate for long histories, the chain of diagonal blocks for short ones.  One GP of 4096 observations (64
-// features): 3.0 ms, 31 TFLOP/s of FP64 without the exponentials (a sequence of 290 launches with 4x4 register tiles and
-// recursive doubling for the inverse: 7.2 ms); 300 observations 0.09 ms (0.41 ms); 64 GPs of 512 0.60 ms (1.26 ms).
+// features): 2.9 ms, 32 TFLOP/s of FP64 without the exponentials (a sequence of 290 launches with 4x4 register tiles and
+// recursive doubling for the inverse: 7.2 ms); 300 observations 0.09 ms (0.41 ms); 64 GPs of 512 0.47 ms (1.26 ms).
 // An append of 128 to 3968 (it was triangular products, a Schur complement and their corrections): 0.6 ms (2.0 ms).
 #include <algorithm>
 
@@ -49,7 +52,7 @@ struct FactorArgs {
     int *wprog;                     // [batch][T] one past the last finished half tile of each column of W
     unsigned* ticket;
     int* status;
-    int first[kMaxTiles + 1];       // tasks per GP before step j
+    int first[kMaxTiles + 2];       // tasks per GP before step j
 };
 
 __device__ __forceinline__ int load_acquire_int(const int* p) { return (int)load_acquire(reinterpret_cast<const unsigned*>(p)); }
@@ -510,7 +513,7 @@ __global__ void __launch_bounds__(kThreads, 2) factor_kernel(const __grid_consta
     double* tile1 = tile0 + TB * kLd;
     const int t = threadIdx.x, w = t / 32, l = t % 32, wm = (w % 4) * 16, wn = (w / 4) * 32;
     const int npad = a.npad, T = a.T;
-    const int total = a.first[T] * a.batch;
+    const int total = a.first[T + 1] * a.batch;
     auto publish = [&](int* p, int v) {   // the tile has been stored by all threads
         __syncthreads();
         if (t == 0) store_release_int(p, v);   // (a release covers what the barrier has made this thread see)
@@ -526,20 +529,20 @@ __global__ void __launch_bounds__(kThreads, 2) factor_kernel(const __grid_consta
         __syncthreads();
         const int task = sh.task;
         if (task >= total) return;
-        int lo = 0, hi = T - 1;   // the step: last j with first[j] * batch <= task
+        int lo = 0, hi = T;   // the step: last j with first[j] * batch <= task
         while (lo < hi) {
             const int mid = (lo + hi + 1) / 2;
             if (a.first[mid] * a.batch <= task) lo = mid;
             else hi = mid - 1;
         }
-        const int j = lo, rest = task - a.first[j] * a.batch;
-        const int top = max(j, a.i0), ncol = T - top;   // tiles of column j still to be made, per GP
+        // step j: the diagonal tiles of column j, row j - 1 of W, the rest of column j (all GPs' first tiles, then their next)
+        const int j = lo, at = (task - a.first[j] * a.batch) / a.batch, g = (task - a.first[j] * a.batch) % a.batch;
+        const int diag = j >= a.i0 && j < T ? 1 : 0, wrow = j > a.i0 ? j - 1 : 0;
         double* Lg;
         double* Wg;
         double c[2][4][2] = {};
-        if (rest < ncol * a.batch) {
-            // tile by tile down the column (all GPs' diagonal tiles first)
-            const int i = top + rest / a.batch, g = rest % a.batch;
+        if (at < diag || at >= diag + wrow) {
+            const int i = at < diag ? j : max(j + 1, a.i0) + at - diag - wrow;
             int* lp = a.lprog + (size_t)g * T;
             Lg = a.L + (size_t)g * npad * npad;
             Wg = a.W + (size_t)g * npad * npad;
@@ -591,7 +594,7 @@ __global__ void __launch_bounds__(kThreads, 2) factor_kernel(const __grid_consta
                 zero_tile(Wg, npad, j, i);
             }
         } else {
-            const int r2 = rest - ncol * a.batch, i = j, col = r2 / a.batch, g = r2 % a.batch;
+            const int i = j - 1, col = at - diag;
             Lg = a.L + (size_t)g * npad * npad;
             Wg = a.W + (size_t)g * npad * npad;
             int* wp = a.wprog + (size_t)g * T;
@@ -678,8 +681,8 @@ r3_status_t factor_device(const FactorProblem& p, void* scratch, int extra_ints,
     a.wprog = a.lprog + (size_t)p.batch * a.T;
     a.status = status;
     a.first[0] = 0;
-    for (int j = 0; j < a.T; ++j)   // column j of L below the finished rows, then row j of W
-        a.first[j + 1] = a.first[j] + (a.T - std::max(j, a.i0)) + (j >= a.i0 ? j : 0);
+    for (int j = 0; j <= a.T; ++j)   // column j of L below the finished rows, row j - 1 of W
+        a.first[j + 1] = a.first[j] + (j < a.T ? a.T - std::max(j, a.i0) : 0) + (j > a.i0 ? j - 1 : 0);
     const size_t xcount = (size_t)p.batch * p.n * p.d;
     const int zeros = (int)(factor_scratch_bytes(p.batch, p.npad) / sizeof(int)) + extra_ints;
     const unsigned gx = (unsigned)std::max<size_t>(1, std::min<size_t>(148, (xcount + 2047) / 2048) / p.batch);
@@ -688,7 +691,7 @@ r3_status_t factor_device(const FactorProblem& p, void* scratch, int extra_ints,
     int sms = 148;
     R3_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device));
     R3_CUDA_TRY(cudaFuncSetAttribute(factor_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFactorSmem));
-    const long long tasks = (long long)a.first[a.T] * a.batch;
+    const long long tasks = (long long)a.first[a.T + 1] * a.batch;
     const unsigned grid = (unsigned)std::min<long long>(tasks, 2ll * sms);
     void* params[] = {&a};
     R3_CUDA_TRY(cudaLaunchCooperativeKernel((const void*)factor_kernel, dim3(grid), dim3(kThreads), params, kFactorSmem, stream));
