@@ -7,8 +7,9 @@
 // Everything in FP64.  A block forms a 64 x 64 tile of the lower triangle of K^-1 on the FP64 tensor path and, with the
 // tile still in registers, its share of every pair sum; M is never stored.  The sums are reduced in a fixed order (per-tile
 // partial sums, then one warp per derivative adds them), so results repeat bit for bit.
-// Bound: FP64 rate, n^3/3 multiply-adds for K^-1 and 7 n^2 d / 2 operations for the pairs.  64 GPs of 512 observations, 32
-// features: 0.35 ms; K^-1 by 4x4 register tiles, M written and read back, and a warp sum per feature and pair tile: 0.79 ms.
+// Bound: FP64 rate, n^3/3 multiply-adds for K^-1 and 6 n^2 d / 2 operations for the pairs (a feature's scale is applied to
+// its sum, not to every pair).  64 GPs of 512 observations, 32 features: 0.34 ms; K^-1 by 4x4 register tiles, M written and
+// read back, and a warp sum per feature and pair tile: 0.79 ms.
 #include <math.h>
 
 #include <algorithm>
@@ -199,11 +200,11 @@ __global__ void __launch_bounds__(kThreads, 2) lml_tile_kernel(const LmlArgs a)
                     for (int j = 0; j < 4; ++j)
 #pragma unroll
                         for (int h = 0; h < 2; ++h) {
-                            const double u = (p - q[j][h]) * s;
-                            acc = fma(c[i][j][h], u * u, acc);
+                            const double u = p - q[j][h];
+                            acc = fma(c[i][j][h] * u, u, acc);
                         }
                 }
-                v[b] = acc;
+                v[b] = acc * (s * s);   // the scale of u_j^2, once per sum
             }
 #pragma unroll
             for (int o = 4; o > 0; o >>= 1) {
