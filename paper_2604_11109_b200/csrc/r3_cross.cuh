@@ -70,16 +70,22 @@ __device__ __forceinline__ void cross_tile(int n, int d, int npad, const float* 
                 }
         }
     }
+#pragma unroll 1
+    for (int u = 0; u < U; ++u) {   // not unrolled: four square roots and exponentials at a time are enough to overlap
+        double part = 0.0, ru[4];
 #pragma unroll
-    for (int u = 0; u < U; ++u) {
-        double part = 0.0;
+        for (int v = 0; v < 4; ++v) {
+            ru[v] = r2[0][v];
+#pragma unroll
+            for (int uu = 1; uu < U; ++uu) ru[v] = uu == u ? r2[uu][v] : ru[v];
+        }
 #pragma unroll
         for (int v = 0; v < 4; ++v) {
             const int k = k0 + tx + 16 * v;
             if (k >= npad) continue;
             double kv = 0.0;
             if (k < n) {
-                const double sq = sqrt(5.0) * sqrt(r2[u][v]);
+                const double sq = sqrt(5.0) * sqrt(ru[v]);
                 kv = sf2 * fma(sq, fma(sq, 1.0 / 3.0, 1.0), 1.0) * exp(-sq);
                 if (alpha) part = fma(kv, alpha[k], part);
             }

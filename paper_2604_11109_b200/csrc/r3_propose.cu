@@ -12,12 +12,13 @@
 // incumbent) only drops: a candidate outside the R best of the first scoring can be picked only if some
 // pick's EI falls below the (R+1)-th initial EI.  So: one full scoring with its top-(R+1), then the q picks on the
 // shortlist alone, in FP64, in two kernels:
-//   build_kernel  (cooperative) k* of the shortlist, V = W k*, C0 for all its pairs, as tiles on the FP64 tensor path;
+//   build_kernel  (cooperative) k* of the shortlist and k(z, z') of its pairs, which depend on nothing and are made together;
+//                 then V = W k*; then C0 = k - V V^T; the products as tiles on the FP64 tensor path;
 //   pick_kernel   (one cluster per GP) the q picks: a candidate per thread and part, the columns c_u in shared memory, one
 //                 cluster barrier per pick.
 // Bound: R n^2 / 2 + R^2 n / 2 FP64 multiply-adds, then the latency of a pick.  One GP of 4096 observations, 1023
 // shortlisted, 128 picks: 6.1 ms as 259 launches (R n multiply-adds per pick), 1.8 ms now; 72 observations, 256
-// shortlisted, 8 picks: 100 us in 19 launches and 62 us.
+// shortlisted, 8 picks: 100 us in 19 launches and 46 us (62 us with k(z, z') made beside V V^T, after the second barrier).
 #include <cooperative_groups.h>
 
 #include <algorithm>
@@ -68,15 +69,32 @@ __global__ void __launch_bounds__(kCrossThreads, 2) build_kernel(const ProposeAr
     const int t = threadIdx.x, w = t / 32, l = t % 32, wm = (w % 4) * 16, wn = (w / 4) * 32;
     const int npad = a.npad, R = a.R, RT = (R + 63) / 64, NT = (npad + 63) / 64;
     unsigned target = 0;
-    // ---- k* and the partial means
-    for (int item = blockIdx.x; item < a.B * RT * NT; item += gridDim.x) {
-        const int g = item / (RT * NT), rt = item % (RT * NT) / NT, kb = item % NT;
-        double* Ks = a.Ks + ((size_t)g * R + rt * 64) * npad;
-        cross_tile<64>(
-            a.n, a.d, npad, a.ell + (size_t)g * a.d, (double)a.sf2[g], a.alpha + (size_t)g * npad,
-            [&](int r) { return short_row(a, g, rt * 64 + r); }, [&](int k) { return a.X + ((size_t)g * a.n + k) * a.d; }, kb,
-            smem, [&](int c, int k, double v) { if (rt * 64 + c < R) Ks[(size_t)c * npad + k] = v; },
-            [&](int c, double s) { if (rt * 64 + c < R) a.mupart[((size_t)g * R + rt * 64 + c) * NT + kb] = s; });
+    // ---- k* and the partial means; k(z, z') of the shortlist's own pairs, tiles (ta, tb) of the lower triangle
+    const int pairs = RT * (RT + 1) / 2, kstar = a.B * RT * NT;
+    auto pair_tile = [&](int p, int& ta, int& tb) {
+        ta = 0;
+        while ((ta + 1) * (ta + 2) / 2 <= p) ++ta;
+        tb = p - ta * (ta + 1) / 2;
+    };
+    for (int item = blockIdx.x; item < kstar + (a.q > 1 ? a.B * pairs : 0); item += gridDim.x) {
+        if (item < kstar) {
+            const int g = item / (RT * NT), rt = item % (RT * NT) / NT, kb = item % NT;
+            double* Ks = a.Ks + ((size_t)g * R + rt * 64) * npad;
+            cross_tile<64>(
+                a.n, a.d, npad, a.ell + (size_t)g * a.d, (double)a.sf2[g], a.alpha + (size_t)g * npad,
+                [&](int r) { return short_row(a, g, rt * 64 + r); }, [&](int k) { return a.X + ((size_t)g * a.n + k) * a.d; }, kb,
+                smem, [&](int c, int k, double v) { if (rt * 64 + c < R) Ks[(size_t)c * npad + k] = v; },
+                [&](int c, double s) { if (rt * 64 + c < R) a.mupart[((size_t)g * R + rt * 64 + c) * NT + kb] = s; });
+        } else {
+            const int g = (item - kstar) / pairs;
+            int ta, tb;
+            pair_tile((item - kstar) % pairs, ta, tb);
+            double* C0 = a.C0 + (size_t)g * R * R;
+            cross_tile<64>(
+                R, a.d, R, a.ell + (size_t)g * a.d, (double)a.sf2[g], nullptr, [&](int r) { return short_row(a, g, ta * 64 + r); },
+                [&](int k) { return short_row(a, g, k); }, tb, smem,
+                [&](int r, int k, double v) { if (ta * 64 + r < R) C0[(size_t)(ta * 64 + r) * R + k] = v; }, [](int, double) {});
+        }
     }
     if (!grid_barrier(a.barrier, target, a.status)) return;
     // ---- V[r][i] = sum_k Ks[r][k] W[i][k], the longest rows of W first, and the partial sums of squares
@@ -107,36 +125,36 @@ __global__ void __launch_bounds__(kCrossThreads, 2) build_kernel(const ProposeAr
     }
     if (a.q < 2) return;
     if (!grid_barrier(a.barrier, target, a.status)) return;
-    // ---- C0 = k(z, z') - V V^T, tiles of the lower triangle, written on both sides
-    const int pairs = RT * (RT + 1) / 2;
+    // ---- C0 = k(z, z') - V V^T, written on both sides
     for (int item = blockIdx.x; item < a.B * pairs; item += gridDim.x) {
-        const int g = item / pairs, p = item % pairs;
-        int ta = 0;
-        while ((ta + 1) * (ta + 2) / 2 <= p) ++ta;
-        const int tb = p - ta * (ta + 1) / 2;
-        double c[2][4][2] = {};
+        const int g = item / pairs;
+        int ta, tb;
+        pair_tile(item % pairs, ta, tb);
         const double* Vg = a.V + (size_t)g * R * npad;
-        nt_tile(Vg + (size_t)ta * 64 * npad, R - ta * 64, Vg + (size_t)tb * 64 * npad, R - tb * 64, npad, npad, smem, c);
-        double* tile = reinterpret_cast<double*>(smem + 20 * 1024);   // [64][65], behind the staged coordinates (17 KB)
+        double* C0 = a.C0 + (size_t)g * R * R;
+        double c[2][4][2] = {}, k0[2][4][2];
 #pragma unroll
         for (int i = 0; i < 2; ++i)
 #pragma unroll
             for (int j = 0; j < 4; ++j)
 #pragma unroll
-                for (int h = 0; h < 2; ++h) tile[(wm + 8 * i + l / 4) * 65 + wn + 8 * j + 2 * (l % 4) + h] = c[i][j][h];
-        double* C0 = a.C0 + (size_t)g * R * R;
-        cross_tile<64>(
-            R, a.d, R, a.ell + (size_t)g * a.d, (double)a.sf2[g], nullptr, [&](int r) { return short_row(a, g, ta * 64 + r); },
-            [&](int k) { return short_row(a, g, k); }, tb, smem,
-            [&](int r, int k, double v) {
-                const int row = ta * 64 + r;
-                if (row >= R) return;
-                v -= tile[r * 65 + k - tb * 64];
-                C0[(size_t)row * R + k] = v;
-                if (ta != tb) C0[(size_t)k * R + row] = v;
-            },
-            [](int, double) {});
-        __syncthreads();
+                for (int h = 0; h < 2; ++h) {
+                    const int row = ta * 64 + wm + 8 * i + l / 4, col = tb * 64 + wn + 8 * j + 2 * (l % 4) + h;
+                    k0[i][j][h] = row < R && col < R ? __ldcg(C0 + (size_t)row * R + col) : 0.0;
+                }
+        nt_tile(Vg + (size_t)ta * 64 * npad, R - ta * 64, Vg + (size_t)tb * 64 * npad, R - tb * 64, npad, npad, smem, c);
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const int row = ta * 64 + wm + 8 * i + l / 4, col = tb * 64 + wn + 8 * j + 2 * (l % 4) + h;
+                    if (row >= R || col >= R) continue;
+                    const double v = k0[i][j][h] - c[i][j][h];
+                    C0[(size_t)row * R + col] = v;
+                    if (ta != tb) C0[(size_t)col * R + row] = v;
+                }
     }
 }
 
@@ -335,8 +353,8 @@ r3_status_t propose_shortlist(r3_gp* gp, const float* Xcand, long long m, const 
     int sms = 148;
     R3_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, gp->device));
     R3_CUDA_TRY(cudaFuncSetAttribute(build_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCrossStageBytes));
-    const long long items = (long long)B * ((R + 63) / 64) * NT;
-    const unsigned grid = (unsigned)std::min<long long>(2ll * sms, std::max<long long>(items, (long long)B * 4));
+    const long long RT = (R + 63) / 64, items = B * (RT * NT + RT * (RT + 1) / 2);   // of the first phase, the widest
+    const unsigned grid = (unsigned)std::min<long long>(2ll * sms, items);
     void* params[] = {&a};
     R3_CUDA_TRY(cudaLaunchCooperativeKernel((const void*)build_kernel, dim3(grid), dim3(kCrossThreads), params, kCrossStageBytes,
                                             stream));
