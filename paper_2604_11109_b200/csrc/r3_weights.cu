@@ -372,7 +372,11 @@ __global__ void __launch_bounds__(kClusterThreads, 1) weights_cluster_kernel(con
     }
     // the growth of the last pass estimates |W|_2^2 from below; 1.5 covers slow convergence
     if (a.iters > 0 && r == 0 && t == 0) a.wnorm[g] = before > 0.0 ? 1.5 * sqrt(sqrt(sum) / (sqrt(before) * scale)) : 0.0;
-    if (late) atomicOr(a.status, DEV_TIMEOUT);
+    if (late) {   // what is still on its way to this block lands before anyone leaves
+        atomicOr(a.status, DEV_TIMEOUT);
+        const long long t0 = clock64();
+        while (clock64() - t0 < 2000000) __nanosleep(1000);
+    }
     cluster.sync();   // no block leaves while another may still write to it
 }
 
