@@ -164,7 +164,7 @@ r3_status_t state_fit(r3_gp* gp, r3_fit_state& s, int rows_done, bool full, bool
     const bool staged = lml && image == gp->stage_h && bytes + lml_bytes <= kStageBytes;
     if (lml) {
         double* out = nullptr;
-        st = lml_enqueue(s, doubles + wdoubles, &out, stream);
+        st = lml_enqueue(s, doubles + wdoubles, &out, s.fit_status, stream);
         if (st != R3_OK) return done(st);
         TRY_DONE(cudaMemcpyAsync(staged ? (void*)(image + bytes) : (void*)lml, out, lml_bytes, cudaMemcpyDeviceToHost, stream));
     }
@@ -175,6 +175,10 @@ r3_status_t state_fit(r3_gp* gp, r3_fit_state& s, int rows_done, bool full, bool
     const int* fs = mirror(s, s.fit_status, image);
     *bits = fs[0];
     if (pivot) *pivot = fs[1];
+    if (fs[0] & DEV_BOUNDS) {
+        set_error("bounds-checking build: an index check of the fit failed (source line %d of its kernel's file)", fs[2]);
+        return done(R3_ERR_CUDA);
+    }
     if (fs[0] & DEV_TIMEOUT) {
         set_error("a bounded device-side wait of the fit ran out");
         return done(R3_ERR_DEVICE_TIMEOUT);

@@ -289,7 +289,7 @@ r3_status_t topk_device(const float* ei, int batch, long long m, int k, int* idx
 
 // log marginal likelihood and gradient (r3_lml.cu): out_h host [batch][d + 3]
 size_t lml_scratch_doubles(const r3_fit_state& s);
-r3_status_t lml_enqueue(const r3_fit_state& s, double* scratch, double** out, cudaStream_t stream);
+r3_status_t lml_enqueue(const r3_fit_state& s, double* scratch, double** out, int* status, cudaStream_t stream);
 r3_status_t lml_device(r3_gp* gp, double* out_h, cudaStream_t stream);
 
 // greedy batch proposal on a shortlist (r3_propose.cu)

@@ -34,6 +34,7 @@ struct LmlArgs {
     int n, d, npad, tiles;
     double* partial;   // [batch][tiles][d + 2]: the features' sums, sum w M Kf, trace
     double* out;       // [batch][d + 3]
+    int* status;       // status words, for the index checks of the bounds-checking build
 };
 
 __global__ void __launch_bounds__(kThreads, 2) lml_tile_kernel(const LmlArgs a)
@@ -58,9 +59,11 @@ __global__ void __launch_bounds__(kThreads, 2) lml_tile_kernel(const LmlArgs a)
 #pragma unroll
             for (int it = 0; it < 2; ++it) {
                 const int e = t + kThreads * it, r = e / 32, q = e % 32;
-                const bool ok = i0 + 2 * q < npad;      // j0 <= i0: its columns exist where these do
-                cp_async16(sA + (s * 16 + r) * kLd + 2 * q, Wg + (size_t)(r0 + r) * npad + (ok ? i0 + 2 * q : 0), ok);
-                cp_async16(sB + (s * 16 + r) * kLd + 2 * q, Wg + (size_t)(r0 + r) * npad + j0 + 2 * q);
+                // the last tile of a row or column may have 32 columns only
+                const bool oki = i0 + 2 * q < npad, okj = j0 + 2 * q < npad;
+                const size_t row = (size_t)R3_IDX(r0 + r, npad, a.status) * npad;
+                cp_async16(sA + (s * 16 + r) * kLd + 2 * q, Wg + row + R3_IDX(oki ? i0 + 2 * q : 0, npad - 1, a.status), oki);
+                cp_async16(sB + (s * 16 + r) * kLd + 2 * q, Wg + row + R3_IDX(okj ? j0 + 2 * q : 0, npad - 1, a.status), okj);
             }
         };
 #pragma unroll
@@ -102,8 +105,8 @@ __global__ void __launch_bounds__(kThreads, 2) lml_tile_kernel(const LmlArgs a)
 #pragma unroll
         for (int e = 0; e < 8; ++e) {
             const int gi = i0 + q + 8 * e, gj = j0 + q + 8 * e;
-            vi[e] = (gi < n && c0 + f < d) ? __ldg(Xg + (size_t)gi * d + c0 + f) : 0.f;
-            vj[e] = (gj < n && c0 + f < d) ? __ldg(Xg + (size_t)gj * d + c0 + f) : 0.f;
+            vi[e] = (gi < n && c0 + f < d) ? __ldg(Xg + R3_IDX((size_t)gi * d + c0 + f, (size_t)n * d, a.status)) : 0.f;
+            vj[e] = (gj < n && c0 + f < d) ? __ldg(Xg + R3_IDX((size_t)gj * d + c0 + f, (size_t)n * d, a.status)) : 0.f;
         }
 #pragma unroll
         for (int e = 0; e < 8; ++e) {
@@ -225,7 +228,7 @@ __global__ void __launch_bounds__(kThreads, 2) lml_tile_kernel(const LmlArgs a)
         if (t < cmax || (c0 == 0 && t >= 32 && t < 34)) {
             double s = 0.0;
             for (int ww = 0; ww < 8; ++ww) s += red[ww][t];
-            out[t < 32 ? c0 + t : d + t - 32] = s;
+            out[R3_IDX(t < 32 ? c0 + t : d + t - 32, d + 2, a.status)] = s;
         }
         __syncthreads();
     }
@@ -265,9 +268,10 @@ int lml_tiles(int n) { return ((n + kTile - 1) / kTile) * ((n + kTile - 1) / kTi
 size_t lml_scratch_doubles(const r3_fit_state& s) { return (size_t)s.batch * ((size_t)lml_tiles(s.n) * (s.d + 2) + s.d + 3); }
 
 // Asynchronous: *out (device, inside scratch) becomes [batch][d + 3] = {lml, d/dlog ell_1..d, d/dlog sf2, d/dlog sn2}.
-r3_status_t lml_enqueue(const r3_fit_state& s, double* scratch, double** out, cudaStream_t stream)
+r3_status_t lml_enqueue(const r3_fit_state& s, double* scratch, double** out, int* status, cudaStream_t stream)
 {
     LmlArgs a;
+    a.status = status;
     a.X = s.X; a.ell = s.ell_d; a.sf2 = s.sf2_d; a.sn2 = s.sn2_d; a.y = s.y;
     a.W = s.W64; a.L = s.L64; a.alpha = s.alpha64;
     a.n = s.n; a.d = s.d; a.npad = s.npad;
@@ -293,7 +297,7 @@ r3_status_t lml_device(r3_gp* gp, double* out_h, cudaStream_t stream)
     };
     R3_CUDA_TRY(dev_malloc(&scratch, sizeof(double) * lml_scratch_doubles(*gp)));
     double* out = nullptr;
-    const r3_status_t st = lml_enqueue(*gp, scratch, &out, stream);
+    const r3_status_t st = lml_enqueue(*gp, scratch, &out, gp->status_d, stream);
     if (st != R3_OK) return done(st);
     cudaError_t e = cudaMemcpyAsync(out_h, out, sizeof(double) * (size_t)gp->batch * (gp->d + 3), cudaMemcpyDeviceToHost, stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(stream);

@@ -25,10 +25,19 @@ def test_small_cases_pass_under_the_bounds_checking_build():
     which = subprocess.run([sys.executable, "-c", "from paper_2604_11109_b200 import binding as b; b.load(); print(b.LIB_PATH)"],
                            cwd=ROOT, env=env, capture_output=True, text=True, timeout=300)
     assert which.stdout.strip().endswith("libr3gp_check.so"), which.stdout + which.stderr
-    sel = "small_cases or near_observations or random_shapes or paired or wait_that_runs_out or two_live"
-    r = subprocess.run([sys.executable, "-m", "pytest", os.path.join(ROOT, "tests", "test_gpu_parity.py"),
-                        os.path.join(ROOT, "tests", "test_gpu_failure_paths.py"), "-m", "gpu", "-x", "-q", "-k", sel,
-                        "-p", "no:cacheprovider"], cwd=ROOT, env=env, capture_output=True, text=True, timeout=1500)
+    run_checked(["test_gpu_parity.py", "test_gpu_failure_paths.py"],
+                "small_cases or near_observations or random_shapes or paired or wait_that_runs_out or two_live")
+
+
+def run_checked(files, sel):
+    env = dict(os.environ, R3_LIB_VARIANT="check")
+    r = subprocess.run([sys.executable, "-m", "pytest", *(os.path.join(ROOT, "tests", f) for f in files), "-m", "gpu", "-x",
+                        "-q", "-k", sel, "-p", "no:cacheprovider"], cwd=ROOT, env=env, capture_output=True, text=True,
+                       timeout=1500)
     tail = (r.stdout + r.stderr)[-3000:]
     assert r.returncode == 0, tail
     assert " passed" in r.stdout and "failed" not in r.stdout, tail
+
+
+def test_evidence_under_the_bounds_checking_build():
+    run_checked(["test_gpu_lml.py"], "random_problems or half_empty")

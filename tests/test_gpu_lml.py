@@ -98,3 +98,24 @@ def test_ill_conditioned_history_is_as_accurate_as_the_oracle(seed, n, d):
     err_lib, err_oracle = abs(lml[0] - ref), abs(v - ref)
     assert err_lib <= 4.0 * err_oracle + 1e-7 * abs(ref), (lml[0], v, ref)
     assert err_lib <= 2e-3 * abs(ref)
+
+
+@pytest.mark.parametrize("batch,n", [(1, 32), (2, 70), (1, 96), (3, 150), (1, 288)])
+def test_histories_whose_last_tile_is_half_empty(batch, n):
+    """The padded length is an odd multiple of 32, so the last 64 x 64 tile of K^-1 lacks its right and lower half.  In the
+    bounds-checking build r3_gp_check reports an operand copy that leaves the matrix."""
+    rng = np.random.default_rng(900 + n)
+    g = {
+        "X": rng.uniform(0, 1, (batch, n, 6)).astype(np.float32),
+        "y": rng.normal(0, 1, (batch, n)).astype(np.float32),
+        "ell": rng.uniform(0.3, 1.5, (batch, 6)).astype(np.float32),
+        "sf2": rng.uniform(0.5, 2.0, batch).astype(np.float32),
+        "sn2": rng.uniform(1e-3, 1e-1, batch).astype(np.float32),
+    }
+    check(g)
+    gp = b.r3_gp_fit(dev(g["X"]), dev(g["y"]), g["ell"], g["sf2"], g["sn2"])
+    b.r3_gp_lml(gp)
+    b.r3_gp_check(gp)
+    b.r3_gp_optimize(gp, max_evals=2, gtol=1e-6)   # the evaluation that a search for hyper-parameters makes
+    b.r3_gp_check(gp)
+    gp.close()
