@@ -489,6 +489,12 @@ unsigned long long r3_cached_bytes(void);
  */
 long long r3_test_fail_allocation(long long after);
 
+/*
+ * Testing aid: y[i] = p[i]^-1/2 as the factorisation computes the reciprocal roots of its pivots (device arrays [count]),
+ * so that its error can be compared with a bound.  Asynchronous on `cuda_stream`.
+ */
+r3_status_t r3_test_rsqrt(const double* p, double* y, long long count, void* cuda_stream);
+
 const char* r3_status_string(r3_status_t status);
 const char* r3_last_error(void);
 int r3_version(void);

@@ -71,6 +71,7 @@ SIGNATURES = {
     "r3_gp_set_wait_limit": (_i, [_vp, _ll]),
     "r3_gp_test_withhold": (_i, [_vp, _ll]),
     "r3_test_fail_allocation": (_ll, [_ll]),
+    "r3_test_rsqrt": (_i, [_vp, _vp, _ll, _vp]),
     "r3_gp_get_best": (_i, [_vp, _fp]),
     "r3_gp_set_best": (_i, [_vp, _fp]),
     "r3_gp_set_engine": (_i, [_vp, _i]),
@@ -385,6 +386,15 @@ def r3_gp_test_withhold(gp: GP, chunk: int):
 
 def r3_test_fail_allocation(after: int) -> int:
     return int(load().r3_test_fail_allocation(int(after)))
+
+
+def r3_test_rsqrt(p):
+    """Reciprocal roots of a float64 CUDA tensor as the factorisation computes them (testing aid)."""
+    import torch
+    p = p.contiguous()
+    y = torch.empty_like(p)
+    _check(load().r3_test_rsqrt(ctypes.c_void_p(p.data_ptr()), ctypes.c_void_p(y.data_ptr()), p.numel(), _stream()))
+    return y
 
 
 def r3_gp_tensor_info(gp: GP) -> dict:

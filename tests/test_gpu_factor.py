@@ -49,3 +49,21 @@ def test_weights_where_their_split_changes(batch, n):
     gp = b.r3_gp_fit(dev(g["X"]), dev(g["y"]), g["ell"], g["sf2"], g["sn2"])
     check_scoring(gp, g, check_handle(gp, g, n))
     gp.close()
+
+
+def test_reciprocal_roots_of_pivots():
+    """Relative error at most 2^-52: the last Newton step rounds the product h y (relative 2^-53, which enters halved) and the
+    new y (2^-53), and the steps leave 2^-84.  CUDA's own function may be off by one unit in the last place as well."""
+    rng = np.random.default_rng(17)
+    p = np.concatenate([np.exp(rng.uniform(np.log(1e-290), np.log(1e290), 400000)),   # every exponent
+                        rng.uniform(0.25, 4.0, 400000),                               # every mantissa of two binades
+                        2.0 ** rng.integers(-200, 200, 1000), 1.0 + np.arange(-64, 65) * 2.0 ** -52])
+    p1, s = rng.uniform(0.5, 2.0, 100000), rng.uniform(0.3, 0.7, 100000)
+    tail = 10.0 ** rng.uniform(-15, 0, 100000)
+    p = np.concatenate([p, p1 * (s * s / p1 + tail) - s * s])   # determinants of nearly singular pairs
+    p = p[p > 1e-300]
+    y = b.r3_test_rsqrt(dev(p)).cpu().numpy()
+    exact = 1.0 / np.sqrt(p.astype(np.longdouble))
+    assert float(np.abs(y / exact - 1.0).max()) <= 2.0 ** -52
+    assert float(np.abs(y / torch.rsqrt(dev(p)).cpu().numpy() - 1.0).max()) <= 2.0 ** -51
+    assert np.isnan(b.r3_test_rsqrt(dev(np.array([0.0, -1.0, np.nan, -np.inf]))).cpu().numpy()).all()
