@@ -70,6 +70,7 @@ SIGNATURES = {
     "r3_gp_check": (_i, [_vp, _vp]),
     "r3_gp_set_wait_limit": (_i, [_vp, _ll]),
     "r3_gp_test_withhold": (_i, [_vp, _ll]),
+    "r3_gp_test_stall": (_i, [_vp, _i, _ll]),
     "r3_test_fail_allocation": (_ll, [_ll]),
     "r3_test_rsqrt": (_i, [_vp, _vp, _ll, _vp]),
     "r3_gp_get_best": (_i, [_vp, _fp]),
@@ -382,6 +383,10 @@ def r3_gp_set_wait_limit(gp: GP, cycles: int):
 
 def r3_gp_test_withhold(gp: GP, chunk: int):
     _check(load().r3_gp_test_withhold(gp.handle, int(chunk)))
+
+
+def r3_gp_test_stall(gp: GP, where: int, cycles: int):
+    _check(load().r3_gp_test_stall(gp.handle, int(where), int(cycles)))
 
 
 def r3_test_fail_allocation(after: int) -> int:

@@ -105,6 +105,17 @@ static r3_status_t run_score(r3_gp* gp, const float* Xcand, long long m, float* 
     return score_simt(gp, Xcand, m, mu, sigma, ei, ws, ws_bytes, stream);
 }
 
+WaitRule wait_rule(r3_gp* gp, int where)
+{
+    WaitRule rule;
+    if (gp->stall_where == where) {
+        rule.cycles = gp->stall_cycles;
+        rule.withhold = 1;
+        gp->stall_where = -1;
+    }
+    return rule;
+}
+
 }  // namespace r3
 
 using namespace r3;
@@ -596,6 +607,17 @@ r3_status_t r3_gp_test_withhold(r3_gp_t* gp, long long chunk)
         return R3_ERR_UNSUPPORTED;
     }
     gp->withhold_w = chunk;
+    return R3_OK;
+}
+
+r3_status_t r3_gp_test_stall(r3_gp_t* gp, int where, long long cycles)
+{
+    if (!gp || where < 0 || where > STALL_WEIGHTS || cycles < 100000) {
+        set_error("r3_gp_test_stall: need a handle, where in [0, %d] and at least 100000 cycles", STALL_WEIGHTS);
+        return R3_ERR_INVALID_ARG;
+    }
+    gp->stall_where = where;
+    gp->stall_cycles = cycles;
     return R3_OK;
 }
 

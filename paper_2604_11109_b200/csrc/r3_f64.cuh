@@ -46,22 +46,22 @@ __device__ __forceinline__ unsigned load_acquire(const unsigned* p)
     return v;
 }
 
-// Barrier over `blocks` blocks (grid_barrier: all) of a cooperatively launched grid.  `counter` starts at zero and only grows; `target` is the
-// caller's running count.  Bounded like every device-side wait: after about two seconds the status word gets
+// Barrier over `blocks` blocks (grid_barrier: all) of a cooperatively launched grid.  `counter` starts at zero and only grows;
+// `target` is the caller's running count.  Bounded like every device-side wait: when it runs out the status word gets
 // DEV_TIMEOUT and false is returned, on which the block leaves the kernel.
-constexpr long long kGridWaitCycles = 4000000000ll;
-__device__ __forceinline__ bool team_barrier(unsigned* counter, unsigned& target, unsigned blocks, int* status)
+__device__ __forceinline__ bool team_barrier(unsigned* counter, unsigned& target, unsigned blocks, int* status,
+                                             const WaitRule& rule)
 {
     bool ok = true;
     __syncthreads();
     target += blocks;
     if (threadIdx.x == 0) {
         __threadfence();
-        atomicAdd(counter, 1u);
+        if (!(rule.withhold && blockIdx.x == 0)) atomicAdd(counter, 1u);
         if (load_acquire(counter) < target) {
             const long long t0 = clock64();
             while (load_acquire(counter) < target) {
-                if (clock64() - t0 > kGridWaitCycles) {
+                if (clock64() - t0 > rule.cycles) {
                     atomicOr(status, DEV_TIMEOUT);
                     ok = false;
                     break;
@@ -71,9 +71,9 @@ __device__ __forceinline__ bool team_barrier(unsigned* counter, unsigned& target
     }
     return __syncthreads_and(ok);
 }
-__device__ __forceinline__ bool grid_barrier(unsigned* counter, unsigned& target, int* status)
+__device__ __forceinline__ bool grid_barrier(unsigned* counter, unsigned& target, int* status, const WaitRule& rule = WaitRule())
 {
-    return team_barrier(counter, target, gridDim.x, status);
+    return team_barrier(counter, target, gridDim.x, status, rule);
 }
 
 }  // namespace r3

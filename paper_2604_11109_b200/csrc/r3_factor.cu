@@ -52,6 +52,7 @@ struct FactorArgs {
     int *wprog;                     // [batch][T] one past the last finished half tile of each column of W
     unsigned* ticket;
     int* status;
+    WaitRule wait;
     int first[kMaxTiles + 2];       // tasks per GP before step j
 };
 
@@ -61,8 +62,9 @@ __device__ __forceinline__ void store_release_int(int* p, int v)
     asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 
-// Waits (one thread) until *p >= want and returns what it saw; -1 when the wait ran out here or elsewhere.
-__device__ __forceinline__ int wait_progress(const int* p, int want, int* status)
+// Waits (one thread) until *p >= want and returns what it saw; -1 when the wait ran out.  Blocks whose operands never come
+// begin to wait within the time of the tasks that still can be done, so a failed factorisation costs that and one limit.
+__device__ __forceinline__ int wait_progress(const int* p, int want, int* status, const WaitRule& rule)
 {
     int v = load_acquire_int(p);
     if (v >= want) return v;
@@ -71,7 +73,7 @@ __device__ __forceinline__ int wait_progress(const int* p, int want, int* status
         __nanosleep(40);
         v = load_acquire_int(p);
         if (v >= want) return v;
-        if (clock64() - t0 > kGridWaitCycles) {
+        if (clock64() - t0 > rule.cycles) {
             atomicOr(status, DEV_TIMEOUT);
             return -1;
         }
@@ -191,11 +193,11 @@ __device__ __forceinline__ bool accumulate(const FactorArgs& a, int g, int i, in
     const int* wj = a.wprog + (size_t)g * a.T + j;
     // thread 0: the number of half tiles whose operands are there (at least `want`), -1 if a wait ran out
     auto poll = [&](int want) {
-        int v = i < a.i0 ? 2 * a.T : wait_progress(li, want, a.status);
+        int v = i < a.i0 ? 2 * a.T : wait_progress(li, want, a.status, a.wait);
         if (v < 0) return -1;
         int u;
-        if (NT) u = j < a.i0 ? 2 * a.T : (j == i ? v : wait_progress(lj, want, a.status));
-        else u = want <= 2 * a.i0 ? 2 * a.i0 : wait_progress(wj, want, a.status);
+        if (NT) u = j < a.i0 ? 2 * a.T : (j == i ? v : wait_progress(lj, want, a.status, a.wait));
+        else u = want <= 2 * a.i0 ? 2 * a.i0 : wait_progress(wj, want, a.status, a.wait);
         return u < 0 ? -1 : min(u, v);
     };
     auto load = [&](int s, int k) {   // stage s <- columns k .. k + 15
@@ -523,12 +525,12 @@ __global__ void __launch_bounds__(kThreads, 2) factor_kernel(const __grid_consta
     const int t = threadIdx.x, w = t / 32, l = t % 32, wm = (w % 4) * 16, wn = (w / 4) * 32;
     const int npad = a.npad, T = a.T;
     const int total = a.first[T + 1] * a.batch;
-    auto publish = [&](int* p, int v) {   // the tile has been stored by all threads
+    auto publish = [&](int* p, int v, bool announce = true) {   // the tile has been stored by all threads
         __syncthreads();
-        if (t == 0) store_release_int(p, v);   // (a release covers what the barrier has made this thread see)
+        if (t == 0 && announce) store_release_int(p, v);   // (a release covers what the barrier has made this thread see)
     };
     auto await = [&](const int* p, int want) {
-        if (t == 0) sh.ok = wait_progress(p, want, a.status);
+        if (t == 0) sh.ok = wait_progress(p, want, a.status, a.wait);
         __syncthreads();
         return sh.ok >= 0;
     };
@@ -538,6 +540,7 @@ __global__ void __launch_bounds__(kThreads, 2) factor_kernel(const __grid_consta
         __syncthreads();
         const int task = sh.task;
         if (task >= total) return;
+        const bool announce = !(a.wait.withhold && task == 0);   // (a test keeps the first tile back)
         int lo = 0, hi = T;   // the step: last j with first[j] * batch <= task
         while (lo < hi) {
             const int mid = (lo + hi + 1) / 2;
@@ -572,12 +575,12 @@ __global__ void __launch_bounds__(kThreads, 2) factor_kernel(const __grid_consta
                 } else {
                     store_half(Lg, npad, j, j, 0, tile0, t - 32, kThreads - 32);
                     asm volatile("bar.sync 2, 224;" ::: "memory");
-                    if (t == 32) store_release_int(lp + j, 2 * j + 1);
+                    if (t == 32 && announce) store_release_int(lp + j, 2 * j + 1);
                     for (int e = t - 32; e < 32 * 32; e += kThreads - 32) tile0[(e / 32) * kLd + 32 + e % 32] = 0.0;
                 }
                 __syncthreads();
                 store_half(Lg, npad, j, j, 32, tile0, t, kThreads);
-                publish(lp + j, 2 * j + 2);
+                publish(lp + j, 2 * j + 2, announce);
                 for (int e = t; e < 32 * 32; e += kThreads) tile1[(e / 32) * kLd + 32 + e % 32] = 0.0;
                 if (w < 2) invert_block(tile0, sh.rinv, 32 * w, tile1);
                 __syncthreads();
@@ -596,7 +599,7 @@ __global__ void __launch_bounds__(kThreads, 2) factor_kernel(const __grid_consta
                     solve_panel(tile0, tile1, sh.rinv, h);
                     __syncthreads();
                     store_half(Lg, npad, i, j, h, tile0, t, kThreads);
-                    publish(lp + i, 2 * j + 1 + h / 32);
+                    publish(lp + i, 2 * j + 1 + h / 32, announce);
                     if (h == 0) update_right(tile0, tile1, 0);
                 }
                 zero_tile(Lg, npad, j, i);
@@ -689,6 +692,7 @@ r3_status_t factor_device(const FactorProblem& p, void* scratch, int extra_ints,
     a.lprog = reinterpret_cast<int*>(scratch) + 1;
     a.wprog = a.lprog + (size_t)p.batch * a.T;
     a.status = status;
+    a.wait = p.wait;
     a.first[0] = 0;
     for (int j = 0; j <= a.T; ++j)   // column j of L below the finished rows, row j - 1 of W
         a.first[j + 1] = a.first[j] + (j < a.T ? a.T - std::max(j, a.i0) : 0) + (j > a.i0 ? j - 1 : 0);

@@ -137,6 +137,7 @@ r3_status_t state_fit(r3_gp* gp, r3_fit_state& s, int rows_done, bool full, bool
     f.batch = B; f.n = s.n; f.d = s.d; f.npad = npad; f.rows_done = rows_done;
     f.L = s.L64; f.W = s.W64;
     f.best = s.best_d; f.yabs = s.yabs_d;
+    f.wait = wait_rule(gp, STALL_FACTOR);
     r3_status_t st = factor_device(f, ints, B, s.fit_status, gp->device, stream);
     if (st != R3_OK) return done(st);
     WeightProblem w;
@@ -146,6 +147,7 @@ r3_status_t state_fit(r3_gp* gp, r3_fit_state& s, int rows_done, bool full, bool
     w.W32 = full ? s.W32 : nullptr;
     w.wnorm = full ? s.wnorm_d : nullptr;
     w.wmax = full ? s.wmax_d : nullptr;
+    w.wait = wait_rule(gp, STALL_WEIGHTS);
     st = weights_device(w, doubles, (unsigned*)((char*)ints + fbytes), s.fit_status, gp->device, stream);
     if (st != R3_OK) return done(st);
     if (full) {

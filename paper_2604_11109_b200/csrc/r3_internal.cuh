@@ -97,6 +97,14 @@ int* pinned_word_acquire();          // kPinnedInts pinned host ints from a proc
 void pinned_word_release(int* w);
 size_t cached_bytes();
 
+// Waits of a kernel whose blocks wait for one another: they give up after `cycles` (about two seconds unless a test asks for
+// less); withhold (r3_gp_test_stall): one block keeps back what the others wait for.
+constexpr long long kGridWaitCycles = 4000000000ll;
+struct WaitRule {
+    long long cycles = kGridWaitCycles;
+    int withhold = 0;
+};
+
 inline int round_up(int a, int b) { return (a + b - 1) / b * b; }
 inline long long round_up_ll(long long a, long long b) { return (a + b - 1) / b * b; }
 
@@ -166,6 +174,8 @@ struct r3_gp : r3_fit_state {
     // bounded device-side waits of the tensor engine: the limit in cycles, and the test aid that makes one run out
     long long wait_limit_cycles = 4000000000ll;   // about 2 s
     long long withhold_w = -1;
+    int stall_where = -1;             // r3_gp_test_stall: the kernel, and the limit of its waits
+    long long stall_cycles = 0;
 
     // optional timing of the dominant scoring kernel: event pairs recorded around its launches
     bool profile = false;
@@ -179,6 +189,10 @@ struct r3_gp : r3_fit_state {
 
 namespace r3 {
 
+// The rule for the next launch of kernel `where`; a test's request holds for one launch.
+enum : int { STALL_FACTOR = 0, STALL_WEIGHTS = 1 };
+WaitRule wait_rule(r3_gp* gp, int where);
+
 // factor and inverse factor (r3_factor.cu)
 constexpr int kFactorTile = 64;
 struct FactorProblem {
@@ -187,6 +201,7 @@ struct FactorProblem {
     int rows_done;          // rows of L and W that are there already: a multiple of kFactorTile
     double *L, *W;          // [batch][npad][npad]
     float *best, *yabs;     // [batch] min y, max |y|
+    WaitRule wait;
 };
 size_t factor_scratch_bytes(int batch, int npad);
 // Asynchronous; non-finite inputs and non-positive pivots are latched in `status`.
@@ -203,6 +218,7 @@ struct WeightProblem {
     float* W32;             // [batch][npad][npad], or nullptr
     double* wnorm;          // [batch], or nullptr: weights only
     unsigned* wmax;         // [batch] bits of max |W|, zero on entry, or nullptr
+    WaitRule wait;
 };
 size_t weights_scratch_doubles(int batch, int npad);
 // barrier: [batch] words, zero on entry.  Asynchronous.

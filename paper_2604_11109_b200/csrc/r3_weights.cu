@@ -42,6 +42,7 @@ struct WeightArgs {
     double* npart;         // [batch][npad / 16] sums of squares of the new vector
     unsigned* barrier;     // [batch]
     int* status;
+    WaitRule wait;
 };
 
 // u_i = W_i . v / nrm (and W_i . y) for the rows of this warp
@@ -202,6 +203,11 @@ __device__ __forceinline__ bool arrived(uint32_t bar, uint32_t parity)
     return ok != 0;
 }
 
+__device__ __forceinline__ void count_as_arrived(uint32_t bar, uint32_t bytes)
+{
+    asm volatile("mbarrier.complete_tx.relaxed.cta.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
+}
+
 template <int R>
 __global__ void __launch_bounds__(kClusterThreads, 1) weights_cluster_kernel(const WeightArgs a)
 {
@@ -209,6 +215,8 @@ __global__ void __launch_bounds__(kClusterThreads, 1) weights_cluster_kernel(con
     __shared__ double warp_sums[kClusterThreads / 32];
     __shared__ int warp_tops[kClusterThreads / 32];
     __shared__ __align__(8) unsigned long long bars[2];
+    __shared__ int gave_up;   // a wait ran out in some block of the cluster
+    __shared__ int sent;      // passes whose shares this block has sent
     cg::cluster_group cluster = cg::this_cluster();
     const int r = (int)cluster.block_rank(), g = blockIdx.x / R, threads = blockDim.x, warps = threads / 32;
     const int t = threadIdx.x, lane = t % 32, warp = t / 32, npad = a.npad, n = a.n, rows = npad / R, half = npad / 2;
@@ -224,6 +232,7 @@ __global__ void __launch_bounds__(kClusterThreads, 1) weights_cluster_kernel(con
     if (t == 0) {
         mbar_init(smem_u32(&bars[0]), 1);
         mbar_init(smem_u32(&bars[1]), 1);
+        gave_up = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (t < kClusterThreads / 32) {
@@ -267,7 +276,8 @@ __global__ void __launch_bounds__(kClusterThreads, 1) weights_cluster_kernel(con
     const bool second = rows > threads / 8;
     const uint32_t mine = smem_u32(shares + r * npad + 2 * c);
     double2 v = make_double2(0.0, 0.0);   // (thread < half) the new vector's columns 2 t and 2 t + 1
-    bool late = false;                    // a bounded wait ran out: the rest goes through without waiting
+    bool late = false;                    // a bounded wait ran out, here or in another block of the cluster
+    const int sends = a.wait.withhold && r == R - 1 ? 1 : a.iters + 1;   // (a test keeps the last block's shares back)
     auto pass = [&](double scale, int turn) {   // x, v <- W^T (scale W x)
         for (int q = t / 8; q < rows; q += threads / 8) {
             const int i = R * q + r, m = i < n ? i / 2 : -1;
@@ -305,7 +315,7 @@ __global__ void __launch_bounds__(kClusterThreads, 1) weights_cluster_kernel(con
             *reinterpret_cast<double2*>(parts + p * npad + 2 * c) = s;
         }
         __syncthreads();
-        if (p < min(lots, R)) {   // two columns to every lots-th block
+        if (p < min(lots, R) && turn < sends) {   // two columns to every lots-th block
             double2 s = *reinterpret_cast<const double2*>(parts + 2 * c);
 #pragma unroll
             for (int k = 1; k < kMaxParts; ++k)
@@ -320,13 +330,17 @@ __global__ void __launch_bounds__(kClusterThreads, 1) weights_cluster_kernel(con
         }
         if (t < half) {
             const uint32_t parity = (turn >> 1) & 1;
-            if (!late && !arrived(bar, parity)) {
+            if (!arrived(bar, parity)) {
                 const long long t0 = clock64();
-                while (!arrived(bar, parity))
-                    if (clock64() - t0 > kGridWaitCycles) {
+                while (!arrived(bar, parity)) {
+                    late = *reinterpret_cast<volatile int*>(&gave_up) != 0;
+                    if (!late && clock64() - t0 > a.wait.cycles) {
                         late = true;
-                        break;
+                        atomicOr(a.status, DEV_TIMEOUT);
+                        for (int b = 0; b < R; ++b) *reinterpret_cast<volatile int*>(cluster.map_shared_rank(&gave_up, b)) = 1;
                     }
+                    if (late) break;
+                }
             }
             const double* from = shares + buffer * R * npad + 2 * t;
             v = make_double2(0.0, 0.0);
@@ -340,9 +354,11 @@ __global__ void __launch_bounds__(kClusterThreads, 1) weights_cluster_kernel(con
         }
     };
     double sum = 0.0, before = 0.0, scale = 1.0;
+    int entered = 0;   // passes begun
 #pragma unroll 1
     for (int turn = 0; turn <= a.iters; ++turn) {
         pass(scale, turn);
+        entered = turn + 1;
         if (turn == 0) {
             if (t < half) {
                 if (r == 0) {
@@ -362,9 +378,8 @@ __global__ void __launch_bounds__(kClusterThreads, 1) weights_cluster_kernel(con
         if (turn + 1 >= a.iters) {
             before = sum;
             sum = total(fma(v.x, v.x, v.y * v.y));
-        } else {
-            __syncthreads();
         }
+        if (__syncthreads_or(late)) break;
         if (turn < a.iters) {
             const int e = __reduce_max_sync(0xffffffffu, warp_tops[lane % (kClusterThreads / 32)]) >> 20;
             scale = e == 0 ? 1.0 : __hiloint2double(max(2046 - e, 0) << 20, 0);
@@ -372,12 +387,34 @@ __global__ void __launch_bounds__(kClusterThreads, 1) weights_cluster_kernel(con
     }
     // the growth of the last pass estimates |W|_2^2 from below; 1.5 covers slow convergence
     if (a.iters > 0 && r == 0 && t == 0) a.wnorm[g] = before > 0.0 ? 1.5 * sqrt(sqrt(sum) / (sqrt(before) * scale)) : 0.0;
-    if (late) {   // what is still on its way to this block lands before anyone leaves
-        atomicOr(a.status, DEV_TIMEOUT);
-        const long long t0 = clock64();
-        while (clock64() - t0 < 2000000) __nanosleep(1000);
+    // No block leaves while another's shares may still be on their way to it.  A block that has waited for all its passes has
+    // them all; after this barrier everyone else's have been sent as well.
+    if (t == 0) sent = min(entered, sends);
+    cluster.sync();
+    if (gave_up) {   // said in every block before the barrier, so all see the same
+        // All blocks have sent the shares of the passes before the last one begun here.  Of that pass, and of the one after
+        // it (begun by blocks that got their shares), those that were sent are waited for.
+        if (t == 0) {
+            int missing = 0, ahead = 0;
+            for (int b = 0; b < R; ++b) {
+                const int theirs = *cluster.map_shared_rank(&sent, b);
+                missing += theirs < entered ? 1 : 0;
+                ahead += theirs > entered ? 1 : 0;
+            }
+            const uint32_t share = (uint32_t)(npad * sizeof(double));
+            auto land = [&](int turn) {
+                const long long t0 = clock64();
+                while (!arrived(smem_u32(&bars[turn & 1]), (turn >> 1) & 1) && clock64() - t0 < 2000000) {}
+            };
+            if (missing) count_as_arrived(smem_u32(&bars[(entered - 1) & 1]), missing * share);
+            land(entered - 1);
+            if (ahead) {
+                mbar_arrive_expect_tx(smem_u32(&bars[entered & 1]), ahead * share);
+                land(entered);
+            }
+        }
+        cluster.sync();
     }
-    cluster.sync();   // no block leaves while another may still write to it
 }
 
 __global__ void __launch_bounds__(kThreads, 2) weights_kernel(const WeightArgs a)
@@ -413,7 +450,7 @@ __global__ void __launch_bounds__(kThreads, 2) weights_kernel(const WeightArgs a
                 __syncthreads();
                 return true;
             }
-            return team_barrier(a.barrier + g, target, (unsigned)a.team, a.status);
+            return team_barrier(a.barrier + g, target, (unsigned)a.team, a.status, a.wait);
         };
         auto stage = [&](const double* src, double* dst) {
             for (int i = 2 * t; i < npad; i += 2 * kThreads)
@@ -472,6 +509,7 @@ r3_status_t weights_device(const WeightProblem& p, double* scratch, unsigned* ba
     a.npart = a.v + (size_t)p.batch * p.npad;
     a.barrier = barrier;
     a.status = status;
+    a.wait = p.wait;
     int sms = 148;
     R3_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device));
     // W in shared memory, as far as that goes (R = 2: 320 observations, R = 8: 544).  Eight blocks per GP while that leaves

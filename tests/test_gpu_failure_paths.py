@@ -184,3 +184,28 @@ def test_the_cache_makes_room_for_sizes_that_are_still_in_use():
     gp.close()
     b.r3_trim_cache()
     assert b.r3_cached_bytes() == 0
+
+
+@pytest.mark.parametrize("where,batch,n", [
+    (0, 1, 100), (0, 3, 400),     # the factorisation: the first tile of the first GP is never announced
+    (1, 1, 100), (1, 2, 530),     # the weights: a cluster of eight blocks
+    (1, 40, 300),                 # a cluster of two
+    (1, 1, 700),                  # a team of blocks with a barrier
+])
+def test_a_wait_of_an_append_that_runs_out_leaves_the_handle_unchanged(where, batch, n):
+    g = rand_problem(5000 + n, batch, n, 5, 60)
+    k = 70                                        # a whole tile of new rows and more
+    gp = b.r3_gp_fit(dev(g["X"][:, :-k]), dev(g["y"][:, :-k]), g["ell"], g["sf2"], g["sn2"])
+    xc, xn, yn = dev(g["Xcand"]), dev(g["X"][:, -k:]), dev(g["y"][:, -k:])
+    before = [t.clone() for t in b.r3_gp_score(gp, xc)]
+    b.r3_gp_test_stall(gp, where, SHORT_LIMIT)
+    with pytest.raises(b.R3Error) as e:
+        b.r3_gp_append(gp, xn, yn)
+    assert e.value.status == 6
+    assert b.r3_gp_size(gp) == n - k
+    b.r3_gp_check(gp)
+    for old, new in zip(before, b.r3_gp_score(gp, xc)):
+        assert torch.equal(old, new)
+    b.r3_gp_append(gp, xn, yn)                    # the aid was for one launch
+    _scores_match(g, gp, "append after a wait that ran out")
+    gp.close()
