@@ -189,12 +189,16 @@ r3_status_t r3_gp_set_wait_limit(r3_gp_t* gp, long long cycles);
 r3_status_t r3_gp_test_withhold(r3_gp_t* gp, long long chunk);
 
 /*
- * The other kernels whose blocks wait for one another give up after about two seconds, and the call that launched them
- * reports R3_ERR_DEVICE_TIMEOUT.  r3_gp_test_stall is the testing aid for them: in the next launch of kernel `where` that a
+ * The other kernels whose blocks wait for one another give up after about two seconds; fits and appends then
+ * return R3_ERR_DEVICE_TIMEOUT.  r3_gp_test_stall is the testing aid for them: in the next launch of kernel `where` that a
  * call on this handle makes (one launch only) one block keeps back what the others wait for, and the waits of that launch
  * give up after `cycles` (>= 1e5).  Nothing faults and nothing waits longer than the limit.
  *   where 0: the factorisation (r3_gp_append, r3_gp_refit, r3_gp_optimize): the first tile is not announced
  *   where 1: the weights (likewise): a block's share of a pass is not sent, or a block does not arrive at a barrier
+ *   where 2: the accuracy guard (r3_gp_score, r3_gp_score_topk, r3_gp_propose): a block does not arrive at a barrier
+ *   where 3: the covariances of a proposal (r3_gp_propose): likewise
+ * Scoring calls and proposals latch it in the handle, as they do the waits above; the indices that such a call selects are
+ * meaningless, but they are different rows of the pool.
  */
 r3_status_t r3_gp_test_stall(r3_gp_t* gp, int where, long long cycles);
 

@@ -612,8 +612,8 @@ r3_status_t r3_gp_test_withhold(r3_gp_t* gp, long long chunk)
 
 r3_status_t r3_gp_test_stall(r3_gp_t* gp, int where, long long cycles)
 {
-    if (!gp || where < 0 || where > STALL_WEIGHTS || cycles < 100000) {
-        set_error("r3_gp_test_stall: need a handle, where in [0, %d] and at least 100000 cycles", STALL_WEIGHTS);
+    if (!gp || where < 0 || where > STALL_PROPOSE || cycles < 100000) {
+        set_error("r3_gp_test_stall: need a handle, where in [0, %d] and at least 100000 cycles", STALL_PROPOSE);
         return R3_ERR_INVALID_ARG;
     }
     gp->stall_where = where;

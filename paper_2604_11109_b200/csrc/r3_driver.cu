@@ -188,6 +188,10 @@ r3_status_t r3_bo_run(const float* X0, const float* y0, int n0, int d, const flo
             }
             st = r3_gp_propose(gp, work, left, q, 0, opt.lie, idx_d, nullptr, nullptr, cuda_stream);
             if (st != R3_OK) return done(st);
+            if (gp->status_h[0] & DEV_TIMEOUT) {   // as the proposal has just read it
+                set_error("r3_bo_run: a bounded device-side wait ran out");
+                return done(R3_ERR_DEVICE_TIMEOUT);
+            }
         }
         gather_rows_kernel<<<q, 128, 0, stream>>>(work, idx_d, q, d, rows_d);
         ++g_launches;

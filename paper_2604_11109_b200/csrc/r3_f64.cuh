@@ -71,7 +71,7 @@ __device__ __forceinline__ bool team_barrier(unsigned* counter, unsigned& target
     }
     return __syncthreads_and(ok);
 }
-__device__ __forceinline__ bool grid_barrier(unsigned* counter, unsigned& target, int* status, const WaitRule& rule = WaitRule())
+__device__ __forceinline__ bool grid_barrier(unsigned* counter, unsigned& target, int* status, const WaitRule& rule)
 {
     return team_barrier(counter, target, gridDim.x, status, rule);
 }

@@ -190,7 +190,7 @@ struct r3_gp : r3_fit_state {
 namespace r3 {
 
 // The rule for the next launch of kernel `where`; a test's request holds for one launch.
-enum : int { STALL_FACTOR = 0, STALL_WEIGHTS = 1 };
+enum : int { STALL_FACTOR = 0, STALL_WEIGHTS = 1, STALL_GUARD = 2, STALL_PROPOSE = 3 };
 WaitRule wait_rule(r3_gp* gp, int where);
 
 // factor and inverse factor (r3_factor.cu)

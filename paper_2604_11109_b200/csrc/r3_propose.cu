@@ -56,6 +56,7 @@ struct ProposeArrays {
     int *cert;             // [B] the shortlist is certified to lose nothing
     unsigned* barrier;     // grid barrier, zero on entry
     int* status;
+    WaitRule wait;
 };
 
 __device__ __forceinline__ const float* short_row(const ProposeArrays& a, int g, int r)
@@ -96,7 +97,7 @@ __global__ void __launch_bounds__(kCrossThreads, 2) build_kernel(const ProposeAr
                 [&](int r, int k, double v) { if (ta * 64 + r < R) C0[(size_t)(ta * 64 + r) * R + k] = v; }, [](int, double) {});
         }
     }
-    if (!grid_barrier(a.barrier, target, a.status)) return;
+    if (!grid_barrier(a.barrier, target, a.status, a.wait)) return;
     // ---- V[r][i] = sum_k Ks[r][k] W[i][k], the longest rows of W first, and the partial sums of squares
     for (int item = blockIdx.x; item < a.B * RT * NT; item += gridDim.x) {
         const int it = NT - 1 - item / (a.B * RT), g = item % (a.B * RT) / RT, rt = item % RT;
@@ -124,7 +125,7 @@ __global__ void __launch_bounds__(kCrossThreads, 2) build_kernel(const ProposeAr
         __syncthreads();
     }
     if (a.q < 2) return;
-    if (!grid_barrier(a.barrier, target, a.status)) return;
+    if (!grid_barrier(a.barrier, target, a.status, a.wait)) return;
     // ---- C0 = k(z, z') - V V^T, written on both sides
     for (int item = blockIdx.x; item < a.B * pairs; item += gridDim.x) {
         const int g = item / pairs;
@@ -347,6 +348,7 @@ r3_status_t propose_shortlist(r3_gp* gp, const float* Xcand, long long m, const 
     p += up16(sizeof(int) * B);
     a.barrier = (unsigned*)p;
     a.status = gp->status_d;
+    a.wait = wait_rule(gp, STALL_PROPOSE);
     *cert = a.cert;
     R3_CUDA_TRY(cudaMemsetAsync(a.barrier, 0, sizeof(unsigned), stream));
 

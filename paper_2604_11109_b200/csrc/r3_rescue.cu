@@ -65,6 +65,7 @@ struct GuardArgs {
     unsigned* done;               // [batch] slices selected so far
     unsigned* barrier;            // grid barrier
     int* status;                  // the handle's status words
+    WaitRule wait;
     bool have_max;
     double *ks, *qpart, *mupart;  // slab: [slab][npad], [slab][npad / 16], [slab][ceil(npad / 64)]
     int slab;                     // candidates per slab, a multiple of 64
@@ -254,14 +255,14 @@ __device__ __forceinline__ bool rescue(const GuardArgs& a, const int* pref, int 
                 [&](int c, int k, double kv) { a.ks[(slot0 + c) * a.npad + k] = kv; },
                 [&](int c, double part) { a.mupart[(slot0 + c) * nb + kb] = part; });
         }
-        if (!grid_barrier(a.barrier, target, a.status)) return false;
+        if (!grid_barrier(a.barrier, target, a.status, a.wait)) return false;
         for (int item = blockIdx.x; item < nt * row_tiles; item += gridDim.x) {   // the longest rows first
             const int tile = item % nt, rt = row_tiles - 1 - item / nt;
             const double* Wg = a.W64 + (size_t)gp_of(t0 + tile) * a.npad * a.npad;
             if (CT == kTile) rescue_tile(a, Wg, (size_t)tile * CT, rt, smem);
             else rescue_small_tile(a, Wg, (size_t)tile * CT, rt, smem);
         }
-        if (!grid_barrier(a.barrier, target, a.status)) return false;
+        if (!grid_barrier(a.barrier, target, a.status, a.wait)) return false;
         for (int s = blockIdx.x * kThreads + threadIdx.x; s < nt * CT; s += gridDim.x * kThreads) {
             const int tile = s / CT, g = gp_of(t0 + tile), pos = (t0 + tile - pref[g]) * CT + s % CT;
             if (pos >= __ldcg(a.count + g)) continue;
@@ -273,7 +274,7 @@ __device__ __forceinline__ bool rescue(const GuardArgs& a, const int* pref, int 
             write_result(a, g, __ldcg(a.list + (size_t)g * a.m + pos), mu, q);
         }
         // the next slab overwrites the partial sums that other blocks may still be adding up
-        if (t0 + slab_tiles < tiles && !grid_barrier(a.barrier, target, a.status)) return false;
+        if (t0 + slab_tiles < tiles && !grid_barrier(a.barrier, target, a.status, a.wait)) return false;
     }
     return true;
 }
@@ -346,6 +347,21 @@ __global__ void __launch_bounds__(kThreads, 2) guard_kernel(const GuardArgs a)
     const int slices = a.slices_per_gp * a.batch, chunks = a.chunks_per_gp * a.batch;
     const bool own_rescue = a.npad <= kOwnMaxN;
     unsigned target = 0;
+    // A barrier ran out: the results are invalid, and the status word says so, but whoever reads the pool through the selected
+    // indices before the status has been looked at must find k different rows of it.
+    auto give_up = [&]() {
+        if (a.k == 0) return;
+        __syncthreads();
+        if (a.finish) {
+            for (int e = t; e < a.batch * a.k; e += kThreads) a.idx[e] = e % a.k;
+        } else {   // the later levels read these keys
+            for (int s = blockIdx.x; s < slices; s += gridDim.x) {
+                const long long c0 = (long long)(s % a.slices_per_gp) * a.slice;
+                for (int i = t; i < a.K2; i += kThreads)
+                    a.keys[(size_t)s * a.K2 + i] = c0 + i < m ? topk_make_key(0.f, (unsigned)(c0 + i)) : 0ull;
+            }
+        }
+    };
 
     // ---- the pool's largest EI
     if (!a.have_max) {
@@ -358,7 +374,7 @@ __global__ void __launch_bounds__(kThreads, 2) guard_kernel(const GuardArgs a)
             const unsigned top = __reduce_max_sync(0xffffffffu, __float_as_uint(v));   // order-preserving for v >= 0
             if (lane == 0 && top) atomicMax(&a.maxbits[g], top);
         }
-        if (!grid_barrier(a.barrier, target, a.status)) return;
+        if (!grid_barrier(a.barrier, target, a.status, a.wait)) return give_up();
     }
 
     // ---- flag
@@ -420,7 +436,7 @@ __global__ void __launch_bounds__(kThreads, 2) guard_kernel(const GuardArgs a)
             if (own_count > 0) rescue_own(a, g, own, min(own_count, kSmallTile), smem);
         }
     }
-    if (!grid_barrier(a.barrier, target, a.status)) return;
+    if (!grid_barrier(a.barrier, target, a.status, a.wait)) return give_up();
     if (blockIdx.x == 0 && t < min(a.batch, 64)) a.rescued_h[t] = __ldcg(a.total + t);   // pinned host memory
 
     // ---- rescue
@@ -453,12 +469,12 @@ __global__ void __launch_bounds__(kThreads, 2) guard_kernel(const GuardArgs a)
             // 64 x 64 tiles once they give every block two; below that 16 x 16 tiles spread the work
             const long long items = (long long)big * ((a.npad + kTile - 1) / kTile);
             if (items >= 2ll * gridDim.x) {
-                if (!rescue<kTile>(a, pref, big, target, smem)) return;
+                if (!rescue<kTile>(a, pref, big, target, smem)) return give_up();
             } else {
                 const int small = prefix(kSmallTile);
-                if (!rescue<kSmallTile>(a, pref, small, target, smem)) return;
+                if (!rescue<kSmallTile>(a, pref, small, target, smem)) return give_up();
             }
-            if (a.k > 0 && !grid_barrier(a.barrier, target, a.status)) return;
+            if (a.k > 0 && !grid_barrier(a.barrier, target, a.status, a.wait)) return give_up();
         }
     }
     if (a.k == 0) return;
@@ -619,6 +635,7 @@ r3_status_t guard_and_rescue(r3_gp* gp, const float* Xcand, long long m, const G
     a.done = b.done;
     a.barrier = b.barrier;
     a.status = gp->status_d;
+    a.wait = wait_rule(gp, STALL_GUARD);
     a.have_max = have_max;
     a.ks = b.ks; a.qpart = b.qpart; a.mupart = b.mupart;
     a.slab = slab_candidates(gp, m);

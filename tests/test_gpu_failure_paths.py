@@ -209,3 +209,43 @@ def test_a_wait_of_an_append_that_runs_out_leaves_the_handle_unchanged(where, ba
     b.r3_gp_append(gp, xn, yn)                    # the aid was for one launch
     _scores_match(g, gp, "append after a wait that ran out")
     gp.close()
+
+
+@pytest.mark.parametrize("n,m,k", [
+    (40, 600, 16),        # the kernel finishes the selection itself
+    (300, 80000, 300),    # its slices' keys go on to the selection's later levels
+])
+def test_a_guard_barrier_that_runs_out_leaves_indices_inside_the_pool(n, m, k):
+    g = rand_problem(6000 + n, 2, n, 5, m)
+    gp = fit_gpu(g)
+    xc = dev(g["Xcand"])
+    b.r3_gp_score_topk(gp, xc, k)                 # the workspace now holds another call's keys
+    b.r3_gp_check(gp)
+    b.r3_gp_test_stall(gp, 2, SHORT_LIMIT)
+    _, _, _, idx, _ = b.r3_gp_score_topk(gp, xc, k)
+    with pytest.raises(b.R3Error) as e:
+        b.r3_gp_check(gp)
+    assert e.value.status == 6
+    for row in idx.cpu().numpy():
+        assert row.min() >= 0 and row.max() < m and len(set(row.tolist())) == k
+    compare_everything(g, gp, 8, "after a guard barrier that ran out")
+    gp.close()
+
+
+@pytest.mark.parametrize("where", [2, 3])
+def test_a_proposal_whose_barrier_runs_out_names_rows_of_the_pool(where):
+    g = rand_problem(6100, 2, 150, 5, 3000)
+    gp = fit_gpu(g)
+    xc = dev(g["Xcand"])
+    want, _, _ = b.r3_gp_propose(gp, xc, 8)
+    b.r3_gp_test_stall(gp, where, SHORT_LIMIT)
+    idx, _, _ = b.r3_gp_propose(gp, xc, 8)
+    with pytest.raises(b.R3Error) as e:
+        b.r3_gp_check(gp)
+    assert e.value.status == 6
+    for row in np.asarray(idx.cpu()):
+        assert row.min() >= 0 and row.max() < 3000 and len(set(row.tolist())) == 8
+    again, _, _ = b.r3_gp_propose(gp, xc, 8)
+    b.r3_gp_check(gp)
+    assert torch.equal(want, again)
+    gp.close()
