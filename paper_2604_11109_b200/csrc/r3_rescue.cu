@@ -336,9 +336,9 @@ __device__ __forceinline__ void rescue_own(const GuardArgs& a, int g, const int*
     }
 }
 
-__global__ void __launch_bounds__(kThreads, 2) guard_kernel(const GuardArgs a)
+// What guard_kernel does; false: a barrier ran out.
+__device__ __forceinline__ bool guard_pool(const GuardArgs& a, unsigned char* smem)
 {
-    extern __shared__ __align__(16) unsigned char smem[];
     __shared__ int own[kSmallTile], own_count;
     __shared__ int warp_sum[8];
     __shared__ bool last_slice;
@@ -347,21 +347,6 @@ __global__ void __launch_bounds__(kThreads, 2) guard_kernel(const GuardArgs a)
     const int slices = a.slices_per_gp * a.batch, chunks = a.chunks_per_gp * a.batch;
     const bool own_rescue = a.npad <= kOwnMaxN;
     unsigned target = 0;
-    // A barrier ran out: the results are invalid, and the status word says so, but whoever reads the pool through the selected
-    // indices before the status has been looked at must find k different rows of it.
-    auto give_up = [&]() {
-        if (a.k == 0) return;
-        __syncthreads();
-        if (a.finish) {
-            for (int e = t; e < a.batch * a.k; e += kThreads) a.idx[e] = e % a.k;
-        } else {   // the later levels read these keys
-            for (int s = blockIdx.x; s < slices; s += gridDim.x) {
-                const long long c0 = (long long)(s % a.slices_per_gp) * a.slice;
-                for (int i = t; i < a.K2; i += kThreads)
-                    a.keys[(size_t)s * a.K2 + i] = c0 + i < m ? topk_make_key(0.f, (unsigned)(c0 + i)) : 0ull;
-            }
-        }
-    };
 
     // ---- the pool's largest EI
     if (!a.have_max) {
@@ -374,7 +359,7 @@ __global__ void __launch_bounds__(kThreads, 2) guard_kernel(const GuardArgs a)
             const unsigned top = __reduce_max_sync(0xffffffffu, __float_as_uint(v));   // order-preserving for v >= 0
             if (lane == 0 && top) atomicMax(&a.maxbits[g], top);
         }
-        if (!grid_barrier(a.barrier, target, a.status, a.wait)) return give_up();
+        if (!grid_barrier(a.barrier, target, a.status, a.wait)) return false;
     }
 
     // ---- flag
@@ -436,7 +421,7 @@ __global__ void __launch_bounds__(kThreads, 2) guard_kernel(const GuardArgs a)
             if (own_count > 0) rescue_own(a, g, own, min(own_count, kSmallTile), smem);
         }
     }
-    if (!grid_barrier(a.barrier, target, a.status, a.wait)) return give_up();
+    if (!grid_barrier(a.barrier, target, a.status, a.wait)) return false;
     if (blockIdx.x == 0 && t < min(a.batch, 64)) a.rescued_h[t] = __ldcg(a.total + t);   // pinned host memory
 
     // ---- rescue
@@ -469,15 +454,15 @@ __global__ void __launch_bounds__(kThreads, 2) guard_kernel(const GuardArgs a)
             // 64 x 64 tiles once they give every block two; below that 16 x 16 tiles spread the work
             const long long items = (long long)big * ((a.npad + kTile - 1) / kTile);
             if (items >= 2ll * gridDim.x) {
-                if (!rescue<kTile>(a, pref, big, target, smem)) return give_up();
+                if (!rescue<kTile>(a, pref, big, target, smem)) return false;
             } else {
                 const int small = prefix(kSmallTile);
-                if (!rescue<kSmallTile>(a, pref, small, target, smem)) return give_up();
+                if (!rescue<kSmallTile>(a, pref, small, target, smem)) return false;
             }
-            if (a.k > 0 && !grid_barrier(a.barrier, target, a.status, a.wait)) return give_up();
+            if (a.k > 0 && !grid_barrier(a.barrier, target, a.status, a.wait)) return false;
         }
     }
-    if (a.k == 0) return;
+    if (a.k == 0) return true;
 
     // ---- the k largest final EI of every slice
     unsigned long long* keys_s = reinterpret_cast<unsigned long long*>(smem);
@@ -521,6 +506,25 @@ __global__ void __launch_bounds__(kThreads, 2) guard_kernel(const GuardArgs a)
                     if (a.val) a.val[(size_t)g * a.k + i] = ((long long)c < m) ? __ldcg(e + c) : __int_as_float(0x7fc00000);
                 }
             }
+        }
+    }
+    return true;
+}
+
+__global__ void __launch_bounds__(kThreads, 2) guard_kernel(const GuardArgs a)
+{
+    extern __shared__ __align__(16) unsigned char smem[];
+    if (guard_pool(a, smem) || a.k == 0) return;
+    // The results are invalid, and the status word says so, but whoever reads the pool through the selected indices before the
+    // status has been looked at must find k different rows of it.
+    __syncthreads();
+    if (a.finish) {
+        for (int e = threadIdx.x; e < a.batch * a.k; e += kThreads) a.idx[e] = e % a.k;
+    } else {   // the later levels read these keys
+        for (int s = blockIdx.x; s < a.slices_per_gp * a.batch; s += gridDim.x) {
+            const long long c0 = (long long)(s % a.slices_per_gp) * a.slice;
+            for (int i = threadIdx.x; i < a.K2; i += kThreads)
+                a.keys[(size_t)s * a.K2 + i] = c0 + i < a.m ? topk_make_key(0.f, (unsigned)(c0 + i)) : 0ull;
         }
     }
 }
