@@ -76,8 +76,8 @@ typedef enum {
  *
  * Synchronises `cuda_stream` before returning, so that R3_ERR_NOT_PD and
  * R3_ERR_NONFINITE are reported by this call.  No jitter is added: a
- * non-positive-definite K is an error, never silently repaired (a pivot below
- * four roundings of sf2 + noise, such as a duplicated row without noise leaves, counts as non-positive).
+ * non-positive-definite K is an error, never silently repaired: a pivot that is not
+ * positive, or two equal rows of X where signal_var + noise_var equals signal_var in FP64.
  */
 r3_status_t r3_gp_fit(const float* X, const float* y, const float* lengthscales,
                       const float* signal_var, const float* noise_var, int batch, int n, int d,

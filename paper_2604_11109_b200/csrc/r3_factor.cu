@@ -137,6 +137,7 @@ __device__ __forceinline__ void gram_tile(const FactorArgs& a, int g, int ti, in
         }
     }
     const double sf2 = (double)a.sf2[g], sn2 = (double)a.sn2[g];
+    int twin = a.n;   // a row that repeats an earlier one
 #pragma unroll 1
     for (int j = 0; j < 4; ++j)   // not unrolled: four square roots and exponentials at a time are enough to overlap
 #pragma unroll
@@ -150,10 +151,16 @@ __device__ __forceinline__ void gram_tile(const FactorArgs& a, int g, int ti, in
                 const double s = sqrt(5.0) * sqrt(r);
                 double v = sf2 * fma(s, fma(s, 1.0 / 3.0, 1.0), 1.0) * exp(-s);
                 if (row == col) v += sn2;
+                else if (r == 0.0 && col < row) twin = min(twin, row);
                 if (row >= n || col >= n) v = row == col ? 1.0 : 0.0;   // the identity beyond the history
 #pragma unroll
                 for (int jj = 0; jj < 4; ++jj) c[i][jj][h] = jj == j ? -v : c[i][jj][h];
             }
+    // Two equal rows whose noise is lost in the diagonal's rounding: K is singular whatever sign its pivots come out with
+    if (twin < n && sf2 + sn2 == sf2) {
+        atomicOr(&a.status[0], DEV_NOT_PD);
+        atomicMin(&a.status[1], twin);
+    }
 }
 
 // One 16-deep step: A fragments at pa (row stride lda), B fragments either [column][k] (NT) or [k][column].
@@ -345,10 +352,10 @@ __global__ void rsqrt_kernel(const double* __restrict__ p, double* __restrict__ 
 // chain of a step is r2, one column, one update, det and its root, and waits for no broadcast.
 // The two panels of a 64 x 64 block: 15,500 cycles; 17,700 column by column, 22,000 with a shuffle in the chain and unrolled
 // code.  (Letting the second warp follow by a counter instead of the barrier: 24,000, it falls behind.)
-// A pivot of the history must exceed `tiny`, a few roundings of the diagonal entry it was computed from: a duplicated row
-// without noise leaves a pivot of either sign at that level.  cols: 16 x 64 doubles of scratch in shared memory.
+// A pivot's sign decides (gram_tile looks for equal rows without noise, whose pivots are rounding of either sign).
+// cols: 16 x 64 doubles of scratch in shared memory.
 __device__ __forceinline__ void factor_panel(double* tile, int b, int warps, double* cols, double* rinv, const FactorArgs& a,
-                                             int pivot0, double tiny)
+                                             int pivot0)
 {
     const int w = threadIdx.x / 32, l = threadIdx.x % 32;
     if (w >= warps) return;
@@ -420,7 +427,7 @@ __device__ __forceinline__ void factor_panel(double* tile, int b, int warps, dou
         }
         // the pivots' test, once for all: lane = column; beyond the first bad pivot everything is NaN or means nothing
         const double d = tile[row * kLd + row];
-        const bool bad = !(d * d > (pivot0 + row < a.n ? tiny : 0.0) * (1.0 + 1e-15)) || !isfinite(d);
+        const bool bad = !(d > 0.0) || !isfinite(d);
         const unsigned which = __ballot_sync(0xffffffffu, bad);
         if (which && l == 0) {
             atomicOr(&a.status[0], DEV_NOT_PD);
@@ -564,14 +571,13 @@ __global__ void __launch_bounds__(kThreads, 2) factor_kernel(const __grid_consta
             park(c, -1.0, tile0);
             __syncthreads();
             if (i == j) {
-                const double tiny = 4.0 * 2.220446049250313e-16 * ((double)a.sf2[g] + (double)a.sn2[g]);
-                factor_panel(tile0, 0, 2, tile1, sh.rinv, a, j * TB, tiny);
+                factor_panel(tile0, 0, 2, tile1, sh.rinv, a, j * TB);
                 __syncthreads();
                 update_right(tile0, tile0, 32);
                 __syncthreads();
                 // one warp takes the second panel; the others hand the first one out meanwhile
                 if (w == 0) {
-                    factor_panel(tile0, 32, 1, tile1, sh.rinv, a, j * TB, tiny);
+                    factor_panel(tile0, 32, 1, tile1, sh.rinv, a, j * TB);
                 } else {
                     store_half(Lg, npad, j, j, 0, tile0, t - 32, kThreads - 32);
                     asm volatile("bar.sync 2, 224;" ::: "memory");

@@ -67,3 +67,20 @@ def test_reciprocal_roots_of_pivots():
     assert float(np.abs(y / exact - 1.0).max()) <= 2.0 ** -52
     assert float(np.abs(y / torch.rsqrt(dev(p)).cpu().numpy() - 1.0).max()) <= 2.0 ** -51
     assert np.isnan(b.r3_test_rsqrt(dev(np.array([0.0, -1.0, np.nan, -np.inf]))).cpu().numpy()).all()
+
+
+@pytest.mark.parametrize("n", [2, 70])
+@pytest.mark.parametrize("gap", [1.9e-8, 2.0e-8, 2.1e-8, 2.2e-8])
+def test_a_small_positive_pivot_is_positive(n, gap):
+    """Noise-free, all rows far apart but the last, `gap` lengthscales from the first: k = 1 - 5/6 gap^2 = 1 - (3 to 4)e-16,
+    computed with an error of at most 2e-16 (three roundings near one), and the last pivot is 1 - k^2 > 0, a few roundings of
+    the diagonal."""
+    X = (100.0 * np.arange(n, dtype=np.float32))[None, :, None]
+    X[0, -1, 0] = gap
+    y = np.linspace(-1, 1, n, dtype=np.float32)[None]
+    one = np.ones((1, 1), np.float32)
+    gp = b.r3_gp_fit(dev(X), dev(y), one, one[0], np.zeros(1, np.float32))
+    _, L = b.r3_gp_get_factor(gp)
+    assert 0.0 < L[0, -1, -1] ** 2 < 2e-15
+    assert L[0, -1, 0] == pytest.approx(1.0, abs=1e-15)
+    gp.close()
