@@ -84,6 +84,14 @@ static size_t score_workspace_bytes(const r3_gp* gp, long long m)
 
 static size_t align256(size_t v) { return (v + 255) & ~(size_t)255; }
 
+// A refit that failed, and whose previous hyper-parameters could not be fitted again either, leaves nothing to work with.
+static r3_status_t check_fitted(const r3_gp* gp, const char* who)
+{
+    if (gp->fitted) return R3_OK;
+    set_error("%s: the handle's last r3_gp_refit or r3_gp_optimize failed and left it without a fit; r3_gp_refit fits it again", who);
+    return R3_ERR_INVALID_ARG;
+}
+
 static r3_status_t check_score_args(const r3_gp* gp, const void* Xcand, long long m, const void* mu,
                                     const void* sigma, const void* ei)
 {
@@ -95,7 +103,7 @@ static r3_status_t check_score_args(const r3_gp* gp, const void* Xcand, long lon
         set_error("r3_gp_score: m=%lld out of range [1, 2^31)", m);
         return R3_ERR_INVALID_ARG;
     }
-    return R3_OK;
+    return check_fitted(gp, "r3_gp_score");
 }
 
 static r3_status_t run_score(r3_gp* gp, const float* Xcand, long long m, float* mu, float* sigma, float* ei,
@@ -248,6 +256,7 @@ r3_status_t r3_gp_lml(r3_gp_t* gp, double* lml, double* grad, void* cuda_stream)
         set_error("r3_gp_lml: NULL argument");
         return R3_ERR_INVALID_ARG;
     }
+    if (r3_status_t fitted = check_fitted(gp, "r3_gp_lml"); fitted != R3_OK) return fitted;
     const int B = gp->batch, d = gp->d;
     std::vector<double> out((size_t)B * (d + 3));
     const r3_status_t st = lml_device(gp, out.data(), (cudaStream_t)cuda_stream);
@@ -272,6 +281,7 @@ r3_status_t r3_gp_propose(r3_gp_t* gp, const float* Xcand, long long m, int q, i
                   lie);
         return R3_ERR_INVALID_ARG;
     }
+    if (r3_status_t fitted = check_fitted(gp, "r3_gp_propose"); fitted != R3_OK) return fitted;
     const int rmax = (int)(m < 1023 ? m : 1023);
     int R = shortlist;
     if (R == 0) {
@@ -355,6 +365,7 @@ r3_status_t r3_gp_append(r3_gp_t* gp, const float* Xnew, const float* ynew, int 
         set_error("r3_gp_append: need 1 <= k <= %d and n + k <= %d (n=%d, k=%d)", kAppendMax, kMaxN, gp->n, k);
         return R3_ERR_INVALID_ARG;
     }
+    if (r3_status_t fitted = check_fitted(gp, "r3_gp_append"); fitted != R3_OK) return fitted;
     cudaStream_t stream = (cudaStream_t)cuda_stream;
     int bits = 0, pivot = 0;   // the append's own status words: what scoring calls have latched stays where it is
     const r3_status_t st = append_device(gp, Xnew, ynew, k, stream, &bits, &pivot);
@@ -475,6 +486,7 @@ r3_status_t r3_gp_score_topk_host(r3_gp_t* gp, const float* Xcand_host, long lon
         set_error("r3_gp_score_topk_host: m or k out of range");
         return R3_ERR_INVALID_ARG;
     }
+    if (r3_status_t fitted = check_fitted(gp, "r3_gp_score_topk_host"); fitted != R3_OK) return fitted;
     const size_t B = gp->batch;
     const size_t sb = align256(score_workspace_bytes(gp, m));
     const size_t tb = align256(guard_topk_workspace_bytes(gp->batch, m, k));
@@ -723,6 +735,7 @@ r3_status_t r3_gp_get_factor(const r3_gp_t* gp, double* alpha, double* L)
         set_error("r3_gp_get_factor: NULL handle");
         return R3_ERR_INVALID_ARG;
     }
+    if (r3_status_t fitted = check_fitted(gp, "r3_gp_get_factor"); fitted != R3_OK) return fitted;
     R3_CUDA_TRY(cudaDeviceSynchronize());
     const int n = gp->n, npad = gp->npad;
     for (int g = 0; g < gp->batch; ++g) {

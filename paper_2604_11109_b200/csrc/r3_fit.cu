@@ -115,6 +115,8 @@ r3_status_t state_fit(r3_gp* gp, r3_fit_state& s, int rows_done, bool full, bool
     const size_t wdoubles = weights_scratch_doubles(B, npad);
     TRY_DONE(dev_malloc(&doubles, sizeof(double) * (wdoubles + (lml ? lml_scratch_doubles(s) : 0))));
 
+    const bool own = &s == static_cast<r3_fit_state*>(gp);
+    if (own) gp->fitted = false;
     // the block: results cleared, hyper-parameters filled in
     size_t results = 0;
     const size_t bytes = carve_block(s, s.block, &results);
@@ -193,6 +195,7 @@ r3_status_t state_fit(r3_gp* gp, r3_fit_state& s, int rows_done, bool full, bool
             FreeScope no_wait;   // nothing has used them yet
             tc_release(s);
         }
+        if (own) gp->fitted = !(fs[0] & (DEV_NOT_PD | DEV_NONFINITE));
     }
     return done(R3_OK);
 }

@@ -157,6 +157,7 @@ struct r3_fit_state {
 // The handle.  Device arrays are allocated at fit time and freed by r3_gp_free.
 struct r3_gp : r3_fit_state {
     int device = 0;
+    bool fitted = false;       // factor, weights and operands belong together; false while a refit is under way or has failed
     std::vector<float> ell, sf2, sn2;         // host copies [batch][d], [batch], [batch]
     int* status_d = nullptr;   // [4]: status bits of the scoring calls, pivot, line of a failed index check, unused
     int* status_h = nullptr;   // pinned mirror of status_d
@@ -230,7 +231,7 @@ r3_status_t state_alloc(r3_fit_state& s);    // arrays for s.batch, s.n, s.d
 void state_free(r3_fit_state& s);
 // The fit of s (histories in place, hyper-parameters from gp's host copies), rows below rows_done of L and W given.
 // full: everything a handle needs, tensor operands included; otherwise L, W, alpha and the status only (an evaluation of
-// the evidence).  Synchronises; *bits and *pivot are what the device found.  need_tc: a failed allocation of the tensor
+// the evidence, which leaves the handle without a fit).  Synchronises; *bits and *pivot are what the device found.  need_tc: a failed allocation of the tensor
 // operands is an error (otherwise the CUDA-core engine serves the state).
 // lml: if not nullptr receives the evidence and its gradient, host [batch][d + 3] (meaningless when *bits reports a failure).
 r3_status_t state_fit(r3_gp* gp, r3_fit_state& s, int rows_done, bool full, bool need_tc, cudaStream_t stream, int* bits,

@@ -8,6 +8,7 @@
 
 #include <algorithm>
 #include <deque>
+#include <string>
 #include <vector>
 
 #include "r3_internal.cuh"
@@ -175,6 +176,25 @@ private:
     bool started_ = false, done_ = false;
 };
 
+// A handle's hyper-parameters before a refit, for when it fails.
+struct Previous {
+    std::vector<float> ell, sf2, sn2;
+    explicit Previous(const r3_gp* gp) : ell(gp->ell), sf2(gp->sf2), sn2(gp->sn2) {}
+    // Fits the handle with them again and returns `st`, the status of what failed; the error text says how that went.
+    r3_status_t restore(r3_gp* gp, r3_status_t st, cudaStream_t stream) const
+    {
+        const std::string why = r3_last_error();
+        gp->ell = ell;
+        gp->sf2 = sf2;
+        gp->sn2 = sn2;
+        int bits = 0;
+        if (!gp->fitted) state_fit(gp, *gp, 0, true, false, stream, &bits, nullptr);
+        if (gp->fitted) set_error("%s; the previous hyper-parameters were kept", why.c_str());
+        else set_error("%s; fitting the previous hyper-parameters again failed too", why.c_str());
+        return st;
+    }
+};
+
 }  // namespace
 
 }  // namespace r3
@@ -205,23 +225,16 @@ r3_status_t r3_gp_refit(r3_gp_t* gp, const float* lengthscales, const float* sig
         }
     }
     cudaStream_t stream = (cudaStream_t)cuda_stream;
-    const std::vector<float> ell0 = gp->ell, sf0 = gp->sf2, sn0 = gp->sn2;
+    const Previous previous(gp);
     gp->ell.assign(lengthscales, lengthscales + (size_t)B * d);
     gp->sf2.assign(signal_var, signal_var + B);
     gp->sn2.assign(noise_var, noise_var + B);
     int bits = 0, pivot = 0;
-    r3_status_t st = state_fit(gp, *gp, 0, true, true, stream, &bits, &pivot);
-    if (st != R3_OK) return st;
+    const r3_status_t st = state_fit(gp, *gp, 0, true, true, stream, &bits, &pivot);
+    if (st != R3_OK) return previous.restore(gp, st, stream);
     if (bits & DEV_NOT_PD) {
-        gp->ell = ell0;
-        gp->sf2 = sf0;
-        gp->sn2 = sn0;
-        int bits0 = 0;
-        st = state_fit(gp, *gp, 0, true, true, stream, &bits0, nullptr);
-        if (st != R3_OK) return st;
-        set_error("r3_gp_refit: K + noise*I is not positive definite with these hyper-parameters (pivot %d); the "
-                  "previous ones were kept", pivot);
-        return R3_ERR_NOT_PD;
+        set_error("r3_gp_refit: K + noise*I is not positive definite with these hyper-parameters (pivot %d)", pivot);
+        return previous.restore(gp, R3_ERR_NOT_PD, stream);
     }
     return R3_OK;
 }
@@ -240,6 +253,7 @@ r3_status_t r3_gp_optimize(r3_gp_t* gp, int max_evals, double gtol, float* lengt
     }
     cudaStream_t stream = (cudaStream_t)cuda_stream;
     const int B = gp->batch, d = gp->d, P = d + 2;
+    const Previous previous(gp);
     std::vector<Lbfgs> opt;
     for (int g = 0; g < B; ++g) {
         std::vector<double> x(P), lo(P), hi(P);
@@ -275,7 +289,7 @@ r3_status_t r3_gp_optimize(r3_gp_t* gp, int max_evals, double gtol, float* lengt
         load(false);
         int bits = 0;
         st = state_fit(gp, *gp, 0, false, false, stream, &bits, nullptr, out.data());
-        if (st != R3_OK) return st;
+        if (st != R3_OK) return previous.restore(gp, st, stream);
         ++used;
         const bool ok = !(bits & (DEV_NOT_PD | DEV_NONFINITE));
         for (int g = 0; g < B; ++g) {
@@ -288,10 +302,10 @@ r3_status_t r3_gp_optimize(r3_gp_t* gp, int max_evals, double gtol, float* lengt
     load(true);
     int bits = 0;
     st = state_fit(gp, *gp, 0, true, true, stream, &bits, nullptr);
-    if (st != R3_OK) return st;
+    if (st != R3_OK) return previous.restore(gp, st, stream);
     if (bits & (DEV_NOT_PD | DEV_NONFINITE)) {
         set_error("r3_gp_optimize: the starting hyper-parameters do not give a positive definite covariance matrix");
-        return R3_ERR_NOT_PD;
+        return previous.restore(gp, R3_ERR_NOT_PD, stream);
     }
     for (int g = 0; g < B; ++g) {
         if (lengthscales)

@@ -249,3 +249,41 @@ def test_a_proposal_whose_barrier_runs_out_names_rows_of_the_pool(where):
     b.r3_gp_check(gp)
     assert torch.equal(want, again)
     gp.close()
+
+
+@pytest.mark.parametrize("call", ["optimize", "refit"])
+@pytest.mark.parametrize("failure", ["allocation", "wait"])
+def test_a_refit_that_fails_keeps_the_previous_fit(call, failure):
+    g = rand_problem(7000, 2, 150, 10, 300)
+    xc = dev(g["Xcand"])
+
+    def go(gp):
+        if call == "optimize":
+            b.r3_gp_optimize(gp, max_evals=3, gtol=1e-9)
+        else:
+            b.r3_gp_refit(gp, 2.0 * g["ell"], g["sf2"], g["sn2"])
+
+    gp = fit_gpu(g)
+    before = [t.clone() for t in b.r3_gp_score(gp, xc)]
+    factor = b.r3_gp_get_factor(gp)
+    spare = fit_gpu(g)
+    b.r3_test_fail_allocation(-1)
+    go(spare)                                     # how many allocations the call makes
+    total = b.r3_test_fail_allocation(-1)
+    spare.close()
+    for after in range(total) if failure == "allocation" else [None]:
+        if after is None:
+            b.r3_gp_test_stall(gp, 0, SHORT_LIMIT)
+        else:
+            b.r3_test_fail_allocation(after)
+        with pytest.raises(b.R3Error) as e:
+            go(gp)
+        assert e.value.status == (6 if after is None else 4) and "were kept" in str(e.value), after
+        for old, new in zip(factor, b.r3_gp_get_factor(gp)):
+            assert np.array_equal(old, new), after
+        for old, new in zip(before, b.r3_gp_score(gp, xc)):
+            assert torch.equal(old, new), after
+        b.r3_gp_check(gp)
+    b.r3_test_fail_allocation(-1)
+    go(gp)                                        # and the call goes through afterwards
+    gp.close()
