@@ -160,6 +160,7 @@ r3_status_t state_fit(r3_gp* gp, r3_fit_state& s, int rows_done, bool full, bool
         }
         if (tc_supported(s.n, s.d)) {
             st = tc_prepare(s, gp->device, stream);
+            s.tc_short = st == R3_ERR_ALLOC;
             if (st != R3_OK && (need_tc || st != R3_ERR_ALLOC)) return done(st);
         }
     }
@@ -233,6 +234,26 @@ __global__ void embed_kernel(const double* __restrict__ L0, const double* __rest
 
 }  // namespace
 
+// The new state's tensor operands did not fit beside the old state's: now that those are gone, once more.  If there is still no
+// memory for them the append stands and the CUDA-core engine serves the handle (r3_gp_engine tells).
+static r3_status_t operands_again(r3_gp* gp, cudaStream_t stream)
+{
+    r3_status_t st = tc_prepare(*gp, gp->device, stream);
+    if (st != R3_OK) return st == R3_ERR_ALLOC ? R3_OK : st;
+    gp->tc_short = false;
+    if (!gp->tc) return R3_OK;
+    std::vector<unsigned> wmax(gp->batch);
+    unsigned xamax = 0;
+    R3_CUDA_TRY(cudaMemcpyAsync(wmax.data(), gp->wmax_d, sizeof(unsigned) * gp->batch, cudaMemcpyDeviceToHost, stream));
+    R3_CUDA_TRY(cudaMemcpyAsync(&xamax, gp->xamax_d, sizeof(unsigned), cudaMemcpyDeviceToHost, stream));
+    R3_CUDA_TRY(cudaStreamSynchronize(stream));
+    if (!tc_accept(*gp, gp->sf2.data(), wmax.data(), xamax)) {
+        FreeScope no_wait;   // nothing has used them yet
+        tc_release(*gp);
+    }
+    return R3_OK;
+}
+
 r3_status_t append_device(r3_gp* gp, const float* Xnew, const float* ynew, int k, cudaStream_t stream, int* bits, int* pivot)
 {
     r3_fit_state s;
@@ -262,7 +283,7 @@ r3_status_t append_device(r3_gp* gp, const float* Xnew, const float* ynew, int k
     FreeScope no_wait;
     std::swap(static_cast<r3_fit_state&>(*gp), s);
     state_free(s);
-    return R3_OK;
+    return gp->tc_short ? operands_again(gp, stream) : R3_OK;
 }
 
 }  // namespace r3

@@ -152,6 +152,7 @@ struct r3_fit_state {
 
     // tensor-core operands (built by the fit when the tensor engine can serve (n, d))
     void* tc = nullptr;        // r3::TensorOperands*, see r3_score_tc.cu
+    bool tc_short = false;     // they are missing because there was no memory for them
 };
 
 // The handle.  Device arrays are allocated at fit time and freed by r3_gp_free.

@@ -287,3 +287,35 @@ def test_a_refit_that_fails_keeps_the_previous_fit(call, failure):
     b.r3_test_fail_allocation(-1)
     go(gp)                                        # and the call goes through afterwards
     gp.close()
+
+
+def test_an_append_without_memory_for_both_states_operands_keeps_the_tensor_engine():
+    """Whichever single allocation fails, the append either leaves the handle as it was or ends on the engine that serves it:
+    operands that do not fit beside the old state's are made after those are gone."""
+    g = rand_problem(8000, 1, 200, 10, 300)
+    k = 16
+    xn, yn = dev(g["X"][:, -k:]), dev(g["y"][:, -k:])
+
+    def shorter():
+        return b.r3_gp_fit(dev(g["X"][:, :-k]), dev(g["y"][:, :-k]), g["ell"], g["sf2"], g["sn2"])
+
+    gp = shorter()
+    b.r3_test_fail_allocation(-1)
+    b.r3_gp_append(gp, xn, yn)
+    total = b.r3_test_fail_allocation(-1)
+    gp.close()
+    went_through = 0
+    for after in range(total):
+        gp = shorter()
+        b.r3_test_fail_allocation(after)
+        try:
+            b.r3_gp_append(gp, xn, yn)
+            went_through += 1
+        except b.R3Error as e:
+            assert e.status == 4 and b.r3_gp_size(gp) == 200 - k
+            b.r3_gp_append(gp, xn, yn)
+        assert b.r3_gp_engine(gp) == b.ENGINE_TENSOR, after
+        _scores_match(g, gp, f"append with allocation {after} failing")
+        gp.close()
+    b.r3_test_fail_allocation(-1)
+    assert went_through >= 5
