@@ -1199,9 +1199,14 @@ r3_status_t tc_prepare(r3_fit_state& st, int device, cudaStream_t stream)
     if ((e = dev_malloc(&t->wt, sizeof(__half) * B * t->wt_gp_stride)) != cudaSuccess) return fail("cudaMalloc", e);
     if ((e = dev_malloc(&t->kscale, sizeof(float) * B)) != cudaSuccess) return fail("cudaMalloc", e);
     if ((e = dev_malloc(&t->vinv2, sizeof(double) * B)) != cudaSuccess) return fail("cudaMalloc", e);
-    if (t->f8) {
-        if ((e = dev_malloc(&t->wt16, sizeof(__half) * B * t->wt_gp_stride)) != cudaSuccess) return fail("cudaMalloc", e);
-        if ((e = dev_malloc(&t->vinv2_16, sizeof(double) * B)) != cudaSuccess) return fail("cudaMalloc", e);
+    if (t->f8 && (dev_malloc(&t->wt16, sizeof(__half) * B * t->wt_gp_stride) != cudaSuccess ||
+                  dev_malloc(&t->vinv2_16, sizeof(double) * B) != cudaSuccess)) {
+        cudaGetLastError();   // no memory for the second form: every pool is scored with FP8 cross terms
+        FreeScope no_wait;    // nothing has used them yet
+        dev_free(t->wt16);
+        dev_free(t->vinv2_16);
+        t->wt16 = nullptr;
+        t->vinv2_16 = nullptr;
     }
     t->xnmax = reinterpret_cast<float*>(st.xnmax_d);   // lives in the state's block
 
@@ -1214,7 +1219,7 @@ r3_status_t tc_prepare(r3_fit_state& st, int device, cudaStream_t stream)
     wt_build_kernel<<<dim3(t->P * CPP, t->P, B), 256, 0, stream>>>(st.W64, n, st.npad, t->NV, t->wt_gp_stride, st.wmax_d,
                                                                    st.sf2_d, t->kscale, t->vinv2, t->wt, t->f8);
     g_launches += 3;
-    if (t->f8) {
+    if (t->wt16) {
         wt_build_kernel<<<dim3(t->P * CPP, t->P, B), 256, 0, stream>>>(st.W64, n, st.npad, t->NV, t->wt_gp_stride, st.wmax_d,
                                                                        st.sf2_d, t->kscale, t->vinv2_16, t->wt16, false);
         ++g_launches;
@@ -1390,8 +1395,8 @@ r3_status_t score_tc_part(r3_gp* gp, const float* Xcand, long long m, float* mu,
                 const long long whole = rest / prm.tiles_per_gp, part = std::min(m, rest % prm.tiles_per_gp * TILE_M);
                 if (st == R3_OK) st = guard_pilot(gp, m, whole * m + part, gb, mu, sigma, ei, stream);
             }
-            if (st == R3_OK && rest < end) st = launch(true, rest, end, 0);
-            if (st == R3_OK) st = launch(false, begin, end, 1);
+            if (st == R3_OK && rest < end) st = launch(true, rest, end, t->wt16 ? 0 : -1);
+            if (st == R3_OK && t->wt16) st = launch(false, begin, end, 1);
         }
         if (st != R3_OK) return st;
     }

@@ -30,8 +30,8 @@ struct TensorOperands {
                                // second plane is two 8-bit planes [2][KC/16][NV][16]: hi parts (E4M3), then lo parts (E5M2)
     float* kscale = nullptr;   // [B]  2^eK, applied to k* before its split
     double* vinv2 = nullptr;   // [B]  2^(-2 (eK + eW)): scales sum V^2 back
-    __half* wt16 = nullptr;    // with f8: the chunks as FP16 hi/lo planes too, for pools that need them
-    double* vinv2_16 = nullptr;
+    __half* wt16 = nullptr;    // with f8: the chunks as FP16 hi/lo planes too, for pools that need them (nullptr: no memory
+    double* vinv2_16 = nullptr;   // for them when the operands were made)
 };
 
 struct TcParams {

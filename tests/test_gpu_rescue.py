@@ -57,6 +57,28 @@ def test_long_histories_on_pools_that_need_fp16_cross_terms(batch, n, d, m, sn2)
     gp.close()
 
 
+@pytest.mark.parametrize("missing", [1, 2])
+def test_a_long_history_without_memory_for_both_forms_of_its_operands(missing):
+    """The FP16 form's operands are the last two allocations of a fit; without them every pool is scored in the FP8 form."""
+    g = rand_problem(1977, 1, 1900, 4, 20000, sn2=1e-2, spread=2.0)
+    X, y = dev(g["X"]), dev(g["y"])
+    b.r3_test_fail_allocation(-1)
+    b.r3_gp_fit(X, y, g["ell"], g["sf2"], g["sn2"]).close()
+    b.r3_test_fail_allocation(b.r3_test_fail_allocation(-1) - missing)
+    gp = b.r3_gp_fit(X, y, g["ell"], g["sf2"], g["sn2"])
+    b.r3_test_fail_allocation(-1)
+    assert b.r3_gp_engine(gp) == b.ENGINE_TENSOR and b.r3_gp_tensor_info(gp)["f8_cross_terms"] == 1
+    mu, sd, ei, idx, val = (t.cpu().numpy() for t in b.r3_gp_score_topk(gp, dev(g["Xcand"]), 20))
+    b.r3_gp_check(gp)
+    f = o.fit_batch(g["X"], g["y"], g["ell"], g["sf2"], g["sn2"])[0]
+    rows = np.sort(np.random.default_rng(3).choice(20000, size=1000, replace=False))
+    mu_r, sd_r, ei_r = o.score(f, g["Xcand"][0][rows])
+    check_scores(mu[0][rows], sd[0][rows], ei[0][rows], mu_r, sd_r, ei_r, float(np.abs(g["y"][0]).max()),
+                 float(g["sf2"][0]), ei_max=float(ei[0].max()), what="FP8 form only")
+    assert np.array_equal(idx[0], o.topk(ei[0], 20)[0])
+    gp.close()
+
+
 @pytest.mark.parametrize("m,k", [(128, 64), (300, 8), (4096, 1), (4096, 128), (4096, 129), (5000, 320), (20000, 321), (70001, 257)])
 @pytest.mark.parametrize("kind", ["uniform", "crowded", "equal", "clustered"])
 def test_selection_behind_the_guard(m, k, kind):
