@@ -345,6 +345,10 @@ int r3_gp_size(const r3_gp_t* gp);
  * L [batch][n][n] FP64 lower-triangular (upper part zero).  Either may be NULL. */
 r3_status_t r3_gp_get_factor(const r3_gp_t* gp, double* alpha, double* L);
 
+/* Copy each GP's estimate of 1.5 |L^-1|_2 to host wnorm [batch] (diagnostics and tests).  The scoring engines' error estimates
+ * in the variance are proportional to it; the power iteration behind it approaches |L^-1|_2 from below. */
+r3_status_t r3_gp_get_norms(const r3_gp_t* gp, double* wnorm);
+
 /* Kernels launched by this library on the calling thread since the last reset. */
 unsigned long long r3_launch_count(void);
 void r3_launch_count_reset(void);

@@ -78,6 +78,7 @@ SIGNATURES = {
     "r3_gp_set_engine": (_i, [_vp, _i]),
     "r3_gp_engine": (_i, [_vp]),
     "r3_gp_get_factor": (_i, [_vp, _vp, _vp]),
+    "r3_gp_get_norms": (_i, [_vp, _vp]),
     "r3_gp_last_rescued": (_i, [_vp, _vp, ctypes.POINTER(_ll)]),
     "r3_gp_tensor_info": (_i, [_vp, ctypes.POINTER(ctypes.c_int)]),
     "r3_gp_profile": (_i, [_vp, _i]),
@@ -435,6 +436,13 @@ def r3_gp_get_factor(gp: GP):
     L = np.empty((gp.batch, gp.n, gp.n), dtype=np.float64)
     _check(load().r3_gp_get_factor(gp.handle, alpha.ctypes.data_as(_vp), L.ctypes.data_as(_vp)))
     return alpha, L
+
+
+def r3_gp_get_norms(gp: GP) -> np.ndarray:
+    """float64 [batch]: 1.5 times the estimate of |L^-1|_2 that the engines' error estimates use."""
+    out = np.empty((gp.batch,), dtype=np.float64)
+    _check(load().r3_gp_get_norms(gp.handle, out.ctypes.data_as(_vp)))
+    return out
 
 
 def r3_gp_last_rescued(gp: GP) -> int:

@@ -749,4 +749,16 @@ r3_status_t r3_gp_get_factor(const r3_gp_t* gp, double* alpha, double* L)
     return R3_OK;
 }
 
+r3_status_t r3_gp_get_norms(const r3_gp_t* gp, double* wnorm)
+{
+    if (!gp || !wnorm) {
+        set_error("r3_gp_get_norms: NULL argument");
+        return R3_ERR_INVALID_ARG;
+    }
+    if (r3_status_t fitted = check_fitted(gp, "r3_gp_get_norms"); fitted != R3_OK) return fitted;
+    R3_CUDA_TRY(cudaDeviceSynchronize());
+    R3_CUDA_TRY(cudaMemcpy(wnorm, gp->wnorm_d, sizeof(double) * gp->batch, cudaMemcpyDeviceToHost));
+    return R3_OK;
+}
+
 }  // extern "C"

@@ -100,7 +100,10 @@ __device__ __forceinline__ bool misses_contract(float mu, float sd, float dmu, f
 }
 
 // One block looks at the first `rows` candidates (GP after GP) of a pool that the engine has scored in its cheaper form:
-// mode <- 1 when more than one in 32 of them would have to be recomputed, 0 otherwise.  Clears the guard's counters.
+// mode <- 1 when more than one in 32 of them would have to be recomputed, 0 otherwise.  The test is the guard's except that EI
+// is measured against the largest in the sample, over all its GPs: of a GP on a smaller scale than another's it sees errors of
+// mu and sigma only (which decide on the pools that were tried: two GPs a factor of 1e4 apart got the decision that equal
+// scales get).  One decision serves the whole pool, whatever lies behind the sample.  Clears the guard's counters.
 __global__ void __launch_bounds__(1024) pilot_kernel(const GuardArgs a, long long rows, int* __restrict__ mode, int* __restrict__ zero,
                                                      int zeros)
 {

@@ -1384,9 +1384,10 @@ r3_status_t score_tc_part(r3_gp* gp, const float* Xcand, long long m, float* mu,
         } else {
             // The FP8 cross terms save a fifth of the time where the posterior is tame and send most of a pool to the FP64
             // pass where it is not (few features, long lengthscales): 65,536 candidates at n = 4096 with 41,604 recomputed
-            // 41.6 ms, with FP16 cross terms and none recomputed 4.1 ms.  So the pool's first wave of tiles is scored with
-            // them, the guard's own test decides on the device, and of the two launches for the rest (for all of it, in the
-            // FP16 form) one returns at once.  A first wave costs no more alone than as part of the whole.
+            // 41.6 ms, with FP16 cross terms and none recomputed 4.1 ms.  So the pool's first wave of tiles, as they lie in
+            // memory, is scored with them, a test of it (pilot_kernel) decides on the device for the whole pool, and of the two
+            // launches for the rest (for all of it, in the FP16 form) one returns at once.  A first wave costs no more alone
+            // than as part of the whole.
             long long rest = begin;
             if (begin == 0) {
                 rest = std::min<long long>(end, sms);

@@ -3,6 +3,7 @@ GP and for several, against the oracle's factor; the inverse is checked through 
 import numpy as np
 import pytest
 
+from oracle import gp_oracle as o
 from paper_2604_11109_b200 import binding as b
 from tests.test_gpu_append import check_handle, check_scoring, dev, problem
 
@@ -44,10 +45,33 @@ def test_duplicated_row_without_noise_is_not_positive_definite(n, twin):
 @pytest.mark.parametrize("batch,n", [(1, 31), (2, 129), (40, 33), (40, 320), (40, 321), (1, 544), (1, 545)])
 def test_weights_where_their_split_changes(batch, n):
     """One GP or many, around the history lengths at which W stops fitting the shared memory of two and of eight blocks: the
-    weights (check_handle) and, through the scores, the norm estimate."""
+    weights (check_handle), the norm estimate, and the scores."""
     g = problem(2500 + n, batch, n, 4, 40)
     gp = b.r3_gp_fit(dev(g["X"]), dev(g["y"]), g["ell"], g["sf2"], g["sn2"])
-    check_scoring(gp, g, check_handle(gp, g, n))
+    fits = check_handle(gp, g, n)
+    check_norms(gp, fits)
+    check_scoring(gp, g, fits)
+    gp.close()
+
+
+def check_norms(gp, fits):
+    """1.5 times twelve power iterations on W^T W, which never exceed |W|_2 and reach (c^2)^(1/48) of it if a share c^2 of the
+    start vector lies along the leading direction: 0.78 for c^2 = 1e-5.  (W's own error: 1e-4 covers the ill-conditioned.)"""
+    for got, f in zip(b.r3_gp_get_norms(gp), fits):
+        ratio = got * np.linalg.svd(np.tril(f.L), compute_uv=False)[-1]   # |L^-1|_2 = 1 / smallest singular value
+        assert 1.5 * 0.78 <= ratio <= 1.5 * (1 + 1e-4), ratio
+
+
+@pytest.mark.parametrize("batch,n,spread", [(1, 100, 3.0), (40, 300, 5.0), (1, 500, 5.0), (1, 600, 5.0)])
+def test_norm_estimate_of_ill_conditioned_histories(batch, n, spread):
+    g = problem(2700 + n, batch, n, 4, 10)
+    g["ell"] *= np.float32(spread)
+    g["sn2"][:] = 1e-7
+    gp = b.r3_gp_fit(dev(g["X"]), dev(g["y"]), g["ell"], g["sf2"], g["sn2"])
+    check_norms(gp, o.fit_batch(g["X"], g["y"], g["ell"], g["sf2"], g["sn2"]))
+    b.r3_gp_append(gp, dev(g["X"][:, :1] + np.float32(0.5)), dev(g["y"][:, :1]))   # an append makes its own
+    X1, y1 = np.concatenate([g["X"], g["X"][:, :1] + np.float32(0.5)], 1), np.concatenate([g["y"], g["y"][:, :1]], 1)
+    check_norms(gp, o.fit_batch(X1, y1, g["ell"], g["sf2"], g["sn2"]))
     gp.close()
 
 
