@@ -343,6 +343,10 @@ r3_status_t r3_gp_propose(r3_gp_t* gp, const float* Xcand, long long m, int q, i
     TRY_DONE(cudaMemcpyAsync(gp->status_h, gp->status_d, 2 * sizeof(int), cudaMemcpyDeviceToHost, stream));
     TRY_DONE(cudaStreamSynchronize(stream));
 #undef TRY_DONE
+    if (gp->status_h[0] & DEV_BOUNDS) {
+        set_error("bounds-checking build: an index check of the proposal or of an earlier call failed (r3_gp_check tells the line)");
+        return done(R3_ERR_CUDA);
+    }
     if (gp->status_h[0] & DEV_NOT_PD) {
         gp->status_h[0] &= ~DEV_NOT_PD;
         cudaMemcpy(gp->status_d, gp->status_h, sizeof(int), cudaMemcpyHostToDevice);

@@ -101,7 +101,7 @@ __device__ __forceinline__ void cross_tile(int n, int d, int npad, const float* 
 // c += A B^T for 64 rows of A and of B (row-major, leading dimension ld, rows from arows / brows on are zeros), columns
 // [0, K), K a multiple of 16: warp w holds rows 16 (w % 4) + 8 i + l / 4 and columns 32 (w / 4) + 8 j + 2 (l % 4) + h.
 __device__ __forceinline__ void nt_tile(const double* A, int arows, const double* B, int brows, int ld, int K,
-                                        unsigned char* smem, double (&c)[2][4][2])
+                                        unsigned char* smem, double (&c)[2][4][2], int* status)
 {
     double* sA = reinterpret_cast<double*>(smem);         // [stages][64][20]
     double* sB = sA + kCrossStages * kCrossTile * kStageLd;
@@ -112,8 +112,8 @@ __device__ __forceinline__ void nt_tile(const double* A, int arows, const double
 #pragma unroll
         for (int it = 0; it < 2; ++it) {
             const int e = t + kCrossThreads * it, r = e / 8, q = e % 8;
-            cp_async16(sA + (s * kCrossTile + r) * kStageLd + 2 * q, A + (size_t)(r < arows ? r : 0) * ld + k0 + 2 * q, r < arows);
-            cp_async16(sB + (s * kCrossTile + r) * kStageLd + 2 * q, B + (size_t)(r < brows ? r : 0) * ld + k0 + 2 * q, r < brows);
+            cp_async16(sA + (s * kCrossTile + r) * kStageLd + 2 * q, A + (size_t)(r < arows ? r : 0) * ld + R3_IDX(k0 + 2 * q, ld - 1, status), r < arows);
+            cp_async16(sB + (s * kCrossTile + r) * kStageLd + 2 * q, B + (size_t)(r < brows ? r : 0) * ld + R3_IDX(k0 + 2 * q, ld - 1, status), r < brows);
         }
     };
     __syncthreads();   // earlier reads of the stages' bytes are done

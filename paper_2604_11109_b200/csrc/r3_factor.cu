@@ -104,8 +104,8 @@ __device__ __forceinline__ void gram_tile(const FactorArgs& a, int g, int ti, in
 #pragma unroll
         for (int e = 0; e < 8; ++e) {
             const int gi = ti * TB + q0 + 8 * e, gj = tj * TB + q0 + 8 * e;
-            vi[e] = (gi < n && c0 + f0 < d) ? __ldg(Xg + (size_t)gi * d + c0 + f0) : 0.f;
-            vj[e] = (gj < n && c0 + f0 < d) ? __ldg(Xg + (size_t)gj * d + c0 + f0) : 0.f;
+            vi[e] = (gi < n && c0 + f0 < d) ? __ldg(Xg + R3_IDX((size_t)gi * d + c0 + f0, (size_t)n * d, a.status)) : 0.f;
+            vj[e] = (gj < n && c0 + f0 < d) ? __ldg(Xg + R3_IDX((size_t)gj * d + c0 + f0, (size_t)n * d, a.status)) : 0.f;
         }
 #pragma unroll
         for (int e = 0; e < 8; ++e) {
@@ -212,12 +212,13 @@ __device__ __forceinline__ bool accumulate(const FactorArgs& a, int g, int i, in
         for (int it = 0; it < 2; ++it) {
             const int e = t + kThreads * it, r = e / 8, q = e % 8;
             const bool oki = i * TB + r < npad, okj = j * TB + r < npad;
-            cp_async16(sA + (s * TB + r) * kStageLd + 2 * q, Lg + (size_t)(oki ? i * TB + r : 0) * npad + k + 2 * q, oki);
+            auto at = [&](int row, int col) { return (size_t)R3_IDX(row, npad, a.status) * npad + R3_IDX(col, npad - 1, a.status); };
+            cp_async16(sA + (s * TB + r) * kStageLd + 2 * q, Lg + at(oki ? i * TB + r : 0, k + 2 * q), oki);
             if (NT) {
-                cp_async16(sB + s * kBStage + r * kLdb + 2 * q, Lg + (size_t)(okj ? j * TB + r : 0) * npad + k + 2 * q, okj);
+                cp_async16(sB + s * kBStage + r * kLdb + 2 * q, Lg + at(okj ? j * TB + r : 0, k + 2 * q), okj);
             } else {
                 const int rr = e / 32, qq = e % 32;
-                cp_async16(sB + s * kBStage + rr * kLdb + 2 * qq, Wg + (size_t)(k + rr) * npad + j * TB + 2 * qq);
+                cp_async16(sB + s * kBStage + rr * kLdb + 2 * qq, Wg + at(k + rr, j * TB + 2 * qq));
             }
         }
     };
@@ -258,54 +259,56 @@ __device__ __forceinline__ bool accumulate(const FactorArgs& a, int g, int i, in
 }
 
 // Tile (ti, tj) of a matrix into shared memory (zeros beyond npad), asynchronously.
-__device__ __forceinline__ void fetch_tile(const double* Mg, int npad, int ti, int tj, double* dst)
+__device__ __forceinline__ void fetch_tile(const double* Mg, int npad, int ti, int tj, double* dst, int* status)
 {
     for (int e = threadIdx.x; e < TB * (TB / 2); e += kThreads) {
         const int r = e / (TB / 2), q = e % (TB / 2);
         const bool ok = ti * TB + r < npad && tj * TB + 2 * q < npad;
-        cp_async16(dst + r * kLd + 2 * q, Mg + (ok ? (size_t)(ti * TB + r) * npad + tj * TB + 2 * q : 0), ok);
+        cp_async16(dst + r * kLd + 2 * q, Mg + R3_IDX(ok ? (size_t)(ti * TB + r) * npad + tj * TB + 2 * q : 0, (size_t)npad * npad - 1, status), ok);
     }
     cp_async_commit();
 }
 
-__device__ __forceinline__ void store_tile(double* Mg, int npad, int ti, int tj, const double* src)
+__device__ __forceinline__ void store_tile(double* Mg, int npad, int ti, int tj, const double* src, int* status)
 {
     for (int e = threadIdx.x; e < TB * (TB / 2); e += kThreads) {
         const int r = e / (TB / 2), q = e % (TB / 2);
         if (ti * TB + r < npad && tj * TB + 2 * q < npad)
-            *reinterpret_cast<double2*>(Mg + (size_t)(ti * TB + r) * npad + tj * TB + 2 * q) =
+            *reinterpret_cast<double2*>(Mg + R3_IDX((size_t)(ti * TB + r) * npad + tj * TB + 2 * q, (size_t)npad * npad - 1, status)) =
                 *reinterpret_cast<const double2*>(src + r * kLd + 2 * q);
     }
 }
 
 // Of a diagonal tile: columns h .. h + 31 from row h on, as fetch_tile
-__device__ __forceinline__ void fetch_half(const double* Mg, int npad, int tj, int h, double* dst)
+__device__ __forceinline__ void fetch_half(const double* Mg, int npad, int tj, int h, double* dst, int* status)
 {
     for (int e = threadIdx.x; e < (TB - h) * 16; e += kThreads) {
         const int r = h + e / 16, c = h + 2 * (e % 16);
         const bool ok = tj * TB + r < npad && tj * TB + c < npad;
-        cp_async16(dst + r * kLd + c, Mg + (ok ? (size_t)(tj * TB + r) * npad + tj * TB + c : 0), ok);
+        cp_async16(dst + r * kLd + c, Mg + R3_IDX(ok ? (size_t)(tj * TB + r) * npad + tj * TB + c : 0, (size_t)npad * npad - 1, status), ok);
     }
     cp_async_commit();
 }
 
 // Columns h .. h + 31 of a tile, by the threads t of `threads`
-__device__ __forceinline__ void store_half(double* Mg, int npad, int ti, int tj, int h, const double* src, int t, int threads)
+__device__ __forceinline__ void store_half(double* Mg, int npad, int ti, int tj, int h, const double* src, int t, int threads,
+                                           int* status)
 {
     for (int e = t; e < TB * 16; e += threads) {
         const int r = e / 16, c = h + 2 * (e % 16);
         if (ti * TB + r < npad && tj * TB + c < npad)
-            *reinterpret_cast<double2*>(Mg + (size_t)(ti * TB + r) * npad + tj * TB + c) =
+            *reinterpret_cast<double2*>(Mg + R3_IDX((size_t)(ti * TB + r) * npad + tj * TB + c, (size_t)npad * npad - 1, status)) =
                 *reinterpret_cast<const double2*>(src + r * kLd + c);
     }
 }
 
-__device__ __forceinline__ void zero_tile(double* Mg, int npad, int ti, int tj)
+__device__ __forceinline__ void zero_tile(double* Mg, int npad, int ti, int tj, int* status)
 {
     for (int e = threadIdx.x; e < TB * (TB / 2); e += kThreads) {
         const int r = e / (TB / 2), q = e % (TB / 2);
         if (ti * TB + r < npad && tj * TB + 2 * q < npad)
-            *reinterpret_cast<double2*>(Mg + (size_t)(ti * TB + r) * npad + tj * TB + 2 * q) = make_double2(0.0, 0.0);
+            *reinterpret_cast<double2*>(Mg + R3_IDX((size_t)(ti * TB + r) * npad + tj * TB + 2 * q, (size_t)npad * npad - 1, status)) =
+                make_double2(0.0, 0.0);
     }
 }
 
@@ -579,37 +582,37 @@ __global__ void __launch_bounds__(kThreads, 2) factor_kernel(const __grid_consta
                 if (w == 0) {
                     factor_panel(tile0, 32, 1, tile1, sh.rinv, a, j * TB);
                 } else {
-                    store_half(Lg, npad, j, j, 0, tile0, t - 32, kThreads - 32);
+                    store_half(Lg, npad, j, j, 0, tile0, t - 32, kThreads - 32, a.status);
                     asm volatile("bar.sync 2, 224;" ::: "memory");
                     if (t == 32 && announce) store_release_int(lp + j, 2 * j + 1);
                     for (int e = t - 32; e < 32 * 32; e += kThreads - 32) tile0[(e / 32) * kLd + 32 + e % 32] = 0.0;
                 }
                 __syncthreads();
-                store_half(Lg, npad, j, j, 32, tile0, t, kThreads);
+                store_half(Lg, npad, j, j, 32, tile0, t, kThreads, a.status);
                 publish(lp + j, 2 * j + 2, announce);
                 for (int e = t; e < 32 * 32; e += kThreads) tile1[(e / 32) * kLd + 32 + e % 32] = 0.0;
                 if (w < 2) invert_block(tile0, sh.rinv, 32 * w, tile1);
                 __syncthreads();
                 invert_corner(tile0, tile1, tile0);   // L11 is not needed any more
-                store_tile(Wg, npad, j, j, tile1);
+                store_tile(Wg, npad, j, j, tile1, a.status);
                 publish(a.wprog + (size_t)g * T + j, 2 * j + 2);
             } else {
                 // the left half against the first panel while the second is being made
                 for (int h = 0; h < 64; h += 32) {
                     if (j >= a.i0 && !await(lp + j, 2 * j + 1 + h / 32)) return;
-                    fetch_half(Lg, npad, j, h, tile1);
+                    fetch_half(Lg, npad, j, h, tile1, a.status);
                     cp_async_wait<0>();
                     __syncthreads();
                     if (t < 32) sh.rinv[h + t] = 1.0 / tile1[(h + t) * kLd + h + t];
                     __syncthreads();
                     solve_panel(tile0, tile1, sh.rinv, h);
                     __syncthreads();
-                    store_half(Lg, npad, i, j, h, tile0, t, kThreads);
+                    store_half(Lg, npad, i, j, h, tile0, t, kThreads, a.status);
                     publish(lp + i, 2 * j + 1 + h / 32, announce);
                     if (h == 0) update_right(tile0, tile1, 0);
                 }
-                zero_tile(Lg, npad, j, i);
-                zero_tile(Wg, npad, j, i);
+                zero_tile(Lg, npad, j, i, a.status);
+                zero_tile(Wg, npad, j, i, a.status);
             }
         } else {
             const int i = j - 1, col = at - diag;
@@ -618,7 +621,7 @@ __global__ void __launch_bounds__(kThreads, 2) factor_kernel(const __grid_consta
             int* wp = a.wprog + (size_t)g * T;
             if (!accumulate<false>(a, g, i, col, col, i, smem, sh, c)) return;
             if (!await(wp + i, 2 * i + 2)) return;
-            fetch_tile(Wg, npad, i, i, tile0);
+            fetch_tile(Wg, npad, i, i, tile0, a.status);
             park(c, -1.0, tile1);
             cp_async_wait<0>();
             __syncthreads();
@@ -632,7 +635,7 @@ __global__ void __launch_bounds__(kThreads, 2) factor_kernel(const __grid_consta
             __syncthreads();
             park(c, 1.0, tile0);
             __syncthreads();
-            store_tile(Wg, npad, i, col, tile0);
+            store_tile(Wg, npad, i, col, tile0, a.status);
             publish(wp + col, 2 * i + 2);
         }
     }

@@ -61,7 +61,7 @@ struct ProposeArrays {
 
 __device__ __forceinline__ const float* short_row(const ProposeArrays& a, int g, int r)
 {
-    return r < a.R ? a.Xcand + ((size_t)g * a.m + a.sidx[(size_t)g * a.Rk + r]) * a.d : nullptr;
+    return r < a.R ? a.Xcand + ((size_t)g * a.m + R3_IDX(a.sidx[(size_t)g * a.Rk + r], a.m, a.status)) * a.d : nullptr;
 }
 
 __global__ void __launch_bounds__(kCrossThreads, 2) build_kernel(const ProposeArrays a)
@@ -83,8 +83,8 @@ __global__ void __launch_bounds__(kCrossThreads, 2) build_kernel(const ProposeAr
             double* Ks = a.Ks + ((size_t)g * R + rt * 64) * npad;
             cross_tile<64>(
                 a.n, a.d, npad, a.ell + (size_t)g * a.d, (double)a.sf2[g], a.alpha + (size_t)g * npad,
-                [&](int r) { return short_row(a, g, rt * 64 + r); }, [&](int k) { return a.X + ((size_t)g * a.n + k) * a.d; }, kb,
-                smem, [&](int c, int k, double v) { if (rt * 64 + c < R) Ks[(size_t)c * npad + k] = v; },
+                [&](int r) { return short_row(a, g, rt * 64 + r); }, [&](int k) { return a.X + ((size_t)g * a.n + R3_IDX(k, a.n, a.status)) * a.d; }, kb,
+                smem, [&](int c, int k, double v) { if (rt * 64 + c < R) Ks[(size_t)c * npad + R3_IDX(k, npad, a.status)] = v; },
                 [&](int c, double s) { if (rt * 64 + c < R) a.mupart[((size_t)g * R + rt * 64 + c) * NT + kb] = s; });
         } else {
             const int g = (item - kstar) / pairs;
@@ -94,7 +94,7 @@ __global__ void __launch_bounds__(kCrossThreads, 2) build_kernel(const ProposeAr
             cross_tile<64>(
                 R, a.d, R, a.ell + (size_t)g * a.d, (double)a.sf2[g], nullptr, [&](int r) { return short_row(a, g, ta * 64 + r); },
                 [&](int k) { return short_row(a, g, k); }, tb, smem,
-                [&](int r, int k, double v) { if (ta * 64 + r < R) C0[(size_t)(ta * 64 + r) * R + k] = v; }, [](int, double) {});
+                [&](int r, int k, double v) { if (ta * 64 + r < R) C0[(size_t)(ta * 64 + r) * R + R3_IDX(k, R, a.status)] = v; }, [](int, double) {});
         }
     }
     if (!grid_barrier(a.barrier, target, a.status, a.wait)) return;
@@ -103,7 +103,7 @@ __global__ void __launch_bounds__(kCrossThreads, 2) build_kernel(const ProposeAr
         const int it = NT - 1 - item / (a.B * RT), g = item % (a.B * RT) / RT, rt = item % RT;
         double c[2][4][2] = {};
         nt_tile(a.Ks + ((size_t)g * R + rt * 64) * npad, R - rt * 64, a.W + ((size_t)g * npad + it * 64) * npad, npad - it * 64,
-                npad, min(npad, it * 64 + 64), smem, c);
+                npad, min(npad, it * 64 + 64), smem, c, a.status);
         double* red = reinterpret_cast<double*>(smem);   // [2 column warps][64 rows]
 #pragma unroll
         for (int i = 0; i < 2; ++i) {
@@ -143,7 +143,7 @@ __global__ void __launch_bounds__(kCrossThreads, 2) build_kernel(const ProposeAr
                     const int row = ta * 64 + wm + 8 * i + l / 4, col = tb * 64 + wn + 8 * j + 2 * (l % 4) + h;
                     k0[i][j][h] = row < R && col < R ? __ldcg(C0 + (size_t)row * R + col) : 0.0;
                 }
-        nt_tile(Vg + (size_t)ta * 64 * npad, R - ta * 64, Vg + (size_t)tb * 64 * npad, R - tb * 64, npad, npad, smem, c);
+        nt_tile(Vg + (size_t)ta * 64 * npad, R - ta * 64, Vg + (size_t)tb * 64 * npad, R - tb * 64, npad, npad, smem, c, a.status);
 #pragma unroll
         for (int i = 0; i < 2; ++i)
 #pragma unroll
@@ -272,11 +272,11 @@ __global__ void __launch_bounds__(kPickThreads, 1) pick_kernel(const ProposeArra
         if (owner && r == j) picked = true;
         if (step + 1 == a.q) break;
         // ---- c(x) = C0(x, x_j) - sum_u c_u(x) c_u(x_j) / s_u
-        double c = owner ? C0[(size_t)j * R + r] : 0.0;
+        double c = owner ? C0[(size_t)R3_IDX(j, R, a.status) * R + r] : 0.0;
         const int jr = j / Rl, jl = j % Rl;
         const double* theirs = cluster.map_shared_rank(cols, jr);
         for (int u = t; u < step; u += kPickThreads)
-            sh.w[u] = (u < held ? theirs[(size_t)u * Rl + jl] : __ldcg(Cg + (size_t)u * R + j)) * sh.inv_s[u];
+            sh.w[u] = (u < held ? theirs[R3_IDX((size_t)u * Rl + jl, (size_t)held * Rl, a.status)] : __ldcg(Cg + (size_t)u * R + j)) * sh.inv_s[u];
         if (t == 0) sh.inv_s[step] = 1.0 / s;
         __syncthreads();
         double s0 = 0.0, s1 = 0.0;
@@ -294,7 +294,7 @@ __global__ void __launch_bounds__(kPickThreads, 1) pick_kernel(const ProposeArra
         __syncthreads();
         if (owner) {
             for (int p = 0; p < parts; ++p) c -= sh.part[p * Rl + mine];
-            if (step < held) cols[(size_t)step * Rl + mine] = c;
+            if (step < held) cols[R3_IDX((size_t)step * Rl + mine, (size_t)held * Rl, a.status)] = c;
             else Cg[(size_t)step * R + r] = c;
             mu = fma(c, delta, mu);
             var -= c * c / s;

@@ -160,7 +160,7 @@ __device__ __forceinline__ void rescue_tile(const GuardArgs& a, const double* __
     double c[2][4][2] = {};
     // W is lower triangular: columns up to the tile's last row
     nt_tile(Wg + (size_t)i0 * npad, npad - i0, a.ks + (size_t)R3_IDX(slot0, a.slab - (kTile - 1), a.status) * npad, kTile, npad,
-            min(npad, i0 + kTile), smem, c);
+            min(npad, i0 + kTile), smem, c, a.status);
     double* red = reinterpret_cast<double*>(smem);        // [4 row warps][64 candidates]
 #pragma unroll
     for (int j = 0; j < 4; ++j)
@@ -254,9 +254,9 @@ __device__ __forceinline__ bool rescue(const GuardArgs& a, const int* pref, int 
             cross_tile<CT>(
                 a.n, a.d, a.npad, a.ell + (size_t)g * a.d, (double)a.sf2v[g], a.alpha64 + (size_t)g * a.npad,
                 [&](int r) { return r < in_tile ? cand_row(a, g, __ldcg(list_g + r)) : nullptr; },
-                [&](int k) { return a.X + ((size_t)g * a.n + k) * a.d; }, kb, smem,
-                [&](int c, int k, double kv) { a.ks[(slot0 + c) * a.npad + k] = kv; },
-                [&](int c, double part) { a.mupart[(slot0 + c) * nb + kb] = part; });
+                [&](int k) { return a.X + ((size_t)g * a.n + R3_IDX(k, a.n, a.status)) * a.d; }, kb, smem,
+                [&](int c, int k, double kv) { a.ks[R3_IDX((slot0 + c) * a.npad + k, (size_t)a.slab * a.npad, a.status)] = kv; },
+                [&](int c, double part) { a.mupart[R3_IDX((slot0 + c) * nb + kb, (size_t)a.slab * nb, a.status)] = part; });
         }
         if (!grid_barrier(a.barrier, target, a.status, a.wait)) return false;
         for (int item = blockIdx.x; item < nt * row_tiles; item += gridDim.x) {   // the longest rows first
@@ -296,7 +296,7 @@ __device__ __forceinline__ void rescue_own(const GuardArgs& a, int g, const int*
         cross_tile<kSmallTile>(
             a.n, a.d, a.npad, a.ell + (size_t)g * a.d, (double)a.sf2v[g], a.alpha64 + (size_t)g * a.npad,
             [&](int r) { return r < count ? cand_row(a, g, own[r]) : nullptr; },
-            [&](int k) { return a.X + ((size_t)g * a.n + k) * a.d; }, kb, smem, [&](int c, int k, double kv) { ks[c * ld + k] = kv; },
+            [&](int k) { return a.X + ((size_t)g * a.n + R3_IDX(k, a.n, a.status)) * a.d; }, kb, smem, [&](int c, int k, double kv) { ks[R3_IDX(c * ld + k, kSmallTile * ld, a.status)] = kv; },
             [&](int c, double part) { mu_s[c] += part; });
     __syncthreads();
     const double* Wg = a.W64 + (size_t)g * a.npad * a.npad;
@@ -490,7 +490,7 @@ __device__ __forceinline__ bool guard_pool(const GuardArgs& a, unsigned char* sm
         }
         block_select_desc(keys_s, a.slice, a.K2, smem + a.select_offset);
         unsigned long long* out = a.keys + (size_t)s * a.K2;
-        for (int i = t; i < a.K2; i += kThreads) out[i] = keys_s[i];
+        for (int i = t; i < a.K2; i += kThreads) out[i] = keys_s[R3_IDX(i, a.slice, a.status)];
         if (a.finish) {
             __threadfence();
             __syncthreads();
@@ -527,7 +527,7 @@ __global__ void __launch_bounds__(kThreads, 2) guard_kernel(const GuardArgs a)
         for (int s = blockIdx.x; s < a.slices_per_gp * a.batch; s += gridDim.x) {
             const long long c0 = (long long)(s % a.slices_per_gp) * a.slice;
             for (int i = threadIdx.x; i < a.K2; i += kThreads)
-                a.keys[(size_t)s * a.K2 + i] = c0 + i < a.m ? topk_make_key(0.f, (unsigned)(c0 + i)) : 0ull;
+                a.keys[R3_IDX((size_t)s * a.K2 + i, (size_t)a.slices_per_gp * a.batch * a.K2, a.status)] = c0 + i < a.m ? topk_make_key(0.f, (unsigned)(c0 + i)) : 0ull;
         }
     }
 }

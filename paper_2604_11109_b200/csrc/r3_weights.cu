@@ -65,7 +65,7 @@ __device__ __forceinline__ void rows_pass(const WeightArgs& a, int g, int warp_i
         if (i < n) {
 #pragma unroll 8
             for (int k = 2 * lane; k <= i; k += 64) {   // the entry right of the diagonal is a stored zero
-                const double2 w = __ldcg(reinterpret_cast<const double2*>(Wr + k));
+                const double2 w = __ldcg(reinterpret_cast<const double2*>(Wr + R3_IDX(k, npad - 1, a.status)));
                 if (V) {
                     const double2 x = *reinterpret_cast<const double2*>(v + k);
                     s0 = fma(w.x, x.x, s0);
@@ -86,7 +86,7 @@ __device__ __forceinline__ void rows_pass(const WeightArgs& a, int g, int warp_i
                     const double2 w = __ldcg(reinterpret_cast<const double2*>(Wr + k));
                     f = make_float2((float)w.x, (float)w.y);
                 }
-                *reinterpret_cast<float2*>(o + k) = f;
+                *reinterpret_cast<float2*>(o + R3_IDX(k, npad - 1, a.status)) = f;
             }
         }
         double s = s0 + s1, t = t0 + t1;
@@ -114,7 +114,7 @@ __device__ __forceinline__ void columns_pass(const WeightArgs& a, int g, int j0,
     double2 s = make_double2(0.0, 0.0), q = s;
 #pragma unroll 8
     for (int i = j0 + w * 4 + l / 8; i < a.n; i += 4 * kWarps) {
-        const double2 x = __ldcg(reinterpret_cast<const double2*>(Wg + (size_t)i * npad));
+        const double2 x = __ldcg(reinterpret_cast<const double2*>(Wg + (size_t)R3_IDX(i, npad, a.status) * npad));
         if (V) {
             s.x = fma(x.x, u[i], s.x);
             s.y = fma(x.y, u[i], s.y);
@@ -221,12 +221,14 @@ __global__ void __launch_bounds__(kClusterThreads, 1) weights_cluster_kernel(con
     const int r = (int)cluster.block_rank(), g = blockIdx.x / R, threads = blockDim.x, warps = threads / 32;
     const int t = threadIdx.x, lane = t % 32, warp = t / 32, npad = a.npad, n = a.n, rows = npad / R, half = npad / 2;
     const int P = cluster_parts(npad), even = (r & ~1) + 2;
-    double *Ws = vec, *x = Ws + packed_doubles(npad, R), *shares = x + npad, *parts = shares + 2 * R * npad, *u = parts + P * npad;
+    const int packed = packed_doubles(npad, R);
+    double *Ws = vec, *x = Ws + packed, *shares = x + npad, *parts = shares + 2 * R * npad, *u = parts + P * npad;
     auto at = [&](int q) { return R / 2 * q * (q - 1) + q * even; };   // start of row R q + r: its length is even
     const double* Wg = a.W + (size_t)g * npad * npad;
     for (int q = warp; q < rows; q += warps)
         for (int c = lane; c <= (R * q + r) / 2; c += 32)
-            cp_async16(Ws + at(q) + 2 * c, Wg + (size_t)(R * q + r) * npad + 2 * c);
+            cp_async16(Ws + R3_IDX(at(q) + 2 * c, packed - 1, a.status),
+                       Wg + (size_t)R3_IDX(R * q + r, npad, a.status) * npad + R3_IDX(2 * c, npad - 1, a.status));
     cp_async_commit();
     for (int j = t; j < npad; j += threads) x[j] = j < n ? (double)a.y[(size_t)g * n + j] : 0.0;
     if (t == 0) {
@@ -248,7 +250,7 @@ __global__ void __launch_bounds__(kClusterThreads, 1) weights_cluster_kernel(con
             for (int c = lane; c < half; c += 32) {
                 float2 f = make_float2(0.f, 0.f);
                 if (c <= i / 2) {
-                    const double2 w = *reinterpret_cast<const double2*>(Ws + at(q) + 2 * c);
+                    const double2 w = *reinterpret_cast<const double2*>(Ws + R3_IDX(at(q) + 2 * c, packed - 1, a.status));
                     f = make_float2((float)w.x, (float)w.y);
                 }
                 if (i < n) top = fmaxf(top, fmaxf(fabsf(f.x), fabsf(f.y)));
@@ -285,7 +287,8 @@ __global__ void __launch_bounds__(kClusterThreads, 1) weights_cluster_kernel(con
             double s0 = 0.0, s1 = 0.0;
 #pragma unroll 4
             for (int k = t % 8; k <= m; k += 8) {
-                const double2 e = *reinterpret_cast<const double2*>(w + 2 * k), f = *reinterpret_cast<const double2*>(x + 2 * k);
+                const double2 e = *reinterpret_cast<const double2*>(w + R3_IDX(2 * k, packed - 1 - at(q), a.status)),
+                              f = *reinterpret_cast<const double2*>(x + R3_IDX(2 * k, npad - 1, a.status));
                 s0 = fma(e.x, f.x, s0);
                 s1 = fma(e.y, f.y, s1);
             }
@@ -305,8 +308,8 @@ __global__ void __launch_bounds__(kClusterThreads, 1) weights_cluster_kernel(con
             int off = off0, step = step0;
 #pragma unroll 4
             for (int q = q0; q < rows; q += P) {   // the rows from the diagonal on
-                const double2 e = *reinterpret_cast<const double2*>(Ws + off);
-                const double uq = u[q];
+                const double2 e = *reinterpret_cast<const double2*>(Ws + R3_IDX(off, packed - 1, a.status));
+                const double uq = u[R3_IDX(q, rows, a.status)];
                 s.x = fma(e.x, uq, s.x);
                 s.y = fma(e.y, uq, s.y);
                 off += step;

@@ -1,9 +1,10 @@
-"""The bounds-checking build of the library (``build.py --check``, ``-DR3_BOUNDS_CHECK``): the scoring, guard
-and top-k kernels verify their shared-memory, tensor-memory and global indices and report a violation through
-the handle's status instead of faulting.  It stands in for compute-sanitizer, which is not available where the
-library is developed.  The small element-by-element cases (several tiles, ragged tails in every dimension, both
-engines, multi-pass histories) run against that build in a child process: every result must still match the
-oracle and no index check may fire (a fired check makes ``r3_gp_check`` fail with the line of the check).
+"""The bounds-checking build of the library (``build.py --check``, ``-DR3_BOUNDS_CHECK``): the scoring kernels, the guard, the
+factorisation, the weights, the evidence and the proposal verify the indices of their operands and results (shared memory,
+tensor memory and global) and report a violation through a status word instead of faulting.  It stands in for
+compute-sanitizer, which is not available where the library is developed.  The small element-by-element cases (several
+tiles, ragged tails in every dimension, both engines, multi-pass histories) run against that build in a child process: every
+result must still match the oracle and no index check may fire (a fired check makes ``r3_gp_check``, or the fit or proposal
+it happened in, fail with the line of the check).  The selection's own kernels and the Parzen estimator have no checks.
 """
 import os
 import subprocess
@@ -39,5 +40,10 @@ def run_checked(files, sel):
     assert " passed" in r.stdout and "failed" not in r.stdout, tail
 
 
-def test_evidence_under_the_bounds_checking_build():
-    run_checked(["test_gpu_lml.py"], "random_problems or half_empty")
+@pytest.mark.parametrize("files,sel", [
+    (["test_gpu_lml.py"], "random_problems or half_empty"),
+    (["test_gpu_factor.py", "test_gpu_append.py"], "edges or weights or append"),
+    (["test_gpu_propose.py", "test_gpu_rescue.py"], "propos or greedy or pick or recomputed"),
+])
+def test_fits_evidence_proposals_and_rescues_under_the_bounds_checking_build(files, sel):
+    run_checked(files, sel)
