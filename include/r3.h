@@ -151,7 +151,10 @@ r3_status_t r3_topk_noalloc(const float* ei, int batch, long long m, int k, int*
  * the handle's own workspace; asynchronous on `cuda_stream`.  This is the "one
  * BO proposal round" call: idx [batch][k] are the pool members to replay next.
  * The first level of the selection is taken by the accuracy guard's kernel, which
- * runs over the final EI anyway, so a step is four or five kernel launches.  Once
+ * runs over the final EI anyway and finishes small pools by itself.  A step is two
+ * kernel launches on the tensor engine (five for histories of more than 1792
+ * observations), two per GP and one more on the CUDA-core engine, and one or two
+ * more where the guard's slices leave over 4096 keys.  Once
  * the workspace has its size (a first call with this m and k) the call only
  * enqueues work on `cuda_stream` and can be captured in a CUDA graph.
  */
@@ -260,8 +263,9 @@ r3_status_t r3_gp_lml(r3_gp_t* gp, double* lml, double* grad, void* cuda_stream)
 /*
  * r3_gp_refit -- condition the GPs of the handle on the same histories with other hyper-parameters
  * (arguments as for r3_gp_fit; the histories are the ones the handle holds, appended observations
- * included).  Synchronises.  On R3_ERR_NOT_PD the handle is refitted with its previous
- * hyper-parameters and stays usable.
+ * included).  Synchronises.  On any error the handle is refitted with its previous hyper-parameters and stays
+ * usable; if that fails too (r3_last_error says so), calls that need a fit return R3_ERR_INVALID_ARG until a refit
+ * succeeds.  What earlier calls have latched stays for r3_gp_check.
  */
 r3_status_t r3_gp_refit(r3_gp_t* gp, const float* lengthscales, const float* signal_var, const float* noise_var,
                         void* cuda_stream);
@@ -286,7 +290,7 @@ r3_status_t r3_gp_refit(r3_gp_t* gp, const float* lengthscales, const float* sig
  *   evals        host [1]       evaluations used, or NULL
  *
  * On return the handle is fitted with the returned hyper-parameters (never worse than the start).
- * Synchronises.
+ * Synchronises.  On an error the handle is left as r3_gp_refit leaves it.
  */
 r3_status_t r3_gp_optimize(r3_gp_t* gp, int max_evals, double gtol, float* lengthscales, float* signal_var,
                            float* noise_var, double* lml, int* evals, void* cuda_stream);
@@ -490,7 +494,7 @@ r3_status_t r3_tpe_get_model(r3_tpe_t* tpe, int* n_good, int* order, float* comp
 void r3_tpe_free(r3_tpe_t* tpe);
 
 /*
- * Device memory the library has freed is kept (per device, at most 2 GiB, blocks of 1 MiB and more) and
+ * Device memory the library has freed is kept (per device, at most 2 GiB and 4096 blocks of any size) and
  * handed out again by later calls, because allocating and freeing the 100 MB arrays of a fit costs more
  * than the kernels of an append.  r3_trim_cache returns the kept blocks of the current device to the
  * driver; r3_cached_bytes reports how much is kept.

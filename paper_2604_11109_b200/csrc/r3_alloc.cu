@@ -5,8 +5,9 @@
 // kernels of an append -- so freed blocks are kept, per device, and handed out again.  Sizes are
 // rounded up to five significant bits so that neighbouring sizes (a history that grew by a few
 // rows) share a bin; blocks below 1 MiB -- a small history's fit is two dozen of them, and their cudaMalloc and
-// cudaFree calls were most of its time -- are rounded up to a multiple of 512 bytes and kept as well.  dev_free waits for the device like cudaFree does, which makes the block safe to
-// reuse at once.  The cache holds at most kCacheLimit bytes per device: a block that would go over the limit pushes out
+// cudaFree calls were most of its time -- are rounded up to a multiple of 512 bytes and kept as well.  dev_free waits for the device like cudaFree does, which makes the block
+// safe to reuse at once; inside a FreeScope it does not, because whoever opened that knows that nothing in flight uses the
+// block any more.  The cache holds at most kCacheLimit bytes per device: a block that would go over the limit pushes out
 // the ones that have lain there longest (a program whose sizes change would otherwise fill the cache with sizes it no
 // longer asks for, and pay the driver for every block from then on).  r3_trim_cache() returns everything to the driver.
 #include <list>

@@ -21,8 +21,10 @@
 // share out (64 rows of W) x (64 candidates) tiles that run on the FP64 tensor path.  Few listed candidates (less
 // than two tiles per block) get 16 x 16 tiles instead, whose reductions the block's eight warps split, so that W is
 // read once by the whole GPU.  With at most 128 observations a block recomputes the first 16 it flags in a slice by
-// itself, which saves a small call the barriers (64 observations, 4096 candidates: 27.7 us to 19.8 us; with 256 the rows
-// of W cost one block more than the barriers: 45.8 us against 32.9 us).
+// itself, which saves a small call the barriers.  Whole calls, by the flagging block and by all blocks, on 4096 and on 65,536
+// candidates of 16 features: 64 observations 37.1 | 43.6 and 70.2 | 76.4 us, 96 (none and 15 flagged) 30.9 | 31.1 and
+// 72.3 | 74.9, 128 45.6 | 47.7 and 79.2 | 82.2, 160 51.4 | 49.7 and 98.9 | 96.9, 192 51.8 | 49.7 and 107.0 | 104.9,
+// 256 59.5 | 51.7 and 127.5 | 117.4.  (A pool of which a third is flagged loses a little at 96: 65.0 | 60.8.)
 // Bound: the FP64 rate for long lists, one read of W otherwise.  Measured, before (the block that met a flagged candidate
 // recomputed it alone, four at a time) and now: 65,536 candidates at n = 4096, most of them listed, 300-600 ms and
 // 36 ms (31 TFLOP/s of FP64); 2222 candidates at n = 701 1.50 ms and 0.14 ms; one pool of 262,144 with four listed
