@@ -153,8 +153,8 @@ r3_status_t r3_topk_noalloc(const float* ei, int batch, long long m, int k, int*
  * The first level of the selection is taken by the accuracy guard's kernel, which
  * runs over the final EI anyway and finishes small pools by itself.  A step is two
  * kernel launches on the tensor engine (five for histories of more than 1792
- * observations), two per GP and one more on the CUDA-core engine, and one or two
- * more where the guard's slices leave over 4096 keys.  Once
+ * observations), two per GP and slab of its pool and one more on the CUDA-core
+ * engine, and one or two more where the guard's slices leave over 4096 keys.  Once
  * the workspace has its size (a first call with this m and k) the call only
  * enqueues work on `cuda_stream` and can be captured in a CUDA graph.
  */
