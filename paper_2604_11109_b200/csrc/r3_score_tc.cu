@@ -2,17 +2,15 @@
 // accumulation in TMEM), operands staged by bulk asynchronous copies, everything fused in one kernel
 // so that the cross-covariance k* never leaves the SM.
 //
-// One CTA owns a tile of 128 candidates; a TMEM lane IS a candidate.  For that tile it walks the rows
-// of W = L^-1 in passes of NV rows (the V accumulator: 128 lanes x NV TMEM columns) and, inside a pass,
-// the observations in chunks of KC = 32:
+// One CTA owns a tile of 128 candidates; a TMEM lane IS a candidate.  For that tile it walks the rows of W = L^-1 in strips
+// of 128 (a V accumulator: 128 lanes x 128 TMEM columns) and, for a strip, the observations in chunks of KC = 32:
 //
-//   distance MMA   D[cand][k] = z~ . x~_k   (A = scaled candidates, kept in TMEM for the whole tile;
-//                  B = scaled observations, depth d), for KD observations at a time
-//   Matern warps   r^2 = |z~|^2 + |x~_k|^2 - 2 D, k* = sf2 M52(r): read D from TMEM, write k* (scaled,
-//                  FP16 hi/lo planes) as the next A operand into TMEM or shared memory; mu += k* alpha
-//                  on the way
+//   distance MMA   D[cand][k] = z~ . x~_k   (A = scaled candidates, B = scaled observations, both in shared memory, depth d),
+//                  for 64 observations at a time
+//   Matern warps   r^2 = |z~|^2 + |x~_k|^2 - 2 D, k* = sf2 M52(r): read D from TMEM and write k* (scaled, FP16 hi/lo planes)
+//                  over it, where it is the next A operand; mu += k* alpha on the way
 //   variance MMA   V[cand][i] += k*[cand][k] W[i][k]   (B = pre-tiled chunk of W, scaled FP16 hi/lo planes)
-//   end of pass    q += sum_i V[cand][i]^2 read back from TMEM; after the last pass sigma, EI, outputs
+//   end of strip   q += sum_i V[cand][i]^2 read back from TMEM; after the last strip sigma, EI, outputs
 //
 // Precision.  Every product is three MMAs (hi*hi + hi*lo + lo*hi): x = hi + lo with hi = fp16(x) and
 // lo = fp16(x - hi) carries 22 significant bits, and the tensor core accumulates in FP32, so the
@@ -21,17 +19,27 @@
 // scaled back exactly.  The scaled coordinates of the distance product must fit FP16's range; a
 // history that does not is left to the SIMT engine and a candidate that does not is recomputed in FP64.
 //
-// W is lower-triangular, so pass p only needs k < (p+1) NV; k* chunks are regenerated for every pass
-// they take part in instead of being stored.
+// W is lower-triangular, so strip s only needs k < 128 (s + 1).  Strips come in pairs that share the k* chunks; from pair to
+// pair the chunks are generated again instead of being stored.
 //
-// Warp roles: warp 0 streams the operands (lane 0: scaled observations, lane 1: chunks of W), warp 1
-// issues the distance MMAs, warp 2 issues the variance MMAs and owns the TMEM allocation (one thread
-// each), warps 4.. form G Matern/epilogue groups of four warps (one warp per TMEM lane quarter); group
-// g takes every G-th chunk; the k* buffers are one per group (shared memory) or a ring of two shared by
-// the groups (TMEM, where columns are scarce; a group that has computed its chunk keeps it in registers
-// until its slot is free).  Stages are handed over through mbarriers; every wait is bounded: when a limit is hit the
-// CTA raises a status bit, all roles leave their loops, in-flight copies and MMAs are drained (bounded
+// What the layout is for: nothing waits for a whole pass or a whole tile.  The two accumulators are filled by issuers of their
+// own, so that one is read back while the other's products run; the ring of eight k* slots and the second buffer of scaled
+// candidates let the next pair's and the next tile's chunks be made meanwhile; candidates come in and results go out through
+// warps of their own, not through the Matern warps.  TMEM: two accumulators (256 columns) and the ring (8 x 32), all 512.
+// A tile of 512 observations and 32 features takes 33,000 cycles (48,700 as passes of 256 rows with one accumulator, whose
+// Matern warps also brought the candidates in and read the accumulator back); its MMAs alone take 16,400.
+//
+// Warp roles: warp 0 streams the operands (three lanes: scaled observations, chunks of W for either accumulator), warp 1
+// issues the distance MMAs, warps 2 and 3 the variance MMAs of one accumulator each (the issuing roles are whole warps, see
+// mbar_wait_warp); two groups of four warps bring candidates in and results out; three groups of four Matern warps (one warp
+// per TMEM lane quarter) take every third chunk each.  Stages are handed over through mbarriers; every wait is bounded: when
+// a limit is hit the CTA raises a status bit, all roles leave their loops, in-flight copies and MMAs are drained (bounded
 // again), TMEM is freed and the kernel returns.
+//
+// The roles' code has to stay small: together it is about what the SM's instruction cache holds, and what does not fit costs
+// the Matern warps first.  Both halves of a chunk unrolled, norms and weights through shared memory (one more wait in the
+// loop), waits with a long form of their time-out: each of them raised the cache's misses from 0.5 M to 1.4-1.7 M per million
+// candidates' worth of tiles and the kernel's time by 19-27 % (64 pools of 65,536 candidates, 512 observations).
 //
 // Operand layouts are the no-swizzle K-major "core matrix" form: 8 rows x 16 bytes contiguous, 8-row
 // groups 128 bytes apart, 16-byte k-slices one full panel apart.  W and the observations are stored
@@ -51,129 +59,276 @@ namespace r3 {
 
 namespace {
 
+constexpr int kStrip = 128;              // rows of W per accumulator
+constexpr int kSlots = 8;                // ring of k* slots of KC tensor-memory columns
+constexpr uint32_t kRingCol = 2 * kStrip;
+constexpr int kMaxWS = 8, kMaxXS = 3;    // stages of W (half for each accumulator) and of scaled observations
+constexpr int KDC = 2, KD = KDC * KC;    // chunks and observations per distance product, which fills a bank of slots
+constexpr int BANKS = kSlots / KDC;
+constexpr int IO = 2, G = 3;             // groups of four warps: candidates in and results out, Matern
+constexpr int kFirstIo = 4, kFirstMatern = kFirstIo + 4 * IO, kThreads = kFirstMatern * 32 + 128 * G;
+constexpr int kZ32MaxDP = 32;            // features up to which the scaled tile is kept in FP32 too
+constexpr int kPartDP = 64;              // features per stage of scaled observations at most
+
+// barrier slots (8 bytes each)
+enum : uint32_t {
+    BAR_X_FULL = 0, BAR_X_EMPTY = BAR_X_FULL + kMaxXS, BAR_W_FULL = BAR_X_EMPTY + kMaxXS, BAR_W_EMPTY = BAR_W_FULL + kMaxWS,
+    BAR_D_FULL = BAR_W_EMPTY + kMaxWS, BAR_K_EMPTY = BAR_D_FULL + 4, BAR_K_FULL = BAR_K_EMPTY + 4,
+    BAR_V_FULL = BAR_K_FULL + kSlots,   // [accumulator][group that reads it back]
+    BAR_V_EMPTY = BAR_V_FULL + 4, BAR_Z_FULL = BAR_V_EMPTY + 2, BAR_Z_EMPTY = BAR_Z_FULL + 2,
+    BAR_RED_FULL = BAR_Z_EMPTY + 2, BAR_RED_EMPTY = BAR_RED_FULL + 2, BAR_MMA_DONE = BAR_RED_EMPTY + 2,   // MMA_DONE: three, distance and variance issuers
+    BAR_COUNT = BAR_MMA_DONE + 3
+};
+constexpr uint32_t kFlagOffset = 512;    // behind the barriers: int abort, int drain-abort, uint32 tmem base, int last
+static_assert(BAR_COUNT * 8 <= kFlagOffset, "barriers overlap the flags");
+constexpr uint32_t kBarBytes = 1024;
+// Registers per thread once the roles have parted; the block starts with the file split evenly (80 for 768 threads).
+constexpr int kRegsControl = 48, kRegsIo = 80, kRegsMatern = 88;
+static_assert(kRegsControl + IO * kRegsIo + G * kRegsMatern <= 80 * (kThreads / 128), "more registers than the block starts with");
+
+// per buffer of scaled candidates: float[128] squared norms, float[128] thresholds of close pairs, then the tile's scale of
+// k*, 1 / (the power of two in it) and GP
+constexpr uint32_t kZnBuf = TILE_M * 8u + 16u;
+
 // shared-memory map (byte offsets from a 1024-aligned base)
 struct SmemMap {
-    uint32_t z, k, x, w, zs, bar;   // z: reduction scratch; k: k* buffers (absent when k* lives in TMEM); zs: see kZsStride
-    uint32_t x_stage, w_stage;
+    uint32_t z, z32, x, w, red, zn, cache, bar, end;
+    uint32_t z_buf, z32_buf, red_buf, x_stage;
 };
-// With at most 16 (padded) features the scaled candidates of the tile are also kept in FP32 in shared memory,
-// 128 rows of kZsStride floats (the odd stride keeps a warp's 32 rows on 32 banks): close pairs then get their
-// squared distance from direct differences inline, without the out-of-line refinement and its round trips.
-constexpr uint32_t kZsStride = 17;
-constexpr int kZsMaxDP = 16;
-// Registers per thread after the roles have parted: the kernel starts with the register file split evenly
-// (128 per thread for 512 threads, 168 for 384); the four control warps, whose loops are short, give theirs back
-// and the Matern groups, whose chunk loop does not fit 128 without spills, take them.
-constexpr int kRegsControl = 80;
-__host__ __device__ constexpr int regs_matern(int G) { return G == 3 ? 144 : 208; }
-__host__ __device__ inline SmemMap smem_map(int DP, int NV, int G, int KD, int ws, bool kt)
+__host__ __device__ inline SmemMap smem_map(int DP, int parts, int zb, int xs, int ws)
 {
     SmemMap s;
-    s.z = 0;                                       // end-of-tile reduction scratch: G x 128 rows x 4 doubles
-    s.k = (uint32_t)G * 4096u;                     // k* in shared memory: G buffers x 2 planes x [KC/8][128][8] halves
-    s.x = s.k + (kt ? 0u : (uint32_t)G * 16384u);  // XS stages x 2 planes x [DP/8][KD][8] halves
-    s.x_stage = 2u * DP * KD * 2u;
-    s.w = s.x + (uint32_t)XS * s.x_stage;          // ws stages x 2 planes x [KC/8][NV][8] halves
-    s.w_stage = 2u * KC * NV * 2u;
-    s.zs = s.w + (uint32_t)ws * s.w_stage;
-    s.bar = s.zs + (DP <= kZsMaxDP ? TILE_M * kZsStride * 4u : 0u);
+    s.z_buf = 512u * DP;                                  // scaled candidates: FP16 hi plane, lo plane, [DP/8][128][8] each
+    s.z32_buf = DP <= kZ32MaxDP ? 512u * DP : 0u;         // the same in FP32, [DP/4][128][4]
+    s.x_stage = 4u * (DP / parts) * KD;                   // scaled observations: two planes [DP/parts/8][KD][8]
+    s.z = 0;
+    s.z32 = s.z + zb * s.z_buf;
+    s.x = s.z32 + zb * s.z32_buf;
+    s.w = s.x + xs * s.x_stage;                           // chunks of W: two planes [KC/8][rows][8]
+    s.red = s.w + ws * (4u * KC * kStrip);                // per group and row: mu (double), two error scales (float)
+    s.red_buf = (uint32_t)G * TILE_M * 16u;
+    s.zn = s.red + zb * s.red_buf;            // see kZnBuf
+    s.cache = s.zn + 2u * kZnBuf;                    // refined close pairs of the tile (see refine_close_pairs)
+    s.bar = s.cache + (DP <= kZ32MaxDP ? 0u : TILE_M * kCacheSlots * 8u);
+    s.end = s.bar + kBarBytes;
     return s;
 }
-// barriers, flags, TMEM slot, candidate norms; then the tile's cache of refined close pairs
-constexpr uint32_t kCacheOffset = 1024;
-constexpr uint32_t kBarBytes = kCacheOffset + TILE_M * kCacheSlots * 8;
 
-// barrier slots (8 bytes each) inside the barrier block
-enum : uint32_t {
-    BAR_X_FULL = 0, BAR_X_EMPTY = 2, BAR_W_FULL = 4, BAR_W_EMPTY = 10, BAR_D_FULL = 16, BAR_D_EMPTY = 18,
-    BAR_K_FULL = 20, BAR_K_EMPTY = 24, BAR_V_FULL = 28, BAR_V_EMPTY = 29, BAR_Z_READY = 30, BAR_RED_READY = 31,
-    BAR_MMA_DONE = 32,  // two slots: distance issuer, variance issuer
-    BAR_COUNT = 34
-};
-constexpr uint32_t kFlagOffset = BAR_COUNT * 8;       // int abort, int drain-abort, uint32 tmem base
-constexpr uint32_t kZnOffset = 512;                   // float[128] squared norms of the scaled candidates
-
-
-// NV: rows of W per pass (TMEM columns of the V accumulator).  G: number of Matern warp groups; group
-// g owns chunks t = g (mod G) and k* buffer g.  KD: observations per distance product.  KT: the k*
-// buffers (A operand of the variance product) live in TMEM instead of shared memory: shared memory then
-// only feeds the B operands, which is what keeps its 128 B/clk from becoming the limit.
-// NBK: number of k* buffers.  NBK == G: group g owns buffer g.  NBK < G (k* in TMEM, where columns are
-// scarce): the buffers form a ring shared by the groups, chunk t uses buffer t mod NBK; a group that has
-// computed its chunk keeps it in registers until the ring slot is free, so the groups still run ahead.
-// F8: the two cross terms of the variance product (W_hi k_lo, W_lo k_hi) are single FP8 MMAs of depth 32
-// instead of two FP16 MMAs of depth 16 each: four MMAs per chunk instead of six.
-// PUTOFF: a pass's epilogue (read the accumulator back, hand it over) is put off until the group's first chunk of
-// the next pass is on its way, when that chunk can be handed over without the accumulator's release (its k* slot is
-// freed by chunks of the old pass): the MMA issuer then finds the new pass's first chunks waiting when the
-// accumulator is released, instead of waiting for them to be computed after it.  With few passes per tile the
-// refill after a hand-over is a visible part of a tile (4-6 % on histories of two to four passes); with many it is
-// not, and the loop structure it needs costs the long histories more than it saves, hence a kernel variant.
-// ZS: the feature count is at most 16: close pairs are refined inline from the FP32 copy of the scaled tile in
-// shared memory (pools of few features are full of close pairs: on the 16-feature workload 98 % of a warp's
-// 16-entry blocks hold one, and the out-of-line refinement was most of the kernel's time).
-template <int NV, int G, int KD, bool KT, int NBK = G, bool F8 = false, bool PUTOFF = false, bool ZS = false>
-__global__ void __launch_bounds__(128 + 128 * G, 1) score_tc_kernel(const TcParams prm)
+// two FP32 lanes in one 64-bit register pair
+__device__ __forceinline__ uint64_t pack2(float lo, float hi)
 {
-    static_assert(NBK == G || (KT && NBK >= 2 && NBK < G), "ring of k* buffers: TMEM only");
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ void unpack2(uint64_t v, float& lo, float& hi) { asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v)); }
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b)
+{
+    uint64_t r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b)
+{
+    uint64_t r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c)
+{
+    uint64_t r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+// a - h exactly, in one mixed-precision instruction
+__device__ __forceinline__ float minus_half(float a, __half h)
+{
+    float r;
+    asm("fma.rn.f32.f16 %0, %1, %2, %3;" : "=f"(r) : "h"(__half_as_ushort(h)), "h"((unsigned short)0xbc00), "f"(a));
+    return r;
+}
+__device__ __forceinline__ void tc_st16(uint32_t taddr, const uint32_t* r)
+{
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};" ::"r"(taddr),
+                 "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]), "r"(r[9]),
+                 "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])
+                 : "memory");
+}
+
+// The strips (128 rows of W) of a tile come in pairs that share the k* chunks.  Strip a = 2 p needs the first `na` chunks of
+// the history, strip a + 1, where there is one, the first `nb`.
+struct Pair {
+    int a, na, nb;   // nb = 0: a single strip
+    __device__ __forceinline__ Pair(int p, int S, int nc) : a(2 * p), na(min(4 * (a + 1), nc)), nb(a + 1 < S ? min(4 * (a + 2), nc) : 0) {}
+    __device__ __forceinline__ int chunks() const { return nb ? nb : na; }
+};
+
+// Waits and issue for a role that is a whole warp: every lane takes the same path, so that operand addresses and descriptors
+// are computed on the uniform datapath (a role of one lane spent 450 cycles per chunk moving them there, as long as the
+// products took); the instructions that one thread has to issue are predicated on the elected lane.
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile int* abort_flag, long long limit)
+{
+    if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+    const long long t0 = clock64();
+    do {
+        if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+    } while (!__any_sync(0xffffffffu, (*abort_flag != 0) | (clock64() - t0 > limit)));
+    *abort_flag = 1;
+    return false;
+}
+__device__ __forceinline__ uint32_t elect_one()
+{
+    uint32_t r;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(r));
+    return r;
+}
+__device__ __forceinline__ void tc_commit_if(uint32_t leader, uint32_t bar)
+{
+    asm volatile(
+        "{\n\t.reg .pred e;\n\tsetp.ne.b32 e, %1, 0;\n\t"
+        "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(bar), "r"(leader)
+        : "memory");
+}
+__device__ __forceinline__ void tc_mma_f16_if(uint32_t leader, uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accumulate)
+{
+    asm volatile(
+        "{\n\t.reg .pred p, e;\n\tsetp.ne.b32 p, %4, 0;\n\tsetp.ne.b32 e, %5, 0;\n\t"
+        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc),
+        "r"(accumulate), "r"(leader)
+        : "memory");
+}
+__device__ __forceinline__ void tc_mma_f16_ts_if(uint32_t leader, uint32_t d_tmem, uint32_t a_tmem, uint64_t bdesc, uint32_t idesc, uint32_t accumulate)
+{
+    asm volatile(
+        "{\n\t.reg .pred p, e;\n\tsetp.ne.b32 p, %4, 0;\n\tsetp.ne.b32 e, %5, 0;\n\t"
+        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}" ::"r"(d_tmem), "r"(a_tmem), "l"(bdesc), "r"(idesc),
+        "r"(accumulate), "r"(leader)
+        : "memory");
+}
+__device__ __forceinline__ void tc_mma_f8_ts_if(uint32_t leader, uint32_t d_tmem, uint32_t a_tmem, uint64_t bdesc, uint32_t idesc, uint32_t accumulate)
+{
+    asm volatile(
+        "{\n\t.reg .pred p, e;\n\tsetp.ne.b32 p, %4, 0;\n\tsetp.ne.b32 e, %5, 0;\n\t"
+        "@e tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], [%1], %2, %3, p;\n\t}" ::"r"(d_tmem), "r"(a_tmem), "l"(bdesc), "r"(idesc),
+        "r"(accumulate), "r"(leader)
+        : "memory");
+}
+__device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity)
+{
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    return ok != 0;
+}
+
+// Close pairs of a candidate row with the scaled tile in shared memory as FP16 planes: k* recomputed from direct differences.
+// Out of line; per lane, one pair at a time.  z: this row's 16 bytes of the first slice of the hi plane.
+__device__ __noinline__ void refine_close_pairs_smem(float* kv, float v_thresh, float kvscale, const uint8_t* z, int DP,
+                                                     const float* __restrict__ xrow0, unsigned long long* slots, uint32_t key0,
+                                                     bool lookup)
+{
+    uint32_t close = 0;
+#pragma unroll
+    for (int i = 0; i < 16; ++i) close |= (kv[i] > v_thresh) ? (1u << i) : 0u;
+    const uint32_t lo_plane = 256u * DP;
+    for (uint32_t rest = close; rest; rest &= rest - 1) {
+        const int i = __ffs(rest) - 1;
+        if (slots && lookup) {
+            const unsigned long long e = slots[cache_slot(key0 + i)];
+            if ((uint32_t)(e >> 32) == key0 + i) {
+                kv[i] = __uint_as_float((uint32_t)e);
+                continue;
+            }
+        }
+        const float4* xp = reinterpret_cast<const float4*>(xrow0 + (size_t)i * DP);
+        float acc0 = 0.f, acc1 = 0.f;
+#pragma unroll 2
+        for (int j8 = 0; j8 < DP / 8; ++j8) {
+            const uint4 zh = *reinterpret_cast<const uint4*>(z + j8 * 2048u);
+            const uint4 zl = *reinterpret_cast<const uint4*>(z + lo_plane + j8 * 2048u);
+            const float4 xa = __ldg(xp + 2 * j8), xb = __ldg(xp + 2 * j8 + 1);
+            const float x[8] = {xa.x, xa.y, xa.z, xa.w, xb.x, xb.y, xb.z, xb.w};
+            const uint32_t h[4] = {zh.x, zh.y, zh.z, zh.w}, l[4] = {zl.x, zl.y, zl.z, zl.w};
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const float2 a = __half22float2(*reinterpret_cast<const __half2*>(&h[e]));
+                const float2 b = __half22float2(*reinterpret_cast<const __half2*>(&l[e]));
+                float df = (a.x + b.x) - x[2 * e];
+                acc0 = fmaf(df, df, acc0);
+                df = (a.y + b.y) - x[2 * e + 1];
+                acc1 = fmaf(df, df, acc1);
+            }
+        }
+        const float u = sqrtf(acc0 + acc1);
+        kv[i] = kvscale * fmaf(u, fmaf(u, kPolyC2, kPolyC1), 1.f) * exp2f(-u);
+        if (slots) slots[cache_slot(key0 + i)] = ((unsigned long long)(key0 + i) << 32) | __float_as_uint(kv[i]);
+    }
+}
+
+// F8: the two cross terms of the variance product (W_hi k_lo, W_lo k_hi) are single FP8 MMAs of depth 32 instead of two FP16
+// MMAs of depth 16 each: four MMAs per chunk and strip instead of six.
+// Z32: at most 32 features: the scaled candidates are also kept in FP32 and close pairs are refined inline from them (pools of
+// few features are full of close pairs: on 16 features 98 % of a warp's 16-entry blocks hold one).
+template <bool F8, bool Z32>
+__global__ void __launch_bounds__(kThreads, 1) score_tc_kernel(const __grid_constant__ TcParams prm)
+{
     if (prm.mode && *prm.mode != prm.want_mode) return;   // the other form of the kernel serves this pool
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw = smem_u32(smem_raw);
     const uint32_t base = (raw + 1023u) & ~1023u;
     uint8_t* sm = smem_raw + (base - raw);
-    const SmemMap map = smem_map(prm.DP, NV, G, KD, prm.ws, KT);
+    const int DP = prm.DP, parts = prm.parts, DPp = DP / parts, nc = prm.nc, S = prm.S;
+    const int zb = prm.zb, xs = prm.xs, ws = prm.ws;
+    const SmemMap map = smem_map(DP, parts, zb, xs, ws);
     const uint32_t bars = base + map.bar;
     volatile int* abort_flag = reinterpret_cast<volatile int*>(sm + map.bar + kFlagOffset);
     volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(sm + map.bar + kFlagOffset + 8);
-    float* zn_s = reinterpret_cast<float*>(sm + map.bar + kZnOffset);
-    unsigned long long* pair_cache = reinterpret_cast<unsigned long long*>(sm + map.bar + kCacheOffset);
-    float* zs_s = reinterpret_cast<float*>(sm + map.zs);
+    volatile int* last_flag = reinterpret_cast<volatile int*>(sm + map.bar + kFlagOffset + 12);
+    auto zn_buf = [&](int b) { return reinterpret_cast<float*>(sm + map.zn + b * kZnBuf); };
     auto bar = [&](uint32_t slot) { return bars + slot * 8u; };
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    constexpr int CPP = NV / KC;                  // chunks per pass width
-    constexpr int SL = KD / KC;                   // chunks per distance product
-    // TMEM columns: V accumulator [0, NV), two distance buffers [NV, NV + 2 KD), scaled candidates
-    // (FP16 hi plane, then lo plane, DP/2 columns each) from NV + 2 KD, then (KT) G k* buffers of
-    // 2 planes x KC/2 columns
     constexpr uint32_t TMEM_COLS = 512u;
-    constexpr uint32_t ZCOL = NV + 2 * KD;
-    const uint32_t KCOL = ZCOL + (uint32_t)prm.DP;
-    const int DP = prm.DP, P = prm.P, ws = prm.ws;
     const long long wl = prm.wait_limit;
 
     if (threadIdx.x == 0) {
-        for (int i = 0; i < XS; ++i) {
+        for (int i = 0; i < kMaxXS; ++i) {
             mbar_init(bar(BAR_X_FULL + i), 1);
             mbar_init(bar(BAR_X_EMPTY + i), 1);
-            mbar_init(bar(BAR_D_FULL + i), 1);
-            mbar_init(bar(BAR_D_EMPTY + i), 128 * SL);
         }
-        for (int i = 0; i < MAX_STAGES; ++i) {
+        for (int i = 0; i < kMaxWS; ++i) {
             mbar_init(bar(BAR_W_FULL + i), 1);
             mbar_init(bar(BAR_W_EMPTY + i), 1);
         }
         for (int i = 0; i < 4; ++i) {
-            mbar_init(bar(BAR_K_FULL + i), 128);
-            mbar_init(bar(BAR_K_EMPTY + i), 1);
+            mbar_init(bar(BAR_D_FULL + i), 1);
+            mbar_init(bar(BAR_K_EMPTY + i), 2);
         }
-        mbar_init(bar(BAR_V_FULL), 1);
-        mbar_init(bar(BAR_V_EMPTY), 128 * G);
-        mbar_init(bar(BAR_Z_READY), 128);
-        mbar_init(bar(BAR_RED_READY), 128 * G);
-        mbar_init(bar(BAR_MMA_DONE), 1);
-        mbar_init(bar(BAR_MMA_DONE + 1), 1);
+        for (int i = 0; i < kSlots; ++i) mbar_init(bar(BAR_K_FULL + i), 4);
+        for (int i = 0; i < 2; ++i) {
+            mbar_init(bar(BAR_V_FULL + i), 1);
+            mbar_init(bar(BAR_V_FULL + 2 + i), 1);
+            mbar_init(bar(BAR_V_EMPTY + i), 4);
+            mbar_init(bar(BAR_RED_FULL + i), 4 * G);
+            mbar_init(bar(BAR_RED_EMPTY + i), 4);
+            mbar_init(bar(BAR_Z_FULL + i), 4);
+            mbar_init(bar(BAR_Z_EMPTY + i), 1 + 4 * G);
+        }
+        for (int i = 0; i < 3; ++i) mbar_init(bar(BAR_MMA_DONE + i), 1);
         abort_flag[0] = 0;
         abort_flag[1] = 0;   // private flag of the bounded drain waits
-    }
-    if (threadIdx.x < TILE_M * kCacheSlots / 4) {   // no entry yet: a key that no (tile, observation) forms
-        for (int i = 0; i < 4; ++i) pair_cache[threadIdx.x * 4 + i] = ~0ull;
-    }
-    if (threadIdx.x == 0) {
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    // The guard's counters.  Not here with FP8 cross terms: the pilot clears them, and these few instructions cost that
-    // kernel, which the board's power limits, 0.6 % (1,048,576 candidates at n = 4096: 43.4 ms, 43.7 ms with them).
+    if (!Z32) {
+        unsigned long long* pair_cache = reinterpret_cast<unsigned long long*>(sm + map.cache);
+        for (int i = threadIdx.x; i < TILE_M * (int)kCacheSlots; i += blockDim.x) pair_cache[i] = ~0ull;   // a key that no (tile, observation) forms
+    }
+    // the guard's counters (with FP8 cross terms the pilot clears them)
     if constexpr (!F8)
         if (blockIdx.x == 0)
             for (int i = threadIdx.x; i < prm.zero_ints; i += blockDim.x) prm.zero[i] = 0;
@@ -190,338 +345,274 @@ __global__ void __launch_bounds__(128 + 128 * G, 1) score_tc_kernel(const TcPara
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
 
-    // tiles of this CTA: blockIdx.x, blockIdx.x + gridDim.x, ...
-    const long long first_tile = prm.tile_begin + blockIdx.x, tile_step = gridDim.x;
-    const int items_per_tile = CPP * P * (P + 1) / 2;
-    long long tacc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-    long long tlast = prm.trace ? clock64() : 0;
+    // units of this CTA: blockIdx.x, blockIdx.x + gridDim.x, ...; a unit is the pairs [cut[part], cut[part + 1]) of a tile
+    const int tiles = (int)(prm.total_tiles - prm.tile_begin), units = tiles * prm.splits, unit_step = (int)gridDim.x;
+    const uint32_t tiles_per_gp = (uint32_t)prm.tiles_per_gp;
+    auto part_of = [&](int unit) { return prm.splits == 1 ? 0 : prm.splits - 1 - (int)((uint32_t)unit / (uint32_t)tiles); };   // the longest parts first
+    auto tile_of = [&](int unit) { return (uint32_t)prm.tile_begin + (prm.splits == 1 ? (uint32_t)unit : (uint32_t)unit % (uint32_t)tiles); };
 
     if (warp < 4) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsControl));
-    if (warp == 0 && lane == 0) {
-        // ------------------------------------------------------------ producer: scaled observations
-        const uint32_t bytes = map.x_stage;
+    const uint32_t leader = elect_one();
+    if (warp == 0) {
+        // ------------------------------------------------------------ producer: three lanes, a stream each
+        // lane 0: scaled observations; lanes 1 and 2: the chunks of W of the strips that go to accumulator 0 and 1.  The lanes
+        // poll together, so that no stream waits for another.
+        const int me = lane - 1, ring = lane == 0 ? xs : ws / 2;
+        const uint32_t full0 = lane == 0 ? BAR_X_FULL : BAR_W_FULL + me * (kMaxWS / 2), empty0 = lane == 0 ? BAR_X_EMPTY : BAR_W_EMPTY + me * (kMaxWS / 2);
+        const uint32_t dst0 = base + (lane == 0 ? map.x : map.w + me * ring * (4u * KC * kStrip)), stride = lane == 0 ? map.x_stage : 4u * KC * kStrip;
         long long issued = 0;
-        int st = 0;
-        uint32_t ph = 0;   // stage ring: (stage, phase) advance together, no divisions in the loop
-        bool ok = true;
-        for (long long tile = first_tile; ok && tile < prm.total_tiles; tile += tile_step) {
-            const int g = (int)(tile / prm.tiles_per_gp);
-            const __half* src = prm.xt + (size_t)g * (prm.NP / KD) * (bytes / 2);
-            for (int p = 0; ok && p < P; ++p)
-                for (int c = 0; c < (p + 1) * (NV / KD); ++c, ++issued) {
-                    if (!(ok = mbar_wait(bar(BAR_X_EMPTY + st), ph ^ 1u, abort_flag, wl))) break;
-                    mbar_arrive_expect_tx(bar(BAR_X_FULL + st), bytes);
-                    bulk_g2s(base + map.x + (uint32_t)R3_IDX(st, XS, prm.status) * bytes,
-                             src + (size_t)R3_IDX(c, prm.NP / KD, prm.status) * (bytes / 2), bytes, bar(BAR_X_FULL + st));
-                    if (++st == XS) { st = 0; ph ^= 1u; }
+        int st = 0, unit = blockIdx.x, p = 0, strip = 0, strips = 0, c = 0, count = 0;
+        uint32_t ph = 0, bytes = 0, sigma = 0;
+        const __half* src = nullptr;
+        bool have = lane < 3 && unit < units;
+        int p_end = 0, g = 0;
+        auto open_unit = [&] {
+            const int part = part_of(unit);
+            p = prm.cut[part];
+            p_end = prm.cut[part + 1];
+            g = (int)(tile_of(unit) / tiles_per_gp);
+        };
+        if (have) open_unit();
+        auto next_segment = [&] {   // the next run of equal blobs: a pair's observations, or the chunks of one of its strips
+            c = 0;
+            while (have) {
+                if (strip == strips) {   // next pair
+                    if (strips && ++p == p_end) {
+                        if ((unit += unit_step) >= units) { have = false; break; }
+                        open_unit();
+                    }
+                    strip = 0;
+                    strips = lane == 0 || !Pair(p, S, nc).nb ? 1 : 2;
                 }
-        }
-        if (!ok) {  // aborting: let the copies still in flight land before the CTA goes away
-            const int pending = (int)(issued < XS ? issued : XS);
-            for (int u = 0; u < pending; ++u) {
-                if (--st < 0) { st = XS - 1; ph ^= 1u; }
-                mbar_wait(bar(BAR_X_FULL + st), ph, abort_flag + 1, wl);
-            }
-        }
-    } else if (warp == 0 && lane == 1) {
-        // ------------------------------------------------------------ producer: chunks of W
-        const uint32_t bytes = map.w_stage;
-        long long issued = 0;
-        int st = 0;
-        uint32_t ph = 0;
-        bool ok = true;
-        for (long long tile = first_tile; ok && tile < prm.total_tiles; tile += tile_step) {
-            const int g = (int)(tile / prm.tiles_per_gp);
-            const __half* src = prm.wt + (size_t)g * prm.wt_gp_stride;
-            for (int p = 0; ok && p < P; ++p) {
-                const __half* psrc = src + (size_t)(CPP * p * (p + 1) / 2) * (bytes / 2);
-                for (int c = 0; c < (p + 1) * CPP; ++c, ++issued) {
-                    if (issued == prm.withhold_w) { ok = false; break; }   // test aid: the stream of W stops here
-                    if (!(ok = mbar_wait(bar(BAR_W_EMPTY + st), ph ^ 1u, abort_flag, wl))) break;
-                    mbar_arrive_expect_tx(bar(BAR_W_FULL + st), bytes);
-                    (void)R3_IDX(CPP * p * (p + 1) / 2 + c, CPP * P * (P + 1) / 2, prm.status);   // chunk of W within the GP's tiles
-                    bulk_g2s(base + map.w + (uint32_t)R3_IDX(st, ws, prm.status) * bytes, psrc + (size_t)c * (bytes / 2), bytes,
-                             bar(BAR_W_FULL + st));
-                    if (++st == ws) { st = 0; ph ^= 1u; }
+                const Pair pr(p, S, nc);
+                const int s = pr.a + strip++;
+                if (lane == 0) {
+                    src = prm.xt + (size_t)g * prm.NP * 2 * DP;
+                    count = pr.chunks() / KDC * parts;
+                    bytes = map.x_stage;
+                    break;
+                }
+                if ((int)(sigma++ & 1u) == me) {
+                    const int rows = min(kStrip, nc * KC - s * kStrip);
+                    src = prm.wt + (size_t)g * prm.wt_gp_stride +
+                          R3_IDX((size_t)2 * s * (s + 1) * (2 * KC * kStrip), prm.wt_gp_stride, prm.status);
+                    count = min(4 * (s + 1), nc);
+                    bytes = 4u * KC * rows;
+                    break;
                 }
             }
+        };
+        next_segment();
+        bool ok = true;
+        long long t0 = clock64();
+        while (__any_sync(0xffffffffu, have)) {
+            const bool held = lane == 1 && issued == prm.withhold_w;   // test aid: this stream of W stops here
+            bool moved = false;
+            if (have && !held && mbar_test(bar(empty0 + st), ph ^ 1u)) {
+                mbar_arrive_expect_tx(bar(full0 + st), bytes);
+                bulk_g2s(dst0 + (uint32_t)R3_IDX(st, ring, prm.status) * stride, src + (size_t)c * (bytes / 2), bytes, bar(full0 + st));
+                ++issued;
+                if (++st == ring) { st = 0; ph ^= 1u; }
+                if (++c == count) next_segment();
+                moved = true;
+            }
+            if (__any_sync(0xffffffffu, moved)) {
+                t0 = clock64();
+                continue;
+            }
+            if (__any_sync(0xffffffffu, *abort_flag)) { ok = false; break; }
+            if (__any_sync(0xffffffffu, clock64() - t0 > wl)) {
+                *abort_flag = 1;
+                ok = false;
+                break;
+            }
+            __nanosleep(100);
         }
-        if (!ok) {
-            const int pending = (int)(issued < ws ? issued : ws);
+        if (!ok && lane < 3) {  // aborting: let the copies still in flight land before the CTA goes away
+            const int pending = (int)(issued < ring ? issued : ring);
             for (int u = 0; u < pending; ++u) {
-                if (--st < 0) { st = ws - 1; ph ^= 1u; }
-                mbar_wait(bar(BAR_W_FULL + st), ph, abort_flag + 1, wl);
+                if (--st < 0) { st = ring - 1; ph ^= 1u; }
+                mbar_wait(bar(full0 + st), ph, abort_flag + 1, wl);
             }
         }
-    } else if (warp == 1 && lane == 0) {
+    } else if (warp == 1) {
         // ------------------------------------------------------------ MMA issuer: distance products
         constexpr uint32_t IDESC_D = instr_desc_f16(KD);
         // descriptor low word = start >> 4 | (k-slice distance >> 4) << 16
-        const uint32_t zH = tmem + ZCOL, zL = zH + (uint32_t)DP / 2;
+        const uint32_t z_lo0 = desc_addr(base + map.z) | ((2048u >> 4) << 16);
         const uint32_t x_lo0 = desc_addr(base + map.x) | (((KD * 16u) >> 4) << 16);
-        const int ksteps = DP / 16;
-        long long tile_iter = 0;
-        int st = 0, db = 0;
-        uint32_t ph = 0, d_ph = 0;   // X stage ring; parity of the distance-buffer pair
+        const int ksteps = DPp / 16;
+        const uint32_t x_plane = ((uint32_t)DPp * KD * 2u) >> 4, z_plane = (256u * DP) >> 4;
+        int st = 0, bank = 0, zi = 0;
+        uint32_t ph = 0, bank_ph = 0, z_ph = 0;
         bool ok = true;
-        for (long long tile = first_tile; ok && tile < prm.total_tiles; tile += tile_step, ++tile_iter) {
-            TICK(7);
-            if (!(ok = mbar_wait(bar(BAR_Z_READY), (uint32_t)(tile_iter & 1), abort_flag, wl))) break;
-            TICK(3);
+        for (int unit = blockIdx.x; ok && unit < units; unit += unit_step) {
+            const int part = part_of(unit);
+            if (!(ok = mbar_wait_warp(bar(BAR_Z_FULL + zi), z_ph, abort_flag, wl))) break;
             tc_fence_after();
-            for (int u = 0; u < items_per_tile / SL; ++u) {
-                TICK(7);
-                if (!(ok = mbar_wait(bar(BAR_X_FULL + st), ph, abort_flag, wl))) break;
-                TICK(0);
-                if (!(ok = mbar_wait(bar(BAR_D_EMPTY + db), d_ph ^ 1u, abort_flag, wl))) break;
-                TICK(1);
-                LOGEV(8, (long long)(tile_iter * (items_per_tile / SL) + u) * SL);
-                tc_fence_after();
-                const uint32_t xH_lo = x_lo0 + ((st * map.x_stage) >> 4), xL_lo = xH_lo + (((uint32_t)DP * KD * 2u) >> 4);
-                const uint32_t dcol = tmem + NV + db * KD;
-                uint32_t acc = 0;
-#pragma unroll
-                for (int combo = 0; combo < 3; ++combo) {
-                    const uint32_t a0 = combo == 2 ? zL : zH, b0 = combo == 1 ? xL_lo : xH_lo;
-                    for (int jj = 0; jj < ksteps; ++jj) {
-                        tc_mma_f16_ts(dcol, a0 + jj * 8u, pack64(b0 + jj * ((2u * KD * 16u) >> 4), kDescHi), IDESC_D, acc);
-                        acc = 1;
+            for (int p = prm.cut[part]; ok && p < prm.cut[part + 1]; ++p) {
+                const int products = Pair(p, S, nc).chunks() / KDC;
+                for (int u = 0; ok && u < products; ++u) {
+                    if (!(ok = mbar_wait_warp(bar(BAR_K_EMPTY + bank), bank_ph ^ 1u, abort_flag, wl))) break;
+                    const uint32_t dcol = tmem + kRingCol + (uint32_t)R3_IDX(bank, BANKS, prm.status) * KD;
+                    uint32_t acc = 0;
+                    for (int q = 0; q < parts; ++q) {
+                        if (!(ok = mbar_wait_warp(bar(BAR_X_FULL + st), ph, abort_flag, wl))) break;
+                        tc_fence_after();
+                        const uint32_t xH = x_lo0 + ((st * map.x_stage) >> 4);
+                        const uint32_t zH = z_lo0 + ((zi * map.z_buf) >> 4) + q * ksteps * (4096u >> 4);
+                        for (int jj = 0; jj < ksteps; ++jj) {
+                            const uint32_t a = zH + jj * (4096u >> 4), b = xH + jj * ((2u * KD * 16u) >> 4);
+                            tc_mma_f16_if(leader, dcol, pack64(a, kDescHi), pack64(b, kDescHi), IDESC_D, acc);
+                            tc_mma_f16_if(leader, dcol, pack64(a, kDescHi), pack64(b + x_plane, kDescHi), IDESC_D, 1u);
+                            tc_mma_f16_if(leader, dcol, pack64(a + z_plane, kDescHi), pack64(b, kDescHi), IDESC_D, 1u);
+                            acc = 1;
+                        }
+                        tc_commit_if(leader, bar(BAR_X_EMPTY + st));
+                        if (++st == xs) { st = 0; ph ^= 1u; }
                     }
+                    if (!ok) break;
+                    tc_commit_if(leader, bar(BAR_D_FULL + bank));
+                    if (++bank == BANKS) { bank = 0; bank_ph ^= 1u; }
                 }
-                tc_commit(bar(BAR_X_EMPTY + st));
-                tc_commit(bar(BAR_D_FULL + db));
-                TICK(2);
-                LOGEV(7, (long long)(tile_iter * (items_per_tile / SL) + u) * SL);
-                if (++st == XS) { st = 0; ph ^= 1u; }
-                if (++db == 2) { db = 0; d_ph ^= 1u; }
             }
+            if (!ok) break;
+            tc_commit_if(leader, bar(BAR_Z_EMPTY + zi));
+            if (++zi == zb) { zi = 0; z_ph ^= 1u; }
         }
         // every MMA issued by this thread must have completed before TMEM is freed
-        tc_commit(bar(BAR_MMA_DONE));
-        mbar_wait(bar(BAR_MMA_DONE), 0, abort_flag + 1, wl);
-        if (prm.trace)
-            for (int i = 0; i < 8; ++i) prm.trace[((size_t)blockIdx.x * 4 + 3) * 8 + i] = tacc[i];
-    } else if (warp == 2 && lane == 0) {
-        // ------------------------------------------------------------ MMA issuer: variance product
-        const uint32_t k_lo0 = desc_addr(base + map.k) | ((2048u >> 4) << 16);
-        const uint32_t w_lo0 = desc_addr(base + map.w) | (((NV * 16u) >> 4) << 16);
-        uint32_t v_ph = 0;    // parity of the pass counter (V accumulator hand-over)
-        int w_s = 0, k_s = 0, e_s = 0;   // e_s: chunk number mod 4 (ring mode: which "consumed" barrier)
-        uint32_t w_ph = 0, k_ph = 0;
+        tc_commit_if(leader, bar(BAR_MMA_DONE));
+        mbar_wait_warp(bar(BAR_MMA_DONE), 0, abort_flag + 1, wl);
+    } else {
+        // ------------------------------------------------------------ MMA issuers: variance product, one warp per accumulator
+        // The strips of all units go to the two accumulators in turn.  The two issuers share the k* chunks and run at their own
+        // pace: while one's accumulator is being read back, the other's products keep the tensor cores busy.
+        const uint32_t me = warp - 2, ring = ws / 2;
+        const uint32_t w_lo0 = desc_addr(base + map.w + me * ring * (4u * KC * kStrip));
+        const uint32_t wbar = me * (kMaxWS / 2);
+        uint32_t w_s = 0, w_ph = 0, v_ph = 0;
+        uint32_t t_base = 0, sigma = 0;      // chunks before the current pair, strips so far
+        uint32_t zi = 0;                     // which group reads this unit's accumulators back
         bool ok = true;
-        // whether the next chunk's k* and W were already seen complete (tested between this chunk's MMAs, while
-        // the pipe has work queued, so that nothing but the commits sits between two chunks' MMAs)
-        bool k_seen = false, w_seen = false;
-        long long tv = 0;
-        for (long long tile = first_tile; ok && tile < prm.total_tiles; tile += tile_step) {
-            for (int p = 0; ok && p < P; ++p) {
-                const int nchunk = (p + 1) * CPP;
-                for (int c = 0; ok && c < nchunk; ++c) {
-                    const int b = k_s, s = w_s;
-                    TICK(7);
-                    if (c == 0) {
-                        if (!(ok = mbar_wait(bar(BAR_V_EMPTY), v_ph ^ 1u, abort_flag, wl))) break;
-                    }
-                    TICK(3);
-                    if (!k_seen && !(ok = mbar_wait(bar(BAR_K_FULL + b), k_ph, abort_flag, wl))) break;
-                    TICK(4);
-                    LOGEV(0, tv);
-                    if (!w_seen && !(ok = mbar_wait(bar(BAR_W_FULL + s), w_ph, abort_flag, wl))) break;
-                    LOGEV(1, tv);
-                    if (++k_s == NBK) { k_s = 0; k_ph ^= 1u; }
-                    if (++w_s == ws) { w_s = 0; w_ph ^= 1u; }
-                    TICK(5);
-                    tc_fence_after();
-                    // In the pass's diagonal block the rows of W above the chunk's columns are zero (W is lower
-                    // triangular): the MMAs start at the first row that can be non-zero and get narrower.
-                    (void)R3_IDX(s, ws, prm.status);
-                    (void)R3_IDX(b, NBK, prm.status);
-                    const uint32_t skip = c > p * CPP ? (uint32_t)R3_IDX((c - p * CPP) * KC, NV, prm.status) : 0u;
-                    const uint32_t idesc_v = instr_desc_f16(NV - skip);
-                    const uint32_t vcol = tmem + skip;
-                    const uint32_t bH = w_lo0 + ((s * map.w_stage) >> 4) + skip, bL = bH + (((uint32_t)KC * NV * 2u) >> 4);
-                    if (F8) {
-                        // main term: FP16 hi x hi, two MMAs of depth 16; cross terms: one FP8 MMA of depth 32 each
-                        // (planes after the FP16 hi plane: scaled hi parts, then scaled lo parts)
+        for (int unit = blockIdx.x; ok && unit < units; unit += unit_step, zi = zb == 2 ? zi ^ 1u : 0u) {
+            const int part = part_of(unit);
+            for (int p = prm.cut[part]; ok && p < prm.cut[part + 1]; ++p) {
+                const Pair pr(p, S, nc);
+                const uint32_t strips = pr.nb ? 2 : 1, which = (sigma & 1u) == me ? 0u : 1u;
+                sigma += strips;
+                if (which < strips) {
+                    const int s = pr.a + which;
+                    const uint32_t n_own = which ? pr.nb : pr.na, rows = (uint32_t)min(kStrip, nc * KC - s * kStrip);
+                    // arrivals that free a bank of slots: one from each issuer, both from this one where it is the only user
+                    const uint32_t shared = strips == 2 ? (uint32_t)pr.na : 0u;
+                    if (!(ok = mbar_wait_warp(bar(BAR_V_EMPTY + me), v_ph ^ 1u, abort_flag, wl))) break;
+                    for (uint32_t c = 0; c < n_own; ++c) {
+                        const uint32_t t = t_base + c, slot = t % kSlots;
+                        if (!(ok = mbar_wait_warp(bar(BAR_K_FULL + slot), (t / kSlots) & 1u, abort_flag, wl))) break;
+                        if (!(ok = mbar_wait_warp(bar(BAR_W_FULL + wbar + w_s), w_ph, abort_flag, wl))) break;
+                        tc_fence_after();
+                        // In the strip's diagonal block the rows of W above the chunk's columns are zero (W is lower
+                        // triangular): the MMAs start at the first row that can be non-zero and get narrower.
+                        const uint32_t skip = (int)c > 4 * s ? (uint32_t)R3_IDX((c - 4 * s) * KC, rows, prm.status) : 0u;
+                        const uint32_t idesc = instr_desc_f16(rows - skip);
+                        const uint32_t vcol = tmem + me * kStrip + skip;
+                        const uint32_t bH = (w_lo0 + (((uint32_t)R3_IDX(w_s, ring, prm.status) * (4u * KC * kStrip)) >> 4) + skip) | (rows << 16);
+                        const uint32_t aK = tmem + kRingCol + slot * KC;
                         const uint32_t first = c > 0 ? 1u : 0u;
-                        const uint32_t b8H = bH + (((uint32_t)KC * NV * 2u) >> 4), b8L = b8H + (((uint32_t)KC * NV) >> 4);
-                        // k* parts are E5M2; W's hi parts E4M3, its lo parts E5M2
-                        const uint32_t idesc_hl = instr_desc_f8(NV - skip, kFmtE5M2, kFmtE5M2);   // k*_hi x W_lo
-                        const uint32_t idesc_lh = instr_desc_f8(NV - skip, kFmtE5M2, kFmtE4M3);   // k*_lo x W_hi
-                        if (KT) {
-                            const uint32_t aH = tmem + KCOL + (uint32_t)b * KC;
-                            tc_mma_f16_ts(vcol, aH, pack64(bH, kDescHi), idesc_v, first);
-                            tc_mma_f16_ts(vcol, aH + 8u, pack64(bH + ((2u * NV * 16u) >> 4), kDescHi), idesc_v, 1u);
-                            tc_mma_f8_ts(vcol, aH + KC / 2, pack64(b8L, kDescHi), idesc_hl, 1u);
-                            k_seen = mbar_try_wait(bar(BAR_K_FULL + k_s), k_ph);
-                            w_seen = mbar_try_wait(bar(BAR_W_FULL + w_s), w_ph);
-                            tc_mma_f8_ts(vcol, aH + KC / 2 + KC / 4, pack64(b8H, kDescHi), idesc_lh, 1u);
+                        if (F8) {
+                            // main term: FP16 hi x hi, two MMAs of depth 16; cross terms: one FP8 MMA of depth 32 each
+                            // (planes after the FP16 hi plane: hi parts, then lo parts).  A slot holds, 8 columns each, the hi
+                            // parts of the first 16 observations, all hi parts as E5M2, all lo parts as E5M2, the other 16 hi parts.
+                            const uint32_t b8H = bH + ((rows * KC * 2u) >> 4), b8L = b8H + ((rows * KC) >> 4);
+                            tc_mma_f16_ts_if(leader, vcol, aK, pack64(bH, kDescHi), idesc, first);
+                            tc_mma_f16_ts_if(leader, vcol, aK + 24u, pack64(bH + 2u * rows, kDescHi), idesc, 1u);
+                            // k* parts are E5M2; W's hi parts E4M3, its lo parts E5M2
+                            tc_mma_f8_ts_if(leader, vcol, aK + 8u, pack64(b8L, kDescHi), instr_desc_f8(rows - skip, kFmtE5M2, kFmtE5M2), 1u);
+                            tc_mma_f8_ts_if(leader, vcol, aK + 16u, pack64(b8H, kDescHi), instr_desc_f8(rows - skip, kFmtE5M2, kFmtE4M3), 1u);
                         } else {
-                            const uint32_t aH = k_lo0 + ((b * 16384u) >> 4), a8H = aH + (8192u >> 4), a8L = a8H + (4096u >> 4);
-                            tc_mma_f16(vcol, pack64(aH, kDescHi), pack64(bH, kDescHi), idesc_v, first);
-                            tc_mma_f16(vcol, pack64(aH + (4096u >> 4), kDescHi), pack64(bH + ((2u * NV * 16u) >> 4), kDescHi),
-                                       idesc_v, 1u);
-                            tc_mma_f8(vcol, pack64(a8H, kDescHi), pack64(b8L, kDescHi), idesc_hl, 1u);
-                            k_seen = mbar_try_wait(bar(BAR_K_FULL + k_s), k_ph);
-                            w_seen = mbar_try_wait(bar(BAR_W_FULL + w_s), w_ph);
-                            tc_mma_f8(vcol, pack64(a8L, kDescHi), pack64(b8H, kDescHi), idesc_lh, 1u);
-                        }
-                    } else if (KT) {
-                        const uint32_t aH = tmem + KCOL + (uint32_t)b * KC, aL = aH + KC / 2;
+                            // a slot holds, per 16 observations, 8 columns of hi parts and 8 of lo parts
+                            const uint32_t bL = bH + ((rows * KC * 2u) >> 4);
 #pragma unroll
-                        for (int combo = 0; combo < 3; ++combo) {
-                            const uint32_t a0 = combo == 2 ? aL : aH, b0 = combo == 1 ? bL : bH;
+                            for (int combo = 0; combo < 3; ++combo) {
+                                const uint32_t a0 = combo == 2 ? aK + 8u : aK, b0 = combo == 1 ? bL : bH;
 #pragma unroll
-                            for (int jj = 0; jj < KC / 16; ++jj)
-                                tc_mma_f16_ts(vcol, a0 + jj * 8u, pack64(b0 + jj * ((2u * NV * 16u) >> 4), kDescHi), idesc_v,
-                                              (c > 0 || combo > 0 || jj > 0) ? 1u : 0u);
-                            if (combo == 1) {
-                                k_seen = mbar_try_wait(bar(BAR_K_FULL + k_s), k_ph);
-                                w_seen = mbar_try_wait(bar(BAR_W_FULL + w_s), w_ph);
+                                for (int jj = 0; jj < KC / 16; ++jj)
+                                    tc_mma_f16_ts_if(leader, vcol, a0 + jj * 16u, pack64(b0 + jj * 2u * rows, kDescHi), idesc,
+                                                     combo > 0 || jj > 0 ? 1u : first);
                             }
                         }
-                    } else {
-                        const uint32_t aH = k_lo0 + ((b * 16384u) >> 4), aL = aH + (8192u >> 4);
-#pragma unroll
-                        for (int combo = 0; combo < 3; ++combo) {
-                            const uint32_t a0 = combo == 2 ? aL : aH, b0 = combo == 1 ? bL : bH;
-#pragma unroll
-                            for (int jj = 0; jj < KC / 16; ++jj)
-                                tc_mma_f16(vcol, pack64(a0 + jj * (4096u >> 4), kDescHi),
-                                           pack64(b0 + jj * ((2u * NV * 16u) >> 4), kDescHi), idesc_v,
-                                           (c > 0 || combo > 0 || jj > 0) ? 1u : 0u);
-                            if (combo == 1) {
-                                k_seen = mbar_try_wait(bar(BAR_K_FULL + k_s), k_ph);
-                                w_seen = mbar_try_wait(bar(BAR_W_FULL + w_s), w_ph);
-                            }
+                        tc_commit_if(leader, bar(BAR_W_EMPTY + wbar + w_s));
+                        if (++w_s == ring) { w_s = 0; w_ph ^= 1u; }
+                        if (t % KDC == KDC - 1) {   // slots go back to the distance products a bank at a time
+                            const uint32_t kb = bar(BAR_K_EMPTY + (t / KDC) % BANKS);
+                            tc_commit_if(leader, kb);
+                            if (c >= shared) tc_commit_if(leader, kb);
                         }
                     }
-                    tc_commit(bar(BAR_W_EMPTY + s));
-                    tc_commit(bar(BAR_K_EMPTY + (NBK == G ? b : e_s)));
-                    e_s = (e_s + 1) & 3;
-                    if (c == nchunk - 1) {
-                        tc_commit(bar(BAR_V_FULL));
-                        v_ph ^= 1u;
-                    }
-                    TICK(6);
-                    LOGEV(2, tv);
-                    ++tv;
+                    if (!ok) break;
+                    tc_commit_if(leader, bar(BAR_V_FULL + 2 * me + zi));
+                    v_ph ^= 1u;
                 }
+                // chunks that only the other issuer takes: a wait by parity is good for one phase, so none is passed over
+                for (uint32_t c = which < strips ? (which ? pr.nb : pr.na) : 0; ok && c < (uint32_t)pr.chunks(); ++c)
+                    ok = mbar_wait_warp(bar(BAR_K_FULL + (t_base + c) % kSlots), ((t_base + c) / kSlots) & 1u, abort_flag, wl);
+                t_base += pr.chunks();
             }
         }
-        tc_commit(bar(BAR_MMA_DONE + 1));
-        mbar_wait(bar(BAR_MMA_DONE + 1), 0, abort_flag + 1, wl);
-        if (prm.trace)
-            for (int i = 0; i < 8; ++i) prm.trace[((size_t)blockIdx.x * 4 + 0) * 8 + i] = tacc[i];
+        tc_commit_if(leader, bar(BAR_MMA_DONE + 1 + me));
+        mbar_wait_warp(bar(BAR_MMA_DONE + 1 + me), 0, abort_flag + 1, wl);
     }
-    } else {
-        asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(regs_matern(G)));
-        // ------------------------------------------------------------ Matern / epilogue warp groups
-        const int grp = (warp - 4) >> 2;         // 0..G-1
-        const int q4 = warp & 3;                 // TMEM lane quarter == warp % 4
-        const int row = q4 * 32 + lane;          // candidate row in the tile == TMEM lane
-        const uint32_t lane_addr = tmem + ((uint32_t)(q4 * 32) << 16);
-        long long t = grp;                       // next own chunk (global numbering)
-        long long t_tile0 = 0;                   // first chunk of the current tile
-        uint32_t own_ph = 0;                     // parity of this group's own-chunk count
-        uint32_t v_ph = 0;                       // parity of the pass counter
-        long long tile_iter = 0;
-        bool ok = true;
-        bool bad = false;
-        double* red = reinterpret_cast<double*>(sm + map.z);   // scratch of the end-of-tile reduction
-        for (long long tile = first_tile; ok && tile < prm.total_tiles; tile += tile_step, ++tile_iter) {
-            const int g = (int)(tile / prm.tiles_per_gp);
-            const long long cand = (tile % prm.tiles_per_gp) * TILE_M + row;
-            const bool valid = cand < prm.m;
-            const float sf2 = prm.sf2[g];
-            const float kvscale = prm.kscale[g] * sf2;   // k* = sf2 * (k*/sf2), scaled for its FP16 split
-            if (grp == G - 1) {
-                // ---- scale the candidate, split it, store it as the A operand of the distance MMA
-                float zn = 0.f;
-                bool far = false;
-                const float* zrow =
-                    prm.xcand + (size_t)R3_IDX((long long)g * prm.m + (valid ? cand : 0), (long long)prm.batch * prm.m, prm.status) * prm.d;
-                {
-                    // the row this thread will need for the CTA's next tile: start it on its way to L2 now
-                    const long long nt = tile + tile_step;
-                    if (nt < prm.total_tiles) {
-                        const long long nc = (nt % prm.tiles_per_gp) * TILE_M + row;
-                        if (nc < prm.m) {
-                            const char* pf = reinterpret_cast<const char*>(
-                                prm.xcand + ((size_t)(nt / prm.tiles_per_gp) * prm.m + nc) * prm.d);
-                            for (int off = 0; off < prm.d * 4; off += 128)
-                                asm volatile("prefetch.global.L2 [%0];" ::"l"(pf + off));
+    } else if (warp < kFirstMatern) {
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsIo));
+        // ------------------------------------------------------------ candidates in, results out: a row per thread
+        // Two buffers of scaled candidates: the candidates of the unit after the next come in once the present one's last strip
+        // has been read back (its buffer is free when the Matern groups are through with it, and they are ahead of the products);
+        // one buffer: those of the next unit, before that strip.  Two groups take every other unit each.
+        const int io = (warp - kFirstIo) >> 2, row = (threadIdx.x - kFirstIo * 32) & (TILE_M - 1);
+        const uint32_t lane_addr = tmem + ((uint32_t)((warp & 3) * 32) << 16);
+        bool ok = true, bad = false;
+        uint32_t z_ph = 0, v_ph = 0, red_ph = 0;     // parities per buffer b: bit b; v_ph: bit 2 b + accumulator
+        uint32_t sigma = 0;                          // strips of all units so far
+        float zn_in0 = 0.f, zn_in1 = 0.f;            // of the tiles in the buffers (the sign carries the out-of-range mark)
+        const int groups = IO == 2 && zb == 2 ? 2 : 1, own_step = unit_step * groups, ahead = unit_step * zb;
+        auto strips_of = [&](int unit) { return min(S, 2 * prm.cut[part_of(unit) + 1]) - 2 * prm.cut[part_of(unit)]; };
+        int b = groups == 2 ? io : 0;
+        if (io < groups)
+        for (int unit = (int)blockIdx.x + (groups == 2 ? io * unit_step : 0) - ahead; ok && unit < units; unit += own_step) {
+            const bool work = unit >= 0;
+            const float zn_own = b ? zn_in1 : zn_in0;
+            const int next = unit + ahead;
+            const int part = work ? part_of(unit) : 0;
+            const int s0 = work ? 2 * prm.cut[part] : 0, s1 = work ? s0 + strips_of(unit) : 0;
+            const int at = !work ? -1 : zb == 1 ? s1 - 1 : s1;
+            if (groups == 2 && unit >= unit_step) sigma += strips_of(unit - unit_step);   // the other group's
+            double q_acc = 0.0;
+            for (int s = work ? s0 : -1; s <= s1; ++s) {
+                if (s == at && next < units) {
+                    // ---- scale a candidate, split it, store it as the A operand of the distance product
+                    ok = mbar_wait_warp(bar(BAR_Z_EMPTY + b), ((z_ph >> b) & 1u) ^ 1u, abort_flag, wl);
+                    if (!ok) break;
+                    const uint32_t tile = tile_of(next);
+                    const int g = (int)(tile / tiles_per_gp);
+                    const long long cand = (long long)(tile - g * tiles_per_gp) * TILE_M + row;
+                    const bool valid = cand < prm.m;
+                    float zn = 0.f;
+                    bool far = false;
+                    const float* zrow =
+                        prm.xcand + (size_t)R3_IDX((long long)g * prm.m + (valid ? cand : 0), (long long)prm.batch * prm.m, prm.status) * prm.d;
+                    if (next + unit_step < units) {   // the row after that: on its way to L2
+                        const uint32_t nt = tile_of(next + unit_step), ng = nt / tiles_per_gp;
+                        const long long nr = (long long)(nt - ng * tiles_per_gp) * TILE_M + row;
+                        if (nr < prm.m) {
+                            const char* pf = reinterpret_cast<const char*>(prm.xcand + ((size_t)ng * prm.m + nr) * prm.d);
+                            for (int off = 0; off < prm.d * 4; off += 128) asm volatile("prefetch.global.L2 [%0];" ::"l"(pf + off));
                         }
                     }
-                }
-                const float* cen = prm.centre + (size_t)g * DP;
-                const float* scl = prm.scale + (size_t)g * DP;
-                const bool vec = (prm.d % 4) == 0 && (reinterpret_cast<uintptr_t>(prm.xcand) & 15) == 0;
-                // Two forms of the same loop over the row's features.  The long-history kernel keeps the plain one: its
-                // chunk loop sits at the register limit, and the pipelined form, although it runs once per tile, costs
-                // that loop registers (config 5: 45.9 ms to 47.9 ms per pool); everywhere else the row's loads overlap
-                // (config 3: 5.74 ms to 5.52 ms).
-                if constexpr (F8) {
-                    uint32_t zh[8], zl[8];
-                    for (int j8 = 0; j8 < DP / 8; ++j8) {
-                        __half2 hi2[4], lo2[4];
-    #pragma unroll
-                        for (int h = 0; h < 2; ++h) {
-                            const int j4 = 2 * j8 + h;
-                            float z[4];
-                            if (vec && 4 * j4 < prm.d) {
-                                // read once: streaming load, so that the pool does not push W out of L2
-                                const float4 v = __ldcs(reinterpret_cast<const float4*>(zrow + 4 * j4));
-                                z[0] = v.x; z[1] = v.y; z[2] = v.z; z[3] = v.w;
-                            } else {
-    #pragma unroll
-                                for (int e = 0; e < 4; ++e) z[e] = (4 * j4 + e < prm.d) ? __ldcs(zrow + 4 * j4 + e) : 0.f;
-                            }
-                            const float4 c4 = __ldg(reinterpret_cast<const float4*>(cen + R3_IDX(4 * j4, DP - 3, prm.status)));
-                            const float4 s4 = __ldg(reinterpret_cast<const float4*>(scl + R3_IDX(4 * j4, DP - 3, prm.status)));
-                            const float cc[4] = {c4.x, c4.y, c4.z, c4.w}, ss[4] = {s4.x, s4.y, s4.z, s4.w};
-                            float zt[4];
-    #pragma unroll
-                            for (int e = 0; e < 4; ++e) {
-                                bad |= !isfinite(z[e]);
-                                float v = valid ? (z[e] - cc[e]) * ss[e] : 0.f;
-                                if (fabsf(v) > kMaxScaled) {   // outside the FP16 planes' range: clamp, and have it recomputed
-                                    v = copysignf(kMaxScaled, v);
-                                    far = true;
-                                }
-                                zt[e] = v;
-                                zn = fmaf(v, v, zn);
-                            }
-                            split2(zt[0], zt[1], hi2[2 * h], lo2[2 * h]);
-                            split2(zt[2], zt[3], hi2[2 * h + 1], lo2[2 * h + 1]);
-                            if (ZS) {
-    #pragma unroll
-                                for (int e = 0; e < 4; ++e) zs_s[row * kZsStride + 4 * j4 + e] = zt[e];
-                            }
-                        }
-                        // 8 features = 4 columns of each plane; two such groups make one 8-column store
-                        if (j8 & 1) {
-    #pragma unroll
-                            for (int e = 0; e < 4; ++e) {
-                                zh[4 + e] = *reinterpret_cast<const uint32_t*>(&hi2[e]);
-                                zl[4 + e] = *reinterpret_cast<const uint32_t*>(&lo2[e]);
-                            }
-                            // candidate planes: columns [ZCOL, ZCOL + DP) of the 512
-                            (void)R3_IDX(ZCOL + DP / 2 + (j8 >> 1) * 8 + 7, min((int)TMEM_COLS, (int)ZCOL + DP), prm.status);
-                            tc_st8(lane_addr + ZCOL + (uint32_t)(j8 >> 1) * 8u, zh);
-                            tc_st8(lane_addr + ZCOL + (uint32_t)DP / 2 + (uint32_t)(j8 >> 1) * 8u, zl);
-                        } else {
-    #pragma unroll
-                            for (int e = 0; e < 4; ++e) {
-                                zh[e] = *reinterpret_cast<const uint32_t*>(&hi2[e]);
-                                zl[e] = *reinterpret_cast<const uint32_t*>(&lo2[e]);
-                            }
-                        }
-                    }
-                } else {
-                    // 16 features per step (one 8-column store to each plane); the next step's four loads are under way
-                    // while this one is scaled and split, so that the row costs one trip to L2 or HBM and not DP / 8
+                    const float* cen = prm.centre + (size_t)g * DP;
+                    const float* scl = prm.scale + (size_t)g * DP;
+                    const bool vec = (prm.d % 4) == 0 && (reinterpret_cast<uintptr_t>(prm.xcand) & 15) == 0;
+                    uint8_t* zdst = sm + map.z + b * map.z_buf + row * 16;
                     auto load4 = [&](int j4) {
                         float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
                         if (vec && 4 * j4 < prm.d) {
@@ -535,27 +626,24 @@ __global__ void __launch_bounds__(128 + 128 * G, 1) score_tc_kernel(const TcPara
                         }
                         return v;
                     };
-                    float4 nxt[4];
-    #pragma unroll
-                    for (int h = 0; h < 4; ++h) nxt[h] = load4(h);
-                    for (int j16 = 0; j16 < DP / 16; ++j16) {
-                        float4 cur[4];
-    #pragma unroll
-                        for (int h = 0; h < 4; ++h) cur[h] = nxt[h];
-                        if (j16 + 1 < DP / 16) {
-    #pragma unroll
-                            for (int h = 0; h < 4; ++h) nxt[h] = load4(4 * (j16 + 1) + h);
-                        }
-                        uint32_t zh[8], zl[8];
-    #pragma unroll
-                        for (int h = 0; h < 4; ++h) {
-                            const int j4 = 4 * j16 + h;
+                    // 8 features per step; the next step's loads are under way while this one is scaled and split.  (The loop is kept
+                    // short on purpose, as all code of this kernel is: see the top of the file.)
+                    float4 nxt[2] = {load4(0), load4(1)};
+#pragma unroll 1
+                    for (int j8 = 0; j8 < DP / 8; ++j8) {
+                        const float4 cur[2] = {nxt[0], nxt[1]};
+                        nxt[0] = load4(2 * j8 + 2);
+                        nxt[1] = load4(2 * j8 + 3);
+                        __half2 hi[4], lo[4];
+#pragma unroll
+                        for (int h = 0; h < 2; ++h) {
+                            const int j4 = 2 * j8 + h;
                             const float z[4] = {cur[h].x, cur[h].y, cur[h].z, cur[h].w};
                             const float4 c4 = __ldg(reinterpret_cast<const float4*>(cen + R3_IDX(4 * j4, DP - 3, prm.status)));
                             const float4 s4 = __ldg(reinterpret_cast<const float4*>(scl + R3_IDX(4 * j4, DP - 3, prm.status)));
                             const float cc[4] = {c4.x, c4.y, c4.z, c4.w}, ss[4] = {s4.x, s4.y, s4.z, s4.w};
                             float zt[4];
-    #pragma unroll
+#pragma unroll
                             for (int e = 0; e < 4; ++e) {
                                 bad |= !isfinite(z[e]);
                                 float v = valid ? (z[e] - cc[e]) * ss[e] : 0.f;
@@ -566,371 +654,320 @@ __global__ void __launch_bounds__(128 + 128 * G, 1) score_tc_kernel(const TcPara
                                 zt[e] = v;
                                 zn = fmaf(v, v, zn);
                             }
-                            __half2 hi0, lo0, hi1, lo1;
-                            split2(zt[0], zt[1], hi0, lo0);
-                            split2(zt[2], zt[3], hi1, lo1);
-                            zh[2 * h] = *reinterpret_cast<const uint32_t*>(&hi0);
-                            zh[2 * h + 1] = *reinterpret_cast<const uint32_t*>(&hi1);
-                            zl[2 * h] = *reinterpret_cast<const uint32_t*>(&lo0);
-                            zl[2 * h + 1] = *reinterpret_cast<const uint32_t*>(&lo1);
-                            if (ZS) {
-    #pragma unroll
-                                for (int e = 0; e < 4; ++e) zs_s[row * kZsStride + 4 * j4 + e] = zt[e];
-                            }
+                            split2(zt[0], zt[1], hi[2 * h], lo[2 * h]);
+                            split2(zt[2], zt[3], hi[2 * h + 1], lo[2 * h + 1]);
+                            if (Z32)
+                                *reinterpret_cast<float4*>(sm + map.z32 + b * map.z32_buf + (j4 * TILE_M + row) * 16) =
+                                    make_float4(zt[0], zt[1], zt[2], zt[3]);
                         }
-                        // candidate planes: columns [ZCOL, ZCOL + DP) of the 512
-                        (void)R3_IDX(ZCOL + DP / 2 + j16 * 8 + 7, min((int)TMEM_COLS, (int)ZCOL + DP), prm.status);
-                        tc_st8(lane_addr + ZCOL + (uint32_t)j16 * 8u, zh);
-                        tc_st8(lane_addr + ZCOL + (uint32_t)DP / 2 + (uint32_t)j16 * 8u, zl);
+                        *reinterpret_cast<uint4*>(zdst + j8 * 2048u) = *reinterpret_cast<const uint4*>(hi);
+                        *reinterpret_cast<uint4*>(zdst + 256u * DP + j8 * 2048u) = *reinterpret_cast<const uint4*>(lo);
+                    }
+                    float* znb = zn_buf(b);
+                    const float kvscale = prm.kscale[g] * prm.sf2[g];   // k* = sf2 * (k*/sf2), scaled for its FP16 split
+                    znb[row] = zn;
+                    znb[TILE_M + row] = far ? INFINITY : kvscale * kRefine / (zn + prm.xnmax[g]);
+                    if (row == 0) *reinterpret_cast<float4*>(znb + 2 * TILE_M) = make_float4(kvscale, 1.f / prm.kscale[g], __int_as_float(g), 0.f);
+                    zn = far ? -zn : zn;
+                    if (b) zn_in1 = zn;
+                    else zn_in0 = zn;
+                    fence_proxy_async();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(bar(BAR_Z_FULL + b));
+                    z_ph ^= 1u << b;
+                }
+                if (!work || s == s1) break;
+                // ---- a finished strip: q += sum_i V^2, then the accumulator is free
+                const uint32_t v_s = sigma++ & 1u;
+                ok = mbar_wait(bar(BAR_V_FULL + 2 * v_s + b), (v_ph >> (2 * b + v_s)) & 1u, abort_flag, wl);
+                v_ph ^= 1u << (2 * b + v_s);
+                ok = __all_sync(0xffffffffu, ok);
+                if (!ok) break;
+                tc_fence_after();
+                const int rows = min(kStrip, nc * KC - s * kStrip);
+#pragma unroll 1
+                for (int c0 = 0; c0 < rows; c0 += 32) {   // two column blocks per round trip to tensor memory
+                    float v[16], w[16];
+                    tc_ld16_issue(lane_addr + v_s * kStrip + c0, v);
+                    tc_ld16_issue(lane_addr + v_s * kStrip + c0 + 16, w);
+                    tc_wait_ld32(v, w);
+                    uint64_t part0 = 0, part1 = 0;
+#pragma unroll
+                    for (int i = 0; i < 16; i += 2) {
+                        const uint64_t v2 = pack2(v[i], v[i + 1]), w2 = pack2(w[i], w[i + 1]);
+                        part0 = fma2(v2, v2, part0);
+                        part1 = fma2(w2, w2, part1);
+                    }
+                    float a0, a1, b0, b1;
+                    unpack2(part0, a0, a1);
+                    unpack2(part1, b0, b1);
+                    q_acc += (double)(a0 + a1);
+                    q_acc += (double)(b0 + b1);
+                }
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(bar(BAR_V_EMPTY + v_s));
+            }
+            if (!ok) break;
+            if (!work) {
+                if (groups == 1 && zb == 2) b ^= 1;
+                continue;
+            }
+            // ---- the groups' partial sums; a tile whose pairs went to several units is finished by the last of them
+            ok = mbar_wait_warp(bar(BAR_RED_FULL + b), (red_ph >> b) & 1u, abort_flag, wl);
+            if (!ok) break;
+            double mu_acc = 0.0;
+            float a2_acc = 0.f, s2_acc = 0.f;
+#pragma unroll
+            for (int gg = 0; gg < G; ++gg) {
+                const uint8_t* o = sm + map.red + b * map.red_buf + (gg * TILE_M + row) * 16;
+                mu_acc += *reinterpret_cast<const double*>(o);
+                const float2 e2 = *reinterpret_cast<const float2*>(o + 8);
+                a2_acc += e2.x;
+                s2_acc += e2.y;
+            }
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bar(BAR_RED_EMPTY + b));
+            red_ph ^= 1u << b;
+            const uint32_t tile = tile_of(unit);
+            bool finish = true;
+            if (prm.splits > 1) {
+                const size_t slot = (size_t)(unit % tiles) * prm.splits;
+                double* mine = prm.partial + (slot + part) * (3 * TILE_M) + row;
+                __stcg(mine, mu_acc);
+                __stcg(mine + TILE_M, q_acc);
+                __stcg(reinterpret_cast<float2*>(mine + 2 * TILE_M), make_float2(a2_acc, s2_acc));
+                __threadfence();
+                asm volatile("bar.sync %0, 128;" ::"r"(1 + io) : "memory");
+                if (row == 0) last_flag[io] = atomicAdd(prm.arrived + unit % tiles, 1) == prm.splits - 1;
+                asm volatile("bar.sync %0, 128;" ::"r"(1 + io) : "memory");
+                finish = last_flag[io] != 0;
+                asm volatile("bar.sync %0, 128;" ::"r"(1 + io) : "memory");
+                if (finish) {
+                    __threadfence();
+                    mu_acc = q_acc = 0.0;
+                    a2_acc = s2_acc = 0.f;
+#pragma unroll 1
+                    for (int i = 0; i < prm.splits; ++i) {
+                        const double* o = prm.partial + (slot + i) * (3 * TILE_M) + row;
+                        mu_acc += __ldcg(o);
+                        q_acc += __ldcg(o + TILE_M);
+                        const float2 e2 = __ldcg(reinterpret_cast<const float2*>(o + 2 * TILE_M));
+                        a2_acc += e2.x;
+                        s2_acc += e2.y;
                     }
                 }
-                asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-                zn_s[R3_IDX(row, TILE_M, prm.status)] = far ? -zn : zn;   // the sign carries the out-of-range mark
-                tc_fence_before();
-                mbar_arrive(bar(BAR_Z_READY));
             }
-            ok = mbar_wait(bar(BAR_Z_READY), (uint32_t)(tile_iter & 1), abort_flag, wl);
-            ok = __all_sync(0xffffffffu, ok);
+            const int g = (int)(tile / tiles_per_gp);
+            const long long cand = (long long)(tile - g * tiles_per_gp) * TILE_M + row;
+            if (finish && cand < prm.m) {
+                const bool far_cand = zn_own < 0.f;
+                q_acc *= prm.vinv2[g];   // undo the power-of-two scaling of k* and W
+                const size_t f = (size_t)R3_IDX((long long)g * prm.m + cand, (long long)prm.batch * prm.m, prm.status);
+                const CandidateResult res =
+                    finalize_candidate(mu_acc, q_acc, (double)prm.sf2[g], (double)prm.best[R3_IDX(g, prm.batch, prm.status)]);
+                __stcs(prm.mu + f, res.mu);
+                __stcs(prm.sigma + f, res.sigma);
+                __stcs(prm.ei + f, res.ei);
+                const float eps = far_cand ? 1.f : (float)kEpsTc0 + (float)kEpsTc1 * prm.rsqrt_dp * (fabsf(zn_own) + prm.xnmax[g]);
+                prm.err_mu[f] = mu_error_estimate(eps, a2_acc);
+                prm.err_q[f] = q_error_estimate(F8 && !far_cand ? eps + (float)kEpsF8 : eps, (float)prm.wnorm[g], (float)q_acc, s2_acc);
+            }
+            if (groups == 1 && zb == 2) b ^= 1;
+        }
+        if (__any_sync(0xffffffffu, bad) && lane == 0) atomicOr(prm.status, DEV_NONFINITE);
+    } else {
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kRegsMatern));
+        // ------------------------------------------------------------ Matern warp groups
+        const int grp = (warp - kFirstMatern) >> 2;   // 0..G-1
+        const int row = ((warp & 3) << 5) + lane;   // candidate row in the tile == TMEM lane
+        const uint32_t ring_addr = tmem + ((uint32_t)((warp & 3) * 32) << 16) + kRingCol;
+        uint32_t t = grp, t_base = 0;            // next own chunk, and the chunks before the current pair (all units' numbering)
+        int zi = 0;
+        uint32_t z_ph = 0, tile_iter = 0;
+        bool ok = true;
+        for (int unit = blockIdx.x; ok && unit < units; unit += unit_step, ++tile_iter) {
+            const int part = part_of(unit);
+            ok = mbar_wait_warp(bar(BAR_Z_FULL + zi), z_ph, abort_flag, wl);
             if (!ok) break;
-            const bool far_cand = zn_s[row] < 0.f;
-            const float zn = fabsf(zn_s[row]);
-
+            const float* znb = zn_buf(zi);
+            const float zn = znb[row], v_thresh = znb[TILE_M + row];
+            const float4 tile_s = *reinterpret_cast<const float4*>(znb + 2 * TILE_M);
+            const float kvscale = tile_s.x, inv = tile_s.y;   // inv: scaled k* -> k*, a power of two
+            const int g = __float_as_int(tile_s.z);
+            const uint64_t zn2 = pack2(zn, zn), minus2 = pack2(-2.f, -2.f);
+            const uint64_t pc0 = pack2(kvscale, kvscale), pc1 = pack2(kvscale * kPolyC1, kvscale * kPolyC1),
+                           pc2 = pack2(kvscale * kPolyC2, kvscale * kPolyC2);
             const float* xs_g = prm.xs32 + (size_t)g * prm.NP * DP;
-            const float v_thresh = far_cand ? INFINITY : kvscale * kRefine / (zn + prm.xnmax[g]);
-            const float pc0 = kvscale, pc1 = kvscale * kPolyC1, pc2 = kvscale * kPolyC2;
-            const float inv_kscale = 1.f / prm.kscale[g];   // scaled k* -> k*
             const float* xn_g = prm.xnorm + (size_t)g * prm.NP;
             const float* al_g = prm.alpha + (size_t)g * prm.NP;
-            double mu_acc = 0.0, a2_acc = 0.0, s2_acc = 0.0, q_acc = 0.0;
-            int pass_base = 0;   // chunks of this tile before pass p
-            // one chunk of this group: chunk c of pass p (which has nchunk chunks); clears ok when the CTA aborts
-            auto do_chunk = [&](const int c, const int p, const int nchunk) {
-                {
-                    const long long U = t / SL;       // distance product and the slice of its buffer
-                    const int db = (int)(U & 1), slice = (int)(t % SL);
-                    // the next own chunk's norms and weights: pull them towards L1 while this one is worked on
-                    if (lane < 2) {
-                        const int cn = c + G < nchunk ? c + G : (c + G - nchunk);
-                        const float* pf = (lane == 0 ? xn_g : al_g) + cn * KC;
-                        asm volatile("prefetch.global.L1 [%0];" ::"l"(pf));
-                    }
-                    TICK(7);
-                    ok = mbar_wait(bar(BAR_D_FULL + db), (uint32_t)((U >> 1) & 1), abort_flag, wl);
-                    ok = __all_sync(0xffffffffu, ok);
-                    if (!ok) return;
-                    TICK(0);
-                    if (threadIdx.x % 128 == 0) LOGEV(3, t);
+            double mu_acc = 0.0;
+            float a2_acc = 0.f, s2_acc = 0.f;    // scales of the error estimate
+            for (int p = prm.cut[part]; ok && p < prm.cut[part + 1]; ++p) {
+                const uint32_t chunks = (uint32_t)Pair(p, S, nc).chunks();
+                for (; ok && t - t_base < chunks; t += G) {
+                    const int c = (int)(t - t_base);
+                    const uint32_t u = t / KDC;
+                    ok = mbar_wait_warp(bar(BAR_D_FULL + u % BANKS), (u / BANKS) & 1u, abort_flag, wl);
+                    if (!ok) break;
                     tc_fence_after();
-                    const bool fresh = c >= p * CPP;   // first time this chunk is generated for the tile
-                    // k* buffer and the parity of its hand-over: the group's own buffer, or slot t mod NBK of the ring
-                    const int kbuf = NBK == G ? grp : (int)(t % NBK);
-                    const uint32_t kpar = NBK == G ? own_ph : (uint32_t)((t / NBK) & 1);
-                    uint8_t* kb = sm + map.k + (uint32_t)R3_IDX(kbuf, NBK, prm.status) * 16384u + row * 16;
-                    if (KT) (void)R3_IDX(KCOL + kbuf * KC + KC - 1, TMEM_COLS, prm.status);   // the slot's columns in tensor memory
-                    uint32_t kh[KC / 16][8], kl[KC / 16][8];
-                    // both halves of the chunk's dot products in one round trip to TMEM, then the buffer is free
-                    float dots[KC / 16][16];
+                    const uint32_t slot_addr = ring_addr + (t % kSlots) * KC;
+                    float dots[F8 ? 2 : 1][16];
+                    if (F8) {   // the 8-bit planes of both halves lie over the second half's dot products
+                        tc_ld16_issue(slot_addr, dots[0]);
+                        tc_ld16_issue(slot_addr + 16, dots[F8]);
+                        tc_wait_ld32(dots[0], dots[F8]);
+                    }
+                    const bool fresh = c >= 8 * p;   // first time this chunk is generated for the tile
+                    uint32_t f8h[2][4], f8l[2][4];
+                    constexpr int kUnroll = F8 ? 2 : 1;   // one copy of the loop's body where registers allow it: see above
+#pragma unroll kUnroll
+                    for (int h = 0; h < 2; ++h) {
+                        if (!F8) tc_ld16_issue(slot_addr + h * 16, dots[0]);
+                        const float* dot16 = dots[F8 ? h : 0];
+                        const int k0 = (int)R3_IDX(c * KC + h * 16, prm.NP - 15, prm.status);
+                        ulonglong2 xn[4];
 #pragma unroll
-                    for (int h = 0; h < KC / 16; ++h)
-                        tc_ld16_issue(lane_addr + NV + (uint32_t)R3_IDX(db * KD + slice * KC + h * 16, 2 * KD - 15, prm.status), dots[h]);
-                    tc_wait_ld32(dots[0], dots[1]);
-                    tc_fence_before();
-                    mbar_arrive(bar(BAR_D_EMPTY + db));
-                    TICK(1);
+                        for (int q = 0; q < 4; ++q) xn[q] = __ldg(reinterpret_cast<const ulonglong2*>(xn_g + k0 + 4 * q));
+                        if (!F8) tc_wait_ld16(dots[0]);
+                        uint64_t v2[8];   // k* times kvscale (the power of two of its FP16 split), in pairs
 #pragma unroll
-                    for (int h = 0; h < KC / 16; ++h) {
-                        const float* dot = dots[h];
-                        float kv[16];   // k* times kvscale (the power of two of its FP16 split)
-#pragma unroll
-                        for (int q = 0; q < 4; ++q) {
-                            const float4 xn4 =
-                                __ldg(reinterpret_cast<const float4*>(xn_g + R3_IDX(c * KC + h * 16 + 4 * q, prm.NP - 3, prm.status)));
-                            const float xn[4] = {xn4.x, xn4.y, xn4.z, xn4.w};
-#pragma unroll
-                            for (int e = 0; e < 4; ++e) {
-                                // |.|: a slightly negative r^2 (rounding) is a tiny distance either way
-                                const float u = sqrt_approx(fabsf(fmaf(-2.f, dot[4 * q + e], zn + xn[e])));
-                                kv[4 * q + e] = fmaf(u, fmaf(u, pc2, pc1), pc0) * exp2_approx(-u);
-                            }
+                        for (int e = 0; e < 8; ++e) {
+                            float r0, r1;
+                            unpack2(fma2(minus2, pack2(dot16[2 * e], dot16[2 * e + 1]), add2(zn2, e & 1 ? xn[e / 2].y : xn[e / 2].x)), r0, r1);
+                            // |.|: a slightly negative r^2 (rounding) is a tiny distance either way
+                            const float u0 = sqrt_approx(fabsf(r0)), u1 = sqrt_approx(fabsf(r1));
+                            const uint64_t uu = pack2(u0, u1);
+                            v2[e] = mul2(fma2(uu, fma2(uu, pc2, pc1), pc0), pack2(exp2_approx(-u0), exp2_approx(-u1)));
                         }
                         // largest of the sixteen in eight three-input maxima
-                        const float vmax = max3(max3(max3(kv[0], kv[1], kv[2]), max3(kv[3], kv[4], kv[5]), max3(kv[6], kv[7], kv[8])),
-                                                max3(max3(kv[9], kv[10], kv[11]), max3(kv[12], kv[13], kv[14]), kv[15]), 0.f);
-                        if (ZS) {
-                            if (vmax > v_thresh) {   // close pairs of this candidate: direct differences, inline
-                                uint32_t marked = 0;
+                        float m8[8];
 #pragma unroll
-                                for (int i = 0; i < 16; ++i) marked |= (kv[i] > v_thresh) ? (1u << i) : 0u;
-                                const float* zr = zs_s + row * kZsStride;
-                                for (; marked; marked &= marked - 1) {
-                                    const uint32_t i = (uint32_t)__ffs(marked) - 1u;
-                                    const float4* xp = reinterpret_cast<const float4*>(
-                                        xs_g + (size_t)R3_IDX(c * KC + h * 16 + (int)i, prm.NP, prm.status) * kZsMaxDP);
-                                    float acc0 = 0.f, acc1 = 0.f;
-#pragma unroll
-                                    for (int e = 0; e < 4; ++e) {
-                                        const float4 x4 = __ldg(xp + e);
-                                        float df = zr[4 * e] - x4.x;
-                                        acc0 = fmaf(df, df, acc0);
-                                        df = zr[4 * e + 1] - x4.y;
-                                        acc1 = fmaf(df, df, acc1);
-                                        df = zr[4 * e + 2] - x4.z;
-                                        acc0 = fmaf(df, df, acc0);
-                                        df = zr[4 * e + 3] - x4.w;
-                                        acc1 = fmaf(df, df, acc1);
-                                    }
-                                    const float u = sqrtf(acc0 + acc1);
-                                    const float val = kvscale * fmaf(u, fmaf(u, kPolyC2, kPolyC1), 1.f) * exp2f(-u);
-#pragma unroll
-                                    for (int e2 = 0; e2 < 16; ++e2) kv[e2] = (uint32_t)e2 == i ? val : kv[e2];
-                                }
-                            }
-                        } else
-                        if (__any_sync(0xffffffffu, vmax > v_thresh)) {
-                            // rare: close pairs.  Values refined in an earlier pass of this tile come back from the
-                            // cache without a call; what is left goes to the out-of-line refinement through a local
-                            // array, so that the hot path keeps kv in registers.
-                            const uint32_t key0 = (((uint32_t)tile_iter & 0x3ffffu) << 13) | (uint32_t)(c * KC + h * 16);
-                            unsigned long long* slots = P > 1 ? pair_cache + R3_IDX(row, TILE_M, prm.status) * kCacheSlots : nullptr;
-                            (void)R3_IDX(c * KC + h * 16 + 15, prm.NP, prm.status);   // rows of the FP32 observations the refinement reads
-                            bool need = vmax > v_thresh;
-                            if (need && slots && !fresh) {
-                                uint32_t marked = 0;
-#pragma unroll
-                                for (int i = 0; i < 16; ++i) marked |= (kv[i] > v_thresh) ? (1u << i) : 0u;
-                                need = false;
-                                for (; marked; marked &= marked - 1) {
-                                    const uint32_t i = (uint32_t)__ffs(marked) - 1u;
-                                    const unsigned long long e = slots[cache_slot(key0 + i)];
-                                    if ((uint32_t)(e >> 32) != key0 + i) {
-                                        need = true;
-                                        break;
-                                    }
-                                    const float val = __uint_as_float((uint32_t)e);
-#pragma unroll
-                                    for (int e2 = 0; e2 < 16; ++e2) kv[e2] = (uint32_t)e2 == i ? val : kv[e2];
-                                }
-                            }
-                            if (__any_sync(0xffffffffu, need)) {
-                                float tmp[16];
-#pragma unroll
-                                for (int i = 0; i < 16; ++i) tmp[i] = kv[i];
-                                if (slots)
-                                    refine_close_pairs<true>(tmp, v_thresh, kvscale, lane_addr + ZCOL, DP,
-                                                             xs_g + (size_t)(c * KC + h * 16) * DP, slots, key0, !fresh);
-                                else
-                                    refine_close_pairs<false>(tmp, v_thresh, kvscale, lane_addr + ZCOL, DP,
-                                                              xs_g + (size_t)(c * KC + h * 16) * DP, nullptr, 0u, false);
-#pragma unroll
-                                for (int i = 0; i < 16; ++i) kv[i] = tmp[i];
-                            }
+                        for (int e = 0; e < 8; e += 2) {
+                            float a0, a1, b0, b1;
+                            unpack2(v2[e], a0, a1);
+                            unpack2(v2[e + 1], b0, b1);
+                            m8[e / 2] = max3(a0, a1, b0);
+                            m8[4 + e / 2] = b1;
                         }
+                        const float vmax = max3(max3(m8[0], m8[1], m8[2]), max3(m8[3], m8[4], m8[5]), max3(m8[6], m8[7], 0.f));
+                        if (vmax > v_thresh) {   // close pairs of this candidate
+                            float kv[16];
+                            uint32_t marked = 0;
+#pragma unroll
+                            for (int e = 0; e < 8; ++e) unpack2(v2[e], kv[2 * e], kv[2 * e + 1]);
+                            if (Z32) {   // direct differences, inline
+#pragma unroll
+                                for (int i = 0; i < 16; ++i) marked |= (kv[i] > v_thresh) ? (1u << i) : 0u;
+                                const float4* zr = reinterpret_cast<const float4*>(sm + map.z32 + zi * map.z32_buf + row * 16);
+                                for (; marked; marked &= marked - 1) {
+                                    const uint32_t i = (uint32_t)__ffs(marked) - 1u;
+                                    const float4* xp = reinterpret_cast<const float4*>(xs_g + (size_t)(k0 + (int)i) * DP);
+                                    float acc0 = 0.f, acc1 = 0.f;
+#pragma unroll 4
+                                    for (int e = 0; e < DP / 4; ++e) {
+                                        const float4 x4 = __ldg(xp + e), z4 = zr[e * TILE_M];
+                                        float df = z4.x - x4.x;
+                                        acc0 = fmaf(df, df, acc0);
+                                        df = z4.y - x4.y;
+                                        acc1 = fmaf(df, df, acc1);
+                                        df = z4.z - x4.z;
+                                        acc0 = fmaf(df, df, acc0);
+                                        df = z4.w - x4.w;
+                                        acc1 = fmaf(df, df, acc1);
+                                    }
+                                    const float uu = sqrtf(acc0 + acc1);
+                                    const float val = kvscale * fmaf(uu, fmaf(uu, kPolyC2, kPolyC1), 1.f) * exp2f(-uu);
+#pragma unroll
+                                    for (int e2 = 0; e2 < 16; ++e2) kv[e2] = (uint32_t)e2 == i ? val : kv[e2];
+                                }
+                            } else {
+                                // rare: out of line, through a local array; values refined in an earlier pair of strips come back
+                                // from the tile's cache
+                                const uint32_t key0 = ((tile_iter & 0x3ffffu) << 13) | (uint32_t)k0;
+                                unsigned long long* slots = reinterpret_cast<unsigned long long*>(sm + map.cache) + row * kCacheSlots;
+                                refine_close_pairs_smem(kv, v_thresh, kvscale, sm + map.z + zi * map.z_buf + row * 16, DP,
+                                                        xs_g + (size_t)k0 * DP, S > 2 ? slots : nullptr, key0, !fresh);
+                            }
+#pragma unroll
+                            for (int e = 0; e < 8; ++e) v2[e] = pack2(kv[2 * e], kv[2 * e + 1]);
+                        }
+                        __syncwarp();   // the stores to tensor memory are warp-wide
                         if (fresh) {   // warp-uniform: the mean and the error scales see every observation once
-                            float mpart = 0.f, apart = 0.f, spart = 0.f;
+                            uint64_t mp = 0, ap = 0, sp = 0;
 #pragma unroll
                             for (int q = 0; q < 4; ++q) {
-                                const float4 al4 =
-                                    __ldg(reinterpret_cast<const float4*>(al_g + R3_IDX(c * KC + h * 16 + 4 * q, prm.NP - 3, prm.status)));
-                                const float al[4] = {al4.x, al4.y, al4.z, al4.w};
+                                const ulonglong2 al = __ldg(reinterpret_cast<const ulonglong2*>(al_g + k0 + 4 * q));
 #pragma unroll
-                                for (int e = 0; e < 4; ++e) {
-                                    const float v = kv[4 * q + e], va = v * al[e];
-                                    mpart += va;
-                                    apart = fmaf(va, va, apart);
-                                    spart = fmaf(v, v, spart);
+                                for (int e = 0; e < 2; ++e) {
+                                    const uint64_t v = v2[2 * q + e], va = mul2(v, e ? al.y : al.x);
+                                    mp = add2(mp, va);
+                                    ap = fma2(va, va, ap);
+                                    sp = fma2(v, v, sp);
                                 }
                             }
-                            mu_acc += (double)(mpart * inv_kscale);
-                            a2_acc += (double)(apart * inv_kscale * inv_kscale);
-                            s2_acc += (double)(spart * inv_kscale * inv_kscale);
+                            float m0, m1, a0, a1, b0, b1;
+                            unpack2(mp, m0, m1);
+                            unpack2(ap, a0, a1);
+                            unpack2(sp, b0, b1);
+                            mu_acc += (double)(m0 + m1);
+                            a2_acc += a0 + a1;
+                            s2_acc += b0 + b1;
                         }
-                        // split into the two FP16 planes; the stores wait until the whole chunk is computed
-                        // so that the arithmetic does not sit between the buffer's release and its refill
+                        // split into the FP16 planes and over the dot products they came from
+                        uint32_t out[16];
                         if (F8) {
-                            // kl[h][0..3]: the 16 hi parts as E5M2, kl[h][4..7]: the 16 lo parts
 #pragma unroll
-                            for (int e = 0; e < 4; ++e)
-                                split4_f8(kv + 4 * e, kh[h][2 * e], kh[h][2 * e + 1], kl[h][e], kl[h][4 + e]);
+                            for (int e = 0; e < 4; ++e) {
+                                float v4[4];
+                                unpack2(v2[2 * e], v4[0], v4[1]);
+                                unpack2(v2[2 * e + 1], v4[2], v4[3]);
+                                split4_f8(v4, out[2 * e], out[2 * e + 1], f8h[h][e], f8l[h][e]);
+                            }
+                            tc_st8(slot_addr + (h ? 24 : 0), out);
                         } else {
 #pragma unroll
                             for (int e = 0; e < 8; ++e) {
-                                __half2 hi, lo;
-                                split2(kv[2 * e], kv[2 * e + 1], hi, lo);
-                                kh[h][e] = *reinterpret_cast<const uint32_t*>(&hi);
-                                kl[h][e] = *reinterpret_cast<const uint32_t*>(&lo);
+                                float a, b;
+                                unpack2(v2[e], a, b);
+                                const __half2 hi = __floats2half2_rn(a, b);
+                                const __half2 lo = __floats2half2_rn(minus_half(a, __low2half(hi)), minus_half(b, __high2half(hi)));
+                                out[e] = *reinterpret_cast<const uint32_t*>(&hi);
+                                out[8 + e] = *reinterpret_cast<const uint32_t*>(&lo);
                             }
+                            tc_st16(slot_addr + h * 16, out);
                         }
                     }
-                    TICK(2);
-                    if (threadIdx.x % 128 == 0) LOGEV(4, t);
-                    if (NBK == G) {
-                        ok = mbar_wait(bar(BAR_K_EMPTY + kbuf), kpar ^ 1u, abort_flag, wl);
-                    } else if (t >= NBK) {
-                        // Ring shorter than the number of groups: slot t mod NBK is free once chunk t - NBK has
-                        // been consumed.  A parity wait is only valid at most one phase behind, and with one
-                        // barrier per slot this group could be two uses of its slot ahead of the issuer, or the
-                        // issuer two ahead of the group.  The "consumed" barriers are therefore indexed by the
-                        // chunk number mod 4: the chunks 4 apart that share a barrier are never both pending.
-                        const long long te = t - NBK;
-                        ok = mbar_wait(bar(BAR_K_EMPTY + (int)(te & 3)), (uint32_t)((te >> 2) & 1), abort_flag, wl);
-                    }
-                    ok = __all_sync(0xffffffffu, ok);
-                    if (!ok) return;
-                    TICK(3);
-                    if (threadIdx.x % 128 == 0) LOGEV(5, t);
                     if (F8) {
-                        if (KT) {
-                            // FP16 hi plane: 16 columns; then the chunk's 32 E5M2 hi parts (8 columns) and lo parts (8)
-                            uint32_t p8[8];
-                            tc_st8(lane_addr + KCOL + (uint32_t)kbuf * KC, kh[0]);
-                            tc_st8(lane_addr + KCOL + (uint32_t)kbuf * KC + 8, kh[1]);
+                        uint32_t o8[16];
 #pragma unroll
-                            for (int e = 0; e < 4; ++e) { p8[e] = kl[0][e]; p8[4 + e] = kl[1][e]; }
-                            tc_st8(lane_addr + KCOL + (uint32_t)kbuf * KC + KC / 2, p8);
-#pragma unroll
-                            for (int e = 0; e < 4; ++e) { p8[e] = kl[0][4 + e]; p8[4 + e] = kl[1][4 + e]; }
-                            tc_st8(lane_addr + KCOL + (uint32_t)kbuf * KC + KC / 2 + KC / 4, p8);
-                        } else {
-#pragma unroll
-                            for (int h = 0; h < KC / 16; ++h) {
-#pragma unroll
-                                for (int sl = 0; sl < 2; ++sl)
-                                    *reinterpret_cast<uint4*>(kb + (2 * h + sl) * 2048u) =
-                                        make_uint4(kh[h][4 * sl], kh[h][4 * sl + 1], kh[h][4 * sl + 2], kh[h][4 * sl + 3]);
-                                // one 16-byte k-slice of each 8-bit plane per 16 observations
-                                *reinterpret_cast<uint4*>(kb + 8192u + h * 2048u) = make_uint4(kl[h][0], kl[h][1], kl[h][2], kl[h][3]);
-                                *reinterpret_cast<uint4*>(kb + 12288u + h * 2048u) = make_uint4(kl[h][4], kl[h][5], kl[h][6], kl[h][7]);
-                            }
+                        for (int e = 0; e < 4; ++e) {
+                            o8[e] = f8h[0][e];
+                            o8[4 + e] = f8h[1][e];
+                            o8[8 + e] = f8l[0][e];
+                            o8[12 + e] = f8l[1][e];
                         }
-                    } else
-#pragma unroll
-                    for (int h = 0; h < KC / 16; ++h) {
-                        if (KT) {
-                            // 16 columns = 8 packed TMEM columns of each plane
-                            tc_st8(lane_addr + KCOL + (uint32_t)kbuf * KC + h * 8, kh[h]);
-                            tc_st8(lane_addr + KCOL + (uint32_t)kbuf * KC + KC / 2 + h * 8, kl[h]);
-                        } else {
-                            // 16 columns = two 16-byte k-slices of the A operand, hi and lo planes
-#pragma unroll
-                            for (int sl = 0; sl < 2; ++sl) {
-                                *reinterpret_cast<uint4*>(kb + (2 * h + sl) * 2048u) =
-                                    make_uint4(kh[h][4 * sl], kh[h][4 * sl + 1], kh[h][4 * sl + 2], kh[h][4 * sl + 3]);
-                                *reinterpret_cast<uint4*>(kb + 8192u + (2 * h + sl) * 2048u) =
-                                    make_uint4(kl[h][4 * sl], kl[h][4 * sl + 1], kl[h][4 * sl + 2], kl[h][4 * sl + 3]);
-                            }
-                        }
+                        tc_st16(slot_addr + 8, o8);
                     }
-                    if (!ok) return;
-                    if (KT) {
-                        asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-                        tc_fence_before();
-                    } else {
-                        fence_proxy_async();
-                    }
-                    mbar_arrive(bar(BAR_K_FULL + kbuf));
-                    TICK(4);
-                    if (threadIdx.x % 128 == 0) LOGEV(6, t);
-                    t += G;
-                    own_ph ^= 1u;
+                    asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(bar(BAR_K_FULL + t % kSlots));
                 }
-            };
-            // end of a pass: q += sum_i V^2 over this group's share of the columns, then the accumulator is free
-            auto do_epilogue = [&]() {
-                TICK(7);
-                ok = mbar_wait(bar(BAR_V_FULL), v_ph, abort_flag, wl);
-                ok = __all_sync(0xffffffffu, ok);
-                if (!ok) return;
-                TICK(5);
-                tc_fence_after();
-#pragma unroll 1
-                for (int c0 = grp * 16; c0 < NV; c0 += 32 * G) {   // two column blocks per round trip to TMEM
-                    const int c1 = c0 + 16 * G;
-                    (void)R3_IDX(c0 + 15, NV, prm.status);
-                    float v[16], w[16];
-                    float part0 = 0.f, part1 = 0.f;
-                    if (c1 < NV) {
-                        tc_ld16_issue(lane_addr + c0, v);
-                        tc_ld16_issue(lane_addr + c1, w);
-                        tc_wait_ld32(v, w);
-#pragma unroll
-                        for (int i = 0; i < 16; ++i) part1 = fmaf(w[i], w[i], part1);
-                    } else {
-                        tc_ld16(lane_addr + c0, v);
-                    }
-#pragma unroll
-                    for (int i = 0; i < 16; ++i) part0 = fmaf(v[i], v[i], part0);
-                    q_acc += (double)part0;
-                    q_acc += (double)part1;
-                }
-                tc_fence_before();
-                mbar_arrive(bar(BAR_V_EMPTY));
-                TICK(6);
-                v_ph ^= 1u;
-            };
-            if constexpr (!PUTOFF) {
-                for (int p = 0; ok && p < P; ++p) {
-                    const int nchunk = (p + 1) * CPP;
-                    // own chunks of this pass: global t with t - t_tile0 - pass_base in [0, nchunk)
-                    while (ok && t - t_tile0 - pass_base < nchunk) do_chunk((int)(t - t_tile0 - pass_base), p, nchunk);
-                    if (!ok) break;
-                    pass_base += nchunk;
-                    do_epilogue();
-                }
-            } else {
-                // one loop over the group's chunks of the tile, pass after pass, the epilogues in between
-                int p = 0, nchunk = CPP, epilogues_due = 0;
-                while (ok) {
-                    bool first_of_pass = false;
-                    if (t - t_tile0 - pass_base >= nchunk) {   // this group's chunks of pass p are done
-                        pass_base += nchunk;
-                        ++p;
-                        nchunk += CPP;
-                        ++epilogues_due;
-                        first_of_pass = true;
-                    }
-                    const int c = (int)(t - t_tile0 - pass_base);
-                    const bool put_off = first_of_pass && p < P && (NBK == G || c < NBK);
-                    for (int run = epilogues_due - (put_off ? 1 : 0); ok && run > 0; --run) {
-                        --epilogues_due;
-                        do_epilogue();
-                    }
-                    if (!ok || p >= P) break;
-                    do_chunk(c, p, nchunk);
-                }
+                t_base += chunks;
             }
             if (!ok) break;
-            t_tile0 += items_per_tile;
-            // ---- combine the groups' partial sums; group 0 finishes the candidate
-            double* mine = red + (size_t)R3_IDX(grp * TILE_M + row, G * TILE_M, prm.status) * 4;
-            mine[0] = mu_acc; mine[1] = a2_acc; mine[2] = s2_acc; mine[3] = q_acc;
-            mbar_arrive(bar(BAR_RED_READY));
-            if (grp == 0) {   // only the finishing group waits; the others move on to the next tile
-                ok = mbar_wait(bar(BAR_RED_READY), (uint32_t)(tile_iter & 1), abort_flag, wl);
-                ok = __all_sync(0xffffffffu, ok);
-                if (!ok) break;
-                if (valid) {
-                    mu_acc = a2_acc = s2_acc = q_acc = 0.0;
-#pragma unroll
-                    for (int gg = 0; gg < G; ++gg) {
-                        const double* o = red + ((size_t)gg * TILE_M + row) * 4;
-                        mu_acc += o[0]; a2_acc += o[1]; s2_acc += o[2]; q_acc += o[3];
-                    }
-                    q_acc *= prm.vinv2[g];   // undo the power-of-two scaling of k* and W
-                    const size_t f = (size_t)R3_IDX((long long)g * prm.m + cand, (long long)prm.batch * prm.m, prm.status);
-                    const CandidateResult res = finalize_candidate(mu_acc, q_acc, (double)sf2, (double)prm.best[R3_IDX(g, prm.batch, prm.status)]);
-                    __stcs(prm.mu + f, res.mu);
-                    __stcs(prm.sigma + f, res.sigma);
-                    __stcs(prm.ei + f, res.ei);
-                    const double eps =
-                        far_cand ? 1.0 : kEpsTc0 + kEpsTc1 * (double)(zn + prm.xnmax[g]) * rsqrt((double)DP);
-                    prm.err_mu[f] = mu_error_estimate(eps, a2_acc);
-                    prm.err_q[f] = q_error_estimate(F8 && !far_cand ? eps + kEpsF8 : eps, prm.wnorm[g], q_acc, s2_acc);
-                }
-            }
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bar(BAR_Z_EMPTY + zi));
+            ok = mbar_wait_warp(bar(BAR_RED_EMPTY + zi), z_ph ^ 1u, abort_flag, wl);
+            if (!ok) break;
+            uint8_t* o = sm + map.red + zi * map.red_buf + (R3_IDX(grp * TILE_M + row, G * TILE_M, prm.status)) * 16;
+            *reinterpret_cast<double*>(o) = mu_acc * (double)inv;
+            *reinterpret_cast<float2*>(o + 8) = make_float2(a2_acc * inv * inv, s2_acc * inv * inv);
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bar(BAR_RED_FULL + zi));
+            if (++zi == zb) { zi = 0; z_ph ^= 1u; }
         }
-        if (__any_sync(0xffffffffu, bad) && lane == 0) atomicOr(prm.status, DEV_NONFINITE);
-        if (prm.trace && q4 == 0 && lane == 0 && grp < 2)
-            for (int i = 0; i < 8; ++i) prm.trace[((size_t)blockIdx.x * 4 + 1 + grp) * 8 + i] = tacc[i];
     }
 
     // ---------------------------------------------------------------- teardown
@@ -971,7 +1008,7 @@ __global__ void centre_kernel(const float* __restrict__ X, const float* __restri
 // and the largest scaled coordinate (the FP16 planes have a limited range).
 __global__ void xt_build_kernel(const float* __restrict__ X, const float* __restrict__ centre,
                                 const float* __restrict__ scale, const float* __restrict__ alpha32, int n, int d,
-                                int npad_fit, int DP, int NP, int KD, __half* __restrict__ xt,
+                                int npad_fit, int DP, int parts, int NP, int KD, __half* __restrict__ xt,
                                 float* __restrict__ xs32, float* __restrict__ xnorm, float* __restrict__ alpha, unsigned* __restrict__ xamax_bits,
                                 unsigned* __restrict__ xnmax_bits)
 {
@@ -989,9 +1026,10 @@ __global__ void xt_build_kernel(const float* __restrict__ X, const float* __rest
         amax = fmaxf(amax, fabsf(xv));
         xs32[((size_t)g * NP + k) * DP + j] = xv;
         const __half h = __float2half_rn(xv);
-        const size_t off = ((size_t)(j / 8) * KD + r) * 8 + (j % 8);
+        const int DPp = DP / parts, jp = j % DPp;
+        const size_t off = (size_t)(j / DPp) * (2 * DPp * KD) + ((size_t)(jp / 8) * KD + r) * 8 + (jp % 8);
         blob[off] = h;
-        blob[(size_t)DP * KD + off] = __float2half_rn(xv - __half2float(h));
+        blob[(size_t)DPp * KD + off] = __float2half_rn(xv - __half2float(h));
     }
     for (int o = 16; o > 0; o >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o));
     if ((threadIdx.x & 31) == 0) atomicMax(xamax_bits, __float_as_uint(amax));
@@ -1021,81 +1059,79 @@ __host__ __device__ inline void operand_scales(float wmax, float sf2, bool f8, i
     sk = kScaleExp - ek;
 }
 
-// One block per (chunk c, pass p, GP): the KC x NV block of 2^eW W (rows p NV.., columns c KC..) as
-// FP16 hi/lo planes in the B-operand layout; zero outside the lower triangle and outside n.
+// One block per (chunk c, strip s, GP): the block of 2^eW W (rows 128 s.., columns c KC..) as FP16 hi/lo planes in the
+// B-operand layout; zero outside the lower triangle and outside n.  A thread takes eight consecutive columns of a row: it
+// reads 64 contiguous bytes and writes 16 to each plane.
 // With f8 the second plane holds, instead of the FP16 lo parts, two 8-bit planes in the 8-bit form of the same
 // layout (16 k-elements per 16-byte slice): the hi parts as E4M3 (|2^eW W| < 2^8 for these histories), then the
-// lo parts as E5M2.
-__global__ void wt_build_kernel(const double* __restrict__ W64, int n, int npad_fit, int NV, size_t gp_stride,
+// lo parts as E5M2.  strip_rows: 128, or 256 for the paired kernel's passes.
+__global__ void wt_build_kernel(const double* __restrict__ W64, int n, int npad_fit, int strip_rows, int nc, size_t gp_stride,
                                 const unsigned* __restrict__ wmax, const float* __restrict__ sf2, float* __restrict__ kscale,
                                 double* __restrict__ vinv2, __half* __restrict__ wt, bool f8)
 {
-    const int c = blockIdx.x, p = blockIdx.y, g = blockIdx.z;
-    const int CPP = NV / KC;
-    if (c >= (p + 1) * CPP) return;
-    const size_t tile = (size_t)CPP * p * (p + 1) / 2 + c;
-    __half* dst = wt + (size_t)g * gp_stride + tile * (2 * KC * NV);
+    const int c = blockIdx.x, s = blockIdx.y, g = blockIdx.z, per = strip_rows / KC;
+    if (c >= (s + 1) * per) return;
+    const int rows = min(strip_rows, nc * KC - s * strip_rows);
+    __half* dst = wt + (size_t)g * gp_stride + (size_t)per * s * (s + 1) / 2 * (2 * KC * strip_rows) + (size_t)c * (2 * KC * rows);
     const double* Wg = W64 + (size_t)g * npad_fit * npad_fit;
     int sw, sk;
     operand_scales(__uint_as_float(wmax[g]), sf2[g], f8, sw, sk);
     const double sc = ldexp(1.0, sw);
-    if (c == 0 && p == 0 && threadIdx.x == 0) {
+    if (c == 0 && s == 0 && threadIdx.x == 0) {
         kscale[g] = (float)ldexp(1.0, sk);
         vinv2[g] = ldexp(1.0, -2 * (sw + sk));
     }
-    for (int e = threadIdx.x; e < KC * NV; e += blockDim.x) {
-        const int kk = e % KC, r = e / KC;   // consecutive threads walk k: coalesced reads of a W row
-        const int i = p * NV + r, k = c * KC + kk;
-        float w = 0.f;
-        if (i < n && k <= i) w = (float)(Wg[(size_t)i * npad_fit + k] * sc);
-        const __half h = __float2half_rn(w);
-        const size_t off = ((size_t)(kk / 8) * NV + r) * 8 + (kk % 8);
-        dst[off] = h;
+    for (int e = threadIdx.x; e < rows * (KC / 8); e += blockDim.x) {
+        const int k8 = e % (KC / 8), r = e / (KC / 8);
+        const int i = s * strip_rows + r, k = c * KC + k8 * 8;
+        float w[8] = {};
+        if (i < n && k <= i) {   // a row of W has npad_fit >= i + 1 columns, a multiple of 32
+            const double2* src = reinterpret_cast<const double2*>(Wg + (size_t)i * npad_fit + k);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const double2 v = src[q];
+                w[2 * q] = k + 2 * q <= i ? (float)(v.x * sc) : 0.f;
+                w[2 * q + 1] = k + 2 * q + 1 <= i ? (float)(v.y * sc) : 0.f;
+            }
+        }
+        __half2 hi[4];
+        float lo[8];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            hi[q] = __floats2half2_rn(w[2 * q], w[2 * q + 1]);
+            const float2 back = __half22float2(hi[q]);
+            lo[2 * q] = w[2 * q] - back.x;
+            lo[2 * q + 1] = w[2 * q + 1] - back.y;
+            w[2 * q] = back.x;
+            w[2 * q + 1] = back.y;
+        }
+        const size_t off = ((size_t)k8 * rows + r) * 8;
+        *reinterpret_cast<uint4*>(dst + off) = *reinterpret_cast<const uint4*>(hi);
         if (f8) {
-            uint8_t* d8 = reinterpret_cast<uint8_t*>(dst + (size_t)KC * NV);
-            const size_t off8 = ((size_t)(kk / 16) * NV + r) * 16 + (kk % 16);
-            const float hf = __half2float(h);
-            d8[off8] = (uint8_t)(e4m3x4(hf, 0.f, 0.f, 0.f) & 0xffu);
-            d8[(size_t)KC * NV + off8] = (uint8_t)(e5m2x4(w - hf, 0.f, 0.f, 0.f) & 0xffu);
+            uint8_t* d8 = reinterpret_cast<uint8_t*>(dst + (size_t)KC * rows);
+            const size_t off8 = ((size_t)(k8 / 2) * rows + r) * 16 + (k8 % 2) * 8;
+            *reinterpret_cast<uint2*>(d8 + off8) = make_uint2(e4m3x4(w[0], w[1], w[2], w[3]), e4m3x4(w[4], w[5], w[6], w[7]));
+            *reinterpret_cast<uint2*>(d8 + (size_t)KC * rows + off8) =
+                make_uint2(e5m2x4(lo[0], lo[1], lo[2], lo[3]), e5m2x4(lo[4], lo[5], lo[6], lo[7]));
         } else {
-            dst[(size_t)KC * NV + off] = __float2half_rn(w - __half2float(h));
+            __half2 l2[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) l2[q] = __floats2half2_rn(lo[2 * q], lo[2 * q + 1]);
+            *reinterpret_cast<uint4*>(dst + (size_t)KC * rows + off) = *reinterpret_cast<const uint4*>(l2);
         }
     }
 }
 
 TensorOperands* ops_of(const r3_fit_state* gp) { return static_cast<TensorOperands*>(gp->tc); }
 
-void (*kernel_for(int NV, int G, bool kt, int nbk, bool f8, bool putoff, bool zs))(const TcParams)
-{
-    if (zs && kt && nbk == 2 && G == 3 && !f8) {   // at most 16 features, in the preferred shape
-        if (NV == 128) return score_tc_kernel<128, 3, 64, true, 2, false, false, true>;
-        return putoff ? score_tc_kernel<256, 3, 64, true, 2, false, true, true> : score_tc_kernel<256, 3, 64, true, 2, false, false, true>;
-    }
-    if (putoff && !f8 && NV == 256 && G == 3) {   // histories of two to seven passes in the two preferred shapes
-        if (kt && nbk == 2) return score_tc_kernel<256, 3, 64, true, 2, false, true>;
-        if (!kt && nbk == 3) return score_tc_kernel<256, 3, 64, false, 3, false, true>;
-    }
-    if (f8) {   // offered for the shapes of long histories only (tc_prepare)
-        if (kt && nbk == 2 && G == 3) return score_tc_kernel<256, 3, 64, true, 2, true>;
-        if (kt) return G == 3 ? score_tc_kernel<256, 3, 64, true, 3, true> : score_tc_kernel<256, 2, 64, true, 2, true>;
-        return G == 3 ? score_tc_kernel<256, 3, 64, false, 3, true> : score_tc_kernel<256, 2, 64, false, 2, true>;
-    }
-    if (kt && nbk == 2 && G == 3)
-        return NV == 256 ? score_tc_kernel<256, 3, 64, true, 2> : score_tc_kernel<128, 3, 64, true, 2>;
-    if (kt) {
-        if (NV == 256) return G == 3 ? score_tc_kernel<256, 3, 64, true> : score_tc_kernel<256, 2, 64, true>;
-        return G == 3 ? score_tc_kernel<128, 3, 64, true> : score_tc_kernel<128, 2, 64, true>;
-    }
-    if (NV == 256) return G == 3 ? score_tc_kernel<256, 3, 64, false> : score_tc_kernel<256, 2, 64, false>;
-    return G == 3 ? score_tc_kernel<128, 3, 64, false> : score_tc_kernel<128, 2, 64, false>;
-}
-
-constexpr int kF8MinPasses = 8;   // n > 1792: below that the guard hands more candidates to the FP64 pass than the cheaper MMAs save
+constexpr int kF8MinPasses = 8;   // pairs of strips (n > 1792): below that the guard hands more candidates to the FP64 pass than the cheaper MMAs save
 
 // The kernel a set of operands runs on, with or without FP8 cross terms
 void (*kernel_of(const TensorOperands* t, bool f8))(const TcParams)
 {
-    return kernel_for(t->NV, t->G, t->kt, t->nbk, f8, t->P >= 2 && t->P < kF8MinPasses, t->DP <= kZsMaxDP);
+    const bool z32 = t->DP <= kZ32MaxDP;
+    if (f8) return z32 ? score_tc_kernel<true, true> : score_tc_kernel<true, false>;
+    return z32 ? score_tc_kernel<false, true> : score_tc_kernel<false, false>;
 }
 
 int env_int(const char* name, int fallback)
@@ -1136,51 +1172,38 @@ r3_status_t tc_prepare(r3_fit_state& st, int device, cudaStream_t stream)
         return R3_ERR_ALLOC;
     }
     st.tc = t;
-    t->DP = round_up(d, 16);
-    t->NV = n > 128 ? 256 : 128;
-    t->NP = round_up(n, t->NV);
-    t->P = t->NP / t->NV;
-    // Shape, in order of preference (measured on the largest workload: the first two are within 1 %):
-    // k* in shared memory with three Matern groups and at least three W stages; k* in TMEM (needs
-    // V accumulator + two distance buffers + candidates + G k* buffers <= 512 columns), which frees
-    // shared memory for W stages; then whatever fits with two W stages.
-    const size_t budget = 227 * 1024 - 1024 - kBarBytes;
-    const int want_kt = env_int("R3_TC_KT", -1), want_g = env_int("R3_TC_G", 0);
-    t->KD = 64;
-    bool found = false;
-    static const struct { bool kt; int G, min_ws, nbk; } prefs[] = {
-        {true, 3, 3, 2},  {false, 3, 3, 3}, {true, 3, 3, 3}, {true, 2, 3, 2},
-        {false, 2, 3, 2}, {false, 3, 2, 3}, {true, 2, 2, 2}, {false, 2, 2, 2}};
-    const int want_nbk = env_int("R3_TC_NBK", 0);
-    // Stages of W: four by default although shared memory would hold up to six for few features.  Measured, the
-    // fifth and sixth buy nothing on any workload and cost the short histories 3-5 % (256 observations, 16
-    // features: 0.241 ms to 0.228 ms per pool; 512 and 32: 5.79 ms to 5.63 ms; 1024 and 4096 observations:
-    // unchanged down to three).  R3_TC_MAXWS = 2..6 overrides.
-    const int max_ws = std::min(std::max(env_int("R3_TC_MAXWS", 4), 2), MAX_STAGES);
-    for (const auto& pr : prefs) {
-        if (found) break;
-        t->kt = pr.kt;
-        t->G = pr.G;
-        t->nbk = pr.nbk;
-        if (want_kt >= 0 && (int)t->kt != want_kt) continue;
-        if (want_g && t->G != want_g) continue;
-        if (want_nbk && t->nbk != want_nbk) continue;
-        if (t->NV + 2 * t->KD + t->DP + (t->kt ? t->nbk * KC : 0) > 512) continue;
-        for (t->ws = max_ws; t->ws >= 2; --t->ws)
-            if (smem_map(t->DP, t->NV, t->G, t->KD, t->ws, t->kt).bar <= budget) break;
-        found = t->ws >= pr.min_ws;
-    }
-    if (!found) {
-        tc_release(st);   // does not fit: the SIMT engine serves this shape
-        return R3_OK;
-    }
-    t->smem_bytes = smem_map(t->DP, t->NV, t->G, t->KD, t->ws, t->kt).bar + kBarBytes + 1024;
-    // FP8 cross terms: R3_TC_F8 = 0/1 decides; by default histories of at least kF8MinPasses passes take them
+    // R3_TC_PAIR=1 lays the operands out for the paired kernel (r3_score_tc2.cu) where that serves the shape
     const int want_f8 = env_int("R3_TC_F8", -1);
-    t->f8 = t->NV == 256 && (want_f8 >= 0 ? want_f8 != 0 : t->P >= kF8MinPasses);
-    const int CPP = t->NV / KC;
-    const size_t tiles = (size_t)CPP * t->P * (t->P + 1) / 2;
-    t->wt_gp_stride = tiles * (2 * (size_t)KC * t->NV);
+    t->f8 = want_f8 >= 0 ? want_f8 != 0 && n > 128 : (n + 255) / 256 >= kF8MinPasses;
+    t->DP = round_up(d, 16);
+    t->KD = KD;
+    t->NP = round_up(n, 256);
+    t->P = t->NP / 256;
+    int pair_ws = 0;
+    t->pair = env_int("R3_TC_PAIR", 0) != 0 && !t->f8 && tc_pair_fits(t, &pair_ws);
+    if (!t->pair) {
+        t->parts = (t->DP + kPartDP - 1) / kPartDP;
+        t->DP = t->parts * round_up((t->DP + t->parts - 1) / t->parts, 16);
+        t->NP = round_up(n, KD);
+        t->S = (n + kStrip - 1) / kStrip;
+        t->P = (t->S + 1) / 2;
+        t->G = G;
+        const size_t budget = 227 * 1024 - 1024;
+        t->zb = 2;
+        t->xs = 2;
+        t->ws = 6;   // four per accumulator instead of three: no faster (512 observations) or slower (701 by 0.1 ms in 0.6)
+        auto bytes = [&] { return (size_t)smem_map(t->DP, t->parts, t->zb, t->xs, t->ws).end; };
+        if (bytes() > budget) t->zb = 1;
+        while (t->ws > 4 && bytes() > budget) t->ws -= 2;
+        if (bytes() > budget) {
+            tc_release(st);   // does not fit: the SIMT engine serves this shape
+            return R3_OK;
+        }
+        t->smem_bytes = bytes() + 1024;
+    }
+    const int strip_rows = t->pair ? 256 : kStrip, strips = t->pair ? t->P : t->S, chunks = t->NP / KC, per = strip_rows / KC;
+    const int last_rows = t->NP - (strips - 1) * strip_rows;
+    t->wt_gp_stride = (size_t)per * strips * (strips - 1) / 2 * (2 * KC * strip_rows) + (size_t)chunks * (2 * KC * last_rows);
     auto fail = [&](const char* what, cudaError_t e) {
         set_error("%s failed: %s", what, cudaGetErrorString(e));
         cudaStreamSynchronize(stream);
@@ -1214,17 +1237,18 @@ r3_status_t tc_prepare(r3_fit_state& st, int device, cudaStream_t stream)
     // scaled by a power of two that the largest |W| decides
     centre_kernel<<<dim3(t->DP, B), 256, 0, stream>>>(st.X, st.inv_ell, n, d, t->DP, t->centre, t->scale);
     xt_build_kernel<<<dim3(t->NP / t->KD, B), 256, 0, stream>>>(st.X, t->centre, t->scale, st.alpha32, n, d, st.npad, t->DP,
-                                                                t->NP, t->KD, t->xt, t->xs32, t->xnorm, t->alpha, st.xamax_d,
+                                                                t->parts, t->NP, t->KD, t->xt, t->xs32, t->xnorm, t->alpha, st.xamax_d,
                                                                 st.xnmax_d);
-    wt_build_kernel<<<dim3(t->P * CPP, t->P, B), 256, 0, stream>>>(st.W64, n, st.npad, t->NV, t->wt_gp_stride, st.wmax_d,
-                                                                   st.sf2_d, t->kscale, t->vinv2, t->wt, t->f8);
+    wt_build_kernel<<<dim3(chunks, strips, B), 256, 0, stream>>>(st.W64, n, st.npad, strip_rows, chunks, t->wt_gp_stride, st.wmax_d,
+                                                                 st.sf2_d, t->kscale, t->vinv2, t->wt, t->f8);
     g_launches += 3;
     if (t->wt16) {
-        wt_build_kernel<<<dim3(t->P * CPP, t->P, B), 256, 0, stream>>>(st.W64, n, st.npad, t->NV, t->wt_gp_stride, st.wmax_d,
-                                                                       st.sf2_d, t->kscale, t->vinv2_16, t->wt16, false);
+        wt_build_kernel<<<dim3(chunks, strips, B), 256, 0, stream>>>(st.W64, n, st.npad, strip_rows, chunks, t->wt_gp_stride,
+                                                                     st.wmax_d, st.sf2_d, t->kscale, t->vinv2_16, t->wt16, false);
         ++g_launches;
     }
     if ((e = cudaGetLastError()) != cudaSuccess) return fail("operand preparation launch", e);
+    if (t->pair) return R3_OK;
     // The cap on dynamic shared memory belongs to the kernel, not to the handle, and handles with different
     // feature counts share an instantiation with different sizes: raise it to the device's limit (the kernel
     // has no static shared memory), so that no handle's preparation lowers it for another.
@@ -1265,11 +1289,66 @@ void tc_info(const r3_gp* gp, int* info)
     const TensorOperands* t = ops_of(gp);
     for (int i = 0; i < 8; ++i) info[i] = 0;
     if (!t) return;
-    info[0] = t->NV; info[1] = t->P; info[2] = t->DP; info[3] = t->NP;
-    info[4] = t->G; info[5] = t->ws; info[6] = t->kt ? 1 : 0; info[7] = t->f8 ? 1 : 0;
+    info[0] = 256; info[1] = t->P; info[2] = t->DP; info[3] = t->NP;
+    info[4] = t->G; info[5] = t->ws; info[6] = t->pair ? 0 : 1; info[7] = t->f8 ? 1 : 0;
 }
 
-size_t score_tc_workspace_bytes(const r3_gp* gp, long long m) { return guard_workspace_bytes(gp, m); }
+// How many units a tile's pairs of strips are shared out to.  A pool of few tiles leaves SMs idle, and one of a few waves its
+// last wave: the parts of a tile are scored by different CTAs and the last of them adds the sums up.  The choice minimises
+// waves x the longest part, a pair of strips counted as its chunks of k* and a unit as kUnitChunks more (prologue, drain of the
+// pipeline, epilogue).  It depends on the whole pool, not on the piece a launch covers.
+constexpr int kUnitChunks = 8;
+static int plan_splits(const TensorOperands* t, long long tiles, int sms, unsigned char* cut)
+{
+    const int nc = t->NP / KC;
+    auto chunks = [&](int p) { return std::min(8 * (p + 1), nc); };
+    cut[0] = 0;
+    cut[1] = (unsigned char)t->P;
+    long long all = 0;
+    for (int p = 0; p < t->P; ++p) all += chunks(p);
+    int best = 1;
+    if (tiles >= 16ll * sms || t->pair) return best;
+    long long best_cost = (tiles + sms - 1) / sms * (all + kUnitChunks);
+    best_cost -= best_cost / 20;   // sharing out has to gain something
+    for (int k = 2; k <= std::min(t->P, kMaxSplits); ++k) {
+        unsigned char c[kMaxSplits + 2] = {0};
+        long long longest = 0, done = 0;
+        int p = 0;
+        for (int i = 0; i < k; ++i) {   // pairs up to the next k-th of the chunks, at least one, one left for each part behind
+            const long long from = done, goal = all * (i + 1) / k;
+            do done += chunks(p++);
+            while (p < t->P - (k - 1 - i) && done + chunks(p) / 2 <= goal);
+            if (i == k - 1)
+                for (; p < t->P; ++p) done += chunks(p);
+            c[i + 1] = (unsigned char)p;
+            longest = std::max(longest, done - from);
+        }
+        const long long cost = (tiles * k + sms - 1) / sms * (longest + kUnitChunks);
+        if (cost < best_cost) {
+            best_cost = cost;
+            best = k;
+            for (int i = 0; i <= k; ++i) cut[i] = c[i];
+        }
+    }
+    return best;
+}
+
+static int device_sms(int device)
+{
+    int sms = 148;
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
+    return sms;
+}
+
+// guard's workspace, then the sums of split tiles and their counters
+static size_t split_bytes(const r3_gp* gp, long long m)
+{
+    unsigned char cut[kMaxSplits + 2];
+    const long long tiles = score_tc_tiles(gp, m);
+    const int splits = plan_splits(ops_of(gp), tiles, device_sms(gp->device), cut);
+    return splits > 1 ? (size_t)tiles * (splits * 3 * TILE_M * sizeof(double) + sizeof(int)) + 256 : 0;
+}
+size_t score_tc_workspace_bytes(const r3_gp* gp, long long m) { return guard_workspace_bytes(gp, m) + split_bytes(gp, m); }
 
 r3_status_t score_tc(r3_gp* gp, const float* Xcand, long long m, float* mu, float* sigma, float* ei, void* ws,
                      size_t ws_bytes, cudaStream_t stream)
@@ -1279,7 +1358,7 @@ r3_status_t score_tc(r3_gp* gp, const float* Xcand, long long m, float* mu, floa
 
 long long score_tc_tiles(const r3_gp* gp, long long m) { return (m + TILE_M - 1) / TILE_M * gp->batch; }
 
-bool score_tc_can_split(const r3_gp* gp) { return ops_of(gp) != nullptr && env_int("R3_TC_PAIR", 0) == 0; }
+bool score_tc_can_split(const r3_gp* gp) { return ops_of(gp) != nullptr && !ops_of(gp)->pair; }
 
 r3_status_t score_tc_guard(r3_gp* gp, const float* Xcand, long long m, float* mu, float* sigma, float* ei, void* ws,
                            cudaStream_t stream)
@@ -1328,6 +1407,12 @@ r3_status_t score_tc_part(r3_gp* gp, const float* Xcand, long long m, float* mu,
     prm.NP = t->NP;
     prm.P = t->P;
     prm.ws = t->ws;
+    prm.parts = t->parts;
+    prm.S = t->S;
+    prm.nc = t->NP / KC;
+    prm.zb = t->zb;
+    prm.xs = t->xs;
+    prm.rsqrt_dp = (float)(1.0 / sqrt((double)round_up(gp->d, 16)));
     prm.status = gp->status_d;
     prm.tiles_per_gp = (m + TILE_M - 1) / TILE_M;
     prm.total_tiles = prm.tiles_per_gp * gp->batch;
@@ -1345,21 +1430,19 @@ r3_status_t score_tc_part(r3_gp* gp, const float* Xcand, long long m, float* mu,
     prm.zero_ints = guard_zero_ints(gp);
     prm.mode = nullptr;
     prm.want_mode = 0;
-    int sms = 148;
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, gp->device);
-    const unsigned grid = (unsigned)(launch_tiles < sms ? launch_tiles : sms);
-    // R3_TC_TRACE=1 prints, for the first CTA, the cycles each role spent per wait / issue category
-    prm.trace = nullptr;
-    if (getenv("R3_TC_TRACE")) {
-        if (dev_malloc(&prm.trace, sizeof(long long) * (grid * 32 + 32 * 128)) != cudaSuccess) prm.trace = nullptr;
-        if (prm.trace) cudaMemset(prm.trace, 0, sizeof(long long) * (grid * 32 + 32 * 128));
+    const int sms = device_sms(gp->device);
+    prm.splits = plan_splits(t, prm.tiles_per_gp * gp->batch, sms, prm.cut);
+    prm.partial = nullptr;
+    prm.arrived = nullptr;
+    if (prm.splits > 1) {
+        uintptr_t at = (uintptr_t)ws + guard_workspace_bytes(gp, m);
+        at = (at + 255) & ~(uintptr_t)255;
+        prm.partial = reinterpret_cast<double*>(at);
+        prm.arrived = reinterpret_cast<int*>(prm.partial + (size_t)score_tc_tiles(gp, m) * prm.splits * 3 * TILE_M);
     }
-    // The paired kernel (two CTAs of a cluster share a tile and the k* chunks) serves histories with at least
-    // two passes; R3_TC_PAIR=0/1 overrides the choice.
-    int pair_ws = 0;
-    const bool pair = tile_end < 0 && !t->f8 && env_int("R3_TC_PAIR", 0) != 0 && tc_pair_fits(t, &pair_ws);
+    prm.trace = nullptr;
     prof_begin(gp, stream);
-    if (pair) {
+    if (t->pair) {
         const r3_status_t st = launch_tc_pair(t, prm, sms, stream);
         if (st != R3_OK) return st;
     } else {
@@ -1373,8 +1456,9 @@ r3_status_t score_tc_part(r3_gp* gp, const float* Xcand, long long m, float* mu,
                 q.wt = t->wt16;
                 q.vinv2 = t->vinv2_16;
             }
+            if (q.splits > 1) R3_CUDA_TRY(cudaMemsetAsync(q.arrived, 0, sizeof(int) * (end - begin), stream));
             void (*kernel)(const TcParams) = kernel_of(t, f8);
-            R3_LAUNCH(kernel, (unsigned)std::min<long long>(end - begin, sms), 128 + 128 * t->G, t->smem_bytes, stream, q);
+            R3_LAUNCH(kernel, (unsigned)std::min<long long>((end - begin) * q.splits, sms), kThreads, t->smem_bytes, stream, q);
             return R3_OK;
         };
         const long long begin = prm.tile_begin, end = prm.total_tiles;
@@ -1402,25 +1486,6 @@ r3_status_t score_tc_part(r3_gp* gp, const float* Xcand, long long m, float* mu,
         if (st != R3_OK) return st;
     }
     prof_end(gp, stream);
-    if (prm.trace) {
-        std::vector<long long> h((size_t)grid * 32 + 32 * 128);
-        cudaMemcpy(h.data(), prm.trace, sizeof(long long) * h.size(), cudaMemcpyDeviceToHost);
-        for (int i = 0; i < 128; ++i) {
-            fprintf(stderr, "ev %d:", i);
-            for (int e = 0; e < 24; ++e) fprintf(stderr, " %lld", h[(size_t)grid * 32 + e * 128 + i] - h[(size_t)grid * 32 + 128 * 12]);
-            fprintf(stderr, "\n");
-        }
-        dev_free(prm.trace);
-        const char* names[4] = {"mmaV", "matern0", "matern1", "mmaD"};
-        fprintf(stderr, "trace shape NV=%d G=%d KD=%d kt=%d ws=%d DP=%d P=%d smem=%zu\n", t->NV, t->G, t->KD, (int)t->kt, t->ws,
-                t->DP, t->P, t->smem_bytes);
-        for (int cta = 0; cta < (pair ? 2 : 1); ++cta)
-            for (int r = 0; r < 4; ++r) {
-                fprintf(stderr, "trace cta%d %s:", cta, names[r]);
-                for (int i = 0; i < 8; ++i) fprintf(stderr, " %lld", h[((size_t)cta * 4 + r) * 8 + i]);
-                fprintf(stderr, "\n");
-            }
-    }
     if (!guard) return R3_OK;
     return guard_and_rescue(gp, Xcand, m, gb, mu, sigma, ei, false, stream);
 }

@@ -728,7 +728,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(128 + 128 * G2, 1) s
 // Whether the paired kernel serves this handle: at least two passes, and a shape that fits.
 bool tc_pair_fits(const TensorOperands* t, int* ws_out)
 {
-    if (t->NV != NV2 || t->KD != KD2 || t->P < 2) return false;
+    if (t->KD != KD2 || t->P < 2) return false;
     if (NV2 + 2 * KD2 + t->DP > 512) return false;
     const size_t budget = 227 * 1024 - 1024 - kPairBarBytes;
     int ws;

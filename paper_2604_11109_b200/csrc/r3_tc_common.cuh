@@ -13,26 +13,31 @@
 namespace r3 {
 
 struct TensorOperands {
-    int NV = 0, G = 0, KD = 0, DP = 0, NP = 0, P = 0, ws = 0;
-    bool kt = false;           // k* buffers in TMEM
+    int G = 0, KD = 0, DP = 0, NP = 0, P = 0, ws = 0;
+    int parts = 1;             // stages that the features of a distance product are split over
+    int S = 0;                 // strips of 128 rows of W; P = pairs of them
+    int zb = 0, xs = 0;        // buffers of scaled candidates, stages of scaled observations
+    bool pair = false;         // laid out for the paired kernel: chunks of 256 rows of W
     bool f8 = false;           // cross terms of the variance product as FP8 MMAs
-    int nbk = 0;               // number of k* buffers (== G: one per group; smaller: a shared ring)
     size_t smem_bytes = 0;
     size_t wt_gp_stride = 0;   // halves per GP in wt
     float* centre = nullptr;   // [B][DP]  column means of X (zero padded)
     float* scale = nullptr;    // [B][DP]  1/lengthscale (zero padded)
-    __half* xt = nullptr;      // [B][NP/KD][2][DP/8][KD][8]  scaled observations, FP16 hi/lo planes
+    __half* xt = nullptr;      // [B][NP/KD][parts][2][DP/parts/8][KD][8]  scaled observations, FP16 hi/lo planes
     float* xs32 = nullptr;     // [B][NP][DP]  scaled observations in FP32 (refinement of close pairs)
-    float* xnorm = nullptr;    // [B][NP]  |x~_k|^2
+    float* xnorm = nullptr;    // [B][NP/KD][2][KD]  |x~_k|^2, then weights (zero padded); pair: [B][NP] |x~_k|^2
+    float* alpha = nullptr;    // the weights inside xnorm; pair: [B][NP] behind it
     float* xnmax = nullptr;    // [B]      max_k |x~_k|^2
-    float* alpha = nullptr;    // [B][NP]  weights, zero padded
-    __half* wt = nullptr;      // [B][tile(p,c)][2][KC/8][NV][8]  chunks of 2^eW W, FP16 hi/lo planes; with f8 the
-                               // second plane is two 8-bit planes [2][KC/16][NV][16]: hi parts (E4M3), then lo parts (E5M2)
+    __half* wt = nullptr;      // [B][strip s][chunk c <= 4 s + 3][2][KC/8][R][8]  chunks of 2^eW W (R rows of the strip), FP16
+                               // hi/lo planes; with f8 the second plane is two 8-bit planes [2][KC/16][R][16]: hi parts
+                               // (E4M3), then lo parts (E5M2).  pair: [B][pass p][chunk c < 8 (p + 1)][2][KC/8][256][8]
     float* kscale = nullptr;   // [B]  2^eK, applied to k* before its split
     double* vinv2 = nullptr;   // [B]  2^(-2 (eK + eW)): scales sum V^2 back
     __half* wt16 = nullptr;    // with f8: the chunks as FP16 hi/lo planes too, for pools that need them (nullptr: no memory
     double* vinv2_16 = nullptr;   // for them when the operands were made)
 };
+
+constexpr int kMaxSplits = 32;
 
 struct TcParams {
     const float* xcand;
@@ -46,6 +51,12 @@ struct TcParams {
     const float *sf2, *best;
     const double* wnorm;
     int DP, NP, P, ws;
+    int parts, S, nc, zb, xs;   // nc: chunks of the whole history
+    float rsqrt_dp;             // 1 / sqrt of the feature count rounded up to 16 (error estimate)
+    int splits;                 // units that a tile's pairs of strips are shared out to: part i takes [cut[i], cut[i + 1])
+    unsigned char cut[kMaxSplits + 2];
+    double* partial;            // splits > 1: [tiles][splits][3][128] sums of a part, and how many parts of a tile have
+    int* arrived;               // been summed
     int* status;
     int* zero;          // the guard's counters, cleared by the first block (nothing reads them before the guard's kernel)
     int zero_ints;
@@ -103,15 +114,17 @@ __device__ __forceinline__ void mbar_arrive_expect_tx(uint32_t bar, uint32_t byt
 {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
 }
+// how long a waiting thread may sleep before it looks again (it wakes when the phase completes): polling takes issue slots
+constexpr uint32_t kSuspendNs = 2000;
 __device__ __forceinline__ uint32_t mbar_try_wait(uint32_t bar, uint32_t parity)
 {
     uint32_t ok;
     asm volatile(
         "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
         "selp.u32 %0, 1, 0, p;\n\t}"
         : "=r"(ok)
-        : "r"(bar), "r"(parity)
+        : "r"(bar), "r"(parity), "r"(kSuspendNs)
         : "memory");
     return ok;
 }
@@ -230,6 +243,14 @@ __device__ __forceinline__ void tc_wait_ld32(float* a, float* b)
     asm volatile(""
                  : "+f"(b[0]), "+f"(b[1]), "+f"(b[2]), "+f"(b[3]), "+f"(b[4]), "+f"(b[5]), "+f"(b[6]), "+f"(b[7]),
                    "+f"(b[8]), "+f"(b[9]), "+f"(b[10]), "+f"(b[11]), "+f"(b[12]), "+f"(b[13]), "+f"(b[14]), "+f"(b[15])
+                 :
+                 : "memory");
+}
+__device__ __forceinline__ void tc_wait_ld16(float* a)
+{
+    asm volatile("tcgen05.wait::ld.sync.aligned;"
+                 : "+f"(a[0]), "+f"(a[1]), "+f"(a[2]), "+f"(a[3]), "+f"(a[4]), "+f"(a[5]), "+f"(a[6]), "+f"(a[7]),
+                   "+f"(a[8]), "+f"(a[9]), "+f"(a[10]), "+f"(a[11]), "+f"(a[12]), "+f"(a[13]), "+f"(a[14]), "+f"(a[15])
                  :
                  : "memory");
 }

@@ -1,0 +1,50 @@
+"""The tensor engine at the edges of its tiles: strips of 128 rows of W in pairs, chunks of 32 and distance products of 64
+observations, features padded to 16 and split over stages of 64, one or two buffers of scaled candidates, and tiles whose pairs
+of strips are shared out to several thread blocks.  Every element against the FP64 oracle (tolerances of ``tests/parity.py``).
+"""
+import pytest
+
+from paper_2604_11109_b200 import binding as b
+from tests.test_gpu_parity import compare_everything, dev, fit_gpu, rand_problem
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("batch,n,d,m", [
+    (1, 31, 4, 130),          # one chunk of a distance product is padding
+    (1, 64, 16, 129),         # exactly one product; a tile of one candidate
+    (1, 65, 17, 257),         # one observation in the second product
+    (2, 128, 32, 300),        # exactly one strip; the FP32 copy of the candidates at its widest
+    (1, 129, 33, 200),        # a second strip of 64 rows, without that copy
+    (3, 192, 9, 140),         # a strip and a half, several GPs
+    (1, 256, 64, 200),        # exactly one pair; one stage of features at its widest
+    (2, 257, 65, 150),        # a pair and a strip of 64 rows; features split over two stages; pairs shared out
+    (1, 385, 97, 260),        # two pairs; the second stage mostly padding
+    (1, 641, 128, 300),       # an odd number of strips; one buffer of candidates
+    (1, 1025, 21, 100),       # five pairs shared out
+    (1, 1793, 40, 131),       # FP8 cross terms, eight pairs shared out
+    (1, 40, 5, 148 * 128 * 2 + 77),   # more tiles than thread blocks, ragged tail
+    (1, 300, 12, 148 * 128 + 1),      # the same with two pairs
+])
+def test_edges_of_strips_chunks_stages_and_parts(batch, n, d, m):
+    g = rand_problem(7000 + n + d, batch, n, d, m)
+    gp = fit_gpu(g, b.ENGINE_TENSOR)
+    assert b.r3_gp_engine(gp) == b.ENGINE_TENSOR
+    compare_everything(g, gp, min(8, m), f"edges n{n} d{d} m{m}")
+    gp.close()
+
+
+def test_parts_of_a_tile_add_up_to_the_whole():
+    """A pool of one tile, whose pairs of strips go to several thread blocks, and the same rows among enough others that every
+    tile stays with one block: FP64 sums of the same FP32 parts in another order, so at most a last bit apart."""
+    g = rand_problem(91, 1, 900, 24, 148 * 128 * 16)
+    gp = fit_gpu(g, b.ENGINE_TENSOR)
+    whole = [t[0, :100].clone() for t in b.r3_gp_score(gp, dev(g["Xcand"]))]
+    rescued_whole = b.r3_gp_last_rescued(gp)
+    part = [t[0] for t in b.r3_gp_score(gp, dev(g["Xcand"][:, :100]))]
+    if rescued_whole == 0 and b.r3_gp_last_rescued(gp) == 0:   # what the FP64 pass has rewritten does not show the engine's sums
+        for a, c in zip(part[:2], whole[:2]):
+            ulp = torch.finfo(torch.float32).eps * c.abs().clamp_min(1e-30)
+            assert ((a - c).abs() <= ulp).all()
+    gp.close()
