@@ -47,6 +47,9 @@ constexpr int kSortThreads = 1024;
 constexpr int kScoreThreads = 256;
 constexpr int kStage = 512;   // components per shared-memory stage
 constexpr size_t kResidentBytes = 72 * 1024;   // largest model a scoring block keeps whole in shared memory
+// Components of such a model with every set padded to a multiple of four: set i begins at its unpadded place plus 3 i, rounded
+// up to a multiple of four, which leaves room for the padding of the sets before it.
+__host__ __device__ inline int resident_padded(int total, int d) { return (total + 3 * 2 * d + 3) & ~3; }
 
 // Unsigned integer with the same order as the float (-0 and +0 equal).
 __device__ __forceinline__ unsigned ordered_bits(float v)
@@ -364,49 +367,134 @@ __device__ __forceinline__ float lg2_fast(float x)
     return r;
 }
 
-// sum over `count` components of exp2(b - a (x - mean)^2) for R candidates at once.  The components are
-// staged through shared memory by the whole block (all of its threads must call this together): one
-// broadcast LDS.128 per component instead of a global load per thread was worth 14 % on the full pool.
+// Components in shared memory, one array per coefficient: -mean, -a and b of four components in a row are three 16-byte reads
+// and give two pairs of each, ready for the packed FP32 instructions.  Sets are padded to a multiple of four with components
+// that contribute nothing.
+struct Components {
+    float *nmean, *na, *b;
+};
+constexpr float kNullB = -1e4f;   // exp2 of it is 0 either way
+
+__device__ __forceinline__ uint64_t pack2(float lo, float hi)
+{
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ void unpack2(uint64_t v, float& lo, float& hi) { asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v)); }
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b)
+{
+    uint64_t r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b)
+{
+    uint64_t r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c)
+{
+    uint64_t r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ uint64_t both(float v) { return pack2(v, v); }
+
+// exp2 of a pair on the FP32 pipe: x = n + f with n the nearest whole number, 2^f by a polynomial ((2^f - 1) / f interpolated at
+// six Chebyshev nodes of [-1/2, 1/2]; 7.4e-8 relative at most, the special-function unit 1.7e-7), n added to the exponent.
+// Below -127 the result is 0 (n = -127, f = 0), between -127 and -126 less than 2^-126.  x must be below 127.
+__device__ __forceinline__ uint64_t exp2_poly2(uint64_t x2)
+{
+    float x0, x1;
+    unpack2(x2, x0, x1);
+    x2 = pack2(fmaxf(x0, -127.f), fmaxf(x1, -127.f));
+    const uint64_t z = add2(x2, both(12582912.f));           // 1.5 * 2^23: the low bits of z are n
+    const uint64_t n = add2(z, both(-12582912.f));
+    const uint64_t f = fma2(n, both(-1.f), x2);
+    uint64_t p = both(0x1.44138ap-13f);
+    p = fma2(p, f, both(0x1.5f0890p-10f));
+    p = fma2(p, f, both(0x1.3b2a54p-7f));
+    p = fma2(p, f, both(0x1.c6af6cp-5f));
+    p = fma2(p, f, both(0x1.ebfbe0p-3f));
+    p = fma2(p, f, both(0x1.62e430p-1f));
+    p = fma2(p, f, both(1.f));
+    float z0, z1, p0, p1;
+    unpack2(z, z0, z1);
+    unpack2(p, p0, p1);
+    return pack2(__int_as_float(__float_as_int(p0) + (__float_as_int(z0) << 23)),
+                 __int_as_float(__float_as_int(p1) + (__float_as_int(z1) << 23)));
+}
+__device__ __forceinline__ uint64_t exp2_fast2(uint64_t x2)
+{
+    float x0, x1;
+    unpack2(x2, x0, x1);
+    return pack2(ex2_fast(x0), ex2_fast(x1));
+}
+
+// sum over components [lo, hi) (multiples of four) of exp2(b - a (x - mean)^2) for R candidates at once, four partial sums per
+// candidate.  Bound by the special-function unit, which gives a warp an exponential in eight cycles, and by instruction issue;
+// hence pairs, and with two candidates per thread one exponential in eight on the FP32 pipe.  1,048,576 candidates with 2432
+// exponentials each (whole call) and 500,000 with 20,000: scalar instructions 1.02 and 2.79 ms, pairs 0.95 and 2.59 ms, one in
+// four on the FP32 pipe 0.96 and 2.58 ms, one in eight 0.925 and 2.39 ms.
+template <int R>
+__device__ __forceinline__ void mixture_sums(const Components& m, int lo, int hi, const float (&x)[R], uint64_t (&part)[R][2])
+{
+    uint64_t x2[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) x2[r] = both(x[r]);
+    auto group = [&](int c, bool odd) {
+        const ulonglong2 nm = *reinterpret_cast<const ulonglong2*>(m.nmean + c);
+        const ulonglong2 na = *reinterpret_cast<const ulonglong2*>(m.na + c);
+        const ulonglong2 b = *reinterpret_cast<const ulonglong2*>(m.b + c);
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const uint64_t t0 = add2(x2[r], nm.x), t1 = add2(x2[r], nm.y);
+            const uint64_t e0 = fma2(t0, mul2(t0, na.x), b.x), e1 = fma2(t1, mul2(t1, na.y), b.y);
+            part[r][0] = add2(part[r][0], exp2_fast2(e0));
+            part[r][1] = add2(part[r][1], (r % 2 == 1 && odd) ? exp2_poly2(e1) : exp2_fast2(e1));
+        }
+    };
+    int c = lo;
+#pragma unroll 2
+    for (; c + 8 <= hi; c += 8) {
+        group(c, false);
+        group(c + 4, true);
+    }
+    if (c < hi) group(c, false);
+}
+template <int R>
+__device__ __forceinline__ void finish_sums(const uint64_t (&part)[R][2], float (&sum)[R])
+{
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        float a, b;
+        unpack2(add2(part[r][0], part[r][1]), a, b);
+        sum[r] = a + b;
+    }
+}
+
+// The same over `count` components in global memory, which the whole block stages through shared memory (all of its threads
+// must call this together): one broadcast read instead of a global load per thread was worth 14 % on the full pool.
 template <int R>
 __device__ __forceinline__ void mixture_sums_staged(const float4* __restrict__ comp, int count, const float (&x)[R],
-                                                    float (&sum)[R], float4* stage)
+                                                    float (&sum)[R], const Components& stage)
 {
-    // four partial sums per candidate: independent add chains, and half the rounding of one long sum
-    float part[4][R];
-#pragma unroll
-    for (int u = 0; u < 4; ++u)
-#pragma unroll
-        for (int r = 0; r < R; ++r) part[u][r] = 0.f;
+    uint64_t part[R][2] = {};
     for (int c0 = 0; c0 < count; c0 += kStage) {
-        const int nc = min(kStage, count - c0);
+        const int nc = min(kStage, count - c0), nc4 = (nc + 3) & ~3;
         __syncthreads();
-        for (int i = threadIdx.x; i < nc; i += kScoreThreads) stage[i] = __ldg(comp + c0 + i);
+        for (int i = threadIdx.x; i < nc4; i += kScoreThreads) {
+            const float4 q = i < nc ? __ldg(comp + c0 + i) : make_float4(0.f, 1.f, kNullB, 0.f);
+            stage.nmean[i] = -q.x;
+            stage.na[i] = -q.y;
+            stage.b[i] = q.z;
+        }
         __syncthreads();
-        int c = 0;
-        for (; c + 4 <= nc; c += 4) {
-            float4 q[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) q[u] = stage[c + u];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-#pragma unroll
-                for (int r = 0; r < R; ++r) {
-                    const float t = x[r] - q[u].x;
-                    part[u][r] += ex2_fast(fmaf(-t, t * q[u].y, q[u].z));
-                }
-            }
-        }
-        for (; c < nc; ++c) {
-            const float4 q = stage[c];
-#pragma unroll
-            for (int r = 0; r < R; ++r) {
-                const float t = x[r] - q.x;
-                part[c & 3][r] += ex2_fast(fmaf(-t, t * q.y, q.z));
-            }
-        }
+        mixture_sums<R>(stage, 0, nc4, x, part);
     }
-#pragma unroll
-    for (int r = 0; r < R; ++r) sum[r] = (part[0][r] + part[1][r]) + (part[2][r] + part[3][r]);
+    finish_sums<R>(part, sum);
 }
 
 // (T4) score of every candidate.  A block covers R * blockDim.x consecutive candidates; thread t holds
@@ -421,7 +509,8 @@ __global__ void __launch_bounds__(kScoreThreads) tpe_score_kernel(const float* _
 {
     const long long tiles = (m + (long long)R * kScoreThreads - 1) / ((long long)R * kScoreThreads);
     bool bad = false;
-    __shared__ float4 stage[kStage];
+    __shared__ __align__(16) float stage_s[3][kStage];
+    const Components stage{stage_s[0], stage_s[1], stage_s[2]};
     for (long long tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
         const long long base = tile * (long long)R * kScoreThreads + threadIdx.x;
         const float* row[R];
@@ -499,42 +588,6 @@ __global__ void __launch_bounds__(256) tpe_pack_kernel(const float4* __restrict_
     for (int i = threadIdx.x; i < cnt; i += blockDim.x) packed[lo + i] = src[i];
 }
 
-// sum over components [lo, hi) of a model held in shared memory, for R candidates at once
-template <int R>
-__device__ __forceinline__ void mixture_sums_resident(const float4* __restrict__ model, int lo, int hi,
-                                                      const float (&x)[R], float (&sum)[R])
-{
-    float part[4][R];
-#pragma unroll
-    for (int u = 0; u < 4; ++u)
-#pragma unroll
-        for (int r = 0; r < R; ++r) part[u][r] = 0.f;
-    int c = lo;
-    for (; c + 4 <= hi; c += 4) {
-        float4 q[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) q[u] = model[c + u];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-#pragma unroll
-            for (int r = 0; r < R; ++r) {
-                const float t = x[r] - q[u].x;
-                part[u][r] += ex2_fast(fmaf(-t, t * q[u].y, q[u].z));
-            }
-        }
-    }
-    for (; c < hi; ++c) {
-        const float4 q = model[c];
-#pragma unroll
-        for (int r = 0; r < R; ++r) {
-            const float t = x[r] - q.x;
-            part[(c - lo) & 3][r] += ex2_fast(fmaf(-t, t * q.y, q.z));
-        }
-    }
-#pragma unroll
-    for (int r = 0; r < R; ++r) sum[r] = (part[0][r] + part[1][r]) + (part[2][r] + part[3][r]);
-}
-
 // (T4) for a model that fits shared memory (discrete features leave a few components per admissible value):
 // every block loads the packed model once and then walks its tiles without a block-wide barrier.  (Reading
 // four or eight features of a row per load, with the feature loop unrolled to match, measured 10-30 % slower:
@@ -545,12 +598,34 @@ __global__ void __launch_bounds__(kScoreThreads) tpe_score_resident_kernel(
     const float4* __restrict__ packed, int total, const float* __restrict__ table, float* __restrict__ score,
     int* __restrict__ status)
 {
-    extern __shared__ float4 model[];   // [total] components, then [2d + 1] offsets, then [d] level codes
-    int* offs_s = reinterpret_cast<int*>(model + total);
+    extern __shared__ __align__(16) float model[];   // three arrays of padded components, then [2d + 1] offsets, then [d] level codes
+    const int padded = resident_padded(total, d);
+    const Components comps{model, model + padded, model + 2 * padded};
+    int* offs_s = reinterpret_cast<int*>(model + 3 * padded);
     int* code_s = offs_s + 2 * d + 1;
-    for (int i = threadIdx.x; i < total; i += kScoreThreads) model[i] = __ldg(packed + i);
     for (int i = threadIdx.x; i <= 2 * d; i += kScoreThreads) offs_s[i] = __ldg(offs + i);
     for (int i = threadIdx.x; i < d; i += kScoreThreads) code_s[i] = __ldg(levels + i);
+    for (int i = threadIdx.x; i < padded; i += kScoreThreads) {
+        comps.nmean[i] = 0.f;
+        comps.na[i] = -1.f;
+        comps.b[i] = kNullB;
+    }
+    __syncthreads();
+    for (int c = threadIdx.x; c < total; c += kScoreThreads) {
+        const float4 q = __ldg(packed + c);
+        int lo = 0, hi = 2 * d - 1;   // the last set that begins at or before c
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (offs_s[mid] <= c) lo = mid;
+            else hi = mid - 1;
+        }
+        const int at = ((offs_s[lo] + 3 * lo + 3) & ~3) + c - offs_s[lo];
+        comps.nmean[at] = -q.x;
+        comps.na[at] = -q.y;
+        comps.b[at] = q.z;
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i <= 2 * d; i += kScoreThreads) offs_s[i] = (offs_s[i] + 3 * i + 3) & ~3;   // set i, padded to four
     __syncthreads();
     const long long tiles = (m + (long long)R * kScoreThreads - 1) / ((long long)R * kScoreThreads);
     bool bad = false;
@@ -584,8 +659,13 @@ __global__ void __launch_bounds__(kScoreThreads) tpe_score_resident_kernel(
                 }
             } else {
                 float sl[R], sg[R];
-                mixture_sums_resident<R>(model, offs_s[2 * j], offs_s[2 * j + 1], x, sl);
-                mixture_sums_resident<R>(model, offs_s[2 * j + 1], offs_s[2 * j + 2], x, sg);
+                uint64_t part[R][2] = {};
+                mixture_sums<R>(comps, offs_s[2 * j], offs_s[2 * j + 1], x, part);
+                finish_sums<R>(part, sl);
+#pragma unroll
+                for (int r = 0; r < R; ++r) part[r][0] = part[r][1] = 0;
+                mixture_sums<R>(comps, offs_s[2 * j + 1], offs_s[2 * j + 2], x, part);
+                finish_sums<R>(part, sg);
 #pragma unroll
                 for (int r = 0; r < R; ++r) acc[r] += 0.69314718f * (lg2_fast(sl[r]) - lg2_fast(sg[r]));
             }
@@ -830,7 +910,7 @@ r3_status_t r3_tpe_score(r3_tpe_t* tpe, const float* Xcand, long long m, float* 
         // the whole model in shared memory.  Sixteen blocks per SM's worth of grid (several waves of short
         // blocks) measured up to 8 % faster than one resident wave walking the tiles: the model is a small
         // read from L2 and the finer grain balances the SMs better.
-        const size_t smem = resident_bytes(tpe->total, tpe->d);
+        const size_t smem = sizeof(float) * 3 * resident_padded(tpe->total, tpe->d) + sizeof(int) * (3 * (size_t)tpe->d + 1);
         const long long tiles2 = (m + 2ll * kScoreThreads - 1) / (2ll * kScoreThreads);
         const long long tiles1 = (m + kScoreThreads - 1) / kScoreThreads;
 #define R3_TPE_RESIDENT(R, TILES)                                                                              \

@@ -348,3 +348,28 @@ def test_fit_at_the_edges_of_the_sort_and_of_runs(n):
             total = (np.exp2(got[:, 2].astype(np.float64)) * sg * Z * np.sqrt(2 * np.pi)).sum()
             assert abs(total - 1.0) < 1e-5     # b is FP32: 2^-24 |b| ln 2 per component
     t.close()
+
+
+@pytest.mark.parametrize("n,d,m", [
+    (3, 3, 700), (17, 5, 900),                # model in shared memory, one candidate per thread
+    (260, 2, 148 * 8 * 512 + 77),             # the same, two
+    (1500, 4, 900),                           # staged model, one candidate per thread
+    (1201, 6, 148 * 4 * 512 + 5),             # the same, two
+])
+def test_component_counts_that_fill_no_group_of_four(n, d, m):
+    """Continuous values keep a component each: sets of every remainder modulo four and eight, in both kernels and with one
+    and two candidates per thread; some candidates outside [0, 1], where most exponentials underflow."""
+    rng = np.random.default_rng(n)
+    X = rng.uniform(0, 1, (n, d)).astype(np.float32)
+    y = rng.normal(0, 1, n).astype(np.float32)
+    Xc = rng.uniform(0, 1, (m, d)).astype(np.float32)
+    Xc[::97] = rng.uniform(-1, 2, (len(Xc[::97]), d)).astype(np.float32)
+    levels = np.zeros(d, np.int32)
+    tpe = b.r3_tpe_fit(dev(X), dev(y), levels, 0.25, 1.0)
+    got = b.r3_tpe_score(tpe, dev(Xc)).cpu().numpy()
+    b.r3_tpe_check(tpe)
+    tpe.close()
+    rows = np.unique(np.concatenate([np.arange(0, m, 97)[:200], rng.integers(0, m, 500), [m - 1]]))
+    want = T.tpe_score(T.tpe_fit(X, y, levels, 0.25, 1.0), Xc[rows])
+    err = np.abs(got[rows] - want) / (atol(n, levels) + RTOL * np.abs(want))
+    assert err.max() <= 1.0, float(err.max())
