@@ -6,7 +6,8 @@
 // two numbers close to sf2 (a candidate on top of an observation), nor where mu = k*.alpha cancels
 // heavily (an ill-conditioned history with large weights).  Each engine therefore writes, next to
 // its results, an estimate of its own rounding error in mu and in q.  Once the whole pool is scored, guard_kernel
-//   finds    the pool's largest EI (the EI tolerance is relative to it), unless the engine already has,
+//   finds    the pool's largest EI (the EI tolerance is relative to it), unless the engine already has or has left the largest of
+//            each of its tiles, of which every block takes the largest by itself (a pass over the pool and a grid barrier less),
 //   flags    the candidates whose estimated error exceeds half of the accuracy contract
 //            (1e-4 relative on mu and sigma with absolute floors, 1e-5 max(EI) on EI) in a list per GP,
 //   rescues  them: recomputes them from the raw inputs entirely in FP64 -- direct-difference distances with
@@ -68,7 +69,9 @@ struct GuardArgs {
     unsigned* barrier;            // grid barrier
     int* status;                  // the handle's status words
     WaitRule wait;
-    bool have_max;
+    bool have_max;                // maxbits holds the largest EI already, or tile_max does:
+    const float* tile_max;        // [batch][tiles_per_gp] the engine's largest EI of each tile, or nullptr
+    int tiles_per_gp;
     double *ks, *qpart, *mupart;  // slab: [slab][npad], [slab][npad / 16], [slab][ceil(npad / 64)]
     int slab;                     // candidates per slab, a multiple of 64
     int k, K2;                    // top-k request (k = 0: none); K2 = min(k, slice): keys a slice yields
@@ -368,11 +371,24 @@ __device__ __forceinline__ bool guard_pool(const GuardArgs& a, unsigned char* sm
     }
 
     // ---- flag
+    float pool_max = 0.f;
+    int max_of = -1;   // the GP that it belongs to
     for (int s = blockIdx.x; s < chunks; s += gridDim.x) {
         const int g = s / a.chunks_per_gp;
+        if (a.tile_max && g != max_of) {   // every block takes the largest of the tiles' largest by itself
+            float v = 0.f;
+#pragma unroll 8
+            for (int i = t; i < a.tiles_per_gp; i += kThreads) v = fmaxf(v, __ldg(a.tile_max + (size_t)g * a.tiles_per_gp + i));
+            const unsigned top = __reduce_max_sync(0xffffffffu, __float_as_uint(v));
+            __syncthreads();
+            if (lane == 0) warp_sum[warp] = (int)top;
+            __syncthreads();
+            for (int w = 0; w < 8; ++w) pool_max = w ? fmaxf(pool_max, __int_as_float(warp_sum[w])) : __int_as_float(warp_sum[0]);
+            max_of = g;
+        }
         const long long c0 = (long long)(s % a.chunks_per_gp) * a.chunk, c1 = min(m, c0 + a.chunk);
         const float sf2 = a.sf2v[g], best = a.bestv[g];
-        const float tol_ei = 1e-5f * __uint_as_float(__ldcg(a.maxbits + g));
+        const float tol_ei = 1e-5f * (a.tile_max ? pool_max : __uint_as_float(__ldcg(a.maxbits + g)));
         const float mu_floor = 1e-6f * a.yabsv[g], sd_floor = 1e-6f * sqrtf(sf2);
         if (own_rescue) {
             __syncthreads();
@@ -620,7 +636,7 @@ r3_status_t guard_pilot(r3_gp* gp, long long m, long long rows, const GuardBuffe
 }
 
 r3_status_t guard_and_rescue(r3_gp* gp, const float* Xcand, long long m, const GuardBuffers& b, float* mu,
-                             float* sigma, float* ei, bool have_max, cudaStream_t stream)
+                             float* sigma, float* ei, const float* tile_max, long long tiles_per_gp, bool have_max, cudaStream_t stream)
 {
     const int B = gp->batch;
     const TopkRequest req = gp->topk_req;
@@ -645,7 +661,9 @@ r3_status_t guard_and_rescue(r3_gp* gp, const float* Xcand, long long m, const G
     a.barrier = b.barrier;
     a.status = gp->status_d;
     a.wait = wait_rule(gp, STALL_GUARD);
-    a.have_max = have_max;
+    a.have_max = have_max || tile_max;
+    a.tile_max = tile_max;
+    a.tiles_per_gp = (int)tiles_per_gp;
     a.ks = b.ks; a.qpart = b.qpart; a.mupart = b.mupart;
     a.slab = slab_candidates(gp, m);
     a.k = req.k;

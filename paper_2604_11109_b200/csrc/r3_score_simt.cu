@@ -257,7 +257,7 @@ r3_status_t score_simt(r3_gp* gp, const float* Xcand, long long m, float* mu, fl
             prof_end(gp, stream);
         }
     }
-    return guard_and_rescue(gp, Xcand, m, w.guard, mu, sigma, ei, true, stream);
+    return guard_and_rescue(gp, Xcand, m, w.guard, mu, sigma, ei, nullptr, 0, true, stream);
 }
 
 }  // namespace r3

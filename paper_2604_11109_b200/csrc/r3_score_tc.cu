@@ -289,6 +289,7 @@ __global__ void __launch_bounds__(kThreads, 1) score_tc_kernel(const __grid_cons
     volatile int* abort_flag = reinterpret_cast<volatile int*>(sm + map.bar + kFlagOffset);
     volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(sm + map.bar + kFlagOffset + 8);
     volatile int* last_flag = reinterpret_cast<volatile int*>(sm + map.bar + kFlagOffset + 12);
+    volatile unsigned* top_s = reinterpret_cast<volatile unsigned*>(sm + map.bar + kFlagOffset + 32);   // largest EI of a warp's rows, [group][4]
     auto zn_buf = [&](int b) { return reinterpret_cast<float*>(sm + map.zn + b * kZnBuf); };
     auto bar = [&](uint32_t slot) { return bars + slot * 8u; };
 
@@ -760,6 +761,7 @@ __global__ void __launch_bounds__(kThreads, 1) score_tc_kernel(const __grid_cons
             }
             const int g = (int)(tile / tiles_per_gp);
             const long long cand = (long long)(tile - g * tiles_per_gp) * TILE_M + row;
+            float ei_mine = 0.f;
             if (finish && cand < prm.m) {
                 const bool far_cand = zn_own < 0.f;
                 q_acc *= prm.vinv2[g];   // undo the power-of-two scaling of k* and W
@@ -769,9 +771,19 @@ __global__ void __launch_bounds__(kThreads, 1) score_tc_kernel(const __grid_cons
                 __stcs(prm.mu + f, res.mu);
                 __stcs(prm.sigma + f, res.sigma);
                 __stcs(prm.ei + f, res.ei);
+                if (res.ei == res.ei) ei_mine = res.ei;
                 const float eps = far_cand ? 1.f : (float)kEpsTc0 + (float)kEpsTc1 * prm.rsqrt_dp * (fabsf(zn_own) + prm.xnmax[g]);
                 prm.err_mu[f] = mu_error_estimate(eps, a2_acc);
                 prm.err_q[f] = q_error_estimate(F8 && !far_cand ? eps + (float)kEpsF8 : eps, (float)prm.wnorm[g], (float)q_acc, s2_acc);
+            }
+            if (finish) {   // EI >= 0: the order of the bits is the order of the values
+                const unsigned top = __reduce_max_sync(0xffffffffu, __float_as_uint(ei_mine));
+                if (lane == 0) top_s[io * 4 + (warp & 3)] = top;
+                asm volatile("bar.sync %0, 128;" ::"r"(1 + io) : "memory");
+                if (row == 0)
+                    prm.tile_max[R3_IDX(tile, (long long)tiles_per_gp * prm.batch, prm.status)] =
+                        __uint_as_float(max(max(top_s[io * 4], top_s[io * 4 + 1]), max(top_s[io * 4 + 2], top_s[io * 4 + 3])));
+                asm volatile("bar.sync %0, 128;" ::"r"(1 + io) : "memory");   // read before the next tile's are written
             }
             if (groups == 1 && zb == 2) b ^= 1;
         }
@@ -1340,7 +1352,8 @@ static int device_sms(int device)
     return sms;
 }
 
-// guard's workspace, then the sums of split tiles and their counters
+// guard's workspace, then the tiles' largest EI, the sums of split tiles and their counters
+static size_t max_bytes(const r3_gp* gp, long long m) { return ((size_t)score_tc_tiles(gp, m) * sizeof(float) + 511) & ~(size_t)255; }
 static size_t split_bytes(const r3_gp* gp, long long m)
 {
     unsigned char cut[kMaxSplits + 2];
@@ -1348,7 +1361,13 @@ static size_t split_bytes(const r3_gp* gp, long long m)
     const int splits = plan_splits(ops_of(gp), tiles, device_sms(gp->device), cut);
     return splits > 1 ? (size_t)tiles * (splits * 3 * TILE_M * sizeof(double) + sizeof(int)) + 256 : 0;
 }
-size_t score_tc_workspace_bytes(const r3_gp* gp, long long m) { return guard_workspace_bytes(gp, m) + split_bytes(gp, m); }
+size_t score_tc_workspace_bytes(const r3_gp* gp, long long m) { return guard_workspace_bytes(gp, m) + max_bytes(gp, m) + split_bytes(gp, m); }
+
+static float* tile_max_of(const r3_gp* gp, long long m, void* ws)   // nullptr: the paired kernel leaves none
+{
+    if (ops_of(gp)->pair) return nullptr;
+    return reinterpret_cast<float*>(((uintptr_t)ws + guard_workspace_bytes(gp, m) + 255) & ~(uintptr_t)255);
+}
 
 r3_status_t score_tc(r3_gp* gp, const float* Xcand, long long m, float* mu, float* sigma, float* ei, void* ws,
                      size_t ws_bytes, cudaStream_t stream)
@@ -1363,7 +1382,7 @@ bool score_tc_can_split(const r3_gp* gp) { return ops_of(gp) != nullptr && !ops_
 r3_status_t score_tc_guard(r3_gp* gp, const float* Xcand, long long m, float* mu, float* sigma, float* ei, void* ws,
                            cudaStream_t stream)
 {
-    return guard_and_rescue(gp, Xcand, m, guard_carve(gp, m, ws), mu, sigma, ei, false, stream);
+    return guard_and_rescue(gp, Xcand, m, guard_carve(gp, m, ws), mu, sigma, ei, tile_max_of(gp, m, ws), (m + TILE_M - 1) / TILE_M, false, stream);
 }
 
 r3_status_t score_tc_part(r3_gp* gp, const float* Xcand, long long m, float* mu, float* sigma, float* ei, void* ws,
@@ -1432,10 +1451,11 @@ r3_status_t score_tc_part(r3_gp* gp, const float* Xcand, long long m, float* mu,
     prm.want_mode = 0;
     const int sms = device_sms(gp->device);
     prm.splits = plan_splits(t, prm.tiles_per_gp * gp->batch, sms, prm.cut);
+    prm.tile_max = tile_max_of(gp, m, ws);
     prm.partial = nullptr;
     prm.arrived = nullptr;
     if (prm.splits > 1) {
-        uintptr_t at = (uintptr_t)ws + guard_workspace_bytes(gp, m);
+        uintptr_t at = (uintptr_t)ws + guard_workspace_bytes(gp, m) + max_bytes(gp, m);
         at = (at + 255) & ~(uintptr_t)255;
         prm.partial = reinterpret_cast<double*>(at);
         prm.arrived = reinterpret_cast<int*>(prm.partial + (size_t)score_tc_tiles(gp, m) * prm.splits * 3 * TILE_M);
@@ -1487,7 +1507,7 @@ r3_status_t score_tc_part(r3_gp* gp, const float* Xcand, long long m, float* mu,
     }
     prof_end(gp, stream);
     if (!guard) return R3_OK;
-    return guard_and_rescue(gp, Xcand, m, gb, mu, sigma, ei, false, stream);
+    return guard_and_rescue(gp, Xcand, m, gb, mu, sigma, ei, prm.tile_max, prm.tiles_per_gp, false, stream);
 }
 
 }  // namespace r3

@@ -57,6 +57,7 @@ struct TcParams {
     unsigned char cut[kMaxSplits + 2];
     double* partial;            // splits > 1: [tiles][splits][3][128] sums of a part, and how many parts of a tile have
     int* arrived;               // been summed
+    float* tile_max;            // [tiles of the pool] largest EI of each, for the guard
     int* status;
     int* zero;          // the guard's counters, cleared by the first block (nothing reads them before the guard's kernel)
     int zero_ints;
