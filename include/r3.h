@@ -217,10 +217,10 @@ r3_engine_t r3_gp_engine(const r3_gp_t* gp);
 
 /*
  * Diagnostics: the shape the tensor-core engine runs this handle in (all zero when it does not serve it).
- * info[0] NV   rows of the inverse factor per pass (columns of the accumulator in tensor memory)
- * info[1] P    passes per tile of 128 candidates (the chunks of k* are generated (P + 1) / 2 times on average)
- * info[2] DP   feature count padded to a multiple of 16 (depth of the distance product)
- * info[3] NP   history length padded to a multiple of NV
+ * info[0] NV   rows of the inverse factor that share the generated chunks of k* (a pair of accumulators in tensor memory)
+ * info[1] P    passes over k* per tile of 128 candidates (its chunks are generated (P + 1) / 2 times on average)
+ * info[2] DP   feature count padded to a multiple of 16, of 32 beyond 64 (depth of the distance product)
+ * info[3] NP   history length padded to a multiple of 64 (of 256 with the paired kernel)
  * info[4] G    Matern warp groups;  info[5] W stages in shared memory;  info[6] 1: k* operand in tensor memory
  * info[7] 1: the cross terms of the variance product are FP8 MMAs (histories of eight passes and more)
  */
