@@ -1354,12 +1354,29 @@ static int device_sms(int device)
 
 // guard's workspace, then the tiles' largest EI, the sums of split tiles and their counters
 static size_t max_bytes(const r3_gp* gp, long long m) { return ((size_t)score_tc_tiles(gp, m) * sizeof(float) + 511) & ~(size_t)255; }
-static size_t split_bytes(const r3_gp* gp, long long m)
+// With FP8 cross terms, the tiles that are scored first and decide for the pool: what is left over when the pool is cut into
+// whole waves, so that the rest is whole waves, but at least a quarter of one.  Their pairs of strips are shared out over all
+// SMs.  (A whole wave of tiles: 0.8 ms of the 10.5 ms of a round at n = 4096 whose 512 tiles are then scored with FP16 cross
+// terms, 0.36 ms now; 1,048,576 candidates that keep them 55 waves and a third instead of 56.)
+static long long pilot_tiles(const r3_gp* gp, long long m, int sms)
+{
+    const long long tiles = score_tc_tiles(gp, m);
+    return std::min(tiles, std::max<long long>(sms / 4, tiles % sms));
+}
+// tiles times parts whose sums a call has to hold
+static size_t split_slots(const r3_gp* gp, long long m)
 {
     unsigned char cut[kMaxSplits + 2];
-    const long long tiles = score_tc_tiles(gp, m);
-    const int splits = plan_splits(ops_of(gp), tiles, device_sms(gp->device), cut);
-    return splits > 1 ? (size_t)tiles * (splits * 3 * TILE_M * sizeof(double) + sizeof(int)) + 256 : 0;
+    const TensorOperands* t = ops_of(gp);
+    const int sms = device_sms(gp->device);
+    const long long tiles = score_tc_tiles(gp, m), first = t->f8 ? pilot_tiles(gp, m, sms) : 0;
+    const int splits = plan_splits(t, tiles, sms, cut), first_splits = t->f8 ? plan_splits(t, first, sms, cut) : 1;
+    return std::max<size_t>(splits > 1 ? tiles * splits : 0, first_splits > 1 ? first * first_splits : 0);
+}
+static size_t split_bytes(const r3_gp* gp, long long m)
+{
+    const size_t slots = split_slots(gp, m);
+    return slots ? slots * 3 * TILE_M * sizeof(double) + score_tc_tiles(gp, m) * sizeof(int) + 256 : 0;
 }
 size_t score_tc_workspace_bytes(const r3_gp* gp, long long m) { return guard_workspace_bytes(gp, m) + max_bytes(gp, m) + split_bytes(gp, m); }
 
@@ -1454,11 +1471,11 @@ r3_status_t score_tc_part(r3_gp* gp, const float* Xcand, long long m, float* mu,
     prm.tile_max = tile_max_of(gp, m, ws);
     prm.partial = nullptr;
     prm.arrived = nullptr;
-    if (prm.splits > 1) {
+    if (const size_t slots = t->pair ? 0 : split_slots(gp, m)) {
         uintptr_t at = (uintptr_t)ws + guard_workspace_bytes(gp, m) + max_bytes(gp, m);
         at = (at + 255) & ~(uintptr_t)255;
         prm.partial = reinterpret_cast<double*>(at);
-        prm.arrived = reinterpret_cast<int*>(prm.partial + (size_t)score_tc_tiles(gp, m) * prm.splits * 3 * TILE_M);
+        prm.arrived = reinterpret_cast<int*>(prm.partial + slots * 3 * TILE_M);
     }
     prm.trace = nullptr;
     prof_begin(gp, stream);
@@ -1466,8 +1483,9 @@ r3_status_t score_tc_part(r3_gp* gp, const float* Xcand, long long m, float* mu,
         const r3_status_t st = launch_tc_pair(t, prm, sms, stream);
         if (st != R3_OK) return st;
     } else {
-        auto launch = [&](bool f8, long long begin, long long end, int want_mode) -> r3_status_t {
+        auto launch = [&](bool f8, long long begin, long long end, int want_mode, bool first = false) -> r3_status_t {
             TcParams q = prm;
+            if (first) q.splits = plan_splits(t, end - begin, sms, q.cut);
             q.tile_begin = begin;
             q.total_tiles = end;
             q.mode = want_mode < 0 ? nullptr : gb.mode;
@@ -1488,14 +1506,14 @@ r3_status_t score_tc_part(r3_gp* gp, const float* Xcand, long long m, float* mu,
         } else {
             // The FP8 cross terms save a fifth of the time where the posterior is tame and send most of a pool to the FP64
             // pass where it is not (few features, long lengthscales): 65,536 candidates at n = 4096 with 41,604 recomputed
-            // 41.6 ms, with FP16 cross terms and none recomputed 4.1 ms.  So the pool's first wave of tiles, as they lie in
-            // memory, is scored with them, a test of it (pilot_kernel) decides on the device for the whole pool, and of the two
-            // launches for the rest (for all of it, in the FP16 form) one returns at once.  A first wave costs no more alone
-            // than as part of the whole.
+            // 41.6 ms, with FP16 cross terms and none recomputed 4.1 ms.  So the pool's first tiles, as they lie in
+            // memory, are scored with them, a test of it (pilot_kernel) decides on the device for the whole pool, and of the two
+            // launches for the rest (for all of it, in the FP16 form) one returns at once.  A first part costs no more alone
+            // than as part of the whole (pilot_tiles).
             long long rest = begin;
             if (begin == 0) {
-                rest = std::min<long long>(end, sms);
-                st = launch(true, 0, rest, -1);
+                rest = std::min(end, pilot_tiles(gp, m, sms));   // of the whole pool, whatever this launch covers
+                st = launch(true, 0, rest, -1, true);
                 // candidates of the first `rest` tiles that lie together in memory: whole GPs and a part of the next
                 const long long whole = rest / prm.tiles_per_gp, part = std::min(m, rest % prm.tiles_per_gp * TILE_M);
                 if (st == R3_OK) st = guard_pilot(gp, m, whole * m + part, gb, mu, sigma, ei, stream);
