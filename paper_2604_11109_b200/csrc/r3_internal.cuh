@@ -272,7 +272,7 @@ size_t guard_topk_workspace_bytes(int batch, long long m, int k);
 r3_status_t guard_pilot(r3_gp* gp, long long m, long long rows, const GuardBuffers& b, const float* mu, const float* sigma,
                         const float* ei, cudaStream_t stream);
 GuardBuffers guard_carve(const r3_gp* gp, long long m, void* ws);
-// have_max: the engine has raised maxbits to the pool's largest EI; tile_max: it has left the largest of each tile instead
+// have_max: the engine has raised maxbits to the pool's largest EI; tile_max: it has left the largest of each tile instead, one per 32 rows
 r3_status_t guard_and_rescue(r3_gp* gp, const float* Xcand, long long m, const GuardBuffers& b, float* mu,
                              float* sigma, float* ei, const float* tile_max, long long tiles_per_gp, bool have_max, cudaStream_t stream);
 

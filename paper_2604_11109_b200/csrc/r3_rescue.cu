@@ -70,7 +70,7 @@ struct GuardArgs {
     int* status;                  // the handle's status words
     WaitRule wait;
     bool have_max;                // maxbits holds the largest EI already, or tile_max does:
-    const float* tile_max;        // [batch][tiles_per_gp] the engine's largest EI of each tile, or nullptr
+    const float4* tile_max;       // [batch][tiles_per_gp] the engine's largest EI of each tile, one per 32 rows, or nullptr
     int tiles_per_gp;
     double *ks, *qpart, *mupart;  // slab: [slab][npad], [slab][npad / 16], [slab][ceil(npad / 64)]
     int slab;                     // candidates per slab, a multiple of 64
@@ -377,8 +377,11 @@ __device__ __forceinline__ bool guard_pool(const GuardArgs& a, unsigned char* sm
         const int g = s / a.chunks_per_gp;
         if (a.tile_max && g != max_of) {   // every block takes the largest of the tiles' largest by itself
             float v = 0.f;
-#pragma unroll 8
-            for (int i = t; i < a.tiles_per_gp; i += kThreads) v = fmaxf(v, __ldg(a.tile_max + (size_t)g * a.tiles_per_gp + i));
+#pragma unroll 4
+            for (int i = t; i < a.tiles_per_gp; i += kThreads) {
+                const float4 q = __ldg(a.tile_max + (size_t)g * a.tiles_per_gp + i);
+                v = fmaxf(fmaxf(v, fmaxf(q.x, q.y)), fmaxf(q.z, q.w));
+            }
             const unsigned top = __reduce_max_sync(0xffffffffu, __float_as_uint(v));
             __syncthreads();
             if (lane == 0) warp_sum[warp] = (int)top;
@@ -662,7 +665,7 @@ r3_status_t guard_and_rescue(r3_gp* gp, const float* Xcand, long long m, const G
     a.status = gp->status_d;
     a.wait = wait_rule(gp, STALL_GUARD);
     a.have_max = have_max || tile_max;
-    a.tile_max = tile_max;
+    a.tile_max = reinterpret_cast<const float4*>(tile_max);
     a.tiles_per_gp = (int)tiles_per_gp;
     a.ks = b.ks; a.qpart = b.qpart; a.mupart = b.mupart;
     a.slab = slab_candidates(gp, m);

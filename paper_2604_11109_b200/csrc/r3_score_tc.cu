@@ -34,7 +34,10 @@
 // mbar_wait_warp); two groups of four warps bring candidates in and results out; three groups of four Matern warps (one warp
 // per TMEM lane quarter) take every third chunk each.  Stages are handed over through mbarriers; every wait is bounded: when
 // a limit is hit the CTA raises a status bit, all roles leave their loops, in-flight copies and MMAs are drained (bounded
-// again), TMEM is freed and the kernel returns.
+// again), TMEM is freed and the kernel returns.  Between set-up and teardown no warp waits for another in any other way: whether
+// a wait ran out is decided by each warp for itself, so a barrier without a limit (bar.sync) could be entered by one warp of a
+// group after another has left.  Warps of a group therefore share nothing but mbarriers: a warp finishes its own 32 rows,
+// counts the parts of its own rows of a shared tile, and leaves its own largest EI.
 //
 // The roles' code has to stay small: together it is about what the SM's instruction cache holds, and what does not fit costs
 // the Matern warps first.  Both halves of a chunk unrolled, norms and weights through shared memory (one more wait in the
@@ -79,7 +82,7 @@ enum : uint32_t {
     BAR_RED_FULL = BAR_Z_EMPTY + 2, BAR_RED_EMPTY = BAR_RED_FULL + 2, BAR_MMA_DONE = BAR_RED_EMPTY + 2,   // MMA_DONE: three, distance and variance issuers
     BAR_COUNT = BAR_MMA_DONE + 3
 };
-constexpr uint32_t kFlagOffset = 512;    // behind the barriers: int abort, int drain-abort, uint32 tmem base, int last
+constexpr uint32_t kFlagOffset = 512;    // behind the barriers: int abort, int drain-abort, uint32 tmem base
 static_assert(BAR_COUNT * 8 <= kFlagOffset, "barriers overlap the flags");
 constexpr uint32_t kBarBytes = 1024;
 // Registers per thread once the roles have parted; the block starts with the file split evenly (80 for 768 threads).
@@ -288,8 +291,6 @@ __global__ void __launch_bounds__(kThreads, 1) score_tc_kernel(const __grid_cons
     const uint32_t bars = base + map.bar;
     volatile int* abort_flag = reinterpret_cast<volatile int*>(sm + map.bar + kFlagOffset);
     volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(sm + map.bar + kFlagOffset + 8);
-    volatile int* last_flag = reinterpret_cast<volatile int*>(sm + map.bar + kFlagOffset + 12);
-    volatile unsigned* top_s = reinterpret_cast<volatile unsigned*>(sm + map.bar + kFlagOffset + 32);   // largest EI of a warp's rows, [group][4]
     auto zn_buf = [&](int b) { return reinterpret_cast<float*>(sm + map.zn + b * kZnBuf); };
     auto bar = [&](uint32_t slot) { return bars + slot * 8u; };
 
@@ -714,7 +715,8 @@ __global__ void __launch_bounds__(kThreads, 1) score_tc_kernel(const __grid_cons
                 if (groups == 1 && zb == 2) b ^= 1;
                 continue;
             }
-            // ---- the groups' partial sums; a tile whose pairs went to several units is finished by the last of them
+            // ---- the groups' partial sums; a tile whose pairs went to several units is finished by the last of them, each 32
+            // rows by the warp that sees its last part arrive
             ok = mbar_wait_warp(bar(BAR_RED_FULL + b), (red_ph >> b) & 1u, abort_flag, wl);
             if (!ok) break;
             double mu_acc = 0.0;
@@ -739,11 +741,10 @@ __global__ void __launch_bounds__(kThreads, 1) score_tc_kernel(const __grid_cons
                 __stcg(mine + TILE_M, q_acc);
                 __stcg(reinterpret_cast<float2*>(mine + 2 * TILE_M), make_float2(a2_acc, s2_acc));
                 __threadfence();
-                asm volatile("bar.sync %0, 128;" ::"r"(1 + io) : "memory");
-                if (row == 0) last_flag[io] = atomicAdd(prm.arrived + unit % tiles, 1) == prm.splits - 1;
-                asm volatile("bar.sync %0, 128;" ::"r"(1 + io) : "memory");
-                finish = last_flag[io] != 0;
-                asm volatile("bar.sync %0, 128;" ::"r"(1 + io) : "memory");
+                __syncwarp();
+                int before = 0;   // parts of these 32 rows that are already there
+                if (lane == 0) before = atomicAdd(prm.arrived + R3_IDX((unit % tiles) * 4 + (warp & 3), tiles * 4, prm.status), 1);
+                finish = __shfl_sync(0xffffffffu, before, 0) == prm.splits - 1;
                 if (finish) {
                     __threadfence();
                     mu_acc = q_acc = 0.0;
@@ -778,12 +779,8 @@ __global__ void __launch_bounds__(kThreads, 1) score_tc_kernel(const __grid_cons
             }
             if (finish) {   // EI >= 0: the order of the bits is the order of the values
                 const unsigned top = __reduce_max_sync(0xffffffffu, __float_as_uint(ei_mine));
-                if (lane == 0) top_s[io * 4 + (warp & 3)] = top;
-                asm volatile("bar.sync %0, 128;" ::"r"(1 + io) : "memory");
-                if (row == 0)
-                    prm.tile_max[R3_IDX(tile, (long long)tiles_per_gp * prm.batch, prm.status)] =
-                        __uint_as_float(max(max(top_s[io * 4], top_s[io * 4 + 1]), max(top_s[io * 4 + 2], top_s[io * 4 + 3])));
-                asm volatile("bar.sync %0, 128;" ::"r"(1 + io) : "memory");   // read before the next tile's are written
+                if (lane == 0)
+                    prm.tile_max[R3_IDX((long long)tile * 4 + (warp & 3), 4ll * tiles_per_gp * prm.batch, prm.status)] = __uint_as_float(top);
             }
             if (groups == 1 && zb == 2) b ^= 1;
         }
@@ -1352,8 +1349,8 @@ static int device_sms(int device)
     return sms;
 }
 
-// guard's workspace, then the tiles' largest EI, the sums of split tiles and their counters
-static size_t max_bytes(const r3_gp* gp, long long m) { return ((size_t)score_tc_tiles(gp, m) * sizeof(float) + 511) & ~(size_t)255; }
+// guard's workspace, then the tiles' largest EI (one of each 32 rows), the sums of split tiles and their counters
+static size_t max_bytes(const r3_gp* gp, long long m) { return ((size_t)score_tc_tiles(gp, m) * sizeof(float4) + 511) & ~(size_t)255; }
 // With FP8 cross terms, the tiles that are scored first and decide for the pool: what is left over when the pool is cut into
 // whole waves, so that the rest is whole waves, but at least a quarter of one.  Their pairs of strips are shared out over all
 // SMs.  (A whole wave of tiles: 0.8 ms of the 10.5 ms of a round at n = 4096 whose 512 tiles are then scored with FP16 cross
@@ -1376,7 +1373,7 @@ static size_t split_slots(const r3_gp* gp, long long m)
 static size_t split_bytes(const r3_gp* gp, long long m)
 {
     const size_t slots = split_slots(gp, m);
-    return slots ? slots * 3 * TILE_M * sizeof(double) + score_tc_tiles(gp, m) * sizeof(int) + 256 : 0;
+    return slots ? slots * 3 * TILE_M * sizeof(double) + score_tc_tiles(gp, m) * sizeof(int4) + 256 : 0;
 }
 size_t score_tc_workspace_bytes(const r3_gp* gp, long long m) { return guard_workspace_bytes(gp, m) + max_bytes(gp, m) + split_bytes(gp, m); }
 
@@ -1494,7 +1491,7 @@ r3_status_t score_tc_part(r3_gp* gp, const float* Xcand, long long m, float* mu,
                 q.wt = t->wt16;
                 q.vinv2 = t->vinv2_16;
             }
-            if (q.splits > 1) R3_CUDA_TRY(cudaMemsetAsync(q.arrived, 0, sizeof(int) * (end - begin), stream));
+            if (q.splits > 1) R3_CUDA_TRY(cudaMemsetAsync(q.arrived, 0, sizeof(int4) * (end - begin), stream));
             void (*kernel)(const TcParams) = kernel_of(t, f8);
             R3_LAUNCH(kernel, (unsigned)std::min<long long>((end - begin) * q.splits, sms), kThreads, t->smem_bytes, stream, q);
             return R3_OK;

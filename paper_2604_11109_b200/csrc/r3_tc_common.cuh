@@ -55,9 +55,9 @@ struct TcParams {
     float rsqrt_dp;             // 1 / sqrt of the feature count rounded up to 16 (error estimate)
     int splits;                 // units that a tile's pairs of strips are shared out to: part i takes [cut[i], cut[i + 1])
     unsigned char cut[kMaxSplits + 2];
-    double* partial;            // splits > 1: [tiles][splits][3][128] sums of a part, and how many parts of a tile have
-    int* arrived;               // been summed
-    float* tile_max;            // [tiles of the pool] largest EI of each, for the guard
+    double* partial;            // splits > 1: [tiles][splits][3][128] sums of a part, and
+    int* arrived;               // [tiles][4] how many parts of each 32 rows of a tile have been summed
+    float* tile_max;            // [tiles of the pool][4] largest EI of each 32 rows, for the guard
     int* status;
     int* zero;          // the guard's counters, cleared by the first block (nothing reads them before the guard's kernel)
     int zero_ints;

@@ -30,16 +30,21 @@ def _scores_match(g, gp, what):
                      what=what)
 
 
-@pytest.mark.parametrize("n,m,chunk,pair", [
-    (100, 128, 2, False),      # one pass of four chunks, one tile: the third chunk of W never arrives
-    (250, 300, 0, False),      # the very first chunk is withheld; three tiles on three thread blocks
-    (600, 1000, 11, False),    # three passes; the stream stops inside the second
-    (300, 256, 5, True),       # the kernel that runs a tile on a cluster of two thread blocks
+@pytest.mark.parametrize("n,d,m,chunk,pair", [
+    (100, 12, 128, 2, False),    # one pass of four chunks, one tile: the third chunk of W never arrives
+    (250, 12, 300, 0, False),    # the very first chunk is withheld; three tiles on three thread blocks
+    (600, 12, 1000, 11, False),  # three passes; the stream stops inside the second
+    (500, 128, 260, 9, False),   # one buffer of scaled candidates, whose next tile comes in before the last strip is read back
+    (400, 70, 300, 6, False),    # features in two stages
+    (1100, 40, 200, 3, False),   # pairs of strips shared out: no part of a tile arrives
+    (140, 20, 148 * 128 * 3 + 5, 20, False),   # several tiles per thread block; both groups of result warps are under way
+    (1900, 24, 200, 5, False),   # FP8 cross terms
+    (300, 12, 256, 5, True),     # the kernel that runs a tile on a cluster of two thread blocks
 ])
-def test_a_wait_that_runs_out_is_reported_and_the_handle_stays_usable(monkeypatch, n, m, chunk, pair):
+def test_a_wait_that_runs_out_is_reported_and_the_handle_stays_usable(monkeypatch, n, d, m, chunk, pair):
     if pair:
         monkeypatch.setenv("R3_TC_PAIR", "1")
-    g = rand_problem(4000 + n, 1, n, 12, m)
+    g = rand_problem(4000 + n, 1, n, d, m)
     gp = fit_gpu(g, b.ENGINE_TENSOR)
     _scores_match(g, gp, "before")
     b.r3_gp_set_wait_limit(gp, SHORT_LIMIT)
@@ -52,6 +57,36 @@ def test_a_wait_that_runs_out_is_reported_and_the_handle_stays_usable(monkeypatc
     _scores_match(g, gp, "after the timeout")
     b.r3_gp_set_wait_limit(gp, 4_000_000_000)
     _scores_match(g, gp, "default limit")
+    gp.close()
+
+
+@pytest.mark.parametrize("n,d,m", [
+    (1500, 20, 148 * 128 * 4 + 3),   # two buffers of candidates
+    (1000, 128, 148 * 128 * 3),      # one buffer, features in two stages
+    (2500, 40, 148 * 128 * 2 + 9),   # FP8 cross terms
+    (900, 24, 300),                  # pairs of strips shared out
+])
+def test_a_limit_that_runs_out_while_the_pipeline_is_at_work(n, d, m):
+    """The shortest limit there is, less than a tile takes: waits run out in thread blocks whose other warps are still
+    handing stages over.  The call returns by itself, with or without a time-out, and the handle keeps working."""
+    g = rand_problem(4100 + n, 1, n, d, m)
+    gp = fit_gpu(g, b.ENGINE_TENSOR)
+    xc = dev(g["Xcand"])
+    want = [t.clone() for t in b.r3_gp_score(gp, xc)]
+    b.r3_gp_check(gp)
+    b.r3_gp_set_wait_limit(gp, 100_000)
+    for _ in range(5):
+        b.r3_gp_score(gp, xc)
+        try:
+            b.r3_gp_check(gp)
+        except b.R3Error as e:
+            assert e.status == 6
+    b.r3_gp_set_wait_limit(gp, 4_000_000_000)
+    got = b.r3_gp_score(gp, xc)
+    b.r3_gp_check(gp)
+    # the same kernels on the same operands: only what the FP64 pass recomputes may come in another grouping
+    for a, c, scale in zip(got, want, (np.abs(g["y"]).max(), 1.0, float(want[2].max()))):
+        assert ((a - c).abs() <= 1e-6 * (c.abs() + scale)).all()
     gp.close()
 
 
