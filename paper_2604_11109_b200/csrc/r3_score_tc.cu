@@ -506,8 +506,6 @@ __global__ void __launch_bounds__(kThreads, 1) score_tc_kernel(const __grid_cons
                 if (which < strips) {
                     const int s = pr.a + which;
                     const uint32_t n_own = which ? pr.nb : pr.na, rows = (uint32_t)min(kStrip, nc * KC - s * kStrip);
-                    // arrivals that free a bank of slots: one from each issuer, both from this one where it is the only user
-                    const uint32_t shared = strips == 2 ? (uint32_t)pr.na : 0u;
                     if (!(ok = mbar_wait_warp(bar(BAR_V_EMPTY + me), v_ph ^ 1u, abort_flag, wl))) break;
                     for (uint32_t c = 0; c < n_own; ++c) {
                         const uint32_t t = t_base + c, slot = t % kSlots;
@@ -546,19 +544,21 @@ __global__ void __launch_bounds__(kThreads, 1) score_tc_kernel(const __grid_cons
                         }
                         tc_commit_if(leader, bar(BAR_W_EMPTY + wbar + w_s));
                         if (++w_s == ring) { w_s = 0; w_ph ^= 1u; }
-                        if (t % KDC == KDC - 1) {   // slots go back to the distance products a bank at a time
-                            const uint32_t kb = bar(BAR_K_EMPTY + (t / KDC) % BANKS);
-                            tc_commit_if(leader, kb);
-                            if (c >= shared) tc_commit_if(leader, kb);
-                        }
+                        // slots go back to the distance products a bank at a time, when both issuers are through with it
+                        if (t % KDC == KDC - 1) tc_commit_if(leader, bar(BAR_K_EMPTY + (t / KDC) % BANKS));
                     }
                     if (!ok) break;
                     tc_commit_if(leader, bar(BAR_V_FULL + 2 * me + zi));
                     v_ph ^= 1u;
                 }
-                // chunks that only the other issuer takes: a wait by parity is good for one phase, so none is passed over
-                for (uint32_t c = which < strips ? (which ? pr.nb : pr.na) : 0; ok && c < (uint32_t)pr.chunks(); ++c)
-                    ok = mbar_wait_warp(bar(BAR_K_FULL + (t_base + c) % kSlots), ((t_base + c) / kSlots) & 1u, abort_flag, wl);
+                // Chunks that only the other issuer takes (whole banks: strips have even numbers of chunks).  A wait by parity is
+                // good for one phase, so this issuer waits for each of them too, and the bank is not free before it has: a slot
+                // filled twice in between would look to it as if it had not been filled at all.
+                for (uint32_t c = which < strips ? (which ? pr.nb : pr.na) : 0; ok && c < (uint32_t)pr.chunks(); ++c) {
+                    const uint32_t t = t_base + c;
+                    if (!(ok = mbar_wait_warp(bar(BAR_K_FULL + t % kSlots), (t / kSlots) & 1u, abort_flag, wl))) break;
+                    if (t % KDC == KDC - 1 && leader) mbar_arrive(bar(BAR_K_EMPTY + (t / KDC) % BANKS));
+                }
                 t_base += pr.chunks();
             }
         }
