@@ -37,7 +37,7 @@ def _scores_match(g, gp, what):
     (500, 128, 260, 9, False),   # one buffer of scaled candidates, whose next tile comes in before the last strip is read back
     (400, 70, 300, 6, False),    # features in two stages
     (1100, 40, 200, 3, False),   # pairs of strips shared out: no part of a tile arrives
-    (140, 20, 148 * 128 * 3 + 5, 20, False),   # several tiles per thread block; both groups of result warps are under way
+    (140, 20, 148 * 128 * 3 + 5, 6, False),   # several tiles per thread block; both groups of result warps are under way
     (1900, 24, 200, 5, False),   # FP8 cross terms
     (300, 12, 256, 5, True),     # the kernel that runs a tile on a cluster of two thread blocks
 ])
