@@ -22,7 +22,8 @@ struct r3_tpe {
     int n = 0, d = 0, n_good = 0, device = 0;
     float prior_weight = 1.f;
     std::vector<int> levels;
-    int* levels_d = nullptr;   // [d]
+    int tabled = 0;            // features with a table
+    int* levels_d = nullptr;   // [d], then [d]: the features with a table, then those with mixtures (a score adds them up so)
     int* order_d = nullptr;    // [n] history indices by y ascending
     float4* comps_d = nullptr; // [d][n + 2]: good set's components from 0, the bad set's from n_good + 1
     int* counts_d = nullptr;   // [d][2]: components of each set after merging equal ones
@@ -497,11 +498,72 @@ __device__ __forceinline__ void mixture_sums_staged(const float4* __restrict__ c
     finish_sums<R>(part, sum);
 }
 
+// Look-ups of tabulated features do not depend on one another: in a loop of their own they are taken in groups of four, with the
+// next group's values on their way meanwhile, while in one loop with the mixtures each feature waits for the one before it.
+// Bound by the latency of those reads.  400,000 candidates with 59 tables and a mixture of 40 observations 117 us in one loop,
+// 70 us in two.
+struct Features {
+    int at[kMaxD];      // tables first: the features with a table, then those with mixtures; otherwise feature i
+    float top[kMaxD];   // admissible values - 1, -1 for a mixture
+};
+template <bool TABLES_FIRST>
+__device__ __forceinline__ void load_features(Features& s, const int* __restrict__ levels, int d)
+{
+    for (int i = threadIdx.x; i < d; i += kScoreThreads) {
+        s.at[i] = TABLES_FIRST ? __ldg(levels + d + i) : i;
+        s.top[i] = (float)(abs(__ldg(levels + s.at[i])) - 1);
+    }
+}
+// the admissible value nearest to x (top + 1 of them)
+__device__ __forceinline__ int level_of(float x, float top)
+{
+    const float lv = floorf(__fadd_rn(__fmul_rn(x, top), 0.5f));
+    return isfinite(x) ? (int)fminf(fmaxf(lv, 0.f), top) : 0;
+}
+// acc[r] += the tables' contributions to the candidate in row[r] (a row of the pool for every r)
+template <int R>
+__device__ __forceinline__ void add_tabled(const Features& s, int tabled, const float* const (&row)[R], const float* __restrict__ table,
+                                           float (&acc)[R], bool& bad)
+{
+    if (tabled == 0) return;
+    float next[R][4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e)
+#pragma unroll
+        for (int r = 0; r < R; ++r) next[r][e] = e < tabled ? row[r][s.at[e]] : 0.f;
+    for (int i0 = 0; i0 < tabled; i0 += 4) {
+        float x[R][4], found[R][4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                x[r][e] = next[r][e];
+                next[r][e] = i0 + 4 + e < tabled ? row[r][s.at[i0 + 4 + e]] : 0.f;
+            }
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            if (i0 + e >= tabled) continue;
+            const float top = s.top[i0 + e];
+            const float* t = table + (size_t)s.at[i0 + e] * kTpeMaxLevels;
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                bad |= !isfinite(x[r][e]);
+                found[r][e] = __ldg(t + level_of(x[r][e], top));
+            }
+        }
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+#pragma unroll
+            for (int r = 0; r < R; ++r)
+                if (i0 + e < tabled) acc[r] += found[r][e];
+    }
+}
+
 // (T4) score of every candidate.  A block covers R * blockDim.x consecutive candidates; thread t holds
 // candidates t, t + blockDim.x, ... of the block's range so that the result stores coalesce.
 template <int R>
 __global__ void __launch_bounds__(kScoreThreads) tpe_score_kernel(const float* __restrict__ Xc, long long m, int n,
-                                                                  int d, int n_good, const int* __restrict__ levels,
+                                                                  int d, int n_good, const int* __restrict__ levels, int tabled,
                                                                   const float4* __restrict__ comps,
                                                                   const int* __restrict__ counts,
                                                                   const float* __restrict__ table,
@@ -511,6 +573,12 @@ __global__ void __launch_bounds__(kScoreThreads) tpe_score_kernel(const float* _
     bool bad = false;
     __shared__ __align__(16) float stage_s[3][kStage];
     const Components stage{stage_s[0], stage_s[1], stage_s[2]};
+    constexpr bool SPLIT = R == 1;   // the tables in a loop of their own (3000 candidates, 98 tables and two mixtures: 172 -> 135 us)
+    __shared__ Features features;
+    if constexpr (SPLIT) {
+        load_features<true>(features, levels, d);
+        __syncthreads();
+    }
     for (long long tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
         const long long base = tile * (long long)R * kScoreThreads + threadIdx.x;
         const float* row[R];
@@ -523,30 +591,30 @@ __global__ void __launch_bounds__(kScoreThreads) tpe_score_kernel(const float* _
             row[r] = Xc + (size_t)(valid[r] ? cand : 0) * d;
             acc[r] = 0.f;
         }
-        for (int j = 0; j < d; ++j) {
+        if constexpr (SPLIT) add_tabled<R>(features, tabled, row, table, acc, bad);
+        for (int i = SPLIT ? tabled : 0; i < d; ++i) {
+            const int j = SPLIT ? features.at[i] : i;
             float x[R];
 #pragma unroll
             for (int r = 0; r < R; ++r) {
                 x[r] = row[r][j];
                 bad |= valid[r] && !isfinite(x[r]);
             }
-            const int code = __ldg(levels + j);
-            const int C = code < 0 ? -code : code;   // categorical levels, or grid values of an ordinal dimension
-            if (C > 0) {
+            if constexpr (!SPLIT) {
+                const int values = abs(__ldg(levels + j));
+                if (values > 0) {
 #pragma unroll
-                for (int r = 0; r < R; ++r) {
-                    const float lv = floorf(__fadd_rn(__fmul_rn(x[r], (float)(C - 1)), 0.5f));
-                    const int v = isfinite(x[r]) ? (int)fminf(fmaxf(lv, 0.f), (float)(C - 1)) : 0;
-                    acc[r] += __ldg(table + (size_t)j * kTpeMaxLevels + v);
+                    for (int r = 0; r < R; ++r)
+                        acc[r] += __ldg(table + (size_t)j * kTpeMaxLevels + level_of(x[r], (float)(values - 1)));
+                    continue;
                 }
-            } else {
-                const float4* cj = comps + (size_t)j * (n + 2);
-                float sl[R], sg[R];
-                mixture_sums_staged<R>(cj, __ldg(counts + 2 * j), x, sl, stage);
-                mixture_sums_staged<R>(cj + n_good + 1, __ldg(counts + 2 * j + 1), x, sg, stage);
-#pragma unroll
-                for (int r = 0; r < R; ++r) acc[r] += 0.69314718f * (lg2_fast(sl[r]) - lg2_fast(sg[r]));
             }
+            const float4* cj = comps + (size_t)j * (n + 2);
+            float sl[R], sg[R];
+            mixture_sums_staged<R>(cj, __ldg(counts + 2 * j), x, sl, stage);
+            mixture_sums_staged<R>(cj + n_good + 1, __ldg(counts + 2 * j + 1), x, sg, stage);
+#pragma unroll
+            for (int r = 0; r < R; ++r) acc[r] += 0.69314718f * (lg2_fast(sl[r]) - lg2_fast(sg[r]));
         }
 #pragma unroll
         for (int r = 0; r < R; ++r)
@@ -592,19 +660,26 @@ __global__ void __launch_bounds__(256) tpe_pack_kernel(const float4* __restrict_
 // every block loads the packed model once and then walks its tiles without a block-wide barrier.  (Reading
 // four or eight features of a row per load, with the feature loop unrolled to match, measured 10-30 % slower:
 // the kernel is bound by instruction issue, not by the row reads.)
-template <int R>
+// SPLIT: the tables in a loop of their own, behind the mixtures.  It takes more registers and instructions than a branch in one
+// loop, which with two candidates per thread only a model of mostly tables pays back (1,048,576 candidates: 59 tables and a
+// mixture 215 -> 141 us, five and one 33.7 -> 35.7 us, 32 and 32 695 -> 735 us); with one per thread the reads' latency counts
+// for more (60,000 candidates, 32 and 32: 69 -> 62 us).
+template <int R, bool SPLIT>
 __global__ void __launch_bounds__(kScoreThreads) tpe_score_resident_kernel(
-    const float* __restrict__ Xc, long long m, int d, const int* __restrict__ levels, const int* __restrict__ offs,
+    const float* __restrict__ Xc, long long m, int d, const int* __restrict__ levels, int tabled, const int* __restrict__ offs,
     const float4* __restrict__ packed, int total, const float* __restrict__ table, float* __restrict__ score,
     int* __restrict__ status)
 {
-    extern __shared__ __align__(16) float model[];   // three arrays of padded components, then [2d + 1] offsets, then [d] level codes
+    // three arrays of padded components, the features of the mixture loop and where their two sets begin and end, [2d + 1] offsets
+    extern __shared__ __align__(16) float model[];
+    __shared__ Features features;
     const int padded = resident_padded(total, d);
     const Components comps{model, model + padded, model + 2 * padded};
-    int* offs_s = reinterpret_cast<int*>(model + 3 * padded);
-    int* code_s = offs_s + 2 * d + 1;
+    const int first = SPLIT ? tabled : 0;
+    int4* sets = reinterpret_cast<int4*>(model + 3 * padded);   // padded is a multiple of four
+    int* offs_s = reinterpret_cast<int*>(sets + d - first);
     for (int i = threadIdx.x; i <= 2 * d; i += kScoreThreads) offs_s[i] = __ldg(offs + i);
-    for (int i = threadIdx.x; i < d; i += kScoreThreads) code_s[i] = __ldg(levels + i);
+    load_features<SPLIT>(features, levels, d);
     for (int i = threadIdx.x; i < padded; i += kScoreThreads) {
         comps.nmean[i] = 0.f;
         comps.na[i] = -1.f;
@@ -625,7 +700,11 @@ __global__ void __launch_bounds__(kScoreThreads) tpe_score_resident_kernel(
         comps.b[at] = q.z;
     }
     __syncthreads();
-    for (int i = threadIdx.x; i <= 2 * d; i += kScoreThreads) offs_s[i] = (offs_s[i] + 3 * i + 3) & ~3;   // set i, padded to four
+    for (int i = threadIdx.x; i < d - first; i += kScoreThreads) {
+        const int j = features.at[first + i];
+        auto padded_at = [&](int set) { return (offs_s[set] + 3 * set + 3) & ~3; };
+        sets[i] = make_int4(j, padded_at(2 * j), padded_at(2 * j + 1), padded_at(2 * j + 2));
+    }
     __syncthreads();
     const long long tiles = (m + (long long)R * kScoreThreads - 1) / ((long long)R * kScoreThreads);
     bool bad = false;
@@ -641,35 +720,31 @@ __global__ void __launch_bounds__(kScoreThreads) tpe_score_resident_kernel(
             row[r] = Xc + (size_t)(valid[r] ? cand : 0) * d;
             acc[r] = 0.f;
         }
-        for (int j = 0; j < d; ++j) {
+        for (int i = 0; i < d - first; ++i) {
+            const int4 q = sets[i];
             float x[R];
 #pragma unroll
             for (int r = 0; r < R; ++r) {
-                x[r] = row[r][j];
+                x[r] = row[r][SPLIT ? q.x : i];
                 bad |= valid[r] && !isfinite(x[r]);
             }
-            const int code = code_s[j];
-            const int C = code < 0 ? -code : code;
-            if (C > 0) {
+            if (!SPLIT && features.top[i] >= 0.f) {
 #pragma unroll
-                for (int r = 0; r < R; ++r) {
-                    const float lv = floorf(__fadd_rn(__fmul_rn(x[r], (float)(C - 1)), 0.5f));
-                    const int v = isfinite(x[r]) ? (int)fminf(fmaxf(lv, 0.f), (float)(C - 1)) : 0;
-                    acc[r] += __ldg(table + (size_t)j * kTpeMaxLevels + v);
-                }
-            } else {
-                float sl[R], sg[R];
-                uint64_t part[R][2] = {};
-                mixture_sums<R>(comps, offs_s[2 * j], offs_s[2 * j + 1], x, part);
-                finish_sums<R>(part, sl);
-#pragma unroll
-                for (int r = 0; r < R; ++r) part[r][0] = part[r][1] = 0;
-                mixture_sums<R>(comps, offs_s[2 * j + 1], offs_s[2 * j + 2], x, part);
-                finish_sums<R>(part, sg);
-#pragma unroll
-                for (int r = 0; r < R; ++r) acc[r] += 0.69314718f * (lg2_fast(sl[r]) - lg2_fast(sg[r]));
+                for (int r = 0; r < R; ++r) acc[r] += __ldg(table + (size_t)i * kTpeMaxLevels + level_of(x[r], features.top[i]));
+                continue;
             }
+            float sl[R], sg[R];
+            uint64_t part[R][2] = {};
+            mixture_sums<R>(comps, q.y, q.z, x, part);
+            finish_sums<R>(part, sl);
+#pragma unroll
+            for (int r = 0; r < R; ++r) part[r][0] = part[r][1] = 0;
+            mixture_sums<R>(comps, q.z, q.w, x, part);
+            finish_sums<R>(part, sg);
+#pragma unroll
+            for (int r = 0; r < R; ++r) acc[r] += 0.69314718f * (lg2_fast(sl[r]) - lg2_fast(sg[r]));
         }
+        if (SPLIT) add_tabled<R>(features, tabled, row, table, acc, bad);
 #pragma unroll
         for (int r = 0; r < R; ++r)
             if (valid[r]) score[base + (long long)r * kScoreThreads] = acc[r];
@@ -751,6 +826,40 @@ __global__ void __launch_bounds__(256) tpe_table_score_kernel(const float* __res
     if (bad) atomicOr(status, DEV_NONFINITE);
 }
 
+// (T4) when every dimension is tabulated and rows cannot be read as groups of four (d no multiple of 4, or a pool off a 16-byte
+// boundary).  Whatever mixtures the fit kept for a grid are not looked at.  63 features: 2000 candidates 54 us with the kernels
+// that have mixtures in mind, 21 us here; 1,000,000 candidates 345 and 121 us.
+template <int R>
+__global__ void __launch_bounds__(kScoreThreads) tpe_lookup_score_kernel(const float* __restrict__ Xc, long long m, int d,
+                                                                         const int* __restrict__ levels,
+                                                                         const float* __restrict__ table,
+                                                                         float* __restrict__ score, int* __restrict__ status)
+{
+    __shared__ Features features;
+    load_features<true>(features, levels, d);
+    __syncthreads();
+    const long long tiles = (m + (long long)R * kScoreThreads - 1) / ((long long)R * kScoreThreads);
+    bool bad = false;
+    for (long long tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+        const long long base = tile * (long long)R * kScoreThreads + threadIdx.x;
+        const float* row[R];
+        float acc[R];
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const long long cand = base + (long long)r * kScoreThreads;
+            row[r] = Xc + (size_t)(cand < m ? cand : 0) * d;
+            acc[r] = 0.f;
+        }
+        add_tabled<R>(features, d, row, table, acc, bad);
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const long long cand = base + (long long)r * kScoreThreads;
+            if (cand < m) score[cand] = acc[r];
+        }
+    }
+    if (bad) atomicOr(status, DEV_NONFINITE);
+}
+
 size_t resident_bytes(int total, int d) { return sizeof(float4) * (size_t)total + sizeof(int) * (3 * (size_t)d + 1); }
 
 void tpe_destroy(r3_tpe* t)
@@ -769,7 +878,7 @@ r3_status_t tpe_fit_impl(r3_tpe* t, const float* X, const float* y, cudaStream_t
     auto up = [](size_t b) { return (b + 255) & ~(size_t)255; };
     const size_t b_comps = up(sizeof(float4) * (size_t)d * (n + 2)), b_packed = up(kResidentBytes),
                  b_table = up(sizeof(float) * (size_t)d * kTpeMaxLevels), b_order = up(sizeof(int) * n),
-                 b_levels = up(sizeof(int) * d), b_counts = up(sizeof(int) * 2 * (size_t)d),
+                 b_levels = up(sizeof(int) * 2 * (size_t)d), b_counts = up(sizeof(int) * 2 * (size_t)d),
                  b_offs = up(sizeof(int) * (2 * (size_t)d + 1)), b_status = 256,
                  b_lnp = up(sizeof(double) * 2 * (size_t)d * kTpeMaxLevels);
     char* base = nullptr;
@@ -794,7 +903,13 @@ r3_status_t tpe_fit_impl(r3_tpe* t, const float* X, const float* y, cudaStream_t
         set_error("r3_tpe_fit: no pinned host memory");
         return R3_ERR_ALLOC;
     }
-    R3_CUDA_TRY(cudaMemcpyAsync(t->levels_d, t->levels.data(), sizeof(int) * d, cudaMemcpyHostToDevice, stream));
+    std::vector<int> upload(t->levels);
+    for (int tabulated = 1; tabulated >= 0; --tabulated) {
+        for (int j = 0; j < d; ++j)
+            if ((t->levels[j] != 0) == (tabulated == 1)) upload.push_back(j);
+        if (tabulated) t->tabled = (int)upload.size() - d;
+    }
+    R3_CUDA_TRY(cudaMemcpyAsync(t->levels_d, upload.data(), sizeof(int) * 2 * (size_t)d, cudaMemcpyHostToDevice, stream));
     R3_CUDA_TRY(cudaMemsetAsync(t->status_d, 0, sizeof(int), stream));
     R3_LAUNCH(tpe_order_kernel, (n + kOrderRows - 1) / kOrderRows, 256, 0, stream, y, n, t->order_d, t->status_d);
     int count = 1;
@@ -881,8 +996,19 @@ r3_status_t r3_tpe_score(r3_tpe_t* tpe, const float* Xcand, long long m, float* 
         return R3_ERR_INVALID_ARG;
     }
     cudaStream_t stream = (cudaStream_t)cuda_stream;
-    bool all_tables = (tpe->d % 4) == 0 && (reinterpret_cast<uintptr_t>(Xcand) % 16) == 0;
-    for (int j = 0; j < tpe->d && all_tables; ++j) all_tables = tpe->levels[j] != 0;
+    const bool all_tables = tpe->tabled == tpe->d;
+    if (all_tables && (tpe->d % 4 != 0 || reinterpret_cast<uintptr_t>(Xcand) % 16 != 0)) {
+        // two candidates per thread when that still gives every SM several blocks
+        const long long tiles2 = (m + 2ll * kScoreThreads - 1) / (2ll * kScoreThreads);
+        const long long tiles1 = (m + kScoreThreads - 1) / kScoreThreads;
+        if (tiles2 >= 148ll * 8)
+            R3_LAUNCH(tpe_lookup_score_kernel<2>, (unsigned)std::min<long long>(tiles2, 148ll * 16), kScoreThreads, 0, stream,
+                      Xcand, m, tpe->d, tpe->levels_d, tpe->table_d, score, tpe->status_d);
+        else
+            R3_LAUNCH(tpe_lookup_score_kernel<1>, (unsigned)tiles1, kScoreThreads, 0, stream, Xcand, m, tpe->d, tpe->levels_d,
+                      tpe->table_d, score, tpe->status_d);
+        return R3_OK;
+    }
     if (all_tables) {
         // every dimension is a look-up: stream the pool with whole-row loads
         const int d4 = tpe->d / 4;
@@ -910,22 +1036,28 @@ r3_status_t r3_tpe_score(r3_tpe_t* tpe, const float* Xcand, long long m, float* 
         // the whole model in shared memory.  Sixteen blocks per SM's worth of grid (several waves of short
         // blocks) measured up to 8 % faster than one resident wave walking the tiles: the model is a small
         // read from L2 and the finer grain balances the SMs better.
-        const size_t smem = sizeof(float) * 3 * resident_padded(tpe->total, tpe->d) + sizeof(int) * (3 * (size_t)tpe->d + 1);
         const long long tiles2 = (m + 2ll * kScoreThreads - 1) / (2ll * kScoreThreads);
         const long long tiles1 = (m + kScoreThreads - 1) / kScoreThreads;
-#define R3_TPE_RESIDENT(R, TILES)                                                                              \
+#define R3_TPE_RESIDENT(R, SPLIT, TILES)                                                                       \
     do {                                                                                                       \
-        if (smem > 48 * 1024)                                                                                  \
-            R3_CUDA_TRY(cudaFuncSetAttribute(tpe_score_resident_kernel<R>,                                     \
+        const size_t smem = sizeof(float) * 3 * resident_padded(tpe->total, tpe->d) +                          \
+                            sizeof(int4) * (tpe->d - (SPLIT ? tpe->tabled : 0)) +                              \
+                            sizeof(int) * (2 * (size_t)tpe->d + 1);                                            \
+        if (smem + sizeof(Features) > 48 * 1024)   /* static and dynamic together */                           \
+            R3_CUDA_TRY(cudaFuncSetAttribute(tpe_score_resident_kernel<R, SPLIT>,                              \
                                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));         \
         const unsigned grid = (unsigned)std::min<long long>(TILES, 148ll * 16);                                \
-        R3_LAUNCH(tpe_score_resident_kernel<R>, grid, kScoreThreads, smem, stream, Xcand, m, tpe->d,           \
-                  tpe->levels_d, tpe->offs_d, tpe->packed_d, tpe->total, tpe->table_d, score, tpe->status_d);  \
+        R3_LAUNCH((tpe_score_resident_kernel<R, SPLIT>), grid, kScoreThreads, smem, stream, Xcand, m, tpe->d,  \
+                  tpe->levels_d, tpe->tabled, tpe->offs_d, tpe->packed_d, tpe->total, tpe->table_d, score,     \
+                  tpe->status_d);                                                                              \
     } while (0)
-        if (tiles2 >= 148ll * 8)
-            R3_TPE_RESIDENT(2, tiles2);
+        // two candidates per thread when that still gives every SM several blocks; which loop: see the kernel
+        if (tiles2 < 148ll * 8)
+            R3_TPE_RESIDENT(1, true, tiles1);
+        else if (tpe->tabled >= 6 * (tpe->d - tpe->tabled))
+            R3_TPE_RESIDENT(2, true, tiles2);
         else
-            R3_TPE_RESIDENT(1, tiles1);
+            R3_TPE_RESIDENT(2, false, tiles2);
 #undef R3_TPE_RESIDENT
         return R3_OK;
     }
@@ -936,11 +1068,11 @@ r3_status_t r3_tpe_score(r3_tpe_t* tpe, const float* Xcand, long long m, float* 
     if (tiles2 >= 148ll * 4) {
         const unsigned grid = (unsigned)(tiles2 < 148ll * 64 ? tiles2 : 148ll * 64);
         R3_LAUNCH(tpe_score_kernel<2>, grid, kScoreThreads, 0, stream, Xcand, m, tpe->n, tpe->d, tpe->n_good,
-                  tpe->levels_d, tpe->comps_d, tpe->counts_d, tpe->table_d, score, tpe->status_d);
+                  tpe->levels_d, tpe->tabled, tpe->comps_d, tpe->counts_d, tpe->table_d, score, tpe->status_d);
     } else {
         const long long tiles1 = (m + kScoreThreads - 1) / kScoreThreads;
         R3_LAUNCH(tpe_score_kernel<1>, (unsigned)tiles1, kScoreThreads, 0, stream, Xcand, m, tpe->n, tpe->d,
-                  tpe->n_good, tpe->levels_d, tpe->comps_d, tpe->counts_d, tpe->table_d, score, tpe->status_d);
+                  tpe->n_good, tpe->levels_d, tpe->tabled, tpe->comps_d, tpe->counts_d, tpe->table_d, score, tpe->status_d);
     }
     return R3_OK;
 }

@@ -373,3 +373,57 @@ def test_component_counts_that_fill_no_group_of_four(n, d, m):
     want = T.tpe_score(T.tpe_fit(X, y, levels, 0.25, 1.0), Xc[rows])
     err = np.abs(got[rows] - want) / (atol(n, levels) + RTOL * np.abs(want))
     assert err.max() <= 1.0, float(err.max())
+
+
+@pytest.mark.parametrize("d,m,shift", [
+    (1, 300, 0), (3, 255, 0), (5, 257, 0), (10, 2000, 0), (63, 1500, 0), (127, 900, 0), (255, 400, 0),
+    (30, 148 * 8 * 512 - 1, 0),               # two candidates per thread, the last tile ragged
+    (8, 1001, 1), (8, 148 * 8 * 512 + 3, 3),  # groups of four features, but rows off a 16-byte boundary
+])
+def test_tables_only_whatever_the_feature_count(d, m, shift):
+    """Categorical and grid features alone, in pools whose rows cannot be read four features at a time."""
+    rng = np.random.default_rng(100 * d + m)
+    n = 90
+    levels = np.array([(2, -5, 17, -64)[j % 4] for j in range(d)], np.int32)
+    L = np.abs(levels)
+    X = (np.floor(rng.uniform(0, 1, (n, d)) * L) / (L - 1)).astype(np.float32)
+    y = rng.normal(0, 1, n).astype(np.float32)
+    Xc = (np.floor(rng.uniform(0, 1, (m, d)) * L) / (L - 1)).astype(np.float32)
+    Xc[::61] += rng.uniform(-0.6, 0.6, Xc[::61].shape).astype(np.float32)   # off the grid and outside [0, 1]
+    tpe = b.r3_tpe_fit(dev(X), dev(y), levels, 0.25, 1.0)
+    store = torch.empty(m * d + shift, device="cuda")
+    pool = store[shift:].view(m, d)
+    pool.copy_(dev(Xc))
+    got = b.r3_tpe_score(tpe, pool).cpu().numpy()
+    b.r3_tpe_check(tpe)
+    rows = np.unique(np.concatenate([np.arange(min(m, 400)), np.arange(0, m, 61)[:200], rng.integers(0, m, 300), [m - 1]]))
+    check_score(got[rows], T.tpe_score(T.tpe_fit(X, y, levels, 0.25, 1.0), Xc[rows]), atol(n, levels))
+    pool[m - 1, d - 1] = float("nan")
+    b.r3_tpe_score(tpe, pool)
+    with pytest.raises(b.R3Error) as e:
+        b.r3_tpe_check(tpe)
+    assert e.value.status == 2
+    tpe.close()
+
+
+@pytest.mark.parametrize("n,d,m,continuous", [
+    (60, 1, 300, 1), (60, 6, 900, 1), (300, 31, 1500, 4),        # model in shared memory, one candidate per thread
+    (200, 9, 148 * 8 * 512 + 9, 1), (60, 5, 148 * 8 * 512 + 9, 2),   # two: tables in a loop of their own, and not
+    (3920, 7, 600, 1), (4000, 7, 600, 1), (4090, 7, 600, 1),     # about 48 KB of it
+    (2500, 10, 700, 2), (2500, 7, 148 * 4 * 512 + 5, 2),         # staged model
+])
+def test_tables_and_mixtures_in_one_model(n, d, m, continuous):
+    """Tabulated features are added up first, whatever their places among those with mixtures."""
+    rng = np.random.default_rng(1000 * d + n)
+    levels = np.array([(2, -5, 17, -64)[j % 4] for j in range(d)], np.int32)
+    levels[rng.permutation(d)[:continuous]] = 0
+    L = np.where(levels == 0, 1 << 22, np.abs(levels))
+    X = (np.floor(rng.uniform(0, 1, (n, d)) * L) / (L - 1)).astype(np.float32)
+    y = rng.normal(0, 1, n).astype(np.float32)
+    Xc = (np.floor(rng.uniform(0, 1, (m, d)) * L) / (L - 1)).astype(np.float32)
+    tpe = b.r3_tpe_fit(dev(X), dev(y), levels, 0.25, 1.0)
+    got = b.r3_tpe_score(tpe, dev(Xc)).cpu().numpy()
+    b.r3_tpe_check(tpe)
+    tpe.close()
+    rows = np.unique(np.concatenate([np.arange(min(m, 300)), rng.integers(0, m, 300), [m - 1]]))
+    check_score(got[rows], T.tpe_score(T.tpe_fit(X, y, levels, 0.25, 1.0), Xc[rows]), atol(n, levels))
