@@ -40,11 +40,11 @@ __device__ __forceinline__ CandidateResult finalize_candidate(double mu, double 
 //   d mu ~ 2 eps sqrt(sum_i (k*_i alpha_i)^2)
 //   d q  ~ 2 eps |W|_2 sqrt(q sum_i k*_i^2)        (from dq = 2 V.(W dk*), |V|^2 = q)
 // The flagging pass compares them with the accuracy contract once the pool's largest EI is known.
-// (Scales, so FP32 is enough; the roots are taken apart because a product of variances can leave its range.)
-__device__ __forceinline__ float mu_error_estimate(float eps, float a2) { return 2.f * eps * sqrtf(a2); }
-__device__ __forceinline__ float q_error_estimate(float eps, float wnorm, float q, float s2)
+// (In FP64: they decide what is recomputed, and sums of squared covariances leave FP32's range from a signal variance of 1e17 on.)
+__device__ __forceinline__ float mu_error_estimate(double eps, double a2) { return (float)(2.0 * eps * sqrt(a2)); }
+__device__ __forceinline__ float q_error_estimate(double eps, double wnorm, double q, double s2)
 {
-    return 2.f * eps * wnorm * (sqrtf(fmaxf(q, 0.f)) * sqrtf(s2));
+    return (float)(2.0 * eps * wnorm * sqrt(fmax(q, 0.0) * s2));
 }
 
 }  // namespace r3

@@ -86,7 +86,8 @@ constexpr uint32_t kFlagOffset = 512;    // behind the barriers: int abort, int 
 static_assert(BAR_COUNT * 8 <= kFlagOffset, "barriers overlap the flags");
 constexpr uint32_t kBarBytes = 1024;
 // Registers per thread once the roles have parted; the block starts with the file split evenly (80 for 768 threads).
-constexpr int kRegsControl = 48, kRegsIo = 80, kRegsMatern = 88;
+// The forms without FP8 cross terms spill nothing with this split (88 for the Matern warps and 80 for results: 20 bytes).
+constexpr int kRegsControl = 48, kRegsIo = 72, kRegsMatern = 96;
 static_assert(kRegsControl + IO * kRegsIo + G * kRegsMatern <= 80 * (kThreads / 128), "more registers than the block starts with");
 
 // per buffer of scaled candidates: float[128] squared norms, float[128] thresholds of close pairs, then the tile's scale of
@@ -108,8 +109,8 @@ __host__ __device__ inline SmemMap smem_map(int DP, int parts, int zb, int xs, i
     s.z32 = s.z + zb * s.z_buf;
     s.x = s.z32 + zb * s.z32_buf;
     s.w = s.x + xs * s.x_stage;                           // chunks of W: two planes [KC/8][rows][8]
-    s.red = s.w + ws * (4u * KC * kStrip);                // per group and row: mu (double), two error scales (float)
-    s.red_buf = (uint32_t)G * TILE_M * 16u;
+    s.red = s.w + ws * (4u * KC * kStrip);                // mu and two error scales of each group and row, doubles
+    s.red_buf = 3u * G * TILE_M * 8u;
     s.zn = s.red + zb * s.red_buf;            // see kZnBuf
     s.cache = s.zn + 2u * kZnBuf;                    // refined close pairs of the tile (see refine_close_pairs)
     s.bar = s.cache + (DP <= kZ32MaxDP ? 0u : TILE_M * kCacheSlots * 8u);
@@ -719,15 +720,13 @@ __global__ void __launch_bounds__(kThreads, 1) score_tc_kernel(const __grid_cons
             // rows by the warp that sees its last part arrive
             ok = mbar_wait_warp(bar(BAR_RED_FULL + b), (red_ph >> b) & 1u, abort_flag, wl);
             if (!ok) break;
-            double mu_acc = 0.0;
-            float a2_acc = 0.f, s2_acc = 0.f;
+            double mu_acc = 0.0, a2_acc = 0.0, s2_acc = 0.0;
 #pragma unroll
             for (int gg = 0; gg < G; ++gg) {
-                const uint8_t* o = sm + map.red + b * map.red_buf + (gg * TILE_M + row) * 16;
-                mu_acc += *reinterpret_cast<const double*>(o);
-                const float2 e2 = *reinterpret_cast<const float2*>(o + 8);
-                a2_acc += e2.x;
-                s2_acc += e2.y;
+                const double* o = reinterpret_cast<const double*>(sm + map.red + b * map.red_buf) + gg * (3 * TILE_M) + row;
+                mu_acc += o[0];
+                a2_acc += o[TILE_M];
+                s2_acc += o[2 * TILE_M];
             }
             __syncwarp();
             if (lane == 0) mbar_arrive(bar(BAR_RED_EMPTY + b));
@@ -736,10 +735,11 @@ __global__ void __launch_bounds__(kThreads, 1) score_tc_kernel(const __grid_cons
             bool finish = true;
             if (prm.splits > 1) {
                 const size_t slot = (size_t)(unit % tiles) * prm.splits;
-                double* mine = prm.partial + (slot + part) * (3 * TILE_M) + row;
+                double* mine = prm.partial + (slot + part) * (4 * TILE_M) + row;
                 __stcg(mine, mu_acc);
                 __stcg(mine + TILE_M, q_acc);
-                __stcg(reinterpret_cast<float2*>(mine + 2 * TILE_M), make_float2(a2_acc, s2_acc));
+                __stcg(mine + 2 * TILE_M, a2_acc);
+                __stcg(mine + 3 * TILE_M, s2_acc);
                 __threadfence();
                 __syncwarp();
                 int before = 0;   // parts of these 32 rows that are already there
@@ -747,16 +747,14 @@ __global__ void __launch_bounds__(kThreads, 1) score_tc_kernel(const __grid_cons
                 finish = __shfl_sync(0xffffffffu, before, 0) == prm.splits - 1;
                 if (finish) {
                     __threadfence();
-                    mu_acc = q_acc = 0.0;
-                    a2_acc = s2_acc = 0.f;
+                    mu_acc = q_acc = a2_acc = s2_acc = 0.0;
 #pragma unroll 1
                     for (int i = 0; i < prm.splits; ++i) {
-                        const double* o = prm.partial + (slot + i) * (3 * TILE_M) + row;
+                        const double* o = prm.partial + (slot + i) * (4 * TILE_M) + row;
                         mu_acc += __ldcg(o);
                         q_acc += __ldcg(o + TILE_M);
-                        const float2 e2 = __ldcg(reinterpret_cast<const float2*>(o + 2 * TILE_M));
-                        a2_acc += e2.x;
-                        s2_acc += e2.y;
+                        a2_acc += __ldcg(o + 2 * TILE_M);
+                        s2_acc += __ldcg(o + 3 * TILE_M);
                     }
                 }
             }
@@ -773,9 +771,9 @@ __global__ void __launch_bounds__(kThreads, 1) score_tc_kernel(const __grid_cons
                 __stcs(prm.sigma + f, res.sigma);
                 __stcs(prm.ei + f, res.ei);
                 if (res.ei == res.ei) ei_mine = res.ei;
-                const float eps = far_cand ? 1.f : (float)kEpsTc0 + (float)kEpsTc1 * prm.rsqrt_dp * (fabsf(zn_own) + prm.xnmax[g]);
+                const double eps = far_cand ? 1.0 : kEpsTc0 + kEpsTc1 * prm.rsqrt_dp * (double)(fabsf(zn_own) + prm.xnmax[g]);
                 prm.err_mu[f] = mu_error_estimate(eps, a2_acc);
-                prm.err_q[f] = q_error_estimate(F8 && !far_cand ? eps + (float)kEpsF8 : eps, (float)prm.wnorm[g], (float)q_acc, s2_acc);
+                prm.err_q[f] = q_error_estimate(F8 && !far_cand ? eps + kEpsF8 : eps, prm.wnorm[g], q_acc, s2_acc);
             }
             if (finish) {   // EI >= 0: the order of the bits is the order of the values
                 const unsigned top = __reduce_max_sync(0xffffffffu, __float_as_uint(ei_mine));
@@ -810,8 +808,7 @@ __global__ void __launch_bounds__(kThreads, 1) score_tc_kernel(const __grid_cons
             const float* xs_g = prm.xs32 + (size_t)g * prm.NP * DP;
             const float* xn_g = prm.xnorm + (size_t)g * prm.NP;
             const float* al_g = prm.alpha + (size_t)g * prm.NP;
-            double mu_acc = 0.0;
-            float a2_acc = 0.f, s2_acc = 0.f;    // scales of the error estimate
+            double mu_acc = 0.0, a2_acc = 0.0, s2_acc = 0.0;   // the last two: scales of the error estimate
             for (int p = prm.cut[part]; ok && p < prm.cut[part + 1]; ++p) {
                 const uint32_t chunks = (uint32_t)Pair(p, S, nc).chunks();
                 for (; ok && t - t_base < chunks; t += G) {
@@ -920,8 +917,8 @@ __global__ void __launch_bounds__(kThreads, 1) score_tc_kernel(const __grid_cons
                             unpack2(ap, a0, a1);
                             unpack2(sp, b0, b1);
                             mu_acc += (double)(m0 + m1);
-                            a2_acc += a0 + a1;
-                            s2_acc += b0 + b1;
+                            a2_acc += (double)(a0 + a1);
+                            s2_acc += (double)(b0 + b1);
                         }
                         // split into the FP16 planes and over the dot products they came from
                         uint32_t out[16];
@@ -970,9 +967,11 @@ __global__ void __launch_bounds__(kThreads, 1) score_tc_kernel(const __grid_cons
             if (lane == 0) mbar_arrive(bar(BAR_Z_EMPTY + zi));
             ok = mbar_wait_warp(bar(BAR_RED_EMPTY + zi), z_ph ^ 1u, abort_flag, wl);
             if (!ok) break;
-            uint8_t* o = sm + map.red + zi * map.red_buf + (R3_IDX(grp * TILE_M + row, G * TILE_M, prm.status)) * 16;
-            *reinterpret_cast<double*>(o) = mu_acc * (double)inv;
-            *reinterpret_cast<float2*>(o + 8) = make_float2(a2_acc * inv * inv, s2_acc * inv * inv);
+            double* o = reinterpret_cast<double*>(sm + map.red + zi * map.red_buf) + R3_IDX(grp * (3 * TILE_M) + row, G * 3 * TILE_M, prm.status);
+            const double inv64 = (double)inv, inv2 = inv64 * inv64;
+            o[0] = mu_acc * inv64;
+            o[TILE_M] = a2_acc * inv2;
+            o[2 * TILE_M] = s2_acc * inv2;
             __syncwarp();
             if (lane == 0) mbar_arrive(bar(BAR_RED_FULL + zi));
             if (++zi == zb) { zi = 0; z_ph ^= 1u; }
@@ -1373,7 +1372,7 @@ static size_t split_slots(const r3_gp* gp, long long m)
 static size_t split_bytes(const r3_gp* gp, long long m)
 {
     const size_t slots = split_slots(gp, m);
-    return slots ? slots * 3 * TILE_M * sizeof(double) + score_tc_tiles(gp, m) * sizeof(int4) + 256 : 0;
+    return slots ? slots * 4 * TILE_M * sizeof(double) + score_tc_tiles(gp, m) * sizeof(int4) + 256 : 0;
 }
 size_t score_tc_workspace_bytes(const r3_gp* gp, long long m) { return guard_workspace_bytes(gp, m) + max_bytes(gp, m) + split_bytes(gp, m); }
 
@@ -1445,7 +1444,7 @@ r3_status_t score_tc_part(r3_gp* gp, const float* Xcand, long long m, float* mu,
     prm.nc = t->NP / KC;
     prm.zb = t->zb;
     prm.xs = t->xs;
-    prm.rsqrt_dp = (float)(1.0 / sqrt((double)round_up(gp->d, 16)));
+    prm.rsqrt_dp = 1.0 / sqrt((double)round_up(gp->d, 16));
     prm.status = gp->status_d;
     prm.tiles_per_gp = (m + TILE_M - 1) / TILE_M;
     prm.total_tiles = prm.tiles_per_gp * gp->batch;
@@ -1472,7 +1471,7 @@ r3_status_t score_tc_part(r3_gp* gp, const float* Xcand, long long m, float* mu,
         uintptr_t at = (uintptr_t)ws + guard_workspace_bytes(gp, m) + max_bytes(gp, m);
         at = (at + 255) & ~(uintptr_t)255;
         prm.partial = reinterpret_cast<double*>(at);
-        prm.arrived = reinterpret_cast<int*>(prm.partial + slots * 3 * TILE_M);
+        prm.arrived = reinterpret_cast<int*>(prm.partial + slots * 4 * TILE_M);
     }
     prm.trace = nullptr;
     prof_begin(gp, stream);

@@ -52,10 +52,10 @@ struct TcParams {
     const double* wnorm;
     int DP, NP, P, ws;
     int parts, S, nc, zb, xs;   // nc: chunks of the whole history
-    float rsqrt_dp;             // 1 / sqrt of the feature count rounded up to 16 (error estimate)
+    double rsqrt_dp;            // 1 / sqrt of the feature count rounded up to 16 (error estimate)
     int splits;                 // units that a tile's pairs of strips are shared out to: part i takes [cut[i], cut[i + 1])
     unsigned char cut[kMaxSplits + 2];
-    double* partial;            // splits > 1: [tiles][splits][3][128] sums of a part, and
+    double* partial;            // splits > 1: [tiles][splits][4][128] sums of a part, and
     int* arrived;               // [tiles][4] how many parts of each 32 rows of a tile have been summed
     float* tile_max;            // [tiles of the pool][4] largest EI of each 32 rows, for the guard
     int* status;

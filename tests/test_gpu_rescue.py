@@ -99,3 +99,27 @@ def test_selection_behind_the_guard(m, k, kind):
     oidx, oval = o.topk(ei, k)
     assert np.array_equal(idx, oidx) and np.array_equal(val, oval.astype(np.float32))
     gp.close()
+
+
+@pytest.mark.parametrize("engine,exponent", [
+    (b.ENGINE_SIMT, 62), (b.ENGINE_TENSOR, 62),
+    (b.ENGINE_TENSOR, 70),   # squares of covariances beyond FP32, in which the other engine forms them
+])
+def test_large_signal_variances_are_not_taken_for_errors(engine, exponent):
+    """Responses in units that make them 2^31 or 2^35 times as large (variances of 5e18 and 1e21): every value scales by a
+    power of two, so the same candidates are flagged and the same results come out."""
+    g = rand_problem(31, 1, 600, 24, 3000, sn2=0.1, spread=1.5)
+    gp = fit_gpu(g, engine)
+    want = [t.clone() for t in b.r3_gp_score(gp, dev(g["Xcand"]))]
+    few = b.r3_gp_last_rescued(gp)
+    assert 2 * few < g["Xcand"].shape[1]   # most of the pool needs no recomputation
+    gp.close()
+    unit = np.float32(2.0) ** (exponent // 2)
+    g["y"], g["sf2"], g["sn2"] = g["y"] * unit, g["sf2"] * unit * unit, g["sn2"] * unit * unit
+    gp = fit_gpu(g, engine)
+    got = b.r3_gp_score(gp, dev(g["Xcand"]))
+    b.r3_gp_check(gp)
+    assert b.r3_gp_last_rescued(gp) == few
+    for a, c in zip(got, want):
+        assert torch.allclose(a / float(unit), c, rtol=1e-6, atol=1e-30)
+    gp.close()
