@@ -522,17 +522,24 @@ r3_status_t r3_gp_score_topk_host(r3_gp_t* gp, const float* Xcand_host, long lon
         ~ClearRequest() { gp->topk_req = TopkRequest(); }
     } clear_request{gp};
     // On the tensor engine a pool of several pieces travels on a second stream while the earlier pieces are
-    // scored (a piece is about seven full waves of tiles on 148 SMs, so that no launch ends on a nearly empty
-    // wave); the accuracy guard runs once over the whole pool, as in the device-buffer call, and the results are
-    // identical.  Everything else: one copy, then the scoring.
-    const long long tiles = pick_engine(gp) == R3_ENGINE_TENSOR ? score_tc_tiles(gp, m) : 0;
-    const long long tiles_per_gp = B ? tiles / (long long)B : 0;
-    // pieces are ranges of tiles that are contiguous in memory: any range for one GP, whole GPs for several
-    long long piece_tiles = 148 * 7;
-    if (B > 1) piece_tiles = std::max<long long>(1, (piece_tiles + tiles_per_gp / 2) / std::max<long long>(tiles_per_gp, 1)) * tiles_per_gp;
-    const bool split = pick_engine(gp) == R3_ENGINE_TENSOR && score_tc_can_split(gp) && tiles > piece_tiles;
-    if (split) {
-        const int pieces = (int)((tiles + piece_tiles - 1) / piece_tiles);
+    // scored; the accuracy guard runs once over the whole pool, as in the device-buffer call, and the results are
+    // identical.  Everything else: one copy, then the scoring.  A piece is seven full waves of tiles, the first with the
+    // tiles that are scored ahead of the others on top, so that only the last one ends on a wave that is not full (of
+    // several GPs: the nearest number of whole GPs, because a piece has to lie together in memory).
+    const bool can_split = pick_engine(gp) == R3_ENGINE_TENSOR && score_tc_can_split(gp);
+    const long long tiles_per_gp = (m + 127) / 128, tiles = tiles_per_gp * (long long)B;
+    int sms = 148;
+    R3_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, gp->device));
+    const long long first = can_split ? score_tc_first_tiles(gp, m) : 0;
+    auto piece_end = [&](int c, long long begin) {   // piece c, which begins at tile `begin`
+        long long end = first + 7ll * sms * (c + 1);
+        if (B > 1) end = std::max(begin + tiles_per_gp, (end + tiles_per_gp / 2) / tiles_per_gp * tiles_per_gp);
+        return std::min(tiles, end);
+    };
+    int pieces = 1;
+    if (can_split)
+        for (long long end = piece_end(0, 0); end < tiles; ++pieces) end = piece_end(pieces, end);
+    if (pieces > 1) {
         if (!gp->copy_stream) R3_CUDA_TRY(cudaStreamCreateWithFlags(&gp->copy_stream, cudaStreamNonBlocking));
         while ((int)gp->copy_events.size() < pieces + 1) {
             cudaEvent_t ev;
@@ -547,15 +554,17 @@ r3_status_t r3_gp_score_topk_host(r3_gp_t* gp, const float* Xcand_host, long lon
             if (B == 1) return std::min<long long>(m, tile * 128);
             return std::min<long long>(rows, tile / tiles_per_gp * m);
         };
-        for (int c = 0; c < pieces; ++c) {
-            const long long lo = first_row(c * piece_tiles), hi = first_row(std::min(tiles, (c + 1) * piece_tiles));
+        for (long long c = 0, begin = 0, end; c < pieces; ++c, begin = end) {
+            end = piece_end((int)c, begin);
+            const long long lo = first_row(begin), hi = first_row(end);
             R3_CUDA_TRY(cudaMemcpyAsync(xc + lo * gp->d, Xcand_host + lo * gp->d, sizeof(float) * (hi - lo) * gp->d,
                                         cudaMemcpyHostToDevice, gp->copy_stream));
             R3_CUDA_TRY(cudaEventRecord(gp->copy_events[c], gp->copy_stream));
         }
-        for (int c = 0; c < pieces; ++c) {
+        for (long long c = 0, begin = 0, end; c < pieces; ++c, begin = end) {
+            end = piece_end((int)c, begin);
             R3_CUDA_TRY(cudaStreamWaitEvent(stream, gp->copy_events[c], 0));
-            st = score_tc_part(gp, xc, m, mu, sg, e, gp->ws, sb, c * piece_tiles, (c + 1) * piece_tiles, false, stream);
+            st = score_tc_part(gp, xc, m, mu, sg, e, gp->ws, sb, begin, end, false, stream);
             if (st != R3_OK) return st;
         }
         st = score_tc_guard(gp, xc, m, mu, sg, e, gp->ws, stream);

@@ -292,6 +292,8 @@ r3_status_t score_tc(r3_gp* gp, const float* Xcand, long long m, float* mu, floa
 // the score_tc_tiles(gp, m) tiles of 128 candidates (tile_end < 0: all of them), the guard optionally left to
 // one score_tc_guard call after the last piece.
 long long score_tc_tiles(const r3_gp* gp, long long m);
+// tiles at the pool's beginning that are scored ahead of the others (0: none)
+long long score_tc_first_tiles(const r3_gp* gp, long long m);
 bool score_tc_can_split(const r3_gp* gp);
 r3_status_t score_tc_part(r3_gp* gp, const float* Xcand, long long m, float* mu, float* sigma, float* ei, void* ws,
                           size_t ws_bytes, long long tile_begin, long long tile_end, bool guard, cudaStream_t stream);

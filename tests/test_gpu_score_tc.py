@@ -48,3 +48,24 @@ def test_parts_of_a_tile_add_up_to_the_whole():
             ulp = torch.finfo(torch.float32).eps * c.abs().clamp_min(1e-30)
             assert ((a - c).abs() <= ulp).all()
     gp.close()
+
+
+@pytest.mark.parametrize("batch,n,d,m", [
+    (1, 1900, 20, (7 * 148 + 200) * 128 - 31),   # FP8 cross terms: the tiles that decide, and seven waves, then one
+    (1, 1900, 70, (7 * 148 + 10) * 128),         # less than what the first piece takes
+    (2, 1850, 12, (5 * 148 + 3) * 128 + 1),      # several GPs: whole ones
+    (1, 700, 20, 16 * 148 * 128 - 500),          # FP16 cross terms, three pieces
+])
+def test_pieces_of_a_host_pool_give_what_the_whole_gives(batch, n, d, m):
+    g = rand_problem(7900 + n + d, batch, n, d, m)
+    gp = fit_gpu(g, b.ENGINE_TENSOR)
+    k = 20
+    want = [t.cpu() for t in b.r3_gp_score_topk(gp, dev(g["Xcand"]), k)]
+    b.r3_gp_check(gp)
+    out = [torch.empty(batch, m).pin_memory() for _ in range(3)]
+    out += [torch.empty(batch, k, dtype=torch.int32).pin_memory(), torch.empty(batch, k).pin_memory()]
+    b.r3_gp_score_topk_host(gp, torch.from_numpy(g["Xcand"]).pin_memory(), k, tuple(out))
+    b.r3_gp_check(gp)
+    for a, c in zip(out, want):
+        assert torch.equal(a, c)
+    gp.close()
