@@ -55,6 +55,7 @@
 #include <string.h>
 
 #include "r3_epilogue.cuh"
+#include "r3_f32x2.cuh"
 #include "r3_internal.cuh"
 #include "r3_tc_common.cuh"
 
@@ -68,7 +69,7 @@ constexpr uint32_t kRingCol = 2 * kStrip;
 constexpr int kMaxWS = 8, kMaxXS = 3;    // stages of W (half for each accumulator) and of scaled observations
 constexpr int KDC = 2, KD = KDC * KC;    // chunks and observations per distance product, which fills a bank of slots
 constexpr int BANKS = kSlots / KDC;
-constexpr int IO = 2, G = 3;             // groups of four warps: candidates in and results out, Matern
+constexpr int IO = 2, G = 3;             // groups of four warps: candidates in and results out (one per buffer), Matern
 constexpr int kFirstIo = 4, kFirstMatern = kFirstIo + 4 * IO, kThreads = kFirstMatern * 32 + 128 * G;
 constexpr int kZ32MaxDP = 32;            // features up to which the scaled tile is kept in FP32 too
 constexpr int kPartDP = 64;              // features per stage of scaled observations at most
@@ -86,7 +87,9 @@ constexpr uint32_t kFlagOffset = 512;    // behind the barriers: int abort, int 
 static_assert(BAR_COUNT * 8 <= kFlagOffset, "barriers overlap the flags");
 constexpr uint32_t kBarBytes = 1024;
 // Registers per thread once the roles have parted; the block starts with the file split evenly (80 for 768 threads).
-// The forms without FP8 cross terms spill nothing with this split (88 for the Matern warps and 80 for results: 20 bytes).
+// The forms without FP8 cross terms spill nothing with this split (88 for the Matern warps and 80 for results: 20 bytes); those
+// with them spill six and eight registers, no fewer with any other split (64/72/88: four and ten) nor with the two halves of a
+// chunk's dot products read one after the other.
 constexpr int kRegsControl = 48, kRegsIo = 72, kRegsMatern = 96;
 static_assert(kRegsControl + IO * kRegsIo + G * kRegsMatern <= 80 * (kThreads / 128), "more registers than the block starts with");
 
@@ -118,32 +121,6 @@ __host__ __device__ inline SmemMap smem_map(int DP, int parts, int zb, int xs, i
     return s;
 }
 
-// two FP32 lanes in one 64-bit register pair
-__device__ __forceinline__ uint64_t pack2(float lo, float hi)
-{
-    uint64_t r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-    return r;
-}
-__device__ __forceinline__ void unpack2(uint64_t v, float& lo, float& hi) { asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v)); }
-__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b)
-{
-    uint64_t r;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b)
-{
-    uint64_t r;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c)
-{
-    uint64_t r;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-    return r;
-}
 // a - h exactly, in one mixed-precision instruction
 __device__ __forceinline__ float minus_half(float a, __half h)
 {
@@ -578,11 +555,11 @@ __global__ void __launch_bounds__(kThreads, 1) score_tc_kernel(const __grid_cons
         uint32_t z_ph = 0, v_ph = 0, red_ph = 0;     // parities per buffer b: bit b; v_ph: bit 2 b + accumulator
         uint32_t sigma = 0;                          // strips of all units so far
         float zn_in0 = 0.f, zn_in1 = 0.f;            // of the tiles in the buffers (the sign carries the out-of-range mark)
-        const int groups = IO == 2 && zb == 2 ? 2 : 1, own_step = unit_step * groups, ahead = unit_step * zb;
+        const int groups = zb, own_step = unit_step * groups, ahead = unit_step * zb;   // a group per buffer
         auto strips_of = [&](int unit) { return min(S, 2 * prm.cut[part_of(unit) + 1]) - 2 * prm.cut[part_of(unit)]; };
-        int b = groups == 2 ? io : 0;
+        const int b = io;
         if (io < groups)
-        for (int unit = (int)blockIdx.x + (groups == 2 ? io * unit_step : 0) - ahead; ok && unit < units; unit += own_step) {
+        for (int unit = (int)blockIdx.x + io * unit_step - ahead; ok && unit < units; unit += own_step) {
             const bool work = unit >= 0;
             const float zn_own = b ? zn_in1 : zn_in0;
             const int next = unit + ahead;
@@ -712,10 +689,7 @@ __global__ void __launch_bounds__(kThreads, 1) score_tc_kernel(const __grid_cons
                 if (lane == 0) mbar_arrive(bar(BAR_V_EMPTY + v_s));
             }
             if (!ok) break;
-            if (!work) {
-                if (groups == 1 && zb == 2) b ^= 1;
-                continue;
-            }
+            if (!work) continue;
             // ---- the groups' partial sums; a tile whose pairs went to several units is finished by the last of them, each 32
             // rows by the warp that sees its last part arrive
             ok = mbar_wait_warp(bar(BAR_RED_FULL + b), (red_ph >> b) & 1u, abort_flag, wl);
@@ -780,7 +754,6 @@ __global__ void __launch_bounds__(kThreads, 1) score_tc_kernel(const __grid_cons
                 if (lane == 0)
                     prm.tile_max[R3_IDX((long long)tile * 4 + (warp & 3), 4ll * tiles_per_gp * prm.batch, prm.status)] = __uint_as_float(top);
             }
-            if (groups == 1 && zb == 2) b ^= 1;
         }
         if (__any_sync(0xffffffffu, bad) && lane == 0) atomicOr(prm.status, DEV_NONFINITE);
     } else {
@@ -1476,7 +1449,6 @@ r3_status_t score_tc_part(r3_gp* gp, const float* Xcand, long long m, float* mu,
         prm.partial = reinterpret_cast<double*>(at);
         prm.arrived = reinterpret_cast<int*>(prm.partial + slots * 4 * TILE_M);
     }
-    prm.trace = nullptr;
     prof_begin(gp, stream);
     if (t->pair) {
         const r3_status_t st = launch_tc_pair(t, prm, sms, stream);

@@ -31,18 +31,6 @@ namespace r3 {
 
 namespace {
 
-#ifndef R3_TC_TRACE
-#define LOGEV2(ev, tt) do { } while (0)
-#else
-// event log of the first cluster: clock of event `ev` (0..7) of CTA `rank` for stream chunk tt in the window
-constexpr long long kLog2T0 = 576 + 300;
-#define LOGEV2(ev, tt)                                                                                        \
-    do {                                                                                                      \
-        if (prm.trace && blockIdx.x < 2 && (tt) >= kLog2T0 && (tt) < kLog2T0 + kLogN)                         \
-            prm.trace[(size_t)gridDim.x * 32 + (blockIdx.x * 12 + (ev)) * kLogN + ((tt) - kLog2T0)] = clock64(); \
-    } while (0)
-#endif
-
 constexpr int NV2 = 256;      // rows of W per pass
 constexpr int KD2 = 64;       // observations per distance product
 constexpr int SL2 = KD2 / KC; // chunks per distance product == Matern groups per CTA
@@ -215,8 +203,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(128 + 128 * G2, 1) s
     const uint32_t tmem = *tmem_slot;
 
     const long long first_tile = blockIdx.x >> 1, tile_step = gridDim.x >> 1;
-    long long tacc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-    long long tlast = prm.trace ? clock64() : 0;
 
     if (warp == 0 && lane == 0) {
         // ------------------------------------------------------------ producer: scaled observations (own products)
@@ -334,24 +320,17 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(128 + 128 * G2, 1) s
                 const int nchunk = superpass_chunks(j, P);
                 for (int c = 0; ok && c < nchunk; ++c, ++tv) {
                     const int b = k_s;
-                    TICK(7);
                     if (c < mine) {
                         const int s = w_s;
                         if (c == 0) {
                             if (!(ok = mbar_wait(bar(PB_V_EMPTY), v_ph ^ 1u, abort_flag, wl))) break;
                         }
-                        TICK(3);
                         if (!(ok = mbar_wait(bar(PB_K_FULL + b), k_ph, abort_flag, wl))) break;
-                        TICK(4);
-                        LOGEV2(0, tv);
                         if (!(ok = mbar_wait(bar(PB_W_FULL + s), w_ph, abort_flag, wl))) break;
-                        TICK(5);
-                        LOGEV2(1, tv);
                         if (++w_s == ws) { w_s = 0; w_ph ^= 1u; }
                         // (the writers of a k* buffer fence their stores towards the async proxy before they arrive,
                         // and the peer's copy arrives through the async proxy: no proxy fence on this side)
                         tc_fence_after();
-                        LOGEV2(7, tv);
                         // In the pass's diagonal block the rows of W above the chunk's columns are zero (W is lower
                         // triangular): the MMAs start at the first row that can be non-zero and get narrower.
                         const uint32_t skip = c > p * CPP2 ? (uint32_t)(c - p * CPP2) * KC : 0u;
@@ -368,23 +347,17 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(128 + 128 * G2, 1) s
                                            pack64(b0 + jj * ((2u * NV2 * 16u) >> 4), kDescHi), idesc_v,
                                            (c > 0 || combo > 0 || jj > 0) ? 1u : 0u);
                         }
-                        LOGEV2(8, tv);
                         tc_commit(bar(PB_W_EMPTY + s));
-                        LOGEV2(9, tv);
                         tc_commit_pair(bar(PB_K_EMPTY + b));
-                        LOGEV2(10, tv);
                         if (c == mine - 1) {
                             tc_commit(bar(PB_V_FULL));
                             v_ph ^= 1u;
                         }
-                        TICK(6);
-                        LOGEV2(2, tv);
                     } else {
                         // my pass does not use this chunk: release the buffer on both CTAs once it has been filled
                         if (!(ok = mbar_wait(bar(PB_K_FULL + b), k_ph, abort_flag, wl))) break;
                         mbar_arrive(bar(PB_K_EMPTY + b));
                         mbar_arrive_cluster(k_empty_peer0 + (uint32_t)b * 8u);
-                        TICK(0);
                     }
                     if (++k_s == NB) { k_s = 0; k_ph ^= 1u; }
                 }
@@ -392,20 +365,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(128 + 128 * G2, 1) s
         }
         tc_commit(bar(PB_MMA_DONE + 1));
         mbar_wait(bar(PB_MMA_DONE + 1), 0, abort_flag + 1, wl);
-        if (prm.trace)
-            for (int i = 0; i < 8; ++i) prm.trace[((size_t)blockIdx.x * 4 + 0) * 8 + i] = tacc[i];
-#ifdef R3_TC_TRACE
-    } else if (warp == 3 && lane == 0) {
-        // observer (trace builds only): when each k* buffer became full in this CTA
-        long long tv = 0;
-        bool ok = true;
-        for (long long tile = first_tile; ok && tile < prm.total_tiles; tile += tile_step)
-            for (int j = 0; ok && j < NSP; ++j)
-                for (int c = 0; ok && c < superpass_chunks(j, P); ++c, ++tv) {
-                    ok = mbar_wait(bar(PB_K_FULL + (int)(tv % NB)), (uint32_t)((tv / NB) & 1), abort_flag, wl);
-                    LOGEV2(11, tv);
-                }
-#endif
     } else if (warp >= 4) {
         // ------------------------------------------------------------ Matern / epilogue warp groups
         const int grp = (warp - 4) >> 2;         // 0..G2-1: which chunk of each own product
@@ -507,11 +466,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(128 + 128 * G2, 1) s
             // group of the pair), so that the variance MMAs find k* waiting when the accumulator is free again.
             bool epilogue_due = false;
             auto pass_epilogue = [&]() {
-                TICK(7);
                 ok = mbar_wait(bar(PB_V_FULL), v_ph, abort_flag, wl);
                 ok = __all_sync(0xffffffffu, ok);
                 if (!ok) return;
-                TICK(5);
                 tc_fence_after();
 #pragma unroll 1
                 for (int c0 = grp * 16; c0 < NV2; c0 += 32 * G2) {   // two column blocks per round trip to TMEM
@@ -532,7 +489,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(128 + 128 * G2, 1) s
                 tc_fence_before();
                 mbar_arrive(bar(PB_V_EMPTY));
                 v_ph ^= 1u;
-                TICK(6);
             };
             for (int j = 0; ok && j < NSP; ++j) {
                 const int nchunk = superpass_chunks(j, P);
@@ -544,12 +500,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(128 + 128 * G2, 1) s
                     const int b = (int)(t % NB);
                     const uint32_t k_par = (uint32_t)((t / NB) & 1);
                     const int db = (int)(own & 1);
-                    TICK(7);
                     ok = mbar_wait(bar(PB_D_FULL + db), (uint32_t)((own >> 1) & 1), abort_flag, wl);
                     ok = __all_sync(0xffffffffu, ok);
                     if (!ok) break;
-                    TICK(0);
-                    if (q4 == 0 && lane == 0) LOGEV2(3, t);
                     ++own;
                     tc_fence_after();
                     const bool fresh = c >= 2 * j * CPP2;   // first super-pass that generates this chunk
@@ -562,7 +515,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(128 + 128 * G2, 1) s
                     tc_wait_ld32(dots[0], dots[1]);
                     tc_fence_before();
                     mbar_arrive(bar(PB_D_EMPTY + db));
-                    TICK(1);
 #pragma unroll
                     for (int h = 0; h < KC / 16; ++h) {
                         const float* dot = dots[h];
@@ -616,13 +568,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(128 + 128 * G2, 1) s
                         }
                     }
                     // both CTAs must have finished with the previous chunk in this ring position
-                    TICK(2);
-                    if (q4 == 0 && lane == 0) LOGEV2(4, t);
                     ok = mbar_wait_cluster(bar(PB_K_EMPTY + b), k_par ^ 1u, abort_flag, wl);
                     ok = __all_sync(0xffffffffu, ok);
                     if (!ok) break;
-                    TICK(3);
-                    if (q4 == 0 && lane == 0) LOGEV2(5, t);
                     // the peer's barrier learns of the 16 KB to come now: the remote arrive takes hundreds of cycles,
                     // which pass while this group stores the chunk
                     if (q4 == 1 && lane == 0) mbar_arrive_expect_tx_cluster(k_full_peer0 + (uint32_t)b * 8u, 16384u);
@@ -639,19 +587,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(128 + 128 * G2, 1) s
                     if (!ok) break;
                     // The chunk is complete in this CTA's buffer: publish it here, and send a copy to the
                     // same ring position of the peer with one bulk copy that completes the peer's barrier.
-                    if (q4 == 0 && lane == 0) LOGEV2(7, t);
                     fence_proxy_async();
-                    if (q4 == 0 && lane == 0) LOGEV2(8, t);
                     asm volatile("bar.sync %0, 128;" ::"r"(1 + grp) : "memory");
                     if (q4 == 0 && lane == 0) {
-                        LOGEV2(9, t);
                         mbar_arrive(bar(PB_K_FULL + b));
                         const uint32_t peer_bar = k_full_peer0 + (uint32_t)b * 8u;
-                        LOGEV2(10, t);
                         bulk_s2peer(kbuf_peer0 + b * 16384u, base + map.k + b * 16384u, 16384u, peer_bar);
-                        LOGEV2(6, t);
                     }
-                    TICK(4);
                     if (epilogue_due) {   // the previous super-pass's accumulator, now that the next k* is on its way
                         epilogue_due = false;
                         pass_epilogue();
@@ -707,8 +649,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(128 + 128 * G2, 1) s
             }
         }
         if (__any_sync(0xffffffffu, bad) && lane == 0) atomicOr(prm.status, DEV_NONFINITE);
-        if (prm.trace && q4 == 0 && lane == 0)
-            for (int i = 0; i < 8; ++i) prm.trace[((size_t)blockIdx.x * 4 + 1 + grp) * 8 + i] = tacc[i];
     }
 
     // ---------------------------------------------------------------- teardown

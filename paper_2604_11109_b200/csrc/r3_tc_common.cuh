@@ -25,8 +25,8 @@ struct TensorOperands {
     float* scale = nullptr;    // [B][DP]  1/lengthscale (zero padded)
     __half* xt = nullptr;      // [B][NP/KD][parts][2][DP/parts/8][KD][8]  scaled observations, FP16 hi/lo planes
     float* xs32 = nullptr;     // [B][NP][DP]  scaled observations in FP32 (refinement of close pairs)
-    float* xnorm = nullptr;    // [B][NP/KD][2][KD]  |x~_k|^2, then weights (zero padded); pair: [B][NP] |x~_k|^2
-    float* alpha = nullptr;    // the weights inside xnorm; pair: [B][NP] behind it
+    float* xnorm = nullptr;    // [B][NP]  |x~_k|^2
+    float* alpha = nullptr;    // [B][NP]  weights, zero padded
     float* xnmax = nullptr;    // [B]      max_k |x~_k|^2
     __half* wt = nullptr;      // [B][strip s][chunk c <= 4 s + 3][2][KC/8][R][8]  chunks of 2^eW W (R rows of the strip), FP16
                                // hi/lo planes; with f8 the second plane is two 8-bit planes [2][KC/16][R][16]: hi parts
@@ -65,7 +65,6 @@ struct TcParams {
     int want_mode;
     long long tiles_per_gp, total_tiles;   // total_tiles: one past the last tile of this launch
     long long tile_begin;                  // first tile of this launch (the single-CTA kernel; 0 for a whole pool)
-    long long* trace;   // optional [grid][4 roles][8] cycle counters (diagnostics)
     long long wait_limit;   // cycles after which a device-side wait gives up (r3_gp_set_wait_limit)
     long long withhold_w;   // >= 0: every CTA's stream of W stops before that chunk of its own sequence, so that the
                             // consumer's wait runs out (r3_gp_test_withhold, one call); -1 otherwise
@@ -79,8 +78,7 @@ namespace {
 
 constexpr int KC = 32;        // observations per chunk of the variance product
 constexpr int TILE_M = 128;   // candidates per CTA tile
-constexpr int XS = 2;         // stages of scaled observations
-constexpr int MAX_STAGES = 6; // stages of W
+constexpr int XS = 2;         // stages of scaled observations (paired kernel)
 
 // Scaled coordinates are x^ = (x - centre) * sqrt(5) log2(e) / lengthscale, so that u = |z^ - x^| is the
 // Matern argument in base-2 units: s = sqrt(5) r = u ln 2, exp(-s) = 2^-u, 1 + s + s^2/3 = 1 + c1 u + c2 u^2.
@@ -180,49 +178,13 @@ __device__ __forceinline__ void tc_mma_f16_ts(uint32_t d_tmem, uint32_t a_tmem, 
         ::"r"(d_tmem), "r"(a_tmem), "l"(bdesc), "r"(idesc), "r"(accumulate)
         : "memory");
 }
-// kind::f8f6f4, K = 32; the instruction descriptor is the FP16 one plus the operands' format codes
-// (instr_desc_f8)
-__device__ __forceinline__ void tc_mma_f8(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
-                                          uint32_t accumulate)
-{
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], %1, %2, %3, p;\n\t}"
-        ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
-        : "memory");
-}
-// A operand from TMEM (lane = row, one 32-bit column = four consecutive 8-bit k-elements)
-__device__ __forceinline__ void tc_mma_f8_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t bdesc, uint32_t idesc,
-                                             uint32_t accumulate)
-{
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], [%1], %2, %3, p;\n\t}"
-        ::"r"(d_tmem), "r"(a_tmem), "l"(bdesc), "r"(idesc), "r"(accumulate)
-        : "memory");
-}
 __device__ __forceinline__ void tc_st8(uint32_t taddr, const uint32_t* r)
 {
     asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"r"(taddr), "r"(r[0]),
                  "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7])
                  : "memory");
 }
-__device__ __forceinline__ void tc_ld16(uint32_t taddr, float* v)
-{
-    uint32_t r[16];
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-          "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-        : "r"(taddr)
-        : "memory");
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-    for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
-}
-// The same load without the wait: several can be in flight; tc_wait_ld32 ends them.
+// Sixteen columns, without a wait: several loads can be in flight; tc_wait_ld16 or tc_wait_ld32 ends them.
 __device__ __forceinline__ void tc_ld16_issue(uint32_t taddr, float* v)
 {
     asm volatile(
@@ -435,32 +397,6 @@ __device__ __noinline__ void refine_close_pairs(float* kv, float v_thresh, float
         if (CACHE) slots[cache_slot(key0 + i)] = ((unsigned long long)(key0 + i) << 32) | __float_as_uint(kv[i]);
     }
 }
-
-// Per-role cycle accounting, compiled in only with -DR3_TC_TRACE (it costs issue slots on the hot path).
-#ifndef R3_TC_TRACE
-#define TICK(cat) do { } while (0)
-#define LOGEV(ev, tt) do { } while (0)
-#else
-// event log of the first CTA: clock of event `ev` for global chunk number tt in [kLogT0, kLogT0 + kLogN)
-constexpr long long kLogT0 = 1088 + 600, kLogN = 128;
-#define LOGEV(ev, tt)                                                                                         \
-    do {                                                                                                      \
-        if (prm.trace && blockIdx.x == 0 && (tt) >= kLogT0 && (tt) < kLogT0 + kLogN)                          \
-            prm.trace[(size_t)gridDim.x * 32 + (ev) * kLogN + ((tt) - kLogT0)] = clock64();                   \
-    } while (0)
-#ifdef R3_TC_TRACE_EVENTS_ONLY
-#define TICK(cat) do { } while (0)
-#else
-#define TICK(cat)                                                                          \
-    do {                                                                                   \
-        if (prm.trace) {                                                                   \
-            const long long now__ = clock64();                                             \
-            tacc[cat] += now__ - tlast;                                                    \
-            tlast = now__;                                                                 \
-        }                                                                                  \
-    } while (0)
-#endif
-#endif
 
 }  // namespace
 
