@@ -58,9 +58,10 @@ constexpr uint32_t kPairBarBytes = 1024;
 enum : uint32_t {
     PB_X_FULL = 0, PB_X_EMPTY = 2, PB_W_FULL = 4, PB_W_EMPTY = 10, PB_D_FULL = 16, PB_D_EMPTY = 18,
     PB_K_FULL = 20, PB_K_EMPTY = 24, PB_V_FULL = 28, PB_V_EMPTY = 29, PB_Z_READY = 30, PB_RED_READY = 31,
-    PB_RED_PEER = 32, PB_MMA_DONE = 33, PB_COUNT = 35
+    PB_RED_PEER = 32, PB_MMA_DONE = 33, PB_STAGED = 35, PB_COUNT = 37   // STAGED: one per Matern group
 };
-constexpr uint32_t kPairFlagOffset = PB_COUNT * 8;
+constexpr uint32_t kPairFlagOffset = PB_COUNT * 8;   // int abort, int drain-abort, uint32 tmem base, -, int64 last chunk from the peer [G2]
+static_assert(kPairFlagOffset % 8 == 0 && kPairFlagOffset + 16 + G2 * 8 <= 512, "flags overlap the norms");
 constexpr uint32_t kPairZnOffset = 512;
 
 // ---- cluster-scope PTX
@@ -123,6 +124,10 @@ __device__ __forceinline__ void st_cluster_f64(uint32_t cluster_addr, double v)
 {
     asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(cluster_addr), "d"(v) : "memory");
 }
+__device__ __forceinline__ void st_cluster_s64(uint32_t cluster_addr, long long v)
+{
+    asm volatile("st.shared::cluster.s64 [%0], %1;" ::"r"(cluster_addr), "l"(v) : "memory");
+}
 // arrive on the same barrier of both CTAs of the pair once the MMAs issued so far have completed
 __device__ __forceinline__ void tc_commit_pair(uint32_t bar)
 {
@@ -182,6 +187,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(128 + 128 * G2, 1) s
         mbar_init(bar(PB_RED_PEER), 128);
         mbar_init(bar(PB_MMA_DONE), 1);
         mbar_init(bar(PB_MMA_DONE + 1), 1);
+        for (int i = 0; i < G2; ++i) mbar_init(bar(PB_STAGED + i), 4);
         abort_flag[0] = 0;
         abort_flag[1] = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -376,6 +382,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(128 + 128 * G2, 1) s
         long long Ug = 0;                        // global product counter (same sequence in both CTAs)
         long long tg = 0;                        // global chunk counter at the start of the current super-pass
         long long own = 0;                       // own products so far (distance-buffer ring)
+        long long staged = 0, sent = -1;         // own chunks written so far, and the last one on its way to the peer
         uint32_t v_ph = 0;
         long long tile_iter = 0;
         bool ok = true, bad = false;
@@ -587,13 +594,22 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(128 + 128 * G2, 1) s
                     if (!ok) break;
                     // The chunk is complete in this CTA's buffer: publish it here, and send a copy to the
                     // same ring position of the peer with one bulk copy that completes the peer's barrier.
+                    // Whether a wait ran out is decided warp by warp, so the group's warps meet at a bounded wait.
                     fence_proxy_async();
-                    asm volatile("bar.sync %0, 128;" ::"r"(1 + grp) : "memory");
-                    if (q4 == 0 && lane == 0) {
-                        mbar_arrive(bar(PB_K_FULL + b));
-                        const uint32_t peer_bar = k_full_peer0 + (uint32_t)b * 8u;
-                        bulk_s2peer(kbuf_peer0 + b * 16384u, base + map.k + b * 16384u, 16384u, peer_bar);
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(bar(PB_STAGED + grp));
+                    if (q4 == 0) {
+                        ok = mbar_wait(bar(PB_STAGED + grp), (uint32_t)(staged & 1), abort_flag, wl);
+                        ok = __all_sync(0xffffffffu, ok);
+                        if (!ok) break;
+                        if (lane == 0) {
+                            mbar_arrive(bar(PB_K_FULL + b));
+                            const uint32_t peer_bar = k_full_peer0 + (uint32_t)b * 8u;
+                            bulk_s2peer(kbuf_peer0 + b * 16384u, base + map.k + b * 16384u, 16384u, peer_bar);
+                            sent = t;
+                        }
                     }
+                    ++staged;
                     if (epilogue_due) {   // the previous super-pass's accumulator, now that the next k* is on its way
                         epilogue_due = false;
                         pass_epilogue();
@@ -649,6 +665,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(128 + 128 * G2, 1) s
             }
         }
         if (__any_sync(0xffffffffu, bad) && lane == 0) atomicOr(prm.status, DEV_NONFINITE);
+        if (q4 == 0 && lane == 0) st_cluster_s64(map_to_cta(base + map.bar + kPairFlagOffset + 16 + grp * 8, peer), sent);
     }
 
     // ---------------------------------------------------------------- teardown
@@ -656,7 +673,16 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(128 + 128 * G2, 1) s
     tc_fence_before();
     __syncthreads();
     if (threadIdx.x == 0 && *abort_flag) atomicOr(prm.status, DEV_TIMEOUT);
-    cluster_sync_all();   // the peer may still be writing into this CTA's shared memory until it gets here
+    cluster_sync_all();   // the peer issues nothing more into this CTA's shared memory once it gets here
+    // A group's next chunk goes into the same ring position, after both CTAs are through with the one before: after an abort at
+    // most its last copy is still on its way.  Neither CTA leaves before those have landed.
+    if (threadIdx.x < G2) {
+        const long long last = *reinterpret_cast<volatile long long*>(sm + map.bar + kPairFlagOffset + 16 + threadIdx.x * 8);
+        if (last >= 0) mbar_wait_cluster(bar(PB_K_FULL + (int)(last % NB)), (uint32_t)((last / NB) & 1), abort_flag + 1, wl);
+    }
+    __syncwarp();
+    __syncthreads();
+    cluster_sync_all();
     if (warp == 2) {
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TMEM_COLS) : "memory");

@@ -60,15 +60,18 @@ def test_a_wait_that_runs_out_is_reported_and_the_handle_stays_usable(monkeypatc
     gp.close()
 
 
-@pytest.mark.parametrize("n,d,m", [
-    (1500, 20, 148 * 128 * 4 + 3),   # two buffers of candidates
-    (1000, 128, 148 * 128 * 3),      # one buffer, features in two stages
-    (2500, 40, 148 * 128 * 2 + 9),   # FP8 cross terms
-    (900, 24, 300),                  # pairs of strips shared out
+@pytest.mark.parametrize("n,d,m,pair", [
+    (1500, 20, 148 * 128 * 4 + 3, False),   # two buffers of candidates
+    (1000, 128, 148 * 128 * 3, False),      # one buffer, features in two stages
+    (2500, 40, 148 * 128 * 2 + 9, False),   # FP8 cross terms
+    (900, 24, 300, False),                  # pairs of strips shared out
+    (1200, 20, 148 * 64 * 4 + 3, True),     # clusters of two thread blocks, which send each other chunks
 ])
-def test_a_limit_that_runs_out_while_the_pipeline_is_at_work(n, d, m):
+def test_a_limit_that_runs_out_while_the_pipeline_is_at_work(monkeypatch, n, d, m, pair):
     """The shortest limit there is, less than a tile takes: waits run out in thread blocks whose other warps are still
     handing stages over.  The call returns by itself, with or without a time-out, and the handle keeps working."""
+    if pair:
+        monkeypatch.setenv("R3_TC_PAIR", "1")
     g = rand_problem(4100 + n, 1, n, d, m)
     gp = fit_gpu(g, b.ENGINE_TENSOR)
     xc = dev(g["Xcand"])
