@@ -2,6 +2,7 @@
 observations, features padded to 16 and split over stages of 64, one or two buffers of scaled candidates, and tiles whose pairs
 of strips are shared out to several thread blocks.  Every element against the FP64 oracle (tolerances of ``tests/parity.py``).
 """
+import numpy as np
 import pytest
 
 from paper_2604_11109_b200 import binding as b
@@ -37,16 +38,20 @@ def test_edges_of_strips_chunks_stages_and_parts(batch, n, d, m):
 
 def test_parts_of_a_tile_add_up_to_the_whole():
     """A pool of one tile, whose pairs of strips go to several thread blocks, and the same rows among enough others that every
-    tile stays with one block: FP64 sums of the same FP32 parts in another order, so at most a last bit apart."""
-    g = rand_problem(91, 1, 900, 24, 148 * 128 * 16)
+    tile stays with one block: FP64 sums of the same FP32 parts in another order, so at most a last bit apart.  A smooth, noisy
+    response, of which nothing is recomputed: what the FP64 pass has rewritten would not show the engine's sums."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    g = rand_problem(91, 1, 900, 24, sms * 128 * 16, sn2=0.1)
+    g["Xcand"] = np.clip(g["Xcand"], 0, 1)
+    g["y"] = (0.2 * g["y"] + 2 * np.sin(3 * g["X"].sum(2) / np.sqrt(24))).astype(np.float32)
     gp = fit_gpu(g, b.ENGINE_TENSOR)
     whole = [t[0, :100].clone() for t in b.r3_gp_score(gp, dev(g["Xcand"]))]
-    rescued_whole = b.r3_gp_last_rescued(gp)
+    assert b.r3_gp_last_rescued(gp) == 0
     part = [t[0] for t in b.r3_gp_score(gp, dev(g["Xcand"][:, :100]))]
-    if rescued_whole == 0 and b.r3_gp_last_rescued(gp) == 0:   # what the FP64 pass has rewritten does not show the engine's sums
-        for a, c in zip(part[:2], whole[:2]):
-            ulp = torch.finfo(torch.float32).eps * c.abs().clamp_min(1e-30)
-            assert ((a - c).abs() <= ulp).all()
+    assert b.r3_gp_last_rescued(gp) == 0
+    for a, c in zip(part[:2], whole[:2]):
+        ulp = torch.finfo(torch.float32).eps * c.abs().clamp_min(1e-30)
+        assert ((a - c).abs() <= ulp).all()
     gp.close()
 
 
