@@ -557,8 +557,8 @@ def main():
         # at the FP16/BF16 tensor rate -- the count stays the same when the two cross terms run as FP8 MMAs at
         # twice the rate (then the tensor time actually issued is that of two FP16 MMAs: `issued_f16_equivalent`).
         # The distance products and the diagonal blocks' zero halves are not in the count; `issued_total_tflops`
-        # is everything the pipe was given, in FP16-rate equivalents: per chunk of 32 observations of a tile,
-        # 128 x NV x 32 MACs of the variance product three (two with FP8 cross terms) times over, and
+        # is everything the pipe was given, in FP16-rate equivalents: 128 x 32 MACs of the variance product per row of W
+        # that a chunk of 32 observations is multiplied with, three (two with FP8 cross terms) times over, and
         # 128 x 32 x DP MACs of the distance product three times, for every (re)generation of the chunk.
         info = b.r3_gp_tensor_info(gp)
         f8 = bool(info["f8_cross_terms"])
@@ -567,11 +567,16 @@ def main():
         issued = 3.0 * alg_flops
         achieved = issued * cands_per_launch / (per_launch_ms * 1e-3) / 1e12
         peak = peaks["bf16_tflops"]
-        NV, P, DP = info["NV"], info["P"], info["DP"]
-        chunks_per_tile = (NV // 32) * P * (P + 1) // 2
+        P, DP, chunks = info["P"], info["DP"], info["NP"] // 32
+        chunks_per_tile = sum(min(8 * (p + 1), chunks) for p in range(P))   # once for each pair of strips of 128 rows of W
+        w_chunk_rows = issued_rows = 0                                      # stored, and without the zeros above the diagonal
+        for s in range((chunks + 3) // 4):
+            rows, diagonal = min(128, info["NP"] - 128 * s), min(4, chunks - 4 * s)
+            w_chunk_rows += (4 * s + diagonal) * rows
+            issued_rows += 4 * s * rows + sum(rows - 32 * c for c in range(diagonal))
         tiles_per_launch = B * ((m + 127) // 128) * args.steps / max(kernel_launches, 1)
-        per_chunk = (2.0 if f8 else 3.0) * 2 * 128 * NV * 32 + 3.0 * 2 * 128 * 32 * DP
-        issued_total = per_chunk * chunks_per_tile * tiles_per_launch / (per_launch_ms * 1e-3) / 1e12
+        per_tile = 2.0 * 128 * 32 * ((2.0 if f8 else 3.0) * issued_rows + 3.0 * DP * chunks_per_tile)
+        issued_total = per_tile * tiles_per_launch / (per_launch_ms * 1e-3) / 1e12
         roofline = {"bound": "tensor", "kernel": "score_tc_kernel", "achieved": achieved, "peak": peak,
                     "unit": "TFLOP/s", "frac": achieved / peak, "traffic": None,
                     "note": "3 n^2 flops per candidate: the three FP16-rate MMAs per product that a 22-bit variance "
@@ -581,12 +586,12 @@ def main():
                     "issued_total_tflops": issued_total,
                     "frac_of_sustained_peak": achieved / peaks["bf16_tflops_sustained"],
                     "shape": info}
-        # DRAM bytes per launch, modelled: the pre-tiled operands are read once per launch (their sizes follow
-        # from the shape: chunks of W as 2 x 32 x NV x 2 bytes each, observation planes, FP32 observations), and
-        # an ncu capture of this kernel on 32,768 candidates of the largest workload measured 244 B read and
-        # 18.6 B written per candidate beside them (algorithmic: 4 d read, 20 written).
-        operands = B * ((NV // 32) * P * (P + 1) // 2 * 2 * 32 * NV * 2 + info["NP"] * DP * (4 + 4) + info["NP"] * 8)
-        roofline["traffic"] = float(operands + (4 * d * 244.0 / 256.0 + 18.6) * cands_per_launch)
+        # DRAM bytes per launch, modelled: the pre-tiled operands are read once (chunks of W as 128 B per row and chunk,
+        # observation planes, FP32 observations, norms and weights), 4 d bytes read and 20 written per candidate.  An ncu
+        # capture of 108 and of 148 tiles of the largest workload read 40.2 and 41.4 MB (model: 40.3 and 41.6); their
+        # results were still in L2.
+        operands = B * (w_chunk_rows * 32 * 4 + info["NP"] * DP * (4 + 4) + info["NP"] * 8)
+        roofline["traffic"] = float(operands + (4 * d + 20) * cands_per_launch)
         roofline["traffic_kind"] = "modelled from operand sizes and a small-case ncu capture"
     else:
         alg_flops = float(npad) * npad
