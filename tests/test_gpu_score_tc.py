@@ -25,6 +25,8 @@ pytestmark = pytest.mark.gpu
     (1, 641, 128, 300),       # an odd number of strips; one buffer of candidates
     (1, 1025, 21, 100),       # five pairs shared out
     (1, 1793, 40, 131),       # FP8 cross terms, eight pairs shared out
+    (1, 300, 3, 200), (1, 300, 8, 200), (1, 300, 12, 200),   # one, two and four groups of four features in close pairs
+    (1, 1800, 7, 140),                # the same with FP8 cross terms
     (1, 40, 5, 148 * 128 * 2 + 77),   # more tiles than thread blocks, ragged tail
     (1, 300, 12, 148 * 128 + 1),      # the same with two pairs
 ])
