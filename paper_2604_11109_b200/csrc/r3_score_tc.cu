@@ -88,7 +88,7 @@ static_assert(BAR_COUNT * 8 <= kFlagOffset, "barriers overlap the flags");
 constexpr uint32_t kBarBytes = 1024;
 // Registers per thread once the roles have parted; the block starts with the file split evenly (80 for 768 threads).
 // The forms without FP8 cross terms spill nothing with this split (88 for the Matern warps and 80 for results: 20 bytes); those
-// with them spill six and eight registers, no fewer with any other split (64/72/88: ten and four) nor with the two halves of a
+// with them spill five to eight registers, no fewer with any other split (64/72/88: ten and four) nor with the two halves of a
 // chunk's dot products read one after the other.
 constexpr int kRegsControl = 48, kRegsIo = 72, kRegsMatern = 96;
 static_assert(kRegsControl + IO * kRegsIo + G * kRegsMatern <= 80 * (kThreads / 128), "more registers than the block starts with");
